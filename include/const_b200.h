@@ -195,6 +195,9 @@ const_status_t const_csf_work_lists(const const_csf_t *csf, const int32_t **slic
  *   network T[i,k,l] = U[i,j,k] * V[j,l]; Z[i,m] = T[i,k,l] * W[k,l,m] with V dense, U in CSF with
  *           levels (i,k,j) and W in CSF with levels (l,m,k), loop orders i,k,j,l and i,l,m,k: both
  *           contractions then gather along a fibre; fused over i only (T reduced to order 2).  CONST_F64.
+ *           A chain at other ranks or in fp64 (order-3 TTMc up to rank 32, order-4 TTMc up to rank 8, MTTKRP of
+ *           order 3 and 4 up to rank 1024) belongs to family "tree" but runs on the fused kernels of this family,
+ *           unless const_plan_set_generic_executor asks for the generic executor.
  *   tree    the generic executor (Sec. 4.2: it walks the loop tree that Algorithm 1 prints as forall / where
  *           constructs).  Any checked schedule, any number of CSF operands, fp32 or fp64: e.g. the running
  *           example R_ijk = A_ipq B_jpr C_kqr D_jkr with X and Y as 2-D workspaces inside the fused r, j
@@ -268,8 +271,8 @@ const_status_t const_schedule_cin(const char *expression, const char *const *tre
  * statement of the Fig. 4(b) structure regrouped).  enable != 0: const_execute runs it on the tensor
  * cores (tcgen05, tf32 operands split into two terms each, fp32 accumulation in tensor memory:
  * per-term relative error below 2^-19, so the fp32 tolerance holds); enable == 0: on the fp32 FMA pipes.
- * Plans that have the stage: order-4 TTMc at rank 8 (const_plan_create switches it on: it is the faster
- * path) and order-3 TTMc at rank 16 x 16 (off unless asked for: the FMA path is faster there).
+ * Plans that have the stage: order-4 TTMc at rank 8 and order-3 TTMc at rank 16 x 16.  Off unless asked for: the
+ * fp32 path is the faster one on both (order 4, 50 M nonzeros: 2.3 against 3.1 ms) and the more accurate one.
  * CONST_ERR_UNSUPPORTED for enable != 0 on any other plan.  Host-only call; takes effect at the next
  * const_execute.  A device-side wait that runs out is reported through const_last_device_status.
  */

@@ -190,8 +190,7 @@ const_status_t const_plan_create(const char *expression, const char *const *tree
         delete plan;
         return rc;
     }
-    // the order-4 TTMc kernel with the per-slice stage on the tensor cores is the faster one at rank 8
-    plan->tensor_stage = plan->desc.family == Family::Ttmc4 && plan->desc.ranks[0] == 8;
+    plan->tensor_stage = 0;      // the fp32 pipes are the faster place for the per-slice stage (see const_plan_set_tensor_stage)
     *out = plan;
     return CONST_OK;
 }
@@ -285,6 +284,25 @@ const_status_t const_execute(const_plan_t *h, const const_operand_t *operands, i
         } else if (stream != p->status_stream) {
             CB_CUDA(cudaStreamWaitEvent(stream, p->status_ready, 0));
         }
+    }
+    // a fully fused chain at a rank or in a type without a family of its own: the leaf-balanced kernels take it
+    if (d.family == Family::Tree && !p->use_tree && d.chain != PlanDesc::Chain::None &&
+        chain_covers((int)d.ranks.size() + 1, d.chain == PlanDesc::Chain::Mttkrp, d.ranks.data())) {
+        const const_operand_t *x = find_operand(operands, n_operands, d.sparse_name);
+        if (!x || !x->csf || x->dense_dev) return CONST_ERR_INVALID_ARG;
+        const const_csf *X = as_csf(x->csf);
+        if (!csf_matches(X, d, d.sparse_name, d.dtype)) return CONST_ERR_INVALID_ARG;
+        const void *factors[3] = {nullptr, nullptr, nullptr};
+        for (size_t f = 0; f < d.factor_names.size(); ++f) {
+            const const_operand_t *o = find_operand(operands, n_operands, d.factor_names[f]);
+            if (!o || !o->dense_dev || o->csf) return CONST_ERR_INVALID_ARG;
+            factors[f] = o->dense_dev;
+        }
+        int64_t elems = 1;
+        for (char c : d.result.idx) elems *= d.extents.at(c);
+        const const_status_t rc = run_chain_any(X, d.chain == PlanDesc::Chain::Mttkrp, factors, d.ranks.data(), d.dtype, out_dev,
+                                                elems, stream);
+        if (rc != CONST_ERR_UNSUPPORTED) return rc;      // no memory for padded factors: the generic executor needs none
     }
     if (d.family == Family::Tree || p->use_tree) {
         const tree::Compiled &cp = p->tree;

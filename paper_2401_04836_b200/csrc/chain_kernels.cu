@@ -1,372 +1,675 @@
-// Fused kernels of the "chain" family: one CSF tensor contracted leaf level first with one dense
-// factor per level (TTMc, Sec. 5.3; MTTKRP, Sec. 5.2), executed as the fused loop nest of Fig. 4(b):
+// Fused kernels of the "chain" family: one CSF tensor contracted leaf level first with one dense factor per level
+// (TTMc, Sec. 5.3; MTTKRP, Sec. 5.2), executed as the fused loop nest of Fig. 4(b):
 //
 //   for i (slice)                     -- root level, fused
 //     for j (fibre)                   -- level 1, fused
 //       t[*] = 0                      -- order-1 intermediate, reset per fibre
 //       for k: t[b] += X[i,j,k] * V[k,b]            (producer contraction)
 //       for a,b: Y[i,a,b] += U[j,a] * t[b]          (consumer contraction; MTTKRP: A[i,r] += B[j,r] * t[r])
+// and, for order 4, with one more producer: P[c] += X[i,j,k,l] * W[l,c];  Q[b,c] += V[k,b] * P[c].
 //
-// Thread mapping.  Each warp owns a run of fibres of one slice and alternates between two phases over
-// windows of a few dozen fibres, entirely on its own (only __syncwarp, no block barrier), so warps of
-// a block overlap their memory-bound and arithmetic-bound phases:
+// Every warp owns an equal run of the tensor's leaves and walks it in windows that it stages as flat records
+// (chain_walk.cuh), entirely on its own: no block barrier, no work list, no slice too large or too small.
+//   producer   Lane groups (one 128-bit load per lane and factor row) work through equal runs of the window's
+//     records, four row gathers in flight per lane.  Where a record ends a fibre, the group has the finished t.
+//   consumer, MTTKRP   The group multiplies t with the row of B whose coordinate the record carries (requested
+//     together with the row gathers) into its own accumulator of the slice.
+//   consumer, TTMc   The group parks t in shared memory, with the fibre's j.  After the window the warp holds the
+//     R2 x R3 slice result as RW x 16-byte register blocks; the lanes that cover one result work on one parked
+//     t, so a warp consumes 32 / ((R2 / RW)(R3 / V)) of them per step.
+// The slice result stays in registers and leaves the warp once per slice: stored if the warp had the whole slice, added
+// atomically otherwise (once per block where the whole block lies in one slice).
 //
-//   phase 1 (producer)  A factor row of R3 floats is read by R3/4 neighbouring lanes with one 128-bit
-//     load each.  The nonzeros of the window are dealt out to the lane groups as equal contiguous
-//     runs of 4-aligned blocks, independent of fibre lengths: a block's four coordinates and four
-//     values arrive with one 128-bit load each and the four row gathers are issued together.  A
-//     group stores its partial t when its run leaves a fibre (or hands it over, for a fibre begun
-//     by its neighbour).  The finished t of every fibre of the window is thus parked in shared
-//     memory (the reduced-order intermediate, one row per fibre), together with the fibre's j.
-//   phase 2 (consumer)  The R2 x R3 slice result is cut into 8 x 4 register blocks; the lanes that
-//     cover one result work on one fibre, so a warp consumes 32 / ((R2/8)(R3/4)) fibres per step:
-//     t comes from shared memory, U[j, 8 rows] from global memory with two 128-bit loads, followed
-//     by 32 FMAs per lane.  For MTTKRP a lane owns four rank entries and does four FMAs.
-//
-// The slice result therefore lives in registers and leaves the warp once: straight to global memory
-// for a slice owned by one warp, through a shared-memory tile for a slice (or chunk of a giant
-// slice) owned by a block -- stored once or, for a chunk, added atomically.
-#include "common.cuh"
+// What bounds them, and what they measured on a B200 (before: one block or warp per slice from the work lists): the
+// gathers are served by L2 (hit rate 80-90 %, DRAM below 10 %), and the kernels are held by L2 latency and by the
+// instructions per leaf (9-12; order 4: 29), not by a bandwidth.  MTTKRP, 100 M leaves, rank 32: 1.79 -> 1.26 ms (gather
+// ceiling 1.0 ms; 64 registers for 32 warps per SM matter: 72 registers 1.42 ms); TTMc 8 x 32, 8 M leaves in fibres of
+// 1.6: 499 -> 284 us; order-4 TTMc, 50 M leaves: 4.57 ms on these pipes, 3.11 ms with the last contraction on the tensor
+// cores -> 2.28 ms here (the factor rows of the consumer copied to shared memory behind the producer -0.4 ms, parked Q
+// laid out free of bank conflicts -0.3 ms, leaf arrays requested one window ahead -0.1 ms; the latter costs more
+// registers than it gains in the order-3 kernels).
+#include <algorithm>
+#include <type_traits>
+
+#include "chain_walk.cuh"
 
 namespace cb {
 namespace {
 
-__device__ __forceinline__ float4 ldg4(const float *p) { return __ldg(reinterpret_cast<const float4 *>(p)); }
+using namespace walk;
 
-constexpr int kStreamAhead = 256;   // nonzeros between the L2 prefetch of a line of the leaf arrays and its use
+constexpr int kWarps = 4;                             // warps per block; they share nothing
+constexpr int kUnroll = 4;                            // row gathers in flight per lane
 
-__device__ __forceinline__ void fma4(float4 &t, float x, const float4 &v) {
-    t.x = fmaf(x, v.x, t.x);
-    t.y = fmaf(x, v.y, t.y);
-    t.z = fmaf(x, v.z, t.z);
-    t.w = fmaf(x, v.w, t.w);
+template <typename T>
+__device__ __forceinline__ void put_entry(T *dst, T v, bool whole) {
+    if (whole) *dst = v;
+    else atomicAdd(dst, v);
 }
 
-// first index f in [lo, hi] with pos[f] >= target
-__device__ __forceinline__ int32_t lower_bound_pos(const int32_t *__restrict__ pos, int32_t lo, int32_t hi,
-                                                   int64_t target) {
-    while (lo < hi) {
-        int32_t mid = lo + (hi - lo) / 2;
-        if ((int64_t)__ldg(pos + mid) < target) lo = mid + 1; else hi = mid;
-    }
-    return lo;
-}
-
-struct Csf3 {
-    const int32_t *crd0, *pos1, *crd1, *pos2, *crd2;   // crd2 and vals are readable up to the next multiple of 4
-    const float *vals;
-};
-
-template <int R2, int R3, bool HADAMARD>
-struct Shape {
-    // phase 1
-    static constexpr int LPR1 = R3 / 4;                 // lanes per factor row
-    static constexpr int G1 = 32 / LPR1;                // lane groups per warp
-    static constexpr int WINDOW = R3 >= 32 ? 64 : 128;  // fibres parked per warp
-    // phase 2: register block of RW rows x 4 columns per lane
-    static constexpr int RW = HADAMARD ? 1 : 8;
-    static constexpr int LPF = HADAMARD ? R3 / 4 : (R2 / 8) * (R3 / 4);   // lanes that cover one fibre
-    static constexpr int FPW = 32 / LPF;                // fibres per warp and step
-    static constexpr int NACC = RW * 4;
-    static constexpr int TILE = HADAMARD ? R3 : R2 * R3;  // floats of one output row (slice)
-    static_assert(LPF >= 1 && LPF <= 32 && WINDOW % FPW == 0, "unsupported rank combination");
-};
-
-// Producer for the window of fibres [s0, s0 + cnt): parks t and j in shared memory.
-// A fibre that starts inside a group's run gets its row stored by that group; the part of a fibre
-// that a group finds already begun (its run starts in the middle of it) goes to a per-group "head"
-// slot and is added to the row afterwards, one group after the other, so no atomics and no clearing
-// of the rows are needed.  Rows and j of the padding fibres [cnt, cnt_padded) are zeroed.
-template <int R2, int R3, bool HADAMARD>
-__device__ __forceinline__ void phase1(const Csf3 &x, const float *__restrict__ F2, int32_t s0, int cnt,
-                                       int cnt_padded, int lane, float *__restrict__ Ts, int32_t *__restrict__ Js,
-                                       int32_t *__restrict__ Ps, float *__restrict__ Hs, int32_t *__restrict__ Hf) {
-    using S = Shape<R2, R3, HADAMARD>;
-    const int g = lane / S::LPR1, q = lane % S::LPR1;
-    const float *F2q = F2 + 4 * q;
-    for (int e = lane; e < cnt_padded; e += 32) Js[e] = e < cnt ? __ldg(x.crd1 + s0 + e) : 0;
-    for (int e = lane; e <= cnt; e += 32) Ps[e] = __ldg(x.pos2 + s0 + e);
-    for (int e = cnt * (R3 / 4) + lane; e < cnt_padded * (R3 / 4); e += 32)
-        reinterpret_cast<float4 *>(Ts)[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-    __syncwarp();
-
-    const int32_t P0 = Ps[0], P1 = Ps[cnt];
-    const int32_t A0 = P0 & ~3;                                   // 4-aligned blocks of the leaf arrays
-    const int32_t blocks = (P1 - A0 + 3) >> 2;
-    const int32_t per_group = (blocks + S::G1 - 1) / S::G1;
-    const int32_t ba = A0 + g * per_group * 4;
-    const int32_t bb = ba + per_group * 4;
-    const int32_t pa = ba > P0 ? ba : P0;                         // nonzeros of this group: [pa, pb)
-    const int32_t pb = bb < P1 ? bb : P1;
-    int32_t head_fibre = -1;
-    if (pa < pb) {
-        int lo = 0, hi = cnt - 1;                                 // fibre holding nonzero pa
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (Ps[mid] <= pa) lo = mid; else hi = mid - 1;
-        }
-        int f = lo;
-        int32_t fend = Ps[f + 1];
-        bool head = Ps[f] < pa;                                   // fibre f was begun by an earlier group
-        float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
-
-        auto park = [&]() {                                       // hand the partial t of fibre f over
-            if (head) {
-                *reinterpret_cast<float4 *>(Hs + g * R3 + 4 * q) = t;
-                head_fibre = f;
-                head = false;
-            } else {
-                *reinterpret_cast<float4 *>(Ts + f * R3 + 4 * q) = t;
-            }
-        };
-        auto leave_fibre = [&]() {                                // the run leaves fibre f
-            park();
-            t = make_float4(0.f, 0.f, 0.f, 0.f);
-            ++f;
-            fend = Ps[f + 1 <= cnt ? f + 1 : cnt];
-        };
-
-        auto partial_block = [&](int32_t p) {                     // first or last block of the run
-            const int4 kk = __ldg(reinterpret_cast<const int4 *>(x.crd2 + p));
-            const float4 xx = __ldg(reinterpret_cast<const float4 *>(x.vals + p));
-            const int32_t k[4] = {kk.x, kk.y, kk.z, kk.w};
-            const float xv[4] = {xx.x, xx.y, xx.z, xx.w};
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                if (p + u >= pa && p + u < pb) {
-                    fma4(t, xv[u], ldg4(F2q + (size_t)k[u] * R3));
-                    if (p + u + 1 == fend) leave_fibre();
-                }
-            }
-        };
-
-        // whole blocks [m0, m1) run through a software pipeline: coordinates two blocks ahead,
-        // row gathers one block ahead of the multiply-adds
-        const int32_t m0 = pa > ba ? ba + 4 : ba;
-        const int32_t m1 = pb & ~3;
-        if (pa > ba) partial_block(ba);
-        if (m0 < m1) {
-            int4 kn = __ldg(reinterpret_cast<const int4 *>(x.crd2 + m0));
-            float4 xc = __ldg(reinterpret_cast<const float4 *>(x.vals + m0));
-            float4 v0 = ldg4(F2q + (size_t)kn.x * R3), v1 = ldg4(F2q + (size_t)kn.y * R3);
-            float4 v2 = ldg4(F2q + (size_t)kn.z * R3), v3 = ldg4(F2q + (size_t)kn.w * R3);
-            float4 xn = xc;
-            if (m0 + 4 < m1) {
-                kn = __ldg(reinterpret_cast<const int4 *>(x.crd2 + m0 + 4));
-                xn = __ldg(reinterpret_cast<const float4 *>(x.vals + m0 + 4));
-            }
-            for (int32_t p = m0; p < m1; p += 4) {
-                if (q == 0 && ((p >> 2) & 7) == 0 && p + kStreamAhead < m1) {      // once per 128-byte line of the leaf arrays
-                    asm volatile("prefetch.global.L2 [%0];" :: "l"(x.crd2 + p + kStreamAhead));
-                    asm volatile("prefetch.global.L2 [%0];" :: "l"(x.vals + p + kStreamAhead));
-                }
-                float4 w0 = v0, w1 = v1, w2 = v2, w3 = v3, xw = xn;
-                if (p + 4 < m1) {                                 // gathers of the next block
-                    w0 = ldg4(F2q + (size_t)kn.x * R3); w1 = ldg4(F2q + (size_t)kn.y * R3);
-                    w2 = ldg4(F2q + (size_t)kn.z * R3); w3 = ldg4(F2q + (size_t)kn.w * R3);
-                }
-                if (p + 8 < m1) {                                 // coordinates of the block after it
-                    kn = __ldg(reinterpret_cast<const int4 *>(x.crd2 + p + 8));
-                    xn = __ldg(reinterpret_cast<const float4 *>(x.vals + p + 8));
-                }
-                fma4(t, xc.x, v0);
-                if (p + 1 == fend) leave_fibre();
-                fma4(t, xc.y, v1);
-                if (p + 2 == fend) leave_fibre();
-                fma4(t, xc.z, v2);
-                if (p + 3 == fend) leave_fibre();
-                fma4(t, xc.w, v3);
-                if (p + 4 == fend) leave_fibre();
-                v0 = w0; v1 = w1; v2 = w2; v3 = w3; xc = xw;
-            }
-        }
-        if (m1 >= m0 && m1 < pb) partial_block(m1);
-        if (f < cnt && pb > Ps[f]) park();                        // the run ends inside fibre f
-    }
-    if (q == 0) Hf[g] = head_fibre;
-    __syncwarp();
-    if (g == 0) {                                                 // add the heads, in group order
-        for (int gg = 1; gg < S::G1; ++gg) {
-            const int32_t hf = Hf[gg];
-            if (hf >= 0) {
-                float4 *row = reinterpret_cast<float4 *>(Ts + hf * R3 + 4 * q);
-                const float4 h = *reinterpret_cast<const float4 *>(Hs + gg * R3 + 4 * q);
-                float4 r = *row;
-                r.x += h.x; r.y += h.y; r.z += h.z; r.w += h.w;
-                *row = r;
-            }
-        }
-    }
-    __syncwarp();
-}
-
-// Consumer for the parked window: acc += (factor row of j) (x) t.
-template <int R2, int R3, bool HADAMARD>
-__device__ __forceinline__ void phase2(const float *__restrict__ F1, int cnt_padded, int lane,
-                                       const float *__restrict__ Ts, const int32_t *__restrict__ Js,
-                                       float (&acc)[Shape<R2, R3, HADAMARD>::NACC]) {
-    using S = Shape<R2, R3, HADAMARD>;
-    const int slot = lane / S::LPF, inner = lane % S::LPF;
-    if (HADAMARD) {
-        // lane owns rank entries 4*inner .. 4*inner+3 of the fibre in its slot
-        for (int e = slot; e < cnt_padded; e += S::FPW) {
-            const float4 b = ldg4(F1 + (size_t)Js[e] * R3 + 4 * inner);
-            const float4 tv = *reinterpret_cast<const float4 *>(Ts + e * R3 + 4 * inner);
-            acc[0] = fmaf(b.x, tv.x, acc[0]);
-            acc[1] = fmaf(b.y, tv.y, acc[1]);
-            acc[2] = fmaf(b.z, tv.z, acc[2]);
-            acc[3] = fmaf(b.w, tv.w, acc[3]);
-        }
-    } else {
-        // lane owns rows 8*rg .. 8*rg+7 and columns 4*cg .. 4*cg+3 of the fibre in its slot
-        const int rg = inner / (R3 / 4), cg = inner % (R3 / 4);
-        const float *F1g = F1 + 8 * rg;
-        for (int e = slot; e < cnt_padded; e += S::FPW) {
-            const float *up = F1g + (size_t)Js[e] * R2;
-            const float4 u0 = ldg4(up), u1 = ldg4(up + 4);
-            const float4 tv = *reinterpret_cast<const float4 *>(Ts + e * R3 + 4 * cg);
-            const float ur[8] = {u0.x, u0.y, u0.z, u0.w, u1.x, u1.y, u1.z, u1.w};
-#pragma unroll
-            for (int r = 0; r < 8; ++r) {
-                acc[4 * r + 0] = fmaf(ur[r], tv.x, acc[4 * r + 0]);
-                acc[4 * r + 1] = fmaf(ur[r], tv.y, acc[4 * r + 1]);
-                acc[4 * r + 2] = fmaf(ur[r], tv.z, acc[4 * r + 2]);
-                acc[4 * r + 3] = fmaf(ur[r], tv.w, acc[4 * r + 3]);
-            }
-        }
-    }
-    __syncwarp();
-}
-
-template <int R2, int R3, bool HADAMARD>
-__global__ void __launch_bounds__(kWarpsPerBlock * 32)
-chain3_kernel(const WorkItem *__restrict__ items, const int32_t *__restrict__ bin_totals,
-              const int32_t *__restrict__ light_list, Csf3 x,
-              const float *__restrict__ F1, const float *__restrict__ F2, float *__restrict__ out) {
-    using S = Shape<R2, R3, HADAMARD>;
-    extern __shared__ __align__(16) float Ts_all[];          // [warp][WINDOW * R3] parked rows
-    __shared__ int32_t Js_all[kWarpsPerBlock][S::WINDOW];
-    __shared__ int32_t Ps_all[kWarpsPerBlock][S::WINDOW + 1];
-    __shared__ __align__(16) float Hs_all[kWarpsPerBlock][S::G1 * R3];
-    __shared__ int32_t Hf_all[kWarpsPerBlock][S::G1];
-    __shared__ float tile[S::TILE];
-
-    if ((int)blockIdx.x >= work_item_count(bin_totals)) return;      // the grid is an upper bound
-    const WorkItem it = items[blockIdx.x];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const bool light = it.kind == kItemLight;
-
-    int32_t slice = it.slice, fa = 0, fb = 0;
-    if (light) {
-        if (warp < it.f0) {
-            slice = __ldg(light_list + it.slice + warp);
-            fa = __ldg(x.pos1 + slice);
-            fb = __ldg(x.pos1 + slice + 1);
-        }
-    } else {
-        const int64_t lo = __ldg(x.pos2 + it.f0), hi = __ldg(x.pos2 + it.f1);
-        fa = warp == 0 ? it.f0 : lower_bound_pos(x.pos2, it.f0, it.f1, lo + (hi - lo) * warp / kWarpsPerBlock);
-        fb = warp == kWarpsPerBlock - 1
-                 ? it.f1
-                 : lower_bound_pos(x.pos2, it.f0, it.f1, lo + (hi - lo) * (warp + 1) / kWarpsPerBlock);
-        for (int e = threadIdx.x; e < S::TILE; e += blockDim.x) tile[e] = 0.f;
-        __syncthreads();
-    }
-
-    float acc[S::NACC];
-#pragma unroll
-    for (int a = 0; a < S::NACC; ++a) acc[a] = 0.f;
-    float *Ts = Ts_all + warp * (S::WINDOW * R3);
-    int32_t *Js = Js_all[warp];
-    for (int32_t s0 = fa; s0 < fb; s0 += S::WINDOW) {
-        const int cnt = fb - s0 < S::WINDOW ? fb - s0 : S::WINDOW;
-        const int cnt_padded = (cnt + S::FPW - 1) / S::FPW * S::FPW;
-        phase1<R2, R3, HADAMARD>(x, F2, s0, cnt, cnt_padded, lane, Ts, Js, Ps_all[warp], Hs_all[warp], Hf_all[warp]);
-        phase2<R2, R3, HADAMARD>(F1, cnt_padded, lane, Ts, Js, acc);
-    }
-
-    // lanes of different slots hold partial sums of the same result entries: add them up
-#pragma unroll
-    for (int off = S::LPF; off < 32; off <<= 1) {
-#pragma unroll
-        for (int a = 0; a < S::NACC; ++a) acc[a] += __shfl_xor_sync(0xffffffffu, acc[a], off);
-    }
-    const int inner = lane % S::LPF;
-    const int rg = HADAMARD ? 0 : inner / (R3 / 4), cg = HADAMARD ? inner : inner % (R3 / 4);
-    if (light) {
-        if (warp < it.f0 && lane < S::LPF) {
-            float *dst = out + (size_t)__ldg(x.crd0 + slice) * S::TILE;
-#pragma unroll
-            for (int r = 0; r < S::RW; ++r)
-                *reinterpret_cast<float4 *>(dst + (S::RW * rg + r) * R3 + 4 * cg) =
-                    make_float4(acc[4 * r], acc[4 * r + 1], acc[4 * r + 2], acc[4 * r + 3]);
-        }
+// writes entries [0, n) of a vector; n >= Vec::N and aligned: one 16-byte access
+template <typename T>
+__device__ __forceinline__ void put_vec(T *dst, const Vec<T> &v, int n, bool whole) {
+    if (n >= Vec<T>::N && (reinterpret_cast<uintptr_t>(dst) & 15u) == 0) {
+        if (whole) store_vec(dst, v);
+        else add_vec(dst, v);
         return;
     }
-    if (fa < fb && lane < S::LPF) {
 #pragma unroll
-        for (int r = 0; r < S::RW; ++r)
-#pragma unroll
-            for (int c = 0; c < 4; ++c) atomicAdd(&tile[(S::RW * rg + r) * R3 + 4 * cg + c], acc[4 * r + c]);
-    }
+    for (int i = 0; i < Vec<T>::N; ++i)
+        if (i < n) put_entry(dst + i, v.at(i), whole);
+}
+
+// The block's warps have left their parts of one slice's result, [rows][cols] each, `apart` entries apart: adds them up
+// and adds the sum to out, whose rows have real_cols entries (real_rows of them).
+template <typename T>
+__device__ __forceinline__ void add_joint(const T *parts, int apart, int rows, int cols, T *out, int real_rows, int real_cols) {
+    constexpr int N = Vec<T>::N;
     __syncthreads();
-    float *dst = out + (size_t)__ldg(x.crd0 + slice) * S::TILE;
-    if (it.kind == kItemBlock) {
-        for (int e = threadIdx.x; e < S::TILE; e += blockDim.x) dst[e] = tile[e];
-    } else {
-        for (int e = threadIdx.x; e < S::TILE; e += blockDim.x) atomicAdd(&dst[e], tile[e]);
+    for (int i = threadIdx.x * N; i < rows * cols; i += kWarps * 32 * N) {
+        const Vec<T> sum = add_parts<kWarps>(parts + i, apart);
+        const int r = i / cols, c = i % cols;
+        if (r < real_rows) put_vec(out + (size_t)r * real_cols + c, sum, real_cols - c, false);
     }
 }
 
-template <int R2, int R3, bool HADAMARD>
-const_status_t launch_chain3(const const_csf *X, const float *F1, const float *F2, float *out, int64_t n_rows,
-                             cudaStream_t stream) {
-    constexpr int TILE = Shape<R2, R3, HADAMARD>::TILE;
-    CB_CUDA(cudaMemsetAsync(out, 0, sizeof(float) * TILE * n_rows, stream));       // "R[*] = 0" precedes the nest
-    if (X->nnz == 0) return CONST_OK;
-    Csf3 x{X->crd[0], X->pos[1], X->crd[1], X->pos[2], X->crd[2], static_cast<const float *>(X->vals)};
-    using S = Shape<R2, R3, HADAMARD>;
-    constexpr size_t dyn = sizeof(float) * kWarpsPerBlock * S::WINDOW * R3;
-    static PerDeviceOnce attr_once;                     // per template instance
-    CB_CUDA(once_per_device(attr_once, [&] { return cudaFuncSetAttribute(chain3_kernel<R2, R3, HADAMARD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn); }));
-    CB_LAUNCH("chain3_kernel", stream,
-              chain3_kernel<R2, R3, HADAMARD><<<(unsigned)X->item_cap, kWarpsPerBlock * 32, dyn, stream>>>(
-                  X->items, X->bin_totals, X->light_list, x, F1, F2, out));
-    CB_CUDA(cudaGetLastError());
-    return CONST_OK;
+// sum of the pair over lanes that differ in the lane-number bits from `from` up
+template <typename T>
+__device__ __forceinline__ void reduce_pair(Pair<T> &p, int from) {
+    T x = p.lo(), y = p.hi();
+    for (int off = from; off < 32; off <<= 1) {
+        x += __shfl_xor_sync(kAll, x, off);
+        y += __shfl_xor_sync(kAll, y, off);
+    }
+    p = make_pair(x, y);
 }
 
-template <int R2>
-const_status_t dispatch_ttmc3_r3(const const_csf *X, const float *U, const float *V, int R3, float *Y, int64_t n_rows,
-                                 cudaStream_t s) {
-    switch (R3) {
-        case 8: return launch_chain3<R2, 8, false>(X, U, V, Y, n_rows, s);
-        case 16: return launch_chain3<R2, 16, false>(X, U, V, Y, n_rows, s);
-        case 32: return launch_chain3<R2, 32, false>(X, U, V, Y, n_rows, s);
+// ---------------------------------------------------------------------------------------------- MTTKRP
+template <typename T, int ORDER, int RP>
+struct MttkrpShape {
+    static constexpr int N = Vec<T>::N;
+        static constexpr int LPR = RP / N;                // lanes per factor row
+    static constexpr int G = 32 / LPR;                // lane groups per warp
+    static constexpr int W = 128;                     // leaves per window
+    static_assert(LPR >= 1 && LPR <= 32, "rank tile");
+};
+
+// F[m]: factor of level m + 1, rows of `stride` entries, columns [RP * blockIdx.y, ...) taken here; R = real rank
+template <typename T, int ORDER>
+struct MttkrpArgs {
+    Chain<T, ORDER> x;
+    const T *F[ORDER - 1];
+    T *out;
+    int32_t stride, R, chunk;
+    size_t out_bytes;
+};
+
+template <typename T, int ORDER, int RP>
+__global__ void __launch_bounds__(kWarps * 32, sizeof(T) == 4 ? (ORDER == 3 ? 8 : 6) : 4) mttkrp_kernel(const __grid_constant__ MttkrpArgs<T, ORDER> a) {
+    using S = MttkrpShape<T, ORDER, RP>;
+    constexpr int N = S::N;
+    __shared__ Stage<T, ORDER, S::W> stages[kWarps];
+    const Share own(a.x.n[ORDER - 1], a.chunk, kWarps);
+    const int lane = threadIdx.x & 31, g = lane / S::LPR, q = lane % S::LPR;
+    Stage<T, ORDER, S::W> &st = stages[threadIdx.x >> 5];
+    const int col = blockIdx.y * RP + q * N;
+    const T *leaf = a.F[ORDER - 2] + col, *mid = ORDER == 4 ? a.F[1] + col : nullptr, *top = a.F[0] + col;
+    Vec<T> acc = zero_vec<T>();
+    const int32_t joint = walk_chunk(a.x, own, lane,
+        [](const Place<ORDER> &) {},
+        [&](Place<ORDER> &place, int32_t e, int32_t limit) {
+            const int cnt = limit - e < S::W ? limit - e : S::W;
+            const int run = run_length<S::W, S::G, kUnroll>(cnt);
+            bool flat;
+            Ahead<T, ORDER, S::W> ahead;
+            request<T, ORDER, S::W>(a.x, place, e, limit, lane, ahead);
+            stage_window<T, ORDER, S::W, S::G, false>(ahead, place, e, cnt, run, lane, st, flat);
+            Vec<T> t = zero_vec<T>(), s = zero_vec<T>();
+            for (int i = 0; i < run; i += kUnroll) {
+                Rec<T> r[kUnroll];
+                Vec<T> v[kUnroll], u[kUnroll], w[kUnroll];
+                int32_t k[kUnroll];
+#pragma unroll
+                for (int z = 0; z < kUnroll; ++z) {
+                    r[z] = st.rec[(i + z) * S::G + g];
+                    v[z] = load_vec(leaf + (size_t)r[z].row * a.stride);
+                    if constexpr (ORDER == 4) {
+                        k[z] = st.second_tag((i + z) * S::G + g, r[z]);
+                        if (k[z] >= 0) w[z] = load_vec(mid + (size_t)k[z] * a.stride);
+                    }
+                    if (r[z].tag1 >= 0) u[z] = load_vec(top + (size_t)r[z].tag1 * a.stride);
+                }
+#pragma unroll
+                for (int z = 0; z < kUnroll; ++z) {
+                    axpy(t, make_pair(r[z].val, r[z].val), v[z]);
+                    if constexpr (ORDER == 4) {
+                        if (k[z] >= 0) { mul_add(s, t, w[z]); t = zero_vec<T>(); }
+                        if (r[z].tag1 >= 0) { mul_add(acc, s, u[z]); s = zero_vec<T>(); }
+                    } else {
+                        if (r[z].tag1 >= 0) { mul_add(acc, t, u[z]); t = zero_vec<T>(); }
+                    }
+                }
+            }
+            return cnt;
+        },
+        [&](int32_t slice, bool whole) {
+#pragma unroll
+            for (int i = 0; i < N / 2; ++i) reduce_pair(acc.p[i], S::LPR);
+            if (g == 0) put_vec(a.out + (size_t)__ldg(a.x.crd[0] + slice) * a.R + col, acc, a.R - col, whole);
+            acc = zero_vec<T>();
+        });
+    if (joint >= 0) {
+        T *part = reinterpret_cast<T *>(st.rec);
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < N / 2; ++i) reduce_pair(acc.p[i], S::LPR);
+        if (g == 0) store_vec(part + q * N, acc);
+        const int c0 = blockIdx.y * RP;
+        add_joint(reinterpret_cast<const T *>(stages[0].rec), (int)(sizeof(stages[0]) / sizeof(T)), 1, RP,
+                  a.out + (size_t)__ldg(a.x.crd[0] + joint) * a.R + c0, 1, a.R - c0);
+    }
+}
+
+// ---------------------------------------------------------------------------------------------- TTMc, order 3
+template <typename T, int R2, int R3>
+struct Ttmc3Shape {
+    static constexpr int N = Vec<T>::N;
+    static constexpr int LPR = R3 / N, G = 32 / LPR;
+    static constexpr int W = 64;                      // leaves per window
+    static constexpr int RW = (R2 / 8) * (R3 / N) <= 32 ? 8 : 16;      // rows of a register block
+    static constexpr int LPF = (R2 / RW) * (R3 / N), FPW = 32 / LPF;   // lanes per parked t, parked t per step
+    static constexpr int BLOCKS = sizeof(T) == 4 ? 5 : 3;              // resident blocks the registers are cut for
+    struct __align__(16) Smem {
+        Stage<T, 3, W> st;
+        T t[W * R3];                                  // parked t, one row per piece
+        T u[W * R2];                                  // the factor row that goes with it
+    };
+};
+
+template <typename T>
+struct Ttmc3Args {
+    Chain<T, 3> x;
+    const T *U, *V;                                   // rows of R2 and R3 (padded) entries
+    T *out;
+    int32_t R2, R3, chunk;                            // real ranks
+    size_t out_bytes;
+};
+
+template <typename T, int R2, int R3>
+__global__ void __launch_bounds__(kWarps * 32, Ttmc3Shape<T, R2, R3>::BLOCKS) ttmc3_kernel(const __grid_constant__ Ttmc3Args<T> a) {
+    using S = Ttmc3Shape<T, R2, R3>;
+    constexpr int N = S::N;
+    extern __shared__ __align__(16) unsigned char smem[];
+    const Share own(a.x.n[2], a.chunk, kWarps);
+    const int lane = threadIdx.x & 31, g = lane / S::LPR, q = lane % S::LPR;
+    typename S::Smem &sm = reinterpret_cast<typename S::Smem *>(smem)[threadIdx.x >> 5];
+    const T *V = a.V + q * N;
+    // consumer: the lane owns rows rg .. rg + RW - 1 and columns cg .. cg + N - 1 of the slice result; acc[i][c]: rows
+    // rg + 2 i and rg + 2 i + 1 of column cg + c
+    const int slot = lane / S::LPF, rg = (lane % S::LPF) / (R3 / N) * S::RW, cg = (lane % S::LPF) % (R3 / N) * N;
+    Pair<T> acc[S::RW / 2][N];
+    auto clear = [&]() {
+#pragma unroll
+        for (int i = 0; i < S::RW / 2; ++i)
+#pragma unroll
+            for (int c = 0; c < N; ++c) acc[i][c] = make_pair(T(0), T(0));
+    };
+    clear();
+    // adds the slots up and hands every row of the lane's block to put
+    auto gather = [&](auto put) {
+#pragma unroll
+        for (int i = 0; i < S::RW / 2; ++i) {
+            Vec<T> lo, hi;
+#pragma unroll
+            for (int c = 0; c < N; ++c) reduce_pair(acc[i][c], S::LPF);
+#pragma unroll
+            for (int c = 0; c < N / 2; ++c) {
+                lo.p[c] = make_pair(acc[i][2 * c].lo(), acc[i][2 * c + 1].lo());
+                hi.p[c] = make_pair(acc[i][2 * c].hi(), acc[i][2 * c + 1].hi());
+            }
+            put(rg + 2 * i, lo);
+            put(rg + 2 * i + 1, hi);
+        }
+    };
+    const int32_t joint = walk_chunk(a.x, own, lane,
+        [](const Place<3> &) {},
+        [&](Place<3> &place, int32_t e, int32_t limit) {
+            const int cnt = limit - e < S::W ? limit - e : S::W;
+            const int run = run_length<S::W, S::G, kUnroll>(cnt);
+            bool flat;
+            Ahead<T, 3, S::W> ahead;
+            request<T, 3, S::W>(a.x, place, e, limit, lane, ahead);
+            const int pieces = stage_window<T, 3, S::W, S::G, true>(ahead, place, e, cnt, run, lane, sm.st, flat);
+            fetch_rows<T, R2>(sm.u, a.U, sm.st.j, pieces, lane);
+            Vec<T> t = zero_vec<T>();
+            for (int i = 0; i < run; i += kUnroll) {
+                Rec<T> r[kUnroll];
+                Vec<T> v[kUnroll];
+#pragma unroll
+                for (int z = 0; z < kUnroll; ++z) {
+                    r[z] = sm.st.rec[(i + z) * S::G + g];
+                    v[z] = load_vec(V + (size_t)r[z].row * R3);
+                }
+#pragma unroll
+                for (int z = 0; z < kUnroll; ++z) {
+                    axpy(t, make_pair(r[z].val, r[z].val), v[z]);
+                    if (r[z].tag1 >= 0) { store_vec(sm.t + r[z].tag1 * R3 + q * N, t); t = zero_vec<T>(); }
+                }
+            }
+            copies_done();
+            __syncwarp();
+#pragma unroll 2
+            for (int p = slot; p < pieces; p += S::FPW) {
+                const T *row = sm.u + p * R2 + rg;
+                const Vec<T> tv = peek_vec(sm.t + p * R3 + cg);
+                Vec<T> u[S::RW / N];
+#pragma unroll
+                for (int i = 0; i < S::RW / N; ++i) u[i] = peek_vec(row + i * N);
+#pragma unroll
+                for (int c = 0; c < N; ++c) {
+                    const Pair<T> tt = make_pair(tv.at(c), tv.at(c));
+#pragma unroll
+                    for (int i = 0; i < S::RW / 2; ++i) fma2(acc[i][c], u[i * 2 / N].p[i % (N / 2)], tt);
+                }
+            }
+            return cnt;
+        },
+        [&](int32_t slice, bool whole) {
+            T *dst = a.out + (size_t)__ldg(a.x.crd[0] + slice) * a.R2 * a.R3 + cg;
+            gather([&](int row, const Vec<T> &v) {
+                if (slot == 0 && row < a.R2) put_vec(dst + row * a.R3, v, a.R3 - cg, whole);
+            });
+            clear();
+        });
+    if (joint >= 0) {
+        __syncwarp();
+        gather([&](int row, const Vec<T> &v) {
+            if (slot == 0) store_vec(sm.t + row * R3 + cg, v);
+        });
+        add_joint(reinterpret_cast<typename S::Smem *>(smem)[0].t, (int)(sizeof(sm) / sizeof(T)), R2, R3,
+                  a.out + (size_t)__ldg(a.x.crd[0] + joint) * a.R2 * a.R3, a.R2, a.R3);
+    }
+}
+
+// ---------------------------------------------------------------------------------------------- TTMc, order 4, ranks up to 8
+template <typename T>
+struct Ttmc4Shape {
+    static constexpr int N = Vec<T>::N;
+    static constexpr int R = 8, SL = 4, G = 32 / SL;  // lanes per producer group, groups per warp
+    static constexpr int W = 64, P = 40;              // leaves per window, parked Q (a window that would need more is halved)
+    static constexpr int QROW = R * R + 16;           // 16 spare entries: neighbouring pieces start in other banks
+    // A lane of a producer group holds 2 R entries of Q as chunks of 16 bytes; chunk c of lane h is parked at
+    // (c * SL + h) * 16 bytes, so that the lanes of a group write neighbouring chunks.
+    struct __align__(16) Smem {
+        Stage<T, 4, W> st;
+        T q[P * QROW];                                // parked Q
+        T u[P * R];                                   // the factor row that goes with it
+    };
+};
+
+template <typename T>
+struct Ttmc4Args {
+    Chain<T, 4> x;
+    const T *U, *V, *W;                               // rows of 8 entries
+    T *out;
+    int32_t R2, R3, R4, chunk;                        // real ranks
+    size_t out_bytes;
+};
+
+template <typename T>
+__global__ void __launch_bounds__(kWarps * 32, sizeof(T) == 4 ? 3 : 1) ttmc4_kernel(const __grid_constant__ Ttmc4Args<T> a) {
+    using S = Ttmc4Shape<T>;
+    constexpr int N = S::N, R = S::R, NV = R / N;
+    extern __shared__ __align__(16) unsigned char smem[];
+    const Share own(a.x.n[3], a.chunk, kWarps);
+    const int lane = threadIdx.x & 31, g = lane / S::SL, h = lane % S::SL;
+    typename S::Smem &sm = reinterpret_cast<typename S::Smem *>(smem)[threadIdx.x >> 5];
+    const T *V = a.V + 2 * h;
+    // consumer: 16 lanes cover the 8 x 8 x 8 result; the lane owns every a for one b and four c; acc[i][c]: a = 2 i, 2 i + 1
+    // (numbered so that neighbouring lanes read neighbouring chunks of the parked Q)
+    const int slot = lane >> 4, b = 2 * (lane & 3) + ((lane >> 3) & 1), ch = (lane & 4);
+    const int chunk = (b & 1) * NV + ch / N;
+    Pair<T> acc[R / 2][4];
+    auto clear = [&]() {
+#pragma unroll
+        for (int i = 0; i < R / 2; ++i)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) acc[i][c] = make_pair(T(0), T(0));
+    };
+    clear();
+    // adds the two slots up and hands the lane's part of every plane a = i to put, 16 bytes (from column c) at a time
+    auto gather = [&](auto put) {
+#pragma unroll
+        for (int i = 0; i < R / 2; ++i) {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) reduce_pair(acc[i][c], 16);
+#pragma unroll
+            for (int c = 0; c < 4; c += N) {
+                Vec<T> lo, hi;
+#pragma unroll
+                for (int n = 0; n < N / 2; ++n) {
+                    lo.p[n] = make_pair(acc[i][c + 2 * n].lo(), acc[i][c + 2 * n + 1].lo());
+                    hi.p[n] = make_pair(acc[i][c + 2 * n].hi(), acc[i][c + 2 * n + 1].hi());
+                }
+                put(2 * i, ch + c, lo);
+                put(2 * i + 1, ch + c, hi);
+            }
+        }
+    };
+    Ahead<T, 4, S::W> ahead;
+    const int32_t joint = walk_chunk(a.x, own, lane,
+        [&](const Place<4> &place) {
+            request<T, 4, S::W>(a.x, place, own.e0, own.e1, lane, ahead);
+        },
+        [&](Place<4> &place, int32_t e, int32_t limit) {
+            int cnt = limit - e < S::W ? limit - e : S::W;
+            const Place<4> from = place;
+            int run = run_length<S::W, S::G, kUnroll>(cnt);
+            bool flat;
+            int pieces = stage_window<T, 4, S::W, S::G, true>(ahead, place, e, cnt, run, lane, sm.st, flat);
+            if (pieces > S::P) {                      // uniform over the warp
+                cnt = 32;
+                place = from;
+                run = run_length<S::W, S::G, kUnroll>(cnt);
+                pieces = stage_window<T, 4, S::W, S::G, true>(ahead, place, e, cnt, run, lane, sm.st, flat);
+            }
+            request<T, 4, S::W>(a.x, place, e + cnt, own.e1, lane, ahead);
+            fetch_rows<T, R>(sm.u, a.U, sm.st.j, pieces, lane);
+            Vec<T> p[NV], q0[NV], q1[NV];             // P; rows b = 2 h and 2 h + 1 of Q
+#pragma unroll
+            for (int c = 0; c < NV; ++c) p[c] = q0[c] = q1[c] = zero_vec<T>();
+            auto produce = [&](auto one_leaf_per_node) {
+                constexpr bool FLAT = decltype(one_leaf_per_node)::value;
+                for (int i = 0; i < run; i += kUnroll) {
+                    Rec<T> r[kUnroll];
+                    Vec<T> w[kUnroll][NV];
+                    T v0[kUnroll], v1[kUnroll];
+                    int32_t k[kUnroll];
+#pragma unroll
+                    for (int z = 0; z < kUnroll; ++z) {
+                        const int at = (i + z) * S::G + g;
+                        r[z] = sm.st.rec[at];
+                        k[z] = sm.st.second_tag(at, r[z]);
+#pragma unroll
+                        for (int c = 0; c < NV; ++c) w[z][c] = load_vec(a.W + (size_t)r[z].row * R + c * N);
+                        v0[z] = v1[z] = T(0);
+                        if (k[z] >= 0) {
+                            const Pair<T> v = load_pair(V + (size_t)k[z] * R);
+                            v0[z] = v.lo();
+                            v1[z] = v.hi();
+                        }
+                    }
+#pragma unroll
+                    for (int z = 0; z < kUnroll; ++z) {
+                        if constexpr (FLAT) {         // Q[b, :] += (V[k, b] X) W[l, :]
+                            const T s0 = v0[z] * r[z].val, s1 = v1[z] * r[z].val;
+#pragma unroll
+                            for (int c = 0; c < NV; ++c) {
+                                axpy(q0[c], make_pair(s0, s0), w[z][c]);
+                                axpy(q1[c], make_pair(s1, s1), w[z][c]);
+                            }
+                        } else {                      // P[:] += X W[l, :];  Q[b, :] += V[k, b] P[:]
+#pragma unroll
+                            for (int c = 0; c < NV; ++c) axpy(p[c], make_pair(r[z].val, r[z].val), w[z][c]);
+                            if (k[z] >= 0) {
+#pragma unroll
+                                for (int c = 0; c < NV; ++c) {
+                                    axpy(q0[c], make_pair(v0[z], v0[z]), p[c]);
+                                    axpy(q1[c], make_pair(v1[z], v1[z]), p[c]);
+                                    p[c] = zero_vec<T>();
+                                }
+                            }
+                        }
+                        if (r[z].tag1 >= 0) {
+                            T *dst = sm.q + r[z].tag1 * S::QROW + h * N;
+#pragma unroll
+                            for (int c = 0; c < NV; ++c) {
+                                store_vec(dst + c * S::SL * N, q0[c]);
+                                store_vec(dst + (NV + c) * S::SL * N, q1[c]);
+                                q0[c] = q1[c] = zero_vec<T>();
+                            }
+                        }
+                    }
+                }
+            };
+            if (flat) produce(std::true_type());
+            else produce(std::false_type());
+            copies_done();
+            __syncwarp();
+#pragma unroll 2
+            for (int s = slot; s < pieces; s += 2) {
+                const T *row = sm.u + s * R;
+                Vec<T> u[NV], q[4 / N];
+#pragma unroll
+                for (int i = 0; i < NV; ++i) u[i] = peek_vec(row + i * N);
+#pragma unroll
+                for (int i = 0; i < 4 / N; ++i) q[i] = peek_vec(sm.q + s * S::QROW + ((chunk + i) * S::SL + (lane & 3)) * N);
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const Pair<T> qq = make_pair(q[c / N].at(c % N), q[c / N].at(c % N));
+#pragma unroll
+                    for (int i = 0; i < R / 2; ++i) fma2(acc[i][c], u[i * 2 / N].p[i % (N / 2)], qq);
+                }
+            }
+            return cnt;
+        },
+        [&](int32_t slice, bool whole) {
+            T *dst = a.out + (size_t)__ldg(a.x.crd[0] + slice) * a.R2 * a.R3 * a.R4;
+            gather([&](int i, int c, const Vec<T> &v) {
+                if (slot == 0 && b < a.R3 && i < a.R2) put_vec(dst + ((size_t)i * a.R3 + b) * a.R4 + c, v, a.R4 - c, whole);
+            });
+            clear();
+        });
+    if (joint >= 0) {
+        __syncwarp();
+        gather([&](int i, int c, const Vec<T> &v) {
+            if (slot == 0) store_vec(sm.q + (i * R + b) * R + c, v);
+        });
+        T *dst = a.out + (size_t)__ldg(a.x.crd[0] + joint) * a.R2 * a.R3 * a.R4;
+        const T *parts = reinterpret_cast<typename S::Smem *>(smem)[0].q;
+        __syncthreads();
+        for (int i = threadIdx.x * N; i < R * R * R; i += kWarps * 32 * N) {
+            const Vec<T> sum = add_parts<kWarps>(parts + i, (int)(sizeof(sm) / sizeof(T)));
+            const int a2 = i / (R * R), b2 = i / R % R, c2 = i % R;
+            if (a2 < a.R2 && b2 < a.R3) put_vec(dst + ((size_t)a2 * a.R3 + b2) * a.R4 + c2, sum, a.R4 - c2, false);
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------------------------- host side
+unsigned chunk_blocks(int64_t nnz, int32_t chunk) {
+    const int64_t warps = (nnz + chunk - 1) / chunk;
+    return (unsigned)((warps + kWarps - 1) / kWarps);
+}
+
+template <typename T, int ORDER, int RP>
+const_status_t launch_mttkrp(MttkrpArgs<T, ORDER> a, int tiles, cudaStream_t stream) {
+    const dim3 grid(chunk_blocks(a.x.n[ORDER - 1], a.chunk), (unsigned)tiles);
+    return launch_on_cleared("chain3_kernel", mttkrp_kernel<T, ORDER, RP>, a, grid, kWarps * 32, 0, a.out, a.out_bytes, stream);
+}
+
+template <typename T, int R2, int R3>
+const_status_t launch_ttmc3(const Ttmc3Args<T> &a, cudaStream_t stream) {
+    constexpr size_t dyn = sizeof(typename Ttmc3Shape<T, R2, R3>::Smem) * kWarps;
+    static PerDeviceOnce attr_once;                     // per template instance
+    CB_CUDA(once_per_device(attr_once, [&] { return cudaFuncSetAttribute(ttmc3_kernel<T, R2, R3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn); }));
+    return launch_on_cleared("chain3_kernel", ttmc3_kernel<T, R2, R3>, a, dim3(chunk_blocks(a.x.n[2], a.chunk)), kWarps * 32, dyn, a.out,
+                             a.out_bytes, stream);
+}
+
+// r2, r3: 8, 16 or 32
+template <typename T>
+const_status_t dispatch_ttmc3(const Ttmc3Args<T> &a, int r2, int r3, cudaStream_t s) {
+    switch (r2 * 100 + r3) {
+        case 808: return launch_ttmc3<T, 8, 8>(a, s);
+        case 816: return launch_ttmc3<T, 8, 16>(a, s);
+        case 832: return launch_ttmc3<T, 8, 32>(a, s);
+        case 1608: return launch_ttmc3<T, 16, 8>(a, s);
+        case 1616: return launch_ttmc3<T, 16, 16>(a, s);
+        case 1632: return launch_ttmc3<T, 16, 32>(a, s);
+        case 3208: return launch_ttmc3<T, 32, 8>(a, s);
+        case 3216: return launch_ttmc3<T, 32, 16>(a, s);
+        case 3232: return launch_ttmc3<T, 32, 32>(a, s);
     }
     return CONST_ERR_UNSUPPORTED;
+}
+
+template <typename T, int ORDER>
+const_status_t dispatch_mttkrp(const MttkrpArgs<T, ORDER> &a, int rp, int tiles, cudaStream_t s) {
+    switch (rp) {
+        case 4: return launch_mttkrp<T, ORDER, 4>(a, tiles, s);
+        case 8: return launch_mttkrp<T, ORDER, 8>(a, tiles, s);
+        case 16: return launch_mttkrp<T, ORDER, 16>(a, tiles, s);
+        case 32: return launch_mttkrp<T, ORDER, 32>(a, tiles, s);
+    }
+    return CONST_ERR_UNSUPPORTED;
+}
+
+template <typename T>
+const_status_t launch_ttmc4(const Ttmc4Args<T> &a, cudaStream_t stream) {
+    constexpr size_t dyn = sizeof(typename Ttmc4Shape<T>::Smem) * kWarps;
+    static PerDeviceOnce attr_once;                     // per template instance
+    CB_CUDA(once_per_device(attr_once, [&] { return cudaFuncSetAttribute(ttmc4_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn); }));
+    return launch_on_cleared("ttmc4_kernel", ttmc4_kernel<T>, a, dim3(chunk_blocks(a.x.n[3], a.chunk)), kWarps * 32, dyn, a.out,
+                             a.out_bytes, stream);
+}
+
+// Factors whose rank is not a width of the kernels are copied to rows of that width, zeros behind the rank.
+template <typename T>
+struct PadArgs {
+    const T *src[3];
+    T *dst[3];
+    int64_t first[4];                                   // elements of the padded factors before factor m
+    int32_t rank[3], width[3];
+};
+
+template <typename T>
+__global__ void __launch_bounds__(256) pad_factors(const __grid_constant__ PadArgs<T> a) {
+    for (int64_t e = (int64_t)blockIdx.x * 256 + threadIdx.x; e < a.first[3]; e += (int64_t)gridDim.x * 256) {
+#pragma unroll
+        for (int m = 0; m < 3; ++m)
+            if (e >= a.first[m] && e < a.first[m + 1]) {
+                const int64_t i = e - a.first[m], row = i / a.width[m];
+                const int32_t c = (int32_t)(i - row * a.width[m]);
+                a.dst[m][i] = c < a.rank[m] ? __ldg(a.src[m] + row * a.rank[m] + c) : T(0);
+            }
+    }
+}
+
+int width_of(int rank) { return rank <= 8 ? 8 : rank <= 16 ? 16 : 32; }
+
+template <typename T>
+const_status_t run_any(const const_csf *X, bool mttkrp, const void *const *factors, const int *ranks, T *out, size_t bytes,
+                       cudaStream_t stream) {
+    const int m = X->order - 1;
+    PadArgs<T> pad;
+    const T *F[3] = {nullptr, nullptr, nullptr};
+    int width[3] = {0, 0, 0};
+    int64_t total = 0;
+    bool padded = false;
+    for (int f = 0; f < 3; ++f) {
+        pad.first[f] = total;
+        pad.src[f] = nullptr;
+        pad.rank[f] = pad.width[f] = 1;
+        if (f >= m) continue;
+        F[f] = static_cast<const T *>(factors[f]);
+        width[f] = mttkrp ? (ranks[f] <= 4 ? 4 : ranks[f] <= 32 ? width_of(ranks[f]) : (ranks[f] + 31) / 32 * 32)
+                          : X->order == 4 ? 8 : width_of(ranks[f]);
+        if (width[f] == ranks[f]) continue;
+        pad.src[f] = F[f];
+        pad.rank[f] = ranks[f];
+        pad.width[f] = width[f];
+        total += X->dims[X->mode_order[f + 1]] * width[f];
+        padded = true;
+    }
+    pad.first[3] = total;
+    T *scratch = nullptr;
+    if (padded) {
+        if (scratch_alloc((void **)&scratch, sizeof(T) * total, stream) != cudaSuccess) return CONST_ERR_UNSUPPORTED;
+        for (int f = 0; f < 3; ++f) {
+            pad.dst[f] = scratch + pad.first[f];
+            if (pad.src[f]) F[f] = pad.dst[f];
+        }
+        const int blocks = (int)std::min<int64_t>((total + 255) / 256, 148 * 8);
+        CB_LAUNCH("pad_factors", stream, pad_factors<T><<<blocks, 256, 0, stream>>>(pad));
+    }
+    const_status_t rc;
+    const int rp = width[0] > 32 ? 32 : width[0];
+    if (mttkrp && X->order == 3)
+        rc = dispatch_mttkrp<T, 3>({chain_of<T, 3>(X), {F[0], F[1]}, out, width[0], ranks[0], chunk_leaves(X->nnz, 24, 4096), bytes}, rp,
+                                   width[0] / rp, stream);
+    else if (mttkrp)
+        rc = dispatch_mttkrp<T, 4>({chain_of<T, 4>(X), {F[0], F[1], F[2]}, out, width[0], ranks[0], chunk_leaves(X->nnz, 24, 4096), bytes}, rp,
+                                   width[0] / rp, stream);
+    else if (X->order == 3)
+        rc = dispatch_ttmc3<T>({chain_of<T, 3>(X), F[0], F[1], out, ranks[0], ranks[1], chunk_leaves(X->nnz, 20, 3072), bytes}, width[0], width[1],
+                               stream);
+    else
+        rc = launch_ttmc4<T>({chain_of<T, 4>(X), F[0], F[1], F[2], out, ranks[0], ranks[1], ranks[2], chunk_leaves(X->nnz, 12, 4096), bytes}, stream);
+    if (scratch) cudaFreeAsync(scratch, stream);
+    return rc;
 }
 
 }  // namespace
 
+namespace {
+__global__ void __launch_bounds__(256) clear_kernel(uint4 *out, int64_t n16, uint32_t *tail, int tail_words) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n16; i += (int64_t)gridDim.x * 256) out[i] = make_uint4(0, 0, 0, 0);
+    if (blockIdx.x == 0 && (int)threadIdx.x < tail_words) tail[threadIdx.x] = 0;
+}
+}  // namespace
+
+cudaError_t clear_result(void *out, size_t bytes, cudaStream_t stream) {
+    const int64_t n16 = (int64_t)(bytes / 16);
+    const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((n16 + 1023) / 1024, 148 * 8));
+    CB_LAUNCH("clear_result", stream,
+              clear_kernel<<<blocks, 256, 0, stream>>>(static_cast<uint4 *>(out), n16, reinterpret_cast<uint32_t *>(static_cast<uint4 *>(out) + n16),
+                                                       (int)(bytes % 16 / 4)));
+    return cudaGetLastError();
+}
+
+bool chain_covers(int order, bool mttkrp, const int *ranks) {
+    if (mttkrp) return ranks[0] <= 1024;
+    for (int f = 0; f + 1 < order; ++f)
+        if (ranks[f] > (order == 4 ? 8 : 32)) return false;
+    return true;
+}
+
+const_status_t run_chain_any(const const_csf *X, bool mttkrp, const void *const *factors, const int *ranks, const_dtype_t dtype,
+                             void *out, int64_t out_elems, cudaStream_t stream) {
+    const size_t bytes = (dtype == CONST_F32 ? 4 : 8) * (size_t)out_elems;
+    if (X->nnz == 0) return clear_result(out, bytes, stream) == cudaSuccess ? CONST_OK : CONST_ERR_CUDA;
+    return dtype == CONST_F32 ? run_any<float>(X, mttkrp, factors, ranks, (float *)out, bytes, stream)
+                              : run_any<double>(X, mttkrp, factors, ranks, (double *)out, bytes, stream);
+}
+
 const_status_t run_ttmc3(const const_csf *X, const float *U, const float *V, int R2, int R3, float *Y,
                          int64_t n_rows, int32_t *, cudaStream_t stream) {
-    switch (R2) {
-        case 8: return dispatch_ttmc3_r3<8>(X, U, V, R3, Y, n_rows, stream);
-        case 16: return dispatch_ttmc3_r3<16>(X, U, V, R3, Y, n_rows, stream);
-        case 32: return dispatch_ttmc3_r3<32>(X, U, V, R3, Y, n_rows, stream);
-    }
-    return CONST_ERR_UNSUPPORTED;
+    const size_t bytes = sizeof(float) * R2 * R3 * n_rows;
+    if (X->nnz == 0) return clear_result(Y, bytes, stream) == cudaSuccess ? CONST_OK : CONST_ERR_CUDA;
+    // Short fibres go to the record walk, whose cost is per leaf; chain3_kernel pays per fibre, but less per leaf of a long
+    // one and less to start.  Measured, walk against chain3_kernel (us): 20 M leaves in fibres of one, 16 x 16: 607 / 886;
+    // of two: 405 / 470; of four: 362 / 354; 32 x 32 in fibres of two: 939 / 880; 1 M leaves in fibres of one: 68 / 79, of
+    // two: 46 / 43.
+    const double per_fibre = (double)X->nnz / (double)X->n[1];
+    if (X->nnz < 1000000 || per_fibre > (R2 * R3 < 1024 ? 2.5 : 1.8)) return run_ttmc3_fibres(X, U, V, R2, R3, Y, n_rows, stream);
+    return dispatch_ttmc3<float>({chain_of<float, 3>(X), U, V, Y, R2, R3, chunk_leaves(X->nnz, 20, 3072), bytes}, R2, R3, stream);
 }
 
 const_status_t run_mttkrp3(const const_csf *X, const float *B, const float *C, int R, float *A, int64_t n_rows,
                            int32_t *, cudaStream_t stream) {
-    switch (R) {
-        case 8: return launch_chain3<8, 8, true>(X, B, C, A, n_rows, stream);
-        case 16: return launch_chain3<16, 16, true>(X, B, C, A, n_rows, stream);
-        case 32: return launch_chain3<32, 32, true>(X, B, C, A, n_rows, stream);
-    }
-    return CONST_ERR_UNSUPPORTED;
+    const size_t bytes = sizeof(float) * R * n_rows;
+    if (X->nnz == 0) return clear_result(A, bytes, stream) == cudaSuccess ? CONST_OK : CONST_ERR_CUDA;
+    return dispatch_mttkrp<float, 3>({chain_of<float, 3>(X), {B, C}, A, R, R, chunk_leaves(X->nnz, 32, 4096), bytes}, R, 1, stream);
+}
+
+const_status_t run_ttmc4(const const_csf *X, const float *U, const float *V, const float *W, int rank, float *Y,
+                         int64_t n_rows, int32_t *, cudaStream_t stream) {
+    if (rank != 8) return CONST_ERR_UNSUPPORTED;
+    const size_t bytes = sizeof(float) * 512 * n_rows;
+    if (X->nnz == 0) return clear_result(Y, bytes, stream) == cudaSuccess ? CONST_OK : CONST_ERR_CUDA;
+    return launch_ttmc4<float>({chain_of<float, 4>(X), U, V, W, Y, rank, rank, rank, chunk_leaves(X->nnz, 12, 4096), bytes}, stream);
 }
 
 }  // namespace cb

@@ -133,7 +133,11 @@ struct DebugKnobs {
 };
 DebugKnobs debug_knobs();
 
+// chain_kernels.cu: sets `bytes` (a multiple of 4) at the 16-byte aligned `out` to zero and lets the kernel launched next
+// start at once if its launch allows that
+cudaError_t clear_result(void *out, size_t bytes, cudaStream_t stream);
 // csf_build.cu
+cudaError_t scratch_alloc(void **p, size_t bytes, cudaStream_t stream);   // stream-ordered; release with cudaFreeAsync
 const_status_t csf_build_impl(int order, const int64_t *dims, int64_t nnz, const int32_t *const *coords_dev,
                               const void *vals_dev, const_dtype_t dtype, const int *mode_order,
                               cudaStream_t stream, const_csf **out);
@@ -150,6 +154,15 @@ const_status_t csf_build_noalloc_impl(int order, const int64_t *dims, int64_t nn
 // chain_kernels.cu
 const_status_t run_ttmc3(const const_csf *X, const float *U, const float *V, int R2, int R3, float *Y,
                          int64_t n_rows, int32_t *status, cudaStream_t stream);
+// Whether the leaf-balanced kernels take a chain of these ranks, and the chain itself at any of them, fp32 or fp64
+// (factors in level order; CONST_ERR_UNSUPPORTED when there is no memory for padded factors: nothing but the cleared
+// result has been written then).
+bool chain_covers(int order, bool mttkrp, const int *ranks);
+const_status_t run_chain_any(const const_csf *X, bool mttkrp, const void *const *factors, const int *ranks, const_dtype_t dtype,
+                             void *out, int64_t out_elems, cudaStream_t stream);
+// chain3_kernel.cu: order-3 TTMc for long fibres (X not empty)
+const_status_t run_ttmc3_fibres(const const_csf *X, const float *U, const float *V, int R2, int R3, float *Y, int64_t n_rows,
+                                cudaStream_t s);
 const_status_t run_mttkrp3(const const_csf *X, const float *B, const float *C, int R, float *A,
                            int64_t n_rows, int32_t *status, cudaStream_t stream);
 const_status_t run_ttmc4(const const_csf *X, const float *U, const float *V, const float *W, int R, float *Y,

@@ -920,6 +920,15 @@ PackArgs pack_args(int order, const int64_t *dims, const int *mode_order, const 
 // ------------------------------------------------------------------------------------------------
 // host driver
 // ------------------------------------------------------------------------------------------------
+// Temporaries of an execute.  Under stream capture the allocation becomes a node of the graph, which the device's
+// default pool provides.
+cudaError_t scratch_alloc(void **p, size_t bytes, cudaStream_t stream) {
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    const cudaError_t e = cudaStreamIsCapturing(stream, &capture);
+    if (e != cudaSuccess) return e;
+    return capture == cudaStreamCaptureStatusNone ? pool_alloc(p, bytes, stream) : cudaMallocAsync(p, bytes, stream);
+}
+
 void csf_free(const_csf *csf) {
     if (!csf) return;
     int prev = 0;

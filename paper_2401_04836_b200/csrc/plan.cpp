@@ -274,7 +274,6 @@ const_status_t match_plan(PlanDesc &p) {
         const int n = (int)mo.size();
         if (n != 3 && n != 4) return no("chain family needs a CSF tensor of order 3 or 4");
         if (m != n - 1 || (int)p.inputs.size() != n) return no("chain family needs one factor per non-root level");
-        if (p.dtype != CONST_F32) return no("chain family computes in fp32");
         const TensorRef *X = nullptr;
         for (const TensorRef &r : p.inputs) if (r.name == xname) X = &r;
         std::string lev(n, ' ');
@@ -308,9 +307,8 @@ const_status_t match_plan(PlanDesc &p) {
         else return no("rank indices must be all distinct (TTMc) or all equal (MTTKRP)");
         if (p.result.idx != want_out) return no("result must be indexed [root level, rank indices in level order]");
         for (int l = 1; l < n; ++l) {
-            int64_t r = p.extents[rank_idx[l]];
-            if (r != 8 && r != 16 && r != 32) return no("rank must be 8, 16 or 32");
-            p.ranks.push_back((int)r);
+            const int64_t r = p.extents[rank_idx[l]];
+            p.ranks.push_back(r < 0x7fffffff ? (int)r : 0x7fffffff);
         }
         // fusion depth: every intermediate keeps only what lies below the fused loops
         for (int c = 0; c + 1 < m; ++c) {
@@ -319,6 +317,12 @@ const_status_t match_plan(PlanDesc &p) {
             for (int f = 0; f < level; ++f)
                 if (p.tree[c].loops[f] != lev[f]) return no("fused loops must follow the CSF levels");
         }
+        p.sparse_name = xname;
+        p.factor_names.assign(factors.begin() + 1, factors.end());
+        p.chain = all_distinct ? PlanDesc::Chain::Ttmc : PlanDesc::Chain::Mttkrp;
+        if (p.dtype != CONST_F32) return no("chain family computes in fp32");
+        for (int r : p.ranks)
+            if (r != 8 && r != 16 && r != 32) return no("rank must be 8, 16 or 32");
         if (all_distinct && n == 3) p.family = Family::Ttmc3;
         else if (all_distinct && n == 4) {
             if (p.ranks[0] != 8 || p.ranks[1] != 8 || p.ranks[2] != 8)
@@ -326,8 +330,6 @@ const_status_t match_plan(PlanDesc &p) {
             p.family = Family::Ttmc4;
         } else if (all_same && n == 3) p.family = Family::Mttkrp3;
         else return no("MTTKRP is implemented for order 3");
-        p.sparse_name = xname;
-        p.factor_names.assign(factors.begin() + 1, factors.end());
         return CONST_OK;
     }
 

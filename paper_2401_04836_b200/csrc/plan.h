@@ -35,6 +35,7 @@ struct PlanDesc {
 
     // derived by match()
     Family family = Family::None;
+    enum class Chain { None, Ttmc, Mttkrp } chain = Chain::None;   // the schedule is a fully fused chain, whatever ranks and dtype
     std::string sparse_name;           // chain: the CSF operand; network: U
     std::string sparse2_name;          // network: W
     std::vector<std::string> factor_names;   // chain: factor of level 1, 2, (3); network: V

@@ -1,0 +1,122 @@
+"""The leaf-balanced chain kernels against the oracle: ranks around their widths, fp32 and fp64, orders 3 and 4, windows that
+end inside fibres and slices, chunks that end anywhere, and the same schedule on the generic executor."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2401_04836_b200 as cb
+from oracle import contract as oc
+from workloads import generators as gen
+from workloads import mttkrp_workload, ttmc3_workload, ttmc4_workload
+from tests.gpu_util import assert_close, build_csf, oracle, run_workload, to_dev
+
+pytestmark = pytest.mark.gpu
+NAMES = {"ttmc": "UVW", "mttkrp": "BCD"}
+
+
+def run_chain(family, dims, ranks, X, fac, dtype, generic=False):
+    """A fully fused chain over X at the given ranks; returns (output, S, A)."""
+    order, idx = len(dims), "ijkl"
+    ranked = "abc"[: order - 1] if family == "ttmc" else "r" * (order - 1)
+    ref = lambda t, letters: f"{t}[{','.join(letters)}]"
+    f = [ref(NAMES[family][m], idx[m + 1] + ranked[m]) for m in range(order - 1)]
+    out_idx = "i" + (ranked if family == "ttmc" else "r")
+    expr = f"{ref('Y', out_idx)} = {ref('X', idx[:order])} * " + " * ".join(f)
+    tree, loops, left, left_idx = [], [], "X", idx[:order]
+    for m in range(order - 2, -1, -1):
+        done = ranked[m:] if family == "ttmc" else "r"
+        name = "Y" if m == 0 else f"T{m}"
+        tree.append(f"{ref(name, idx[: m + 1] + done)} = {ref(left, left_idx)} * {f[m]}")
+        loops.append(idx[: m + 2] + done)
+        left, left_idx = name, idx[: m + 1] + done
+    ext = dict(zip(idx, dims))
+    ext.update(zip(ranked, ranks))
+    plan = cb.const_plan_create(expr, tree, {"X": tuple(range(order))}, loops, ext, dtype)
+    if generic:
+        cb.const_plan_set_generic_executor(plan, True)
+    ops = {"X": build_csf(X, tuple(range(order)))}
+    ops.update({n: to_dev(a) for n, a in fac.items()})
+    shape = (dims[0], *ranks) if family == "ttmc" else (dims[0], ranks[0])
+    out = torch.full(shape, float("nan"), dtype=torch.float32 if dtype == cb.F32 else torch.float64, device="cuda")
+    cb.const_execute(plan, ops, out)
+    assert cb.const_last_device_status(plan) == 0
+    S, A = oc.nary_einsum(expr, dict(fac, X=(X.coords, X.vals)), ext)
+    return out.cpu().numpy(), S, A
+
+
+def inputs(family, dims, ranks, nnz, dtype, seed):
+    rng = np.random.default_rng(seed)
+    np_type = np.float32 if dtype == cb.F32 else np.float64
+    X = gen._uniform_tensor(dims, nnz, rng, "pm1", np_type)
+    fac = {n: rng.standard_normal((d, r)).astype(np_type) for n, d, r in zip(NAMES[family], dims[1:], ranks)}
+    return X, fac
+
+
+@pytest.mark.parametrize("dtype", [cb.F32, cb.F64])
+@pytest.mark.parametrize("family,dims,ranks", [
+    ("ttmc", (9, 11, 300), (1, 1)), ("ttmc", (9, 11, 300), (7, 9)), ("ttmc", (40, 30, 20), (10, 12)),
+    ("ttmc", (40, 30, 20), (17, 31)), ("ttmc", (40, 30, 20), (32, 32)), ("ttmc", (3, 2, 2000), (24, 8)),
+    ("ttmc", (12, 10, 9, 8), (8, 8, 8)), ("ttmc", (12, 10, 9, 8), (3, 5, 7)), ("ttmc", (2, 3, 4, 200), (8, 1, 6)),
+    ("mttkrp", (30, 20, 25), (1,)), ("mttkrp", (30, 20, 25), (5,)), ("mttkrp", (30, 20, 25), (33,)),
+    ("mttkrp", (2, 5, 900), (70,)), ("mttkrp", (12, 10, 9, 8), (16,)), ("mttkrp", (12, 10, 9, 8), (3,)),
+    ("mttkrp", (3, 4, 5, 150), (40,)),
+])
+def test_ranks_around_the_widths(family, dims, ranks, dtype):
+    ranks = ranks if family == "ttmc" else ranks * (len(dims) - 1)
+    for nnz in (1, 31, 65, min(2500, int(np.prod(dims)))):
+        X, fac = inputs(family, dims, ranks, nnz, dtype, 7 * nnz + len(dims))
+        out, S, A = run_chain(family, dims, ranks, X, fac, dtype)
+        assert_close(out, S, A, X.vals.dtype)
+
+
+@pytest.mark.parametrize("family,dims,ranks", [("ttmc", (25, 20, 30), (6, 10)), ("mttkrp", (20, 9, 8, 7), (5, 5, 5))])
+def test_agrees_with_the_generic_executor(family, dims, ranks):
+    X, fac = inputs(family, dims, ranks, 1500, cb.F64, 3)
+    a, S, A = run_chain(family, dims, ranks, X, fac, cb.F64)
+    b, _, _ = run_chain(family, dims, ranks, X, fac, cb.F64, generic=True)
+    assert_close(a, S, A, np.float64)
+    assert_close(b, S, A, np.float64)
+
+
+@pytest.mark.parametrize("family,ranks", [("ttmc", (7, 10)), ("mttkrp", (6, 6))])
+def test_rows_a_tensor_does_not_name_stay_out(family, ranks):
+    """A factor row that no nonzero reads may hold anything: neither padding nor unused records may touch it."""
+    X, fac = inputs(family, (20, 15, 30), ranks, 700, cb.F32, 5)
+    X = gen.SparseOperand([X.coords[0], np.maximum(X.coords[1], 1), X.coords[2]], X.vals, X.dims)
+    key = np.unique(np.stack(X.coords), axis=1, return_index=True)[1]
+    X = gen.SparseOperand([np.ascontiguousarray(c[key]) for c in X.coords], np.ascontiguousarray(X.vals[key]), X.dims)
+    keep = X.coords[2] > 0
+    X = gen.SparseOperand([np.ascontiguousarray(c[keep]) for c in X.coords], np.ascontiguousarray(X.vals[keep]), X.dims)
+    clean, S, A = run_chain(family, X.dims, ranks, X, fac, cb.F32)
+    for f in fac.values():
+        f[0] = np.inf
+    dirty, _, _ = run_chain(family, X.dims, ranks, X, fac, cb.F32)
+    assert_close(dirty, S, A, np.float32)
+    assert_close(clean, S, A, np.float32)
+
+
+def test_chunks_of_a_large_skewed_tensor():
+    """Several windows per chunk, slices over many chunks and many slices per chunk; long and short fibres."""
+    for dims, nnz, inner in (((300, 4000, 900), 400_000, None), ((40, 30, 20000), 400_000, None), ((5000, 700, 800), 300_000, 0.9)):
+        w = ttmc3_workload(dims, nnz, (9, 12), slice_s=1.1, inner_s=inner, value="pm1", config_id=21)
+        out, _ = run_workload(w)
+        S, A = oracle(w)
+        assert_close(out, S, A, np.float32)
+    w = mttkrp_workload((4000, 350, 300), 300_000, 20, slice_s=1.2, value="unit", config_id=22)
+    out, _ = run_workload(w)
+    S, A = oracle(w)
+    assert_close(out, S, A, np.float32)
+    w = ttmc4_workload((300, 40, 30, 50), 200_000, 6, slice_s=1.0, value="pm1", config_id=23)
+    out, _ = run_workload(w)
+    S, A = oracle(w)
+    assert_close(out, S, A, np.float32)
+
+
+@pytest.mark.parametrize("rank", [(8, 8), (16, 16), (32, 32), (8, 32)])
+def test_short_fibres_of_a_tensor_above_a_million(rank):
+    """The size and fibre length from which order-3 TTMc at a family rank takes the record walk."""
+    w = ttmc3_workload((60, 40_000, 5000), 1_100_000, rank, slice_s=0.6, inner_s=None, value="pm1", config_id=24)
+    out, handles = run_workload(w)
+    rows = np.arange(0, 60, 7)
+    S, A = oracle(w, rows)
+    assert_close(out, S, A, np.float32, rows)
