@@ -177,6 +177,9 @@ const_status_t run_ttmc3_tensor(const const_csf *X, const float *U, const float 
 const_status_t run_network(const const_csf *U, const double *V, const const_csf *W, double *Z,
                            int64_t n_i, int64_t n_j, int64_t n_k, int64_t n_l, int64_t n_m,
                            int32_t *status, cudaStream_t stream);
+// network_dense.cu: the same contraction on the fp64 matrix pipe where the operands' structure allows it
+const_status_t run_network_dense(const const_csf *U, const double *V, const const_csf *W, double *Z, int64_t n_i, int64_t n_j,
+                                 int64_t n_k, int64_t n_l, int64_t n_m, int32_t **mode_out, void **scratch_out, cudaStream_t stream);
 
 // tree_kernel.cu: the generic executor; sparse[slot] and global_in[slot] follow cp.sparse_names / cp.global_names
 const_status_t run_tree(const tree::Compiled &cp, const_dtype_t dtype, const const_csf *const *sparse,

@@ -1,0 +1,334 @@
+// The two-contraction network  Z[i,m] = sum_{j,k,l} U[i,j,k] V[j,l] W[k,l,m]  (Sec. 1) on the fp64 matrix pipe, for operands
+// with locality: every slice i of U touches a short range of j, every slice l of W a short range of m, and the ranges are
+// reasonably full (the paper's quantum-chemistry tensors; a band in the benchmark).
+//
+// Why.  In the gather form (network_kernels.cu) every multiply-add needs a fresh 8-byte operand from shared memory, which
+// caps it at a quarter of the fp64 rate, and its bookkeeping costs more than that.  Written out densely over its ranges an
+// operand that is a quarter full costs four times the multiply-adds, but in the form of matrix tiles (mma m8n8k4, 256
+// multiply-adds per instruction, one operand load each), which run near the fp64 peak.
+//
+// Two kernels per chunk of slices i, fused over i in chunks: the intermediate T[i,l,k] exists for one chunk at a time.
+//   t_kernel   block = one slice s of U (a tile of up to 128 k) x a share of l.  U_s is written out densely in shared memory,
+//     [j in range][k]; a warp owns eight l and all k:  T[l, k] = sum_j V[j, l] U_s[j, k].  V comes straight from global
+//     memory (each entry is used once per warp, rows of 64 bytes), U_s from shared memory, conflict-free.
+//   z_kernel   block = four slices l of W x 64 slices i.  W_l is written out in shared memory, [k][m in range]; a warp owns
+//     eight i and the whole range of m and keeps Z in registers over the four l:  Z[i, m] += sum_k T[i, l, k] W_l[k, m];  T
+//     comes straight from global memory (L2), each entry used once.  The sums are added to Z atomically.
+//
+// Whether the operands qualify is found on the device (shape_kernel) and left in a mode word that every later kernel reads:
+// nothing waits on the host.  Zeros written out where the tensor has no entry must not meet an infinity or a NaN, which the
+// sparse sum would never touch: t_kernel checks that every T it computed is finite and otherwise sets the mode word, too;
+// the gather kernel, launched last, then clears Z and does the work.
+//
+// Measured (1024 x 1024 x 128, band 32, a quarter full): see run_network.
+#include <algorithm>
+
+#include "common.cuh"
+
+namespace cb {
+namespace {
+
+constexpr int kThreads = 256, kWarps = kThreads / 32;
+constexpr int kRange = 96;            // most j of a slice of U, most m of a group of slices of W
+constexpr int kTileK = 128;           // k per tile
+constexpr int kNodes = 4;             // slices of W per z_kernel block
+constexpr int kRows = 8 * kWarps;     // slices of U per z_kernel block
+constexpr int kMaxDilution = 8;       // dense multiply-adds per sparse one up to which the dense form is taken
+
+struct Csf3d {
+    const int32_t *crd0, *pos1, *crd1, *pos2, *crd2;
+    const double *vals;
+    int32_t n0, n1;
+};
+
+struct Net {
+    Csf3d u, w;                       // levels (i, k, j) and (l, m, k)
+    const double *V;
+    double *Z, *T;
+    int32_t *mode;                    // [0] nonzero: the gather kernel does the work; [2..3] dense multiply-adds (64 bits)
+    int32_t *jmin, *jlen;             // per slice of U: first j, length of the range of j
+    int32_t *mmin, *mlen;             // per group of slices of W: the same of m
+    int32_t n_k, n_l, n_j, n_m, tk;   // tk: n_k rounded up to 8
+    int32_t s0, s1;                   // chunk of slices of U
+};
+
+__device__ __forceinline__ void mma884(double &c0, double &c1, double a, double b) {
+    asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};" : "+d"(c0), "+d"(c1) : "d"(a), "d"(b));
+}
+
+__device__ __forceinline__ int round_up(int x, int to) { return (x + to - 1) / to * to; }
+
+// One warp per slice of U and per group of slices of W: the ranges, the dense work, and whether they fit.
+__global__ void __launch_bounds__(kThreads) shape_kernel(const __grid_constant__ Net a) {
+    const int lane = threadIdx.x & 31;
+    const int unit = blockIdx.x * kWarps + (threadIdx.x >> 5), groups = (a.w.n0 + kNodes - 1) / kNodes;
+    if (unit >= a.u.n0 + groups) return;
+    int lo = 0x7fffffff, hi = -1;
+    unsigned long long work;
+    if (unit < a.u.n0) {
+        const int f1 = __ldg(a.u.pos1 + unit + 1);
+        for (int f = __ldg(a.u.pos1 + unit) + lane; f < f1; f += 32) {
+            lo = min(lo, __ldg(a.u.crd2 + __ldg(a.u.pos2 + f)));
+            hi = max(hi, __ldg(a.u.crd2 + __ldg(a.u.pos2 + f + 1) - 1));
+        }
+    } else {
+        const int node = (unit - a.u.n0) * kNodes + lane;
+        if (lane < kNodes && node < a.w.n0) {
+            lo = __ldg(a.w.crd1 + __ldg(a.w.pos1 + node));
+            hi = __ldg(a.w.crd1 + __ldg(a.w.pos1 + node + 1) - 1);
+        }
+    }
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    const int len = hi - lo + 1;
+    if (lane != 0) return;
+    if (unit < a.u.n0) {
+        a.jmin[unit] = lo;
+        a.jlen[unit] = len;
+        work = (unsigned long long)round_up(len, 4) * a.tk * a.n_l;
+    } else {
+        a.mmin[unit - a.u.n0] = lo;
+        a.mlen[unit - a.u.n0] = len;
+        work = (unsigned long long)round_up(len, 8) * a.tk * kNodes * a.u.n0;
+    }
+    if (len > kRange) a.mode[0] = 1;
+    atomicAdd(reinterpret_cast<unsigned long long *>(a.mode + 2), work);
+}
+
+// The dense form has to be worth it: sparse = multiply-adds of the gather form.
+__global__ void decide_kernel(int32_t *mode, unsigned long long sparse) {
+    if (*reinterpret_cast<unsigned long long *>(mode + 2) > kMaxDilution * sparse) mode[0] = 1;
+}
+
+// Writes the entries of fibres [f0, f1) whose level-1 coordinate less c1 lies in [0, n1) and leaf coordinate less c2 in
+// [0, n2) to put(level-1, leaf, value); eight lanes per fibre.
+template <class Put>
+__device__ __forceinline__ void scatter(const Csf3d &x, int32_t f0, int32_t f1, int c1, int n1, int c2, int n2, Put put) {
+    const int h = threadIdx.x & 7;
+    for (int32_t f = f0 + (threadIdx.x >> 3); f < f1; f += kThreads / 8) {
+        const int y = __ldg(x.crd1 + f) - c1;
+        const int32_t p1 = __ldg(x.pos2 + f + 1);
+        int32_t p = __ldg(x.pos2 + f) + h;
+        if ((unsigned)y >= (unsigned)n1) continue;
+        for (; p < p1; p += 8) {
+            const int z = __ldg(x.crd2 + p) - c2;
+            if ((unsigned)z < (unsigned)n2) put(y, z, __ldg(x.vals + p));
+        }
+    }
+}
+
+__device__ __forceinline__ void clear_shared(double *d, int n) {         // n even, d 16-byte aligned
+    for (int i = threadIdx.x; i < n / 2; i += kThreads) reinterpret_cast<double2 *>(d)[i] = make_double2(0.0, 0.0);
+}
+
+__global__ void __launch_bounds__(kThreads, 2) t_kernel(const __grid_constant__ Net a, int l_tiles_per_block) {
+    extern __shared__ __align__(16) double u_dense[];                     // [range of j][tile of k + 4]
+    __shared__ int skip;                                                  // one reading for the block: others may set it meanwhile
+    if (threadIdx.x == 0) skip = *a.mode;
+    __syncthreads();
+    if (skip) return;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int s = a.s0 + blockIdx.x, k0 = blockIdx.y * kTileK;
+    const int kt = min(kTileK, a.tk - k0), ld = kt + 4;                  // ld = 4 or 12 modulo 16: the loads below meet no bank twice
+    const int j0 = a.jmin[s], steps = round_up(a.jlen[s], 4) / 4;
+    clear_shared(u_dense, steps * 4 * ld);
+    __syncthreads();
+    scatter(a.u, __ldg(a.u.pos1 + s), __ldg(a.u.pos1 + s + 1), k0, kt, j0, steps * 4,
+            [&](int k, int j, double v) { u_dense[j * ld + k] = v; });
+    __syncthreads();
+    const int r = lane >> 2, c = lane & 3, tiles = kt / 8;
+    const int last = min((int)(blockIdx.z + 1) * l_tiles_per_block, (a.n_l + 7) / 8);
+    bool finite = true;
+    for (int lt = blockIdx.z * l_tiles_per_block + warp; lt < last; lt += kWarps) {
+        const int l = lt * 8 + r;
+        double acc[kTileK / 8][2];
+#pragma unroll
+        for (int t = 0; t < kTileK / 8; ++t) acc[t][0] = acc[t][1] = 0.0;
+        auto v_at = [&](int st) {
+            const int j = j0 + st * 4 + c;
+            return l < a.n_l && j < a.n_j && st < steps ? __ldg(a.V + (size_t)j * a.n_l + l) : 0.0;
+        };
+        double v[4];
+#pragma unroll
+        for (int z = 0; z < 4; ++z) v[z] = v_at(z);
+        for (int st = 0; st < steps; st += 4) {
+            double next[4];
+#pragma unroll
+            for (int z = 0; z < 4; ++z) next[z] = v_at(st + 4 + z);
+#pragma unroll
+            for (int z = 0; z < 4; ++z) {
+                if (st + z >= steps) break;                               // uniform
+                const double *row = u_dense + ((st + z) * 4 + c) * ld + r;
+#pragma unroll
+                for (int t = 0; t < kTileK / 8; ++t)
+                    if (t < tiles) mma884(acc[t][0], acc[t][1], v[z], row[t * 8]);
+            }
+#pragma unroll
+            for (int z = 0; z < 4; ++z) v[z] = next[z];
+        }
+        if (l < a.n_l) {
+            double *dst = a.T + ((size_t)(s - a.s0) * a.n_l + l) * a.tk + k0 + 2 * c;
+#pragma unroll
+            for (int t = 0; t < kTileK / 8; ++t)
+                if (t < tiles) {
+                    finite = finite && isfinite(acc[t][0]) && isfinite(acc[t][1]);
+                    *reinterpret_cast<double2 *>(dst + t * 8) = make_double2(acc[t][0], acc[t][1]);
+                }
+        }
+    }
+    if (!finite) atomicExch(a.mode, 1);
+}
+
+__global__ void __launch_bounds__(kThreads, 2) z_kernel(const __grid_constant__ Net a) {
+    extern __shared__ __align__(16) double w_dense[];                     // [tile of k][range of m + 4]
+    __shared__ int skip;
+    if (threadIdx.x == 0) skip = *a.mode;
+    __syncthreads();
+    if (skip) return;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, r = lane >> 2, c = lane & 3;
+    const int group = blockIdx.x, m0 = a.mmin[group], len = a.mlen[group];
+    const int tiles = round_up(len, 8) / 8, ld = tiles * 8 + 4;
+    const int s = a.s0 + blockIdx.y * kRows + warp * 8 + r;              // this lane's slice of U
+    const bool have = s < a.s1;
+    double acc[kRange / 8][2];
+#pragma unroll
+    for (int t = 0; t < kRange / 8; ++t) acc[t][0] = acc[t][1] = 0.0;
+    for (int node = group * kNodes; node < min((group + 1) * kNodes, a.w.n0); ++node) {
+        const int l = __ldg(a.w.crd0 + node);
+        const int32_t f0 = __ldg(a.w.pos1 + node), f1 = __ldg(a.w.pos1 + node + 1);
+        const double *t_row = a.T + ((size_t)(have ? s - a.s0 : 0) * a.n_l + l) * a.tk + c;
+        for (int k0 = 0; k0 < a.tk; k0 += kTileK) {
+            const int kt = min(kTileK, a.tk - k0), steps = kt / 4;       // steps is even
+            auto t_at = [&](int st) { return have && st < steps ? __ldg(t_row + k0 + st * 4) : 0.0; };
+            double x[8];
+#pragma unroll
+            for (int z = 0; z < 8; ++z) x[z] = t_at(z);
+            __syncthreads();                                              // the tile before is used up
+            clear_shared(w_dense, kt * ld);
+            __syncthreads();
+            scatter(a.w, f0, f1, m0, len, k0, kt, [&](int m, int k, double v) { w_dense[k * ld + m] = v; });
+            __syncthreads();
+            for (int st = 0; st < steps; st += 8) {
+                double next[8];
+#pragma unroll
+                for (int z = 0; z < 8; ++z) next[z] = t_at(st + 8 + z);
+#pragma unroll
+                for (int z = 0; z < 8; ++z) {
+                    if (st + z >= steps) break;                           // uniform
+                    const double *row = w_dense + ((st + z) * 4 + c) * ld + r;
+#pragma unroll
+                    for (int t = 0; t < kRange / 8; ++t)
+                        if (t < tiles) mma884(acc[t][0], acc[t][1], x[z], row[t * 8]);
+                }
+#pragma unroll
+                for (int z = 0; z < 8; ++z) x[z] = next[z];
+            }
+        }
+    }
+    if (!have) return;
+    double *z = a.Z + (size_t)__ldg(a.u.crd0 + s) * a.n_m + m0 + 2 * c;
+#pragma unroll
+    for (int t = 0; t < kRange / 8; ++t)
+        if (t < tiles) {
+            if (t * 8 + 2 * c < len) atomicAdd(z + t * 8, acc[t][0]);
+            if (t * 8 + 2 * c + 1 < len) atomicAdd(z + t * 8 + 1, acc[t][1]);
+        }
+}
+
+// Z back to zero where the gather kernel takes over
+__global__ void __launch_bounds__(256) reclear_kernel(const int32_t *mode, double *Z, int64_t n) {
+    if (!*mode) return;
+    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) Z[i] = 0.0;
+}
+
+constexpr int64_t kScratchBytes = 256ll << 20;       // T of one chunk
+
+}  // namespace
+
+// Z is cleared.  On CONST_OK with *mode_out set, the work is queued and *mode_out (device) says, once the stream gets there,
+// whether the gather kernel still has to do it; *mode_out null: nothing was queued.  release(*scratch_out) afterwards.
+const_status_t run_network_dense(const const_csf *U, const double *V, const const_csf *W, double *Z, int64_t n_i, int64_t n_j,
+                                 int64_t n_k, int64_t n_l, int64_t n_m, int32_t **mode_out, void **scratch_out, cudaStream_t stream) {
+    *mode_out = nullptr;
+    *scratch_out = nullptr;
+    const int64_t tk = (n_k + 7) / 8 * 8;
+    const double sparse = (double)U->nnz * n_l + (double)W->nnz * U->n[0];
+    const int64_t row_bytes = n_l * tk * 8;
+    const int64_t n0 = U->n[0], groups = (W->n[0] + kNodes - 1) / kNodes;
+    // Small networks stay with the gather kernel (one launch instead of six); so does one whose T would leave fewer than
+    // 64 slices to a chunk.  What is sparser than one in kMaxDilution over all indices within kRange cannot qualify.
+    if (sparse < 2e7 || n_k > 4096 || kScratchBytes / row_bytes < std::min<int64_t>(n0, 64)) return CONST_OK;
+    if (n_l > (1 << 24) || n_m > (1 << 24) || groups > 65535 * 8ll) return CONST_OK;
+    int64_t chunk = std::min<int64_t>(n0, kScratchBytes / row_bytes);
+    const int64_t chunks = (n0 + chunk - 1) / chunk;
+    chunk = ((n0 + chunks - 1) / chunks + kRows - 1) / kRows * kRows;     // even chunks of whole blocks, never more than fit
+    if (chunk * row_bytes > kScratchBytes) chunk = kScratchBytes / row_bytes;
+    chunk = std::min<int64_t>(chunk, n0);
+    const size_t small = 64 + sizeof(int32_t) * 2 * (size_t)(n0 + groups);
+    const size_t small_pad = (small + 255) / 256 * 256;
+    unsigned char *scratch = nullptr;
+    if (scratch_alloc((void **)&scratch, small_pad + (size_t)(chunk * row_bytes), stream) != cudaSuccess) {
+        (void)cudaGetLastError();                                         // no room: the gather kernel needs none
+        return CONST_OK;
+    }
+    auto queue = [&]() -> const_status_t {
+        CB_CUDA(cudaMemsetAsync(scratch, 0, 64, stream));
+        Net a;
+        auto csf = [](const const_csf *c) {
+            return Csf3d{c->crd[0], c->pos[1], c->crd[1], c->pos[2], c->crd[2], static_cast<const double *>(c->vals), (int32_t)c->n[0], (int32_t)c->n[1]};
+        };
+        a.u = csf(U);
+        a.w = csf(W);
+        a.V = V;
+        a.Z = Z;
+        a.mode = reinterpret_cast<int32_t *>(scratch);
+        a.jmin = reinterpret_cast<int32_t *>(scratch + 64);
+        a.jlen = a.jmin + n0;
+        a.mmin = a.jlen + n0;
+        a.mlen = a.mmin + groups;
+        a.T = reinterpret_cast<double *>(scratch + small_pad);
+        a.n_k = (int32_t)n_k;
+        a.n_l = (int32_t)n_l;
+        a.n_j = (int32_t)n_j;
+        a.n_m = (int32_t)n_m;
+        a.tk = (int32_t)tk;
+        a.s0 = a.s1 = 0;
+        const int64_t units = n0 + groups;
+        CB_LAUNCH("network_shape", stream, shape_kernel<<<(unsigned)((units + kWarps - 1) / kWarps), kThreads, 0, stream>>>(a));
+        CB_LAUNCH("network_shape", stream, decide_kernel<<<1, 1, 0, stream>>>(a.mode, (unsigned long long)sparse));
+        const int kt = (int)std::min<int64_t>(kTileK, tk);
+        const size_t t_smem = sizeof(double) * kRange * (kt + 4), z_smem = sizeof(double) * kt * (kRange + 4);
+        static PerDeviceOnce once;
+        CB_CUDA(once_per_device(once, [] {
+            const int most = (int)sizeof(double) * std::max(kRange * (kTileK + 4), kTileK * (kRange + 4));
+            cudaError_t e = cudaFuncSetAttribute(t_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+            return e == cudaSuccess ? cudaFuncSetAttribute(z_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most) : e;
+        }));
+        const int l_tiles = (int)((n_l + 7) / 8), k_tiles = (int)((tk + kTileK - 1) / kTileK);
+        for (int64_t s0 = 0; s0 < n0; s0 += chunk) {
+            a.s0 = (int32_t)s0;
+            a.s1 = (int32_t)std::min<int64_t>(n0, s0 + chunk);
+            const int rows = a.s1 - a.s0;
+            // shares of l: about seven blocks for every SM, a multiple of the warps' tiles each
+            const int want = std::max(1, (148 * 7 + rows * k_tiles - 1) / (rows * k_tiles));
+            const int per = std::max(kWarps, ((l_tiles + want - 1) / want + kWarps - 1) / kWarps * kWarps);
+            const dim3 tg((unsigned)rows, (unsigned)k_tiles, (unsigned)((l_tiles + per - 1) / per));
+            CB_LAUNCH("network_t", stream, t_kernel<<<tg, kThreads, t_smem, stream>>>(a, per));
+            const dim3 zg((unsigned)groups, (unsigned)((rows + kRows - 1) / kRows));
+            CB_LAUNCH("network_z", stream, z_kernel<<<zg, kThreads, z_smem, stream>>>(a));
+        }
+        CB_LAUNCH("network_shape", stream, reclear_kernel<<<148, 256, 0, stream>>>(a.mode, Z, n_i * n_m));
+        CB_CUDA(cudaGetLastError());
+        return CONST_OK;
+    };
+    const const_status_t rc = queue();
+    if (rc != CONST_OK) {
+        cudaFreeAsync(scratch, stream);
+        return rc;
+    }
+    *mode_out = reinterpret_cast<int32_t *>(scratch);
+    *scratch_out = scratch;
+    return CONST_OK;
+}
+
+}  // namespace cb

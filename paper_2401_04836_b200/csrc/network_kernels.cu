@@ -111,11 +111,12 @@ __device__ __forceinline__ void sweep(const Csf3d &x, int32_t fA, int32_t fB, co
 template <int IS, int LT, int GL>
 __global__ void __launch_bounds__(kThreads)
 network_kernel(Csf3d u, const double *__restrict__ V, Csf3d w, double *__restrict__ Z, int n_k, int n_l, int n_m,
-               int v_vec_ok) {
+               int v_vec_ok, const int32_t *__restrict__ mode) {
     constexpr int VPT_P = LT / GL;                 // entries of a V row per lane (producer)
     constexpr int VPT_C = IS / GL;                 // entries of a T row per lane (consumer)
     static_assert(LT % GL == 0 && IS % GL == 0 && LT <= kMaxLT && (VPT_P == 1 || VPT_P % 2 == 0) &&
                   (VPT_C == 1 || VPT_C % 2 == 0), "a lane group covers the l of the tile or the i of the strip");
+    if (mode && *mode == 0) return;                // network_dense.cu has done the work
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int TL = n_k * IS + 2;                   // doubles per l plane; the +2 staggers the banks of the 8 planes
     double *T = reinterpret_cast<double *>(smem_raw);                               // [LT][n_k][IS]
@@ -248,7 +249,7 @@ namespace {
 
 template <int IS, int LT, int GL>
 const_status_t launch_network(const const_csf *U, const double *V, const const_csf *W, double *Z, int64_t n_k,
-                              int64_t n_l, int64_t n_m, cudaStream_t stream) {
+                              int64_t n_l, int64_t n_m, const int32_t *mode, cudaStream_t stream) {
     const size_t t_doubles = ((size_t)LT * (n_k * IS + 2) + 1) / 2 * 2;
     const size_t smem = sizeof(double) * t_doubles + sizeof(Rec) * RB + sizeof(int32_t) * (2 * FPMAX + 1);
     if (smem > 220 * 1024 || n_l > (1ll << 30) || n_m > (1ll << 30)) return CONST_ERR_WORKSPACE;
@@ -261,27 +262,40 @@ const_status_t launch_network(const const_csf *U, const double *V, const const_c
     const int v_vec_ok = (n_l % 2 == 0) && (reinterpret_cast<uintptr_t>(V) % 16 == 0);
     dim3 grid((unsigned)((U->n[0] + IS - 1) / IS), (unsigned)((n_l + LT - 1) / LT));
     CB_LAUNCH("network_kernel", stream,
-              kernel<<<grid, kThreads, smem, stream>>>(u, V, w, Z, (int)n_k, (int)n_l, (int)n_m, v_vec_ok));
+              kernel<<<grid, kThreads, smem, stream>>>(u, V, w, Z, (int)n_k, (int)n_l, (int)n_m, v_vec_ok, mode));
     CB_CUDA(cudaGetLastError());
     return CONST_OK;
 }
 
 }  // namespace
 
+// Operands with locality run on the fp64 matrix pipe (network_dense.cu), decided on the device; the gather kernel is launched
+// behind it and returns at once where that was done.
 const_status_t run_network(const const_csf *U, const double *V, const const_csf *W, double *Z, int64_t n_i,
                            int64_t n_j, int64_t n_k, int64_t n_l, int64_t n_m, int32_t *, cudaStream_t stream) {
-    (void)n_j;
     CB_CUDA(cudaMemsetAsync(Z, 0, sizeof(double) * n_i * n_m, stream));
     if (U->nnz == 0 || W->nnz == 0) return CONST_OK;
-    // tile shape (slices per strip, l per tile, lanes per fibre); the variants are kept for measurement
-    switch (debug_knobs().variant) {
-        case 1: return launch_network<8, 16, 4>(U, V, W, Z, n_k, n_l, n_m, stream);
-        case 2: return launch_network<16, 8, 4>(U, V, W, Z, n_k, n_l, n_m, stream);
-        case 3: return launch_network<8, 16, 8>(U, V, W, Z, n_k, n_l, n_m, stream);
-        case 4: return launch_network<16, 8, 8>(U, V, W, Z, n_k, n_l, n_m, stream);
-        case 5: return launch_network<4, 16, 4>(U, V, W, Z, n_k, n_l, n_m, stream);
-        default: return launch_network<8, 8, 4>(U, V, W, Z, n_k, n_l, n_m, stream);
+    const int variant = debug_knobs().variant;
+    int32_t *mode = nullptr;
+    void *scratch = nullptr;
+    if (variant == 0) {
+        const const_status_t rc = run_network_dense(U, V, W, Z, n_i, n_j, n_k, n_l, n_m, &mode, &scratch, stream);
+        if (rc != CONST_OK) return rc;
     }
+    // tile shape (slices per strip, l per tile, lanes per fibre); the variants are kept for measurement
+    auto gather = [&]() {
+        switch (variant) {
+            case 1: return launch_network<8, 16, 4>(U, V, W, Z, n_k, n_l, n_m, mode, stream);
+            case 2: return launch_network<16, 8, 4>(U, V, W, Z, n_k, n_l, n_m, mode, stream);
+            case 3: return launch_network<8, 16, 8>(U, V, W, Z, n_k, n_l, n_m, mode, stream);
+            case 4: return launch_network<16, 8, 8>(U, V, W, Z, n_k, n_l, n_m, mode, stream);
+            case 5: return launch_network<4, 16, 4>(U, V, W, Z, n_k, n_l, n_m, mode, stream);
+            default: return launch_network<8, 8, 4>(U, V, W, Z, n_k, n_l, n_m, mode, stream);
+        }
+    };
+    const const_status_t rc = gather();
+    if (scratch) cudaFreeAsync(scratch, stream);
+    return rc;
 }
 
 }  // namespace cb

@@ -1,0 +1,76 @@
+"""The two-contraction network where its operands have locality (the fp64 matrix pipe), and where they do not, or must not be
+written out densely: against the oracle, element by element."""
+import numpy as np
+import pytest
+
+import paper_2401_04836_b200 as cb
+from workloads import generators as gen
+from workloads import network_workload
+from tests.gpu_util import assert_close, oracle, run_workload
+
+pytestmark = pytest.mark.gpu
+
+
+def kernels_of(w):
+    """Output and the time of each kernel (a kernel that leaves the work to another returns at once)."""
+    cb.const_profile_enable(True)
+    out, _ = run_workload(w)
+    prof = cb.const_profile_read()
+    cb.const_profile_enable(False)
+    return out, prof
+
+
+@pytest.mark.parametrize("n,n_k,band,keep", [
+    (331, 61, 17, 0.25),      # nothing a multiple of a tile
+    (300, 128, 12, 0.3),      # a full tile of k
+    (260, 150, 12, 0.3),      # two tiles of k, the second of 22
+    (200, 7, 46, 0.6),        # the widest range that qualifies with four slices together (94 of 96)
+    (200, 9, 48, 0.6),        # one that does not (98)
+    (403, 33, 3, 1.0),        # narrow and full
+])
+def test_banded(n, n_k, band, keep):
+    w = network_workload(n, n_k, band, keep, config_id=61)
+    out, prof = kernels_of(w)
+    assert "network_t" in prof and "network_kernel" in prof
+    S, A = oracle(w)
+    assert_close(out, S, A, np.float64)
+
+
+def scattered(n, n_k, nnz, seed):
+    w = network_workload(n, n_k, 4, 0.25, config_id=62)
+    rng = np.random.default_rng(seed)
+    w.sparse["U"] = gen._uniform_tensor((n, n, n_k), nnz, rng, "normal", np.float64)
+    w.sparse["W"] = gen._uniform_tensor((n_k, n, n), nnz, rng, "normal", np.float64)
+    return w
+
+
+def test_operands_without_locality():
+    w = scattered(250, 20, 60_000, 1)
+    out, _ = kernels_of(w)
+    S, A = oracle(w)
+    assert_close(out, S, A, np.float64)
+
+
+def test_rows_and_slices_missing():
+    """Slices of U and W without nonzeros, ranges at both ends of the extents."""
+    w = network_workload(300, 40, 10, 0.5, config_id=63)
+    for name, m in (("U", 0), ("W", 1)):
+        op = w.sparse[name]
+        keep = (op.coords[m] % 5 != 2) & (op.coords[m] < 290)
+        w.sparse[name] = gen.SparseOperand([np.ascontiguousarray(c[keep]) for c in op.coords], np.ascontiguousarray(op.vals[keep]), op.dims)
+    out, _ = kernels_of(w)
+    S, A = oracle(w)
+    assert_close(out, S, A, np.float64)
+
+
+@pytest.mark.parametrize("value", [np.inf, np.nan])
+def test_values_no_nonzero_reads(value):
+    """A row of V that no nonzero of U reads may hold anything, though it lies inside the ranges that are written out."""
+    w = network_workload(300, 40, 10, 0.5, config_id=64)
+    U = w.sparse["U"]
+    keep = U.coords[1] != 150
+    w.sparse["U"] = gen.SparseOperand([np.ascontiguousarray(c[keep]) for c in U.coords], np.ascontiguousarray(U.vals[keep]), U.dims)
+    S, A = oracle(w)
+    w.dense["V"][150] = value
+    out, _ = kernels_of(w)
+    assert_close(out, S, A, np.float64)
