@@ -48,6 +48,7 @@ struct Net {
     int32_t *mode;                    // [0] nonzero: the gather kernel does the work; [2..3] dense multiply-adds (64 bits)
     int32_t *jmin, *jlen;             // per slice of U: first j, length of the range of j
     int32_t *mmin, *mlen;             // per group of slices of W: the same of m
+    uint32_t *u_place, *w_place;      // per entry (place_kernel)
     int32_t n_k, n_l, n_j, n_m, tk;   // tk: n_k rounded up to 8
     int32_t s0, s1;                   // chunk of slices of U
 };
@@ -100,22 +101,57 @@ __global__ void decide_kernel(int32_t *mode, unsigned long long sparse) {
     if (*reinterpret_cast<unsigned long long *>(mode + 2) > kMaxDilution * sparse) mode[0] = 1;
 }
 
-// Writes the entries of fibres [f0, f1) whose level-1 coordinate less c1 lies in [0, n1) and leaf coordinate less c2 in
-// [0, n2) to put(level-1, leaf, value); eight lanes per fibre.
-template <class Put>
-__device__ __forceinline__ void scatter(const Csf3d &x, int32_t f0, int32_t f1, int c1, int n1, int c2, int n2, Put put) {
+// Where every entry goes when its slice is written out: (place in the range) << 12 | k.  One block per slice, eight lanes per
+// fibre.  The kernels below write a slice out many times (once per share of l, once per 64 slices of U); with the place
+// beside the value they do it from two coalesced streams, without walking the fibres.
+__global__ void __launch_bounds__(kThreads) place_kernel(const __grid_constant__ Net a) {
+    if (*a.mode) return;
+    const bool of_u = (int)blockIdx.x < a.u.n0;
+    const int node = of_u ? blockIdx.x : blockIdx.x - a.u.n0;
+    const Csf3d &x = of_u ? a.u : a.w;
+    const int32_t f1 = __ldg(x.pos1 + node + 1);
+    const int first = of_u ? a.jmin[node] : a.mmin[node / kNodes];
+    uint32_t *to = of_u ? a.u_place : a.w_place;
     const int h = threadIdx.x & 7;
-    for (int32_t f = f0 + (threadIdx.x >> 3); f < f1; f += kThreads / 8) {
-        const int y = __ldg(x.crd1 + f) - c1;
+    for (int32_t f = __ldg(x.pos1 + node) + (threadIdx.x >> 3); f < f1; f += kThreads / 8) {
+        const uint32_t y = __ldg(x.crd1 + f);                             // k of a U fibre, m of a W fibre
         const int32_t p1 = __ldg(x.pos2 + f + 1);
-        int32_t p = __ldg(x.pos2 + f) + h;
-        if ((unsigned)y >= (unsigned)n1) continue;
-        for (; p < p1; p += 8) {
-            const int z = __ldg(x.crd2 + p) - c2;
-            if ((unsigned)z < (unsigned)n2) put(y, z, __ldg(x.vals + p));
+        for (int32_t p = __ldg(x.pos2 + f) + h; p < p1; p += 8) {
+            const uint32_t z = __ldg(x.crd2 + p);
+            to[p] = of_u ? (z - first) << 12 | y : (y - first) << 12 | z;
         }
     }
 }
+
+constexpr int kAhead = 8;             // entries per thread requested ahead of their use
+
+struct Entries {                      // this thread's entries p, p + kThreads, ... below `end` of a slice
+    uint32_t place[kAhead];
+    double v[kAhead];
+    int32_t p, end;
+    __device__ __forceinline__ void request(const uint32_t *places, const double *vals, int32_t first, int32_t last) {
+        p = first + threadIdx.x;
+        end = last;
+#pragma unroll
+        for (int q = 0; q < kAhead; ++q) {
+            const int32_t at = p + q * kThreads;
+            place[q] = at < end ? __ldg(places + at) : 0xffffffffu;
+            v[q] = at < end ? __ldg(vals + at) : 0.0;
+        }
+    }
+    // put(place in the range, k - k0, value) for the entries of tile [k0, k0 + kt)
+    template <class Put>
+    __device__ __forceinline__ void write(const uint32_t *places, const double *vals, int k0, int kt, Put put) const {
+        auto one = [&](uint32_t pl, double val) {
+            const int k = (int)(pl & 4095u) - k0;
+            if ((unsigned)k < (unsigned)kt) put((int)(pl >> 12), k, val);
+        };
+#pragma unroll
+        for (int q = 0; q < kAhead; ++q)
+            if (p + q * kThreads < end) one(place[q], v[q]);
+        for (int32_t at = p + kAhead * kThreads; at < end; at += kThreads) one(__ldg(places + at), __ldg(vals + at));
+    }
+};
 
 __device__ __forceinline__ void clear_shared(double *d, int n) {         // n even, d 16-byte aligned
     for (int i = threadIdx.x; i < n / 2; i += kThreads) reinterpret_cast<double2 *>(d)[i] = make_double2(0.0, 0.0);
@@ -131,11 +167,14 @@ __global__ void __launch_bounds__(kThreads, 2) t_kernel(const __grid_constant__ 
     const int s = a.s0 + blockIdx.x, k0 = blockIdx.y * kTileK;
     const int kt = min(kTileK, a.tk - k0), ld = kt + 4;                  // ld = 4 or 12 modulo 16: the loads below meet no bank twice
     const int j0 = a.jmin[s], steps = round_up(a.jlen[s], 4) / 4;
-    clear_shared(u_dense, steps * 4 * ld);
-    __syncthreads();
-    scatter(a.u, __ldg(a.u.pos1 + s), __ldg(a.u.pos1 + s + 1), k0, kt, j0, steps * 4,
-            [&](int k, int j, double v) { u_dense[j * ld + k] = v; });
-    __syncthreads();
+    {
+        Entries e;
+        e.request(a.u_place, a.u.vals, __ldg(a.u.pos2 + __ldg(a.u.pos1 + s)), __ldg(a.u.pos2 + __ldg(a.u.pos1 + s + 1)));
+        clear_shared(u_dense, steps * 4 * ld);
+        __syncthreads();
+        e.write(a.u_place, a.u.vals, k0, kt, [&](int j, int k, double v) { u_dense[j * ld + k] = v; });
+        __syncthreads();
+    }
     const int r = lane >> 2, c = lane & 3, tiles = kt / 8;
     const int last = min((int)(blockIdx.z + 1) * l_tiles_per_block, (a.n_l + 7) / 8);
     bool finite = true;
@@ -193,27 +232,33 @@ __global__ void __launch_bounds__(kThreads, 2) z_kernel(const __grid_constant__ 
     double acc[kRange / 8][2];
 #pragma unroll
     for (int t = 0; t < kRange / 8; ++t) acc[t][0] = acc[t][1] = 0.0;
-    for (int node = group * kNodes; node < min((group + 1) * kNodes, a.w.n0); ++node) {
+    const int n0 = group * kNodes, n1 = min(n0 + kNodes, a.w.n0);
+    int32_t leaf = __ldg(a.w.pos2 + __ldg(a.w.pos1 + n0));
+    for (int node = n0; node < n1; ++node) {
         const int l = __ldg(a.w.crd0 + node);
-        const int32_t f0 = __ldg(a.w.pos1 + node), f1 = __ldg(a.w.pos1 + node + 1);
+        const int32_t leaf1 = __ldg(a.w.pos2 + __ldg(a.w.pos1 + node + 1));
         const double *t_row = a.T + ((size_t)(have ? s - a.s0 : 0) * a.n_l + l) * a.tk + c;
         for (int k0 = 0; k0 < a.tk; k0 += kTileK) {
             const int kt = min(kTileK, a.tk - k0), steps = kt / 4;       // steps is even
             auto t_at = [&](int st) { return have && st < steps ? __ldg(t_row + k0 + st * 4) : 0.0; };
-            double x[8];
+            double x[4];
+            {
+                Entries e;
+                e.request(a.w_place, a.w.vals, leaf, leaf1);
 #pragma unroll
-            for (int z = 0; z < 8; ++z) x[z] = t_at(z);
-            __syncthreads();                                              // the tile before is used up
-            clear_shared(w_dense, kt * ld);
-            __syncthreads();
-            scatter(a.w, f0, f1, m0, len, k0, kt, [&](int m, int k, double v) { w_dense[k * ld + m] = v; });
-            __syncthreads();
-            for (int st = 0; st < steps; st += 8) {
-                double next[8];
+                for (int z = 0; z < 4; ++z) x[z] = t_at(z);
+                __syncthreads();                                          // the tile before is used up
+                clear_shared(w_dense, kt * ld);
+                __syncthreads();
+                e.write(a.w_place, a.w.vals, k0, kt, [&](int m, int k, double v) { w_dense[k * ld + m] = v; });
+                __syncthreads();
+            }
+            for (int st = 0; st < steps; st += 4) {
+                double next[4];
 #pragma unroll
-                for (int z = 0; z < 8; ++z) next[z] = t_at(st + 8 + z);
+                for (int z = 0; z < 4; ++z) next[z] = t_at(st + 4 + z);
 #pragma unroll
-                for (int z = 0; z < 8; ++z) {
+                for (int z = 0; z < 4; ++z) {
                     if (st + z >= steps) break;                           // uniform
                     const double *row = w_dense + ((st + z) * 4 + c) * ld + r;
 #pragma unroll
@@ -221,9 +266,10 @@ __global__ void __launch_bounds__(kThreads, 2) z_kernel(const __grid_constant__ 
                         if (t < tiles) mma884(acc[t][0], acc[t][1], x[z], row[t * 8]);
                 }
 #pragma unroll
-                for (int z = 0; z < 8; ++z) x[z] = next[z];
+                for (int z = 0; z < 4; ++z) x[z] = next[z];
             }
         }
+        leaf = leaf1;
     }
     if (!have) return;
     double *z = a.Z + (size_t)__ldg(a.u.crd0 + s) * a.n_m + m0 + 2 * c;
@@ -264,7 +310,7 @@ const_status_t run_network_dense(const const_csf *U, const double *V, const cons
     chunk = ((n0 + chunks - 1) / chunks + kRows - 1) / kRows * kRows;     // even chunks of whole blocks, never more than fit
     if (chunk * row_bytes > kScratchBytes) chunk = kScratchBytes / row_bytes;
     chunk = std::min<int64_t>(chunk, n0);
-    const size_t small = 64 + sizeof(int32_t) * 2 * (size_t)(n0 + groups);
+    const size_t small = 64 + sizeof(int32_t) * (2 * (size_t)(n0 + groups) + (size_t)(U->nnz + W->nnz));
     const size_t small_pad = (small + 255) / 256 * 256;
     unsigned char *scratch = nullptr;
     if (scratch_alloc((void **)&scratch, small_pad + (size_t)(chunk * row_bytes), stream) != cudaSuccess) {
@@ -286,6 +332,8 @@ const_status_t run_network_dense(const const_csf *U, const double *V, const cons
         a.jlen = a.jmin + n0;
         a.mmin = a.jlen + n0;
         a.mlen = a.mmin + groups;
+        a.u_place = reinterpret_cast<uint32_t *>(a.mlen + groups);
+        a.w_place = a.u_place + U->nnz;
         a.T = reinterpret_cast<double *>(scratch + small_pad);
         a.n_k = (int32_t)n_k;
         a.n_l = (int32_t)n_l;
@@ -296,6 +344,7 @@ const_status_t run_network_dense(const const_csf *U, const double *V, const cons
         const int64_t units = n0 + groups;
         CB_LAUNCH("network_shape", stream, shape_kernel<<<(unsigned)((units + kWarps - 1) / kWarps), kThreads, 0, stream>>>(a));
         CB_LAUNCH("network_shape", stream, decide_kernel<<<1, 1, 0, stream>>>(a.mode, (unsigned long long)sparse));
+        CB_LAUNCH("network_shape", stream, place_kernel<<<(unsigned)(n0 + W->n[0]), kThreads, 0, stream>>>(a));
         const int kt = (int)std::min<int64_t>(kTileK, tk);
         const size_t t_smem = sizeof(double) * kRange * (kt + 4), z_smem = sizeof(double) * kt * (kRange + 4);
         static PerDeviceOnce once;
