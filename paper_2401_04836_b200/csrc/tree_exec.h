@@ -24,6 +24,7 @@ namespace tree {
 constexpr int kMaxIdx = 16, kMaxLoops = 24, kMaxStmts = 12, kMaxSparse = 6, kMaxDense = 20, kMaxInstr = 96;
 constexpr int kMaxRefIdx = 6, kMaxPriv = 6, kMaxFollow = 3, kMaxLevels = 4;
 constexpr int kThreads = 256;
+constexpr int kExclusiveExtent = 32;   // innermost dense extent from which a group of threads has enough to do per iteration of Q
 
 enum RefKind : int8_t { kRefSparse = 0, kRefGlobal = 1, kRefPrivate = 2 };
 
@@ -63,6 +64,13 @@ struct Stmt {
     int8_t fast;
     int32_t sA[3], sB[3];          // out, lhs, rhs
     int8_t pA[3], pB[3];
+    // The result is private to the group, the two loops dealt as one both index it, and the loop Q around them locates
+    // nothing: then Q and the loops outside it run in step in all threads, the fused pair is dealt to the whole group, and
+    // no two threads touch one element between two barriers, so results are updated without atomics (shared memory has
+    // none in fp64: an atomic addition there is a compare-and-swap loop).  References are affine in Q, too (sQ, pQ).
+    int8_t exclusive;
+    int8_t pQ[3];
+    int32_t sQ[3];
 };
 
 enum Op : int8_t { kOpLoopBegin = 0, kOpLoopEnd = 1, kOpZero = 2, kOpStmt = 3 };
@@ -109,6 +117,7 @@ struct Compiled {
     std::vector<int64_t> root_extent;                      // per program: extent of the root index (dense root loop)
     std::string index_names;                               // index id -> letter
     std::vector<std::vector<std::string>> stmt_text;       // per program, per statement: the assignment as it stands in the tree
+    std::vector<std::vector<int64_t>> ws_elems;            // per program, per private workspace: its elements (without row padding)
     std::vector<std::vector<std::string>> ws_text;         // per program, per private workspace: its reduced reference
     std::string error;
 };

@@ -127,8 +127,9 @@ __device__ void run_statement(const Stmt &s, const Program &p, const Bindings &b
     const int m = fuse ? n - 1 : n;
     const int32_t inner_extent = fuse ? p.loops[s.priv[n - 1]].extent : 1;
     int32_t cur[kMaxPriv], end[kMaxPriv];
-    auto first = [&](int d) { return m == 1 ? G::tid() : d == 0 ? warp : d == 1 ? lane : 0; };
-    auto step = [&](int d) { return m == 1 ? G::size() : d == 0 ? warps : d == 1 ? 32 : 1; };
+    const bool exclusive = s.exclusive != 0;
+    auto first = [&](int d) { return exclusive ? 0 : m == 1 ? G::tid() : d == 0 ? warp : d == 1 ? lane : 0; };
+    auto step = [&](int d) { return exclusive ? 1 : m == 1 ? G::size() : d == 0 ? warps : d == 1 ? 32 : 1; };
     auto open = [&](int d) {                                        // range of dealt loop d (not the innermost) under the current bindings
         loop_range(p.loops[s.priv[d]], b, st, cur[d], end[d]);
         cur[d] += first(d);
@@ -198,8 +199,70 @@ __device__ void run_statement(const Stmt &s, const Program &p, const Bindings &b
             for (int32_t it = lo + f; it < hi; it += stp) one(0, 0, it, crdA ? crdA[it] : it);
         }
     };
+    // ---- exclusive: loop Q in step, the pair below it dealt to the whole group, plain updates between barriers
+    auto in_step = [&]() {
+        const Loop &LQ = p.loops[s.priv[n - 3]], &LA = p.loops[s.priv[n - 2]];
+        int32_t q0, q1, lo = 0, hi = 0;
+        loop_range(LQ, b, st, q0, q1);
+        const bool below = LA.driver >= 0 && LA.driver == LQ.driver && LA.level == LQ.level + 1;
+        if (!below) loop_range(LA, b, st, lo, hi);
+        st.idx[LQ.index] = st.idx[LA.index] = st.idx[p.loops[s.priv[n - 1]].index] = 0;
+        const Ref *refs[3] = {&s.out, &s.lhs, &s.rhs};
+        const T *ptr[3];
+        int64_t base[3];
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+            const Ref &ref = *refs[r];
+            if (ref.kind == kRefSparse) {
+                const SparsePtrs &sp = b.sp[ref.slot];
+                ptr[r] = static_cast<const T *>(sp.vals);
+                base[r] = (s.pA[r] | s.pB[r] | s.pQ[r]) ? 0 : st.node[ref.slot][sp.order - 1];
+            } else {
+                ptr[r] = ref.kind == kRefPrivate ? scratch + p.ws[ref.slot].offset : static_cast<const T *>(b.global[ref.slot]);
+                base[r] = address<T>(ref, st);
+            }
+        }
+        T *dst = const_cast<T *>(ptr[0]);
+        const int32_t *crdQ = LQ.driver >= 0 ? b.sp[LQ.driver].crd[LQ.level] : nullptr;
+        const int32_t *crdA = LA.driver >= 0 ? b.sp[LA.driver].crd[LA.level] : nullptr;
+        const int32_t *posA = below ? b.sp[LA.driver].pos[LA.level] : nullptr;
+        const int32_t f = G::tid(), stp = G::size();
+        const int32_t fa = f / inner_extent, fb = f % inner_extent, da = stp / inner_extent, db = stp % inner_extent;
+        // coordinate and range of the next iteration are requested one iteration ahead
+        int32_t next_c = q0, next_hi = hi;
+        if (q0 < q1) {
+            if (crdQ) next_c = crdQ[q0];
+            if (below) { hi = posA[q0]; next_hi = posA[q0 + 1]; }
+        }
+        for (int32_t q = q0; q < q1; ++q) {
+            const int32_t cq = next_c;
+            if (below) { lo = hi; hi = next_hi; }
+            next_c = q + 1;
+            if (q + 1 < q1) {
+                if (crdQ) next_c = crdQ[q + 1];
+                if (below) next_hi = posA[q + 2];
+            }
+            int64_t bq[3];
+#pragma unroll
+            for (int r = 0; r < 3; ++r) bq[r] = base[r] + (int64_t)cq * s.sQ[r] + (int64_t)q * s.pQ[r];
+            int32_t qb = fb;
+            for (int32_t itA = lo + fa; itA < hi;) {
+                const int32_t cA = crdA ? crdA[itA] : itA;
+                int64_t at[3];
+#pragma unroll
+                for (int r = 0; r < 3; ++r) at[r] = bq[r] + (int64_t)cA * s.sA[r] + (int64_t)qb * s.sB[r] + (int64_t)itA * s.pA[r];
+                dst[at[0]] += ptr[1][at[1]] * ptr[2][at[2]];
+                itA += da;
+                qb += db;
+                if (qb >= inner_extent) { qb -= inner_extent; ++itA; }
+            }
+            G::sync();
+        }
+    };
     if (m == 1) {
         innermost();
+    } else if (exclusive && m == 2) {
+        in_step();
     } else {
         int d = 0;
         open(0);
@@ -213,7 +276,10 @@ __device__ void run_statement(const Stmt &s, const Program &p, const Bindings &b
                 cur[d] += step(d);
                 continue;
             }
-            if (d == m - 2) {
+            if (exclusive && d == m - 3) {
+                in_step();
+                ++cur[d];
+            } else if (d == m - 2) {
                 innermost();
                 cur[d] += step(d);
             } else {

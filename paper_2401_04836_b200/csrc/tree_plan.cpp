@@ -148,10 +148,23 @@ struct Compiler {
         for (int k = ref.n - 1; k >= 0; --k) {
             ref.idx[k] = (int8_t)idx_id.at(t.addr_idx[(size_t)k]);
             ref.stride[k] = (int32_t)stride;
-            stride *= extent(t.addr_idx[(size_t)k]);
+            stride *= k + 1 == ref.n ? row_length(r.name) : extent(t.addr_idx[(size_t)k]);
         }
         (void)p;
         return true;
+    }
+
+    // Entries from one row of a tensor to the next (its last index runs along a row).  The rows of a workspace in shared
+    // memory are made odd, so that threads that walk down a column meet different banks (64 x 64 in fp64: all of them met
+    // the same one); not where that could change who executes an iteration or where its workspaces live (run_tree).
+    int64_t row_length(const std::string &name) const {
+        const TensorInfo &t = tensors.at(name);
+        const int64_t n = extent(t.addr_idx.back());
+        if (t.kind != TensorInfo::PrivateWs || t.addr_idx.size() < 2 || n < 16 || elems(t.addr_idx) <= 1024) return n;
+        int64_t bytes = 0;
+        for (const auto &o : tensors)
+            if (o.second.kind == TensorInfo::PrivateWs) bytes += elems(o.second.addr_idx) * (d.dtype == CONST_F32 ? 4 : 8);
+        return bytes <= 88 * 1024 ? n | 1 : n;
     }
 
     // ---- how one forall iterates ----
@@ -219,6 +232,7 @@ struct Compiler {
         int n_loops = 0, n_stmts = 0;
         std::map<int, int> ws_id;         // producing contraction -> workspace id of this program
         std::vector<std::string> stmt_text, ws_text;
+        std::vector<int64_t> ws_elems;
     };
 
     static std::string show(const TensorRef &r) {
@@ -294,6 +308,25 @@ struct Compiler {
                 }
             }
         }
+        if (s.fast && s.fuse_tail && s.n_priv >= 3 && s.out.kind == kRefPrivate) {
+            const Loop &LB = e.p.loops[s.priv[s.n_priv - 1]], &LA = e.p.loops[s.priv[s.n_priv - 2]], &LQ = e.p.loops[s.priv[s.n_priv - 3]];
+            bool has_a = false, has_b = false;
+            for (int x = 0; x < s.out.n; ++x) {
+                has_a = has_a || s.out.idx[x] == LA.index;
+                has_b = has_b || s.out.idx[x] == LB.index;
+            }
+            s.exclusive = has_a && has_b && LQ.n_follow == 0 && LB.extent >= kExclusiveExtent;
+            const TensorRef *names[3] = {&k.out, &k.lhs, &k.rhs};
+            const Ref *refs[3] = {&s.out, &s.lhs, &s.rhs};
+            for (int r = 0; r < 3; ++r) {
+                const Ref &ref = *refs[r];
+                if (ref.kind == kRefSparse)
+                    s.pQ[r] = LQ.driver == ref.slot && LQ.level == (int)tensors.at(names[r]->name).levels.size() - 1;
+                else
+                    for (int x = 0; x < ref.n; ++x)
+                        if (ref.idx[x] == LQ.index) s.sQ[r] = ref.stride[x];
+            }
+        }
         const Contraction &rk = tree.reduced[c];
         e.stmt_text.push_back(show(rk.out) + " += " + show(rk.lhs) + " * " + show(rk.rhs));
         int at;
@@ -329,7 +362,9 @@ struct Compiler {
             if (tensors.at(d.tree[c].out.name).kind == TensorInfo::PrivateWs) {
                 const int id = (int)e.ws_id.size();
                 e.ws_id[c] = id;
-                const int64_t n = elems(tree.reduced[c].out.idx);
+                const std::string &idx = tree.reduced[c].out.idx;
+                const int64_t n = idx.empty() ? 1 : elems(idx) / extent(idx.back()) * row_length(d.tree[c].out.name);
+                e.ws_elems.push_back(elems(idx));
                 e.p.ws[id] = Workspace{e.p.block_scratch, n};
                 e.ws_text.push_back(show(tree.reduced[c].out));
                 e.p.block_scratch += (n + 1) / 2 * 2;           // keeps 16-byte alignment for fp64
@@ -388,6 +423,7 @@ struct Compiler {
         out.root_flattened.push_back(e.p.root_loop2 >= 0);
         out.stmt_text.push_back(e.stmt_text);
         out.ws_text.push_back(e.ws_text);
+        out.ws_elems.push_back(e.ws_elems);
         return true;
     }
 
@@ -431,7 +467,7 @@ std::string describe(const Compiled &c) {
                 text += "loop " + loop_text(p.loops[in.arg]) + "\n";
                 ++depth;
             } else if (in.op == kOpZero) {
-                text += "zero " + c.ws_text[r][(size_t)in.arg] + " (" + std::to_string(p.ws[in.arg].size) + " elements per iteration in flight)\n";
+                text += "zero " + c.ws_text[r][(size_t)in.arg] + " (" + std::to_string(c.ws_elems[r][(size_t)in.arg]) + " elements per iteration in flight)\n";
             } else {
                 const Stmt &st = p.stmts[in.arg];
                 text += c.stmt_text[r][(size_t)in.arg];
