@@ -182,23 +182,36 @@ __global__ void __launch_bounds__(kRsThreads, 3) rs_onesweep(const uint64_t *__r
     // Rank inside the warp: keys with equal digits keep their order (item, lane).  The lanes holding
     // another digit are collected from one ballot per digit bit (the match instruction costs one
     // round per distinct value in the warp, which for random digits is far slower).
+    // In pairs: the ballots of both, then both counter additions, then the ranks, so that the additions' round trips overlap
+    // (77 M keys: 569 -> 559 us a pass; four at a time 566, eight 568: registers.  Lane words built with atomicOr instead of
+    // ballots: 647).
     int rank[kRsItems];
+    constexpr int kBatch = 2;
 #pragma unroll
-    for (int i = 0; i < kRsItems; ++i) {
-        const unsigned dg = (unsigned)(key[i] >> shift) & kDigitMask;
-        unsigned other = 0;
+    for (int i0 = 0; i0 < kRsItems; i0 += kBatch) {
+        unsigned peers[kBatch];
+        uint32_t old[kBatch];
 #pragma unroll
-        for (int b = 0; b < BITS; ++b) {
-            const bool bit = (dg >> b) & 1u;
-            const unsigned m = __ballot_sync(0xffffffffu, bit);
-            other |= bit ? ~m : m;                                     // lanes whose bit b differs from mine
+        for (int z = 0; z < kBatch; ++z) {
+            const unsigned dg = (unsigned)(key[i0 + z] >> shift) & kDigitMask;
+            unsigned other = 0;
+#pragma unroll
+            for (int b = 0; b < BITS; ++b) {
+                const bool bit = (dg >> b) & 1u;
+                const unsigned m = __ballot_sync(0xffffffffu, bit);
+                other |= bit ? ~m : m;                                 // lanes whose bit b differs from mine
+            }
+            peers[z] = ~other;
         }
-        const unsigned peers = ~other;
-        const int leader = __ffs(peers) - 1;
-        uint32_t old = 0;
-        if (lane == leader) old = atomicAdd(&warp_hist[warp][dg], (uint32_t)__popc(peers));
-        old = __shfl_sync(0xffffffffu, old, leader);
-        rank[i] = (int)old + __popc(peers & ((1u << lane) - 1u));
+#pragma unroll
+        for (int z = 0; z < kBatch; ++z) {
+            const unsigned dg = (unsigned)(key[i0 + z] >> shift) & kDigitMask;
+            old[z] = 0;
+            if ((peers[z] & ((1u << lane) - 1u)) == 0) old[z] = atomicAdd(&warp_hist[warp][dg], (uint32_t)__popc(peers[z]));
+        }
+#pragma unroll
+        for (int z = 0; z < kBatch; ++z)
+            rank[i0 + z] = (int)__shfl_sync(0xffffffffu, old[z], __ffs(peers[z]) - 1) + __popc(peers[z] & ((1u << lane) - 1u));
     }
     __syncthreads();
 
