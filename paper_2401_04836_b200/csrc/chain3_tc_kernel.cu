@@ -298,6 +298,8 @@ const_status_t run_ttmc3_tensor(const const_csf *X, const float *U, const float 
     if (R2 != R || R3 != R) return CONST_ERR_UNSUPPORTED;
     CB_CUDA(cudaMemsetAsync(Y, 0, sizeof(float) * TILE * n_rows, stream));
     if (X->nnz == 0) return CONST_OK;
+    const const_status_t bins = csf_ensure_bins(const_cast<const_csf *>(X), stream);
+    if (bins != CONST_OK) return bins;
     Csf3 x{X->crd[0], X->pos[1], X->crd[1], X->pos[2], X->crd[2], static_cast<const float *>(X->vals)};
     constexpr size_t dyn = kWarpBytes * kWarps;
     const DebugKnobs knobs = debug_knobs();

@@ -51,8 +51,12 @@ struct const_csf {
     int32_t *pos[cb::kMaxOrder] = {nullptr, nullptr, nullptr, nullptr};
     int32_t *crd[cb::kMaxOrder] = {nullptr, nullptr, nullptr, nullptr};
     void *vals = nullptr;
-    // load balancing
+    unsigned char *arena = nullptr;    // pos, crd and slice_ptr live in this one allocation
     int32_t *slice_ptr = nullptr;      // [n0 + 1] leaf offset of every root-level slice
+    // load balancing: built on first use (csf_ensure_bins)
+    std::mutex bins_mu;
+    bool bins_valid = false;
+    cudaEvent_t bins_ready = nullptr;  // recorded behind the binning: other streams wait for it
     int32_t *light_list = nullptr;     // [n0] slice ids handled one per warp (the first n_light entries are used)
     cb::WorkItem *items = nullptr;     // [item_cap] (the first n_items entries are used)
     int32_t *bin_scratch = nullptr;    // [2 * (n0 + 1) + 8 + 64] scan outputs, size-class bases and fill counters
@@ -144,6 +148,7 @@ const_status_t csf_build_impl(int order, const int64_t *dims, int64_t nnz, const
 const_status_t csf_from_dense_impl(int order, const int64_t *dims, const void *dense, const_dtype_t dtype,
                                    const int *mode_order, cudaStream_t stream, const_csf **out);
 const_status_t csf_rebin(const_csf *csf, cudaStream_t stream);
+const_status_t csf_ensure_bins(const_csf *csf, cudaStream_t stream);
 const_status_t csf_bin_totals(const_csf *csf);      // fills the host copies n_light .. n_items (waits for the device once)
 void csf_free(const_csf *csf);
 const_status_t csf_build_noalloc_impl(int order, const int64_t *dims, int64_t nnz, const int32_t *const *coords_dev,

@@ -44,12 +44,48 @@ constexpr int kMaxPasses = 8;
 // in as few passes as possible.
 struct DigitPlan { int shift[kMaxPasses]; int bits[kMaxPasses]; int passes; };
 
+// True in the block that is the last of its grid to arrive (`arrived` starts at zero); what the other blocks wrote before
+// is visible to it.
+__device__ __forceinline__ bool last_block(uint32_t *arrived) {
+    __shared__ bool last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(arrived, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (last) __threadfence();
+    return last;
+}
+
+// Exclusive scan of one number per thread over a block of 256; the block's total in `total`.
+__device__ __forceinline__ uint32_t block_scan(uint32_t v, uint32_t &total) {
+    __shared__ uint32_t sums[8];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t inc = v;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const uint32_t t = __shfl_up_sync(0xffffffffu, inc, off);
+        if (lane >= off) inc += t;
+    }
+    __syncthreads();                                  // the sums of a scan before are used up
+    if (lane == 31) sums[warp] = inc;
+    __syncthreads();
+    uint32_t before = 0;
+    total = 0;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) {
+        if (w < warp) before += sums[w];
+        total += sums[w];
+    }
+    return before + inc - v;
+}
+
 // Pack the permuted coordinates of every nonzero into its 64-bit sort key (range-checked) and, in the
 // same read, count the digits of every radix pass.  Per-block counts live in shared memory and are
-// flushed once; the grid is sized to a few blocks per SM so the flush stays small.
+// flushed once; the grid is sized to a few blocks per SM so the flush stays small.  The last block to
+// finish turns every pass's counts into exclusive offsets.
 template <int ORDER>
 __global__ void __launch_bounds__(256) pack_hist(PackArgs a, int64_t nnz, DigitPlan dp, uint64_t *__restrict__ keys,
-                                                 uint32_t *__restrict__ hist, int32_t *status) {
+                                                 uint32_t *hist, int32_t *status, uint32_t *arrived) {
     extern __shared__ uint32_t sh[];                 // [passes][kRsMaxBins]
     for (int x = threadIdx.x; x < dp.passes * kRsMaxBins; x += blockDim.x) sh[x] = 0;
     __syncthreads();
@@ -75,16 +111,24 @@ __global__ void __launch_bounds__(256) pack_hist(PackArgs a, int64_t nnz, DigitP
     __syncthreads();
     for (int x = threadIdx.x; x < dp.passes * kRsMaxBins; x += blockDim.x)
         if (sh[x]) atomicAdd(&hist[x], sh[x]);
+    if (!last_block(arrived)) return;
+    for (int p = 0; p < dp.passes; ++p) {
+        uint2 *h = reinterpret_cast<uint2 *>(hist + p * kRsMaxBins) + threadIdx.x;       // two digits per thread
+        const uint2 c = __ldcg(h);
+        uint32_t total;
+        const uint32_t before = block_scan(c.x + c.y, total);
+        *h = make_uint2(before, before + c.x);
+    }
 }
 
 inline void launch_pack_hist(const PackArgs &pa, int64_t nnz, const DigitPlan &dp, uint64_t *keys, uint32_t *hist,
-                             int32_t *status, cudaStream_t stream) {
+                             int32_t *status, uint32_t *arrived, cudaStream_t stream) {
     const int blocks = (int)std::min<int64_t>((nnz + 255) / 256, 148 * 8);
     const size_t sm = sizeof(uint32_t) * kRsMaxBins * std::max(dp.passes, 1);
     switch (pa.order) {
-        case 2: pack_hist<2><<<blocks, 256, sm, stream>>>(pa, nnz, dp, keys, hist, status); break;
-        case 3: pack_hist<3><<<blocks, 256, sm, stream>>>(pa, nnz, dp, keys, hist, status); break;
-        default: pack_hist<4><<<blocks, 256, sm, stream>>>(pa, nnz, dp, keys, hist, status); break;
+        case 2: pack_hist<2><<<blocks, 256, sm, stream>>>(pa, nnz, dp, keys, hist, status, arrived); break;
+        case 3: pack_hist<3><<<blocks, 256, sm, stream>>>(pa, nnz, dp, keys, hist, status, arrived); break;
+        default: pack_hist<4><<<blocks, 256, sm, stream>>>(pa, nnz, dp, keys, hist, status, arrived); break;
     }
 }
 
@@ -107,20 +151,6 @@ constexpr unsigned kFlagOwn = 1u, kFlagPrefix = 2u;
 
 __device__ __forceinline__ unsigned long long status_word(unsigned epoch, unsigned flag, uint32_t count) {
     return ((unsigned long long)((epoch << 2) | flag) << 32) | count;
-}
-
-// Exclusive scan of each pass's digit histogram: one block per pass.
-__global__ void __launch_bounds__(256) rs_scan_hist(uint32_t *hist) {
-    __shared__ uint32_t sh[kRsMaxBins];
-    uint32_t *h = hist + blockIdx.x * kRsMaxBins;
-    for (int x = threadIdx.x; x < kRsMaxBins; x += blockDim.x) sh[x] = h[x];
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        uint32_t run = 0;
-        for (int d = 0; d < kRsMaxBins; ++d) { uint32_t c = sh[d]; sh[d] = run; run += c; }
-    }
-    __syncthreads();
-    for (int x = threadIdx.x; x < kRsMaxBins; x += blockDim.x) h[x] = sh[x];
 }
 
 // One radix pass over BITS key bits.  Thread t owns digits t, t + 256, ... (DPT of them).
@@ -366,8 +396,9 @@ __global__ void __launch_bounds__(kRsThreads, 3) rs_onesweep(const uint64_t *__r
 // compression: flags -> counts -> scan -> scatter
 // ------------------------------------------------------------------------------------------------
 constexpr int kCpThreads = 256;
-constexpr int kCpIters = 8;                                   // 32-element steps per warp
-constexpr int kCpTile = kCpThreads * kCpIters;                // 2048 elements per block
+constexpr int kCpSteps = 4;                                   // 64-element steps per warp
+constexpr int kCpTile = kCpThreads * kCpSteps * 2;            // 2048 elements per block
+constexpr int kCpScanBlocks = 4096;                           // up to so many blocks the count kernel scans its own counts
 constexpr int kCpLevels = kMaxOrder - 1;                      // levels that need a scan (all but the leaf level)
 constexpr int kCpAheadTiles = 592;                            // L2 prefetch distance of the one-shot tile kernels (half a wave)
 
@@ -380,63 +411,84 @@ __device__ __forceinline__ void prefetch_tile_ahead(const uint64_t *__restrict__
 
 struct LevelShifts { int shift[kMaxOrder]; int order; };
 
-// ballots of "opens a new node at level l" for the 32 elements starting at `base`
-__device__ __forceinline__ void node_flags(const uint64_t *__restrict__ keys, int64_t n, int64_t base, int lane,
-                                           const LevelShifts &ls, uint64_t &key, unsigned ballots[kCpLevels],
-                                           bool &dup) {
-    int64_t e = base + lane;
-    bool in = e < n;
-    key = in ? keys[e] : 0ull;
-    uint64_t prev = __shfl_up_sync(0xffffffffu, key, 1);
-    if (lane == 0 && in && e > 0) prev = keys[e - 1];
-    bool first = (e == 0);
-    dup = in && !first && key == prev;
+// The 256 consecutive keys of a warp, two neighbours per lane and step (16-byte loads, all requested before the first is
+// used), and the key in front of them.
+struct WarpKeys {
+    ulonglong2 k[kCpSteps];
+    uint64_t carry;
+    int64_t base;
+    __device__ __forceinline__ void load(const uint64_t *__restrict__ keys, int64_t n, int64_t warp_base, int lane) {
+        base = warp_base;
+        carry = warp_base > 0 && warp_base <= n ? __ldg(keys + warp_base - 1) : 0ull;
 #pragma unroll
-    for (int l = 0; l < kCpLevels; ++l) {
-        bool f = false;
-        if (l < ls.order - 1) f = in && (first || (key >> ls.shift[l]) != (prev >> ls.shift[l]));
-        ballots[l] = __ballot_sync(0xffffffffu, f);
+        for (int it = 0; it < kCpSteps; ++it) {
+            const int64_t e = warp_base + it * 64 + 2 * lane;
+            k[it] = make_ulonglong2(0ull, 0ull);
+            if (e + 1 < n) k[it] = __ldg(reinterpret_cast<const ulonglong2 *>(keys + e));
+            else if (e < n) k[it].x = __ldg(keys + e);
+        }
     }
-}
-
-// the same flags from a key the caller already holds; `carry` = the element before `base` (unused when base == 0)
-__device__ __forceinline__ void node_flags_of(int64_t n, int64_t base, int lane, const LevelShifts &ls, uint64_t key,
-                                              uint64_t carry, unsigned ballots[kCpLevels]) {
-    const int64_t e = base + lane;
-    const bool in = e < n;
-    uint64_t prev = __shfl_up_sync(0xffffffffu, key, 1);
-    if (lane == 0) prev = carry;
-    const bool first = (e == 0);
-#pragma unroll
-    for (int l = 0; l < kCpLevels; ++l) {
-        bool f = false;
-        if (l < ls.order - 1) f = in && (first || (key >> ls.shift[l]) != (prev >> ls.shift[l]));
-        ballots[l] = __ballot_sync(0xffffffffu, f);
+    // the key in front of this lane's first key of step `it`
+    __device__ __forceinline__ uint64_t before(int it, int lane) const {
+        uint64_t prev = __shfl_up_sync(0xffffffffu, k[it].y, 1);
+        const uint64_t last = it > 0 ? __shfl_sync(0xffffffffu, k[it > 0 ? it - 1 : 0].y, 31) : carry;
+        return lane == 0 ? last : prev;
     }
-}
+};
 
+// Per-block node counts of every level; with few blocks the last one to finish also scans them (launch_csf_count).
+template <int ORDER>
 __global__ void __launch_bounds__(kCpThreads) csf_count(const uint64_t *__restrict__ keys, int64_t n, LevelShifts ls,
-                                                       uint32_t *__restrict__ block_counts, int32_t *status) {
+                                                       uint32_t *block_counts, int32_t *status, uint32_t *totals, uint32_t *arrived) {
     __shared__ uint32_t sh[kCpLevels];
     if (threadIdx.x < kCpLevels) sh[threadIdx.x] = 0;
     prefetch_tile_ahead(keys, n);
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint32_t cnt[kCpLevels] = {0, 0, 0};
-    bool any_dup = false;
-    for (int it = 0; it < kCpIters; ++it) {
-        int64_t base = (int64_t)blockIdx.x * kCpTile + (warp * kCpIters + it) * 32;
-        uint64_t key; unsigned b[kCpLevels]; bool dup;
-        node_flags(keys, n, base, lane, ls, key, b, dup);
-        any_dup |= dup;
+    WarpKeys w;
+    w.load(keys, n, (int64_t)blockIdx.x * kCpTile + warp * kCpSteps * 64, lane);
+    uint32_t cnt[ORDER - 1] = {};
+    bool dup = false;
 #pragma unroll
-        for (int l = 0; l < kCpLevels; ++l) cnt[l] += __popc(b[l]);
+    for (int it = 0; it < kCpSteps; ++it) {
+        const uint64_t prev = w.before(it, lane);
+        const int64_t e = w.base + it * 64 + 2 * lane;
+        const bool in0 = e < n, in1 = e + 1 < n, first = e == 0;
+        dup = dup || (in0 && !first && w.k[it].x == prev) || (in1 && w.k[it].y == w.k[it].x);
+#pragma unroll
+        for (int l = 0; l < ORDER - 1; ++l)
+            cnt[l] += (in0 && (first || (w.k[it].x >> ls.shift[l]) != (prev >> ls.shift[l]))) +
+                      (in1 && (w.k[it].y >> ls.shift[l]) != (w.k[it].x >> ls.shift[l]));
     }
-    if (any_dup) report(status, CONST_ERR_DUPLICATE_COORD);
-    if (lane == 0)
-        for (int l = 0; l < kCpLevels; ++l) atomicAdd(&sh[l], cnt[l]);
+    if (dup) report(status, CONST_ERR_DUPLICATE_COORD);
+#pragma unroll
+    for (int l = 0; l < ORDER - 1; ++l) {
+        const uint32_t c = __reduce_add_sync(0xffffffffu, cnt[l]);
+        if (lane == 0) atomicAdd(&sh[l], c);
+    }
     __syncthreads();
     if (threadIdx.x < kCpLevels) block_counts[(int64_t)blockIdx.x * kCpLevels + threadIdx.x] = sh[threadIdx.x];
+    if (!totals || !last_block(arrived)) return;
+    constexpr int PER = kCpScanBlocks / kCpThreads;                 // consecutive blocks per thread
+#pragma unroll
+    for (int l = 0; l < kCpLevels; ++l) {
+        uint32_t c[PER], mine = 0;
+#pragma unroll
+        for (int k = 0; k < PER; ++k) {
+            const int b = threadIdx.x * PER + k;
+            c[k] = b < (int)gridDim.x ? __ldcg(block_counts + b * kCpLevels + l) : 0;
+            mine += c[k];
+        }
+        uint32_t total;
+        uint32_t run = block_scan(mine, total);
+#pragma unroll
+        for (int k = 0; k < PER; ++k) {
+            const int b = threadIdx.x * PER + k;
+            if (b < (int)gridDim.x) block_counts[b * kCpLevels + l] = run;
+            run += c[k];
+        }
+        if (threadIdx.x == 0) totals[l] = total;
+    }
 }
 
 // In-place exclusive scan of the per-block counts, in two launches: every scan block adds up its chunk of
@@ -528,76 +580,115 @@ struct CsfArrays {
     int bits[kMaxOrder];
 };
 
-// ORDER is a template parameter so that the per-level arrays are indexed by constants and stay in registers.
+// ORDER is a template parameter so that the per-level arrays are indexed by constants and stay in registers.  The thread
+// that holds the last element closes the pos arrays; slice_ptr (may be null) receives the first leaf of every slice.
 template <int ORDER>
 __global__ void __launch_bounds__(kCpThreads) csf_scatter(const uint64_t *__restrict__ keys, int64_t n, LevelShifts ls,
-                                                         const uint32_t *__restrict__ block_base, CsfArrays out) {
-    __shared__ uint32_t wcnt[kCpThreads / 32][kCpLevels];
+                                                         const uint32_t *__restrict__ block_base, CsfArrays out,
+                                                         int32_t *__restrict__ slice_ptr) {
+    constexpr int L = ORDER - 1;                                    // levels that need a scan; L is the leaf level
+    __shared__ uint32_t wcnt[kCpThreads / 32][L];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     prefetch_tile_ahead(keys, n);
-    uint64_t key[kCpIters];
-    unsigned bal[kCpIters][kCpLevels];
-    uint32_t cnt[kCpLevels] = {0, 0, 0};
-    // the warp's kCpIters * 32 consecutive keys and the one in front of them, all requested before the first is used
-    const int64_t warp_base = (int64_t)blockIdx.x * kCpTile + (int64_t)warp * kCpIters * 32;
-    uint64_t carry = warp_base > 0 && warp_base <= n ? keys[warp_base - 1] : 0ull;
+    WarpKeys w;
+    w.load(keys, n, (int64_t)blockIdx.x * kCpTile + warp * kCpSteps * 64, lane);
+    unsigned b0[kCpSteps][L], b1[kCpSteps][L];                      // nodes opened by the lanes' first and second element
+    uint32_t cnt[L] = {};
 #pragma unroll
-    for (int it = 0; it < kCpIters; ++it) {
-        const int64_t e = warp_base + it * 32 + lane;
-        key[it] = e < n ? keys[e] : 0ull;
-    }
+    for (int it = 0; it < kCpSteps; ++it) {
+        const uint64_t prev = w.before(it, lane);
+        const int64_t e = w.base + it * 64 + 2 * lane;
 #pragma unroll
-    for (int it = 0; it < kCpIters; ++it) {
-        node_flags_of(n, warp_base + it * 32, lane, ls, key[it], carry, bal[it]);
-        carry = __shfl_sync(0xffffffffu, key[it], 31);
-#pragma unroll
-        for (int l = 0; l < kCpLevels; ++l) cnt[l] += __popc(bal[it][l]);
+        for (int l = 0; l < L; ++l) {
+            b0[it][l] = __ballot_sync(0xffffffffu, e < n && (e == 0 || (w.k[it].x >> ls.shift[l]) != (prev >> ls.shift[l])));
+            b1[it][l] = __ballot_sync(0xffffffffu, e + 1 < n && (w.k[it].y >> ls.shift[l]) != (w.k[it].x >> ls.shift[l]));
+            cnt[l] += __popc(b0[it][l]) + __popc(b1[it][l]);
+        }
     }
     if (lane == 0)
-        for (int l = 0; l < kCpLevels; ++l) wcnt[warp][l] = cnt[l];
+#pragma unroll
+        for (int l = 0; l < L; ++l) wcnt[warp][l] = cnt[l];
     __syncthreads();
-    uint32_t run[kCpLevels];
+    uint32_t run[L];
 #pragma unroll
-    for (int l = 0; l < kCpLevels; ++l) {
+    for (int l = 0; l < L; ++l) {
         run[l] = block_base[(int64_t)blockIdx.x * kCpLevels + l];
-        for (int w = 0; w < warp; ++w) run[l] += wcnt[w][l];
+        for (int v = 0; v < warp; ++v) run[l] += wcnt[v][l];
     }
-    constexpr int leaf = ORDER - 1;
     const unsigned below = (1u << lane) - 1u;
+    const uint64_t leaf_mask = (1ull << out.bits[L]) - 1ull;
+    const bool pairs = (reinterpret_cast<uintptr_t>(out.crd[L]) & 7u) == 0;     // a caller's array may start anywhere
 #pragma unroll
-    for (int it = 0; it < kCpIters; ++it) {
-        int64_t e = (int64_t)blockIdx.x * kCpTile + (warp * kCpIters + it) * 32 + lane;
-        if (e < n) {
-            uint32_t id[kMaxOrder];
+    for (int it = 0; it < kCpSteps; ++it) {
+        const int64_t e = w.base + it * 64 + 2 * lane;
+        const uint64_t key[2] = {w.k[it].x, w.k[it].y};
+        const int2 leaf = make_int2((int32_t)((key[0] >> ls.shift[L]) & leaf_mask), (int32_t)((key[1] >> ls.shift[L]) & leaf_mask));
+        if (pairs && e + 1 < n) {
+            *reinterpret_cast<int2 *>(out.crd[L] + e) = leaf;
+        } else {
+            if (e < n) out.crd[L][e] = leaf.x;
+            if (e + 1 < n) out.crd[L][e + 1] = leaf.y;
+        }
+        uint32_t opened[L];                                          // nodes opened in front of the element
 #pragma unroll
-            for (int l = 0; l < kCpLevels; ++l) id[l] = run[l] + __popc(bal[it][l] & below);
-            id[leaf] = (uint32_t)e;
-            out.crd[leaf][e] = (int32_t)((key[it] >> ls.shift[leaf]) & ((1ull << out.bits[leaf]) - 1ull));
+        for (int l = 0; l < L; ++l) opened[l] = run[l] + __popc(b0[it][l] & below) + __popc(b1[it][l] & below);
 #pragma unroll
-            for (int l = 0; l < kCpLevels; ++l) {
-                if (l < leaf && ((bal[it][l] >> lane) & 1u)) {
-                    out.crd[l][id[l]] = (int32_t)((key[it] >> ls.shift[l]) & ((1ull << out.bits[l]) - 1ull));
-                    out.pos[l + 1][id[l]] = (int32_t)id[l + 1];
+        for (int h = 0; h < 2; ++h) {
+            bool opens[L];
+#pragma unroll
+            for (int l = 0; l < L; ++l) opens[l] = ((h ? b1[it][l] : b0[it][l]) >> lane) & 1u;
+#pragma unroll
+            for (int l = 0; l < L; ++l) {
+                if (opens[l]) {
+                    // the child that holds this element: opened by it, or (below the level it opens) the leaf itself
+                    const uint32_t child = l + 1 < L ? opened[l + 1 < L ? l + 1 : l] : (uint32_t)(e + h);
+                    out.crd[l][opened[l]] = (int32_t)((key[h] >> ls.shift[l]) & ((1ull << out.bits[l]) - 1ull));
+                    out.pos[l + 1][opened[l]] = (int32_t)child;
+                    if (l == 0 && slice_ptr) slice_ptr[opened[0]] = (int32_t)(e + h);
                 }
+            }
+#pragma unroll
+            for (int l = 0; l < L; ++l) opened[l] += opens[l];
+            if (e + h == n - 1) {
+                out.pos[0][0] = 0;
+                out.pos[0][1] = (int32_t)opened[0];
+#pragma unroll
+                for (int l = 0; l < L; ++l) out.pos[l + 1][opened[l]] = l + 1 < L ? (int32_t)opened[l + 1 < L ? l + 1 : l] : (int32_t)n;
+                if (slice_ptr) slice_ptr[opened[0]] = (int32_t)n;
             }
         }
 #pragma unroll
-        for (int l = 0; l < kCpLevels; ++l) run[l] += __popc(bal[it][l]);
+        for (int l = 0; l < L; ++l) run[l] += __popc(b0[it][l]) + __popc(b1[it][l]);
     }
 }
 
 inline void launch_csf_scatter(int order, int64_t blocks, const uint64_t *keys, int64_t n, const LevelShifts &ls,
-                               const uint32_t *block_base, const CsfArrays &out, cudaStream_t stream) {
+                               const uint32_t *block_base, const CsfArrays &out, int32_t *slice_ptr, cudaStream_t stream) {
     switch (order) {
-        case 1: csf_scatter<1><<<(unsigned)blocks, kCpThreads, 0, stream>>>(keys, n, ls, block_base, out); break;
-        case 2: csf_scatter<2><<<(unsigned)blocks, kCpThreads, 0, stream>>>(keys, n, ls, block_base, out); break;
-        case 3: csf_scatter<3><<<(unsigned)blocks, kCpThreads, 0, stream>>>(keys, n, ls, block_base, out); break;
-        default: csf_scatter<4><<<(unsigned)blocks, kCpThreads, 0, stream>>>(keys, n, ls, block_base, out); break;
+        case 2: csf_scatter<2><<<(unsigned)blocks, kCpThreads, 0, stream>>>(keys, n, ls, block_base, out, slice_ptr); break;
+        case 3: csf_scatter<3><<<(unsigned)blocks, kCpThreads, 0, stream>>>(keys, n, ls, block_base, out, slice_ptr); break;
+        default: csf_scatter<4><<<(unsigned)blocks, kCpThreads, 0, stream>>>(keys, n, ls, block_base, out, slice_ptr); break;
     }
+}
+
+// Node counts per block, scanned, and the level sizes: one launch while the block counts fit one block's scan, else three.
+inline void launch_csf_count(int order, int64_t blocks, const uint64_t *keys, int64_t n, const LevelShifts &ls, uint32_t *block_counts,
+                             int32_t *status, uint32_t *totals, uint32_t *arrived, cudaStream_t stream) {
+    const bool alone = blocks <= kCpScanBlocks;
+    uint32_t *t = alone ? totals : nullptr;
+    CB_LAUNCH("csf_count", stream, {
+        switch (order) {
+            case 2: csf_count<2><<<(unsigned)blocks, kCpThreads, 0, stream>>>(keys, n, ls, block_counts, status, t, arrived); break;
+            case 3: csf_count<3><<<(unsigned)blocks, kCpThreads, 0, stream>>>(keys, n, ls, block_counts, status, t, arrived); break;
+            default: csf_count<4><<<(unsigned)blocks, kCpThreads, 0, stream>>>(keys, n, ls, block_counts, status, t, arrived); break;
+        }
+    });
+    if (!alone) launch_csf_scan(block_counts, blocks, totals, stream);
 }
 
 struct LevelSizes { int64_t n[kMaxOrder]; int order; };
 
+// the pos arrays of a tensor without nonzeros
 __global__ void csf_finish(CsfArrays out, LevelSizes sz) {
     if (threadIdx.x == 0 && blockIdx.x == 0) {
         out.pos[0][0] = 0;
@@ -616,12 +707,6 @@ __device__ __forceinline__ int32_t leaf_of_fiber(const ChainPtrs &c, int32_t f) 
     int32_t x = f;
     for (int l = 2; l < c.order; ++l) x = c.pos[l][x];
     return x;
-}
-
-__global__ void bin_slice_ptr(ChainPtrs c, int64_t n0, int32_t *__restrict__ slice_ptr) {
-    int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s > n0) return;
-    slice_ptr[s] = leaf_of_fiber(c, c.pos[1][s]);
 }
 
 // Light slices are listed by falling size class (class = floor(log2(nonzeros))), so that the slices that
@@ -806,7 +891,8 @@ struct Scratch {            // stream-ordered temporaries of one build
 struct SortBufs {
     uint32_t *hist;                    // [kMaxPasses][kRsMaxBins] digit counts, then exclusive digit offsets
     uint32_t *counters;                // [kMaxPasses] tile tickets
-    unsigned long long *tile_status;   // [ntiles][kRsMaxBins]
+    unsigned long long *tile_status;   // [ntiles][kRsMaxBins], cleared by the caller
+    uint32_t *arrived;                 // [2] blocks that have finished the pack and the count kernel, zero at first
 };
 
 template <typename V, int BITS>
@@ -839,9 +925,6 @@ const_status_t sort_passes(uint64_t *&keys, uint64_t *&keys_alt, const V *vals_s
         CB_CUDA(cudaMemcpyAsync(vals_a, vals_src, sizeof(V) * n, cudaMemcpyDeviceToDevice, stream));
         return CONST_OK;
     }
-    const int64_t ntiles = (n + kRsTile - 1) / kRsTile;
-    CB_CUDA(cudaMemsetAsync(b.tile_status, 0, sizeof(unsigned long long) * ntiles * kRsMaxBins, stream));
-    CB_LAUNCH("rs_scan_hist", stream, rs_scan_hist<<<dp.passes, 256, 0, stream>>>(b.hist));
     const V *vin = vals_src;
     V *vout = vals_a;
     for (int p = 0; p < dp.passes; ++p) {
@@ -879,9 +962,7 @@ const_status_t sort_and_count(uint64_t *&keys, uint64_t *&keys_alt, const void *
         vals_sorted = out;
     }
     if (s != CONST_OK) return s;
-    const int64_t cp_blocks = (nnz + kCpTile - 1) / kCpTile;
-    CB_LAUNCH("csf_count", stream, csf_count<<<(unsigned)cp_blocks, kCpThreads, 0, stream>>>(keys, nnz, ls, block_counts, status));
-    launch_csf_scan(block_counts, cp_blocks, totals, stream);
+    launch_csf_count(ls.order, (nnz + kCpTile - 1) / kCpTile, keys, nnz, ls, block_counts, status, totals, b.arrived + 1, stream);
     return CONST_OK;
 }
 
@@ -948,12 +1029,12 @@ void csf_free(const_csf *csf) {
     cudaGetDevice(&prev);
     cudaSetDevice(csf->device);
     auto drop = [&](void *p) { if (p) cudaFreeAsync(p, csf->stream); };
-    for (int l = 0; l < kMaxOrder; ++l) { drop(csf->pos[l]); drop(csf->crd[l]); }
+    drop(csf->arena);
     drop(csf->vals);
-    drop(csf->slice_ptr);
     drop(csf->light_list);
     drop(csf->items);
     drop(csf->bin_scratch);
+    if (csf->bins_ready) cudaEventDestroy(csf->bins_ready);
     csf->magic = 0;
     delete csf;
     cudaSetDevice(prev);
@@ -983,16 +1064,35 @@ cudaError_t wait_stream(cudaStream_t stream) {
 
 // Upper bound of the number of work items for the current thresholds: a light or heavy slice gives at most
 // one item, a giant slice of z nonzeros ceil(z / chunk) <= z / chunk + 1.
+static const_status_t csf_rebin_locked(const_csf *csf, cudaStream_t stream);
+
 int64_t item_capacity(const const_csf *csf) {
     return csf->n[0] + csf->nnz / std::max<int64_t>(csf->chunk, 1) + 1;
 }
 
+// The work lists are built when something asks for them (a kernel that works from them, const_csf_work_lists,
+// const_csf_bin_counts); most executes need none.  Safe from several threads; a later user on another stream waits, on
+// the device, for the stream that built them.
+const_status_t csf_ensure_bins(const_csf *csf, cudaStream_t stream) {
+    std::lock_guard<std::mutex> lock(csf->bins_mu);
+    if (!csf->bins_valid) return csf_rebin_locked(csf, stream);
+    if (csf->bins_ready && stream != csf->bin_stream) CB_CUDA(cudaStreamWaitEvent(stream, csf->bins_ready, 0));
+    return CONST_OK;
+}
+
 const_status_t csf_rebin(const_csf *csf, cudaStream_t stream) {
+    std::lock_guard<std::mutex> lock(csf->bins_mu);
+    return csf_rebin_locked(csf, stream);
+}
+
+static const_status_t csf_rebin_locked(const_csf *csf, cudaStream_t stream) {
     const int64_t n0 = csf->n[0];
     csf->n_light = csf->n_heavy = csf->n_giant = csf->n_items = 0;
     csf->totals_on_host = n0 == 0;
     csf->bin_stream = stream;
+    csf->bins_valid = true;
     if (n0 == 0) { csf->item_cap = 0; return CONST_OK; }
+    csf->bins_valid = false;                              // until everything below is queued
     // Nothing below waits for the device: the lists are sized by their upper bounds, the fill kernels read
     // the counts the scan left in `totals`, and so do the fused kernels later on.
     const int64_t cap = item_capacity(csf);
@@ -1004,6 +1104,8 @@ const_status_t csf_rebin(const_csf *csf, cudaStream_t stream) {
     }
     csf->item_cap = cap;
     if (!csf->light_list) CB_CUDA(pool_alloc((void **)&csf->light_list, sizeof(int32_t) * n0, stream));
+    if (!csf->bin_scratch) CB_CUDA(pool_alloc((void **)&csf->bin_scratch, sizeof(int32_t) * (2 * (n0 + 1) + 8 + 2 * kBinClasses), stream));
+    if (!csf->bins_ready) CB_CUDA(cudaEventCreateWithFlags(&csf->bins_ready, cudaEventDisableTiming));
     ChainPtrs c;
     c.order = csf->order;
     for (int l = 0; l < kMaxOrder; ++l) c.pos[l] = csf->pos[l];
@@ -1018,16 +1120,19 @@ const_status_t csf_rebin(const_csf *csf, cudaStream_t stream) {
     const int64_t max_groups = (n0 + kWarpsPerBlock - 1) / kWarpsPerBlock;
     CB_LAUNCH("bin_light_items", stream, bin_light_items<<<(unsigned)((max_groups + 255) / 256), 256, 0, stream>>>(csf->items, totals));
     CB_CUDA(cudaGetLastError());
+    CB_CUDA(cudaEventRecord(csf->bins_ready, stream));
+    csf->bins_valid = true;
     return CONST_OK;
 }
 
 // Host copies of the bin totals, for callers that ask (const_csf_bin_counts, const_csf_work_lists).
 const_status_t csf_bin_totals(const_csf *csf) {
-    if (csf->totals_on_host) return CONST_OK;
     int32_t h[4] = {0, 0, 0, 0};
     int prev = 0;
     CB_CUDA(cudaGetDevice(&prev));
     CB_CUDA(cudaSetDevice(csf->device));
+    const const_status_t rc = csf_ensure_bins(csf, csf->bin_stream);
+    if (rc != CONST_OK || csf->totals_on_host) { cudaSetDevice(prev); return rc; }
     cudaError_t e = cudaMemcpyAsync(h, csf->bin_totals, sizeof(h), cudaMemcpyDeviceToHost, csf->bin_stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(csf->bin_stream);
     cudaSetDevice(prev);
@@ -1063,34 +1168,43 @@ const_status_t csf_build_impl(int order, const int64_t *dims, int64_t nnz, const
     {
         Scratch tmp(stream);
         uint64_t *keys = nullptr, *keys_alt = nullptr;
-        void *vals = nullptr, *vals_alt = nullptr, *vals_sorted = nullptr;
-        unsigned char *small = nullptr;          // hist | counters | totals | status, cleared together
+        void *vals_sorted = nullptr;
         uint32_t *block_counts = nullptr;
-        SortBufs sb{nullptr, nullptr, nullptr};
+        SortBufs sb{nullptr, nullptr, nullptr, nullptr};
         const int64_t cp_blocks = (nnz + kCpTile - 1) / kCpTile;
         const int64_t ntiles = (nnz + kRsTile - 1) / kRsTile;
         constexpr size_t kHistBytes = sizeof(uint32_t) * kMaxPasses * kRsMaxBins;
         constexpr size_t kSmallBytes = kHistBytes + 256;
         auto body = [&]() -> const_status_t {
-            CB_CUDA(tmp.alloc((void **)&keys, sizeof(uint64_t) * nnz));
-            CB_CUDA(tmp.alloc((void **)&keys_alt, sizeof(uint64_t) * nnz));
-            CB_CUDA(tmp.alloc(&vals, vsize * (nnz + 4)));
-            CB_CUDA(tmp.alloc(&vals_alt, vsize * (nnz + 4)));
-            CB_CUDA(tmp.alloc((void **)&small, kSmallBytes));
-            CB_CUDA(tmp.alloc((void **)&sb.tile_status, sizeof(unsigned long long) * std::max<int64_t>(ntiles, 1) * kRsMaxBins));
-            CB_CUDA(tmp.alloc((void **)&block_counts, sizeof(uint32_t) * (kCpLevels * std::max<int64_t>(cp_blocks, 1) +
-                                                                        scan_partials_room(cp_blocks))));
-            CB_CUDA(cudaMemsetAsync(small, 0, kSmallBytes, stream));
+            // One allocation for the temporaries: small | tile states (cleared together) | block counts | keys | keys | payload
+            auto room = [](size_t bytes) { return (bytes + 255) / 256 * 256; };
+            const size_t tiles_bytes = room(sizeof(unsigned long long) * std::max<int64_t>(ntiles, 1) * kRsMaxBins);
+            const size_t counts_bytes = room(sizeof(uint32_t) * (kCpLevels * std::max<int64_t>(cp_blocks, 1) + scan_partials_room(cp_blocks)));
+            const size_t keys_bytes = room(sizeof(uint64_t) * nnz);
+            const int passes = nnz > 0 ? kl.digits.passes : 0;
+            const size_t vals_bytes = passes > 1 ? room(vsize * (nnz + 4)) : 0;
+            unsigned char *arena = nullptr;
+            CB_CUDA(tmp.alloc((void **)&arena, room(kSmallBytes) + tiles_bytes + counts_bytes + 2 * keys_bytes + vals_bytes));
+            CB_CUDA(pool_alloc(&csf->vals, vsize * (nnz + 4), stream));         // where the last pass leaves the payload
+            unsigned char *small = arena;                                       // hist | counters | totals | status
+            sb.tile_status = reinterpret_cast<unsigned long long *>(arena + room(kSmallBytes));
+            block_counts = reinterpret_cast<uint32_t *>(arena + room(kSmallBytes) + tiles_bytes);
+            keys = reinterpret_cast<uint64_t *>(arena + room(kSmallBytes) + tiles_bytes + counts_bytes);
+            keys_alt = reinterpret_cast<uint64_t *>(arena + room(kSmallBytes) + tiles_bytes + counts_bytes + keys_bytes);
+            void *spare = passes > 1 ? (void *)(arena + room(kSmallBytes) + tiles_bytes + counts_bytes + 2 * keys_bytes) : csf->vals;
+            void *vals = passes % 2 == 1 || passes == 0 ? csf->vals : spare, *vals_alt = passes % 2 == 1 || passes == 0 ? spare : csf->vals;
+            CB_CUDA(cudaMemsetAsync(small, 0, room(kSmallBytes) + tiles_bytes, stream));
             sb.hist = reinterpret_cast<uint32_t *>(small);
             sb.counters = reinterpret_cast<uint32_t *>(small + kHistBytes);
             uint32_t *totals = reinterpret_cast<uint32_t *>(small + kHistBytes + 64);
             int32_t *status = reinterpret_cast<int32_t *>(small + kHistBytes + 128);
+            sb.arrived = reinterpret_cast<uint32_t *>(small + kHistBytes + 192);
             LevelShifts ls;
             ls.order = order;
             for (int l = 0; l < kMaxOrder; ++l) ls.shift[l] = kl.shift[l];
             if (nnz > 0) {
                 PackArgs pa = pack_args(order, dims, mode_order, coords_dev, kl);
-                CB_LAUNCH("pack_hist", stream, launch_pack_hist(pa, nnz, kl.digits, keys, sb.hist, status, stream));
+                CB_LAUNCH("pack_hist", stream, launch_pack_hist(pa, nnz, kl.digits, keys, sb.hist, status, sb.arrived, stream));
                 const_status_t s = sort_and_count(keys, keys_alt, vals_dev, vals, vals_alt, vals_sorted, nnz, kl.digits,
                                                   dtype, sb, ls, block_counts, totals, status, stream);
                 if (s != CONST_OK) return s;
@@ -1101,36 +1215,36 @@ const_status_t csf_build_impl(int order, const int64_t *dims, int64_t nnz, const
             if (h_small[16] != 0) return (const_status_t)h_small[16];
             for (int l = 0; l < order - 1; ++l) csf->n[l] = h_small[l];
             csf->n[order - 1] = nnz;
+            if (item_capacity(csf) > 0x7fffffffll) return CONST_ERR_UNSUPPORTED;      // more work items than the lists can number
 
             CsfArrays arr;
             for (int l = 0; l < kMaxOrder; ++l) { arr.pos[l] = arr.crd[l] = nullptr; arr.bits[l] = kl.bits[l]; }
+            // pos and crd of every level and slice_ptr behind one another in one allocation
+            size_t at[2 * kMaxOrder + 1], bytes = 0;
+            auto put = [&](int64_t n) { const size_t o = bytes; bytes += (sizeof(int32_t) * (size_t)n + 255) / 256 * 256; return o; };
             for (int l = 0; l < order; ++l) {
-                const int64_t parents = l == 0 ? 1 : csf->n[l - 1];
-                CB_CUDA(pool_alloc((void **)&csf->pos[l], sizeof(int32_t) * (parents + 1), stream));
-                CB_CUDA(pool_alloc((void **)&csf->crd[l], sizeof(int32_t) * (csf->n[l] + 4), stream));
-                arr.pos[l] = csf->pos[l];
-                arr.crd[l] = csf->crd[l];
+                at[2 * l] = put((l == 0 ? 1 : csf->n[l - 1]) + 1);
+                at[2 * l + 1] = put(csf->n[l] + 4);
             }
-            if (nnz > 0)
-                CB_LAUNCH("csf_scatter", stream, launch_csf_scatter(order, cp_blocks, keys, nnz, ls, block_counts, arr, stream));
-            LevelSizes sz;
-            sz.order = order;
-            for (int l = 0; l < kMaxOrder; ++l) sz.n[l] = csf->n[l];
-            CB_LAUNCH("csf_finish", stream, csf_finish<<<1, 32, 0, stream>>>(arr, sz));
-            if (!vals_sorted) vals_sorted = vals;
-            csf->vals = vals_sorted;          // the sorted payload buffer becomes the leaf value array
-            tmp.forget(vals_sorted);
-
-            // per-slice leaf offsets and the default work lists
-            const int64_t n0 = csf->n[0];
-            CB_CUDA(pool_alloc((void **)&csf->slice_ptr, sizeof(int32_t) * (n0 + 1), stream));
-            CB_CUDA(pool_alloc((void **)&csf->bin_scratch, sizeof(int32_t) * (2 * (n0 + 1) + 8 + 2 * kBinClasses), stream));
-            ChainPtrs c;
-            c.order = order;
-            for (int l = 0; l < kMaxOrder; ++l) c.pos[l] = csf->pos[l];
-            CB_LAUNCH("bin_slice_ptr", stream, bin_slice_ptr<<<(unsigned)((n0 + 1 + 255) / 256), 256, 0, stream>>>(c, n0, csf->slice_ptr));
+            at[2 * order] = put(csf->n[0] + 1);
+            CB_CUDA(pool_alloc((void **)&csf->arena, bytes, stream));
+            for (int l = 0; l < order; ++l) {
+                arr.pos[l] = csf->pos[l] = reinterpret_cast<int32_t *>(csf->arena + at[2 * l]);
+                arr.crd[l] = csf->crd[l] = reinterpret_cast<int32_t *>(csf->arena + at[2 * l + 1]);
+            }
+            csf->slice_ptr = reinterpret_cast<int32_t *>(csf->arena + at[2 * order]);
+            if (nnz > 0) {
+                CB_LAUNCH("csf_scatter", stream, launch_csf_scatter(order, cp_blocks, keys, nnz, ls, block_counts, arr, csf->slice_ptr, stream));
+            } else {
+                LevelSizes sz;
+                sz.order = order;
+                for (int l = 0; l < kMaxOrder; ++l) sz.n[l] = 0;
+                CB_LAUNCH("csf_finish", stream, csf_finish<<<1, 32, 0, stream>>>(arr, sz));
+                CB_CUDA(cudaMemsetAsync(csf->slice_ptr, 0, sizeof(int32_t), stream));
+            }
             CB_CUDA(cudaGetLastError());
-            return csf_rebin(csf, stream);
+            csf->bin_stream = stream;
+            return CONST_OK;
         };
         rc = body();
     }
@@ -1203,12 +1317,13 @@ const_status_t csf_build_noalloc_impl(int order, const int64_t *dims, int64_t nn
     uint64_t *keys_alt = reinterpret_cast<uint64_t *>(base + kNaOffKeys1);
     uint32_t *block_counts = reinterpret_cast<uint32_t *>(base + kNaOffBlockCounts);
     SortBufs sb{reinterpret_cast<uint32_t *>(base + kNaOffHist), reinterpret_cast<uint32_t *>(base + kNaOffSmall),
-                reinterpret_cast<unsigned long long *>(base + kNaOffTileStatus)};
+                reinterpret_cast<unsigned long long *>(base + kNaOffTileStatus),
+                reinterpret_cast<uint32_t *>(base + kNaOffSmall + 192)};
     uint32_t *totals = reinterpret_cast<uint32_t *>(base + kNaOffSmall + 64);
     int32_t *status = reinterpret_cast<int32_t *>(base + kNaOffSmall + 128);
     // everything that must start at zero: digit histograms, pass counters, level totals, status word
-    // (the tile states are cleared by the sort itself)
     CB_CUDA(cudaMemsetAsync(base + kNaOffHist, 0, kNaHistBytes + kNaSmallBytes, stream));
+    CB_CUDA(cudaMemsetAsync(sb.tile_status, 0, sizeof(unsigned long long) * ((nnz + kRsTile - 1) / kRsTile) * kRsMaxBins, stream));
 
     const size_t vsize = dtype == CONST_F32 ? 4 : 8;
     const int64_t cp_blocks = (nnz + kCpTile - 1) / kCpTile;
@@ -1217,7 +1332,7 @@ const_status_t csf_build_noalloc_impl(int order, const int64_t *dims, int64_t nn
     for (int l = 0; l < kMaxOrder; ++l) ls.shift[l] = kl.shift[l];
     if (nnz > 0) {
         PackArgs pa = pack_args(order, dims, mode_order, coords_dev, kl);
-        launch_pack_hist(pa, nnz, kl.digits, keys, sb.hist, status, stream);
+        launch_pack_hist(pa, nnz, kl.digits, keys, sb.hist, status, sb.arrived, stream);
         // the payload alternates between the caller's output and the static buffer; start on the side
         // that makes the last pass land in the caller's output
         const bool odd = kl.digits.passes % 2 == 1 || kl.digits.passes == 0;
@@ -1243,8 +1358,8 @@ const_status_t csf_build_noalloc_impl(int order, const int64_t *dims, int64_t nn
         arr.crd[l] = l < order ? crd_out[l] : nullptr;
         arr.bits[l] = kl.bits[l];
     }
-    if (nnz > 0) launch_csf_scatter(order, cp_blocks, keys, nnz, ls, block_counts, arr, stream);
-    csf_finish<<<1, 32, 0, stream>>>(arr, sz);
+    if (nnz > 0) launch_csf_scatter(order, cp_blocks, keys, nnz, ls, block_counts, arr, nullptr, stream);
+    else csf_finish<<<1, 32, 0, stream>>>(arr, sz);
     CB_CUDA(cudaGetLastError());
     if (level_sizes)
         for (int l = 0; l < order; ++l) level_sizes[l] = sz.n[l];
