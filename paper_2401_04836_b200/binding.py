@@ -7,6 +7,7 @@ fallback: if the shared library is missing the import of this module's functions
 from __future__ import annotations
 
 import ctypes
+import functools
 import os
 from typing import Dict, List, Optional, Sequence, Tuple, Union
 
@@ -32,6 +33,11 @@ class _Extent(ctypes.Structure):
 
 class _Operand(ctypes.Structure):
     _fields_ = [("name", ctypes.c_char_p), ("csf", ctypes.c_void_p), ("dense_dev", ctypes.c_void_p)]
+
+
+@functools.lru_cache(maxsize=None)
+def _operand_array(n: int):
+    return _Operand * n
 
 
 _lib = None
@@ -113,18 +119,29 @@ def _check(status: int, where: str) -> None:
         raise ConstError(status, where)
 
 
-def _stream_ptr(stream) -> ctypes.c_void_p:
+_torch = None
+
+
+def _stream_int(stream) -> int:
+    """The cudaStream_t of `stream` (a torch stream or the number itself), of the current stream when it is None."""
+    global _torch
     if stream is None:
-        import torch
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(int(getattr(stream, "cuda_stream", stream)))
+        if _torch is None:
+            import torch
+            _torch = torch
+        stream = _torch.cuda.current_stream()
+    return int(getattr(stream, "cuda_stream", stream))
+
+
+def _stream_ptr(stream) -> ctypes.c_void_p:
+    return ctypes.c_void_p(_stream_int(stream))
 
 
 class CsfHandle:
-    """Owns a const_csf_t*; `order`, `dtype` mirror the build arguments."""
+    """Owns a const_csf_t*; `order`, `dtype`, `stream` mirror the build arguments."""
 
-    def __init__(self, ptr: int, order: int, dtype: int):
-        self.ptr, self.order, self.dtype = ptr, order, dtype
+    def __init__(self, ptr: int, order: int, dtype: int, stream: Optional[int] = None):
+        self.ptr, self.order, self.dtype, self.stream = ptr, order, dtype, stream
 
     def __del__(self):
         try:
@@ -162,10 +179,10 @@ def const_csf_build(coords, vals, dims: Sequence[int], mode_order: Sequence[int]
     mo_a = (ctypes.c_int * order)(*[int(m) for m in mode_order])
     cptr = (ctypes.c_void_p * order)(*[c.data_ptr() for c in coords])
     out = ctypes.c_void_p()
-    st = lib.const_csf_build(order, dims_a, nnz, cptr, ctypes.c_void_p(vals.data_ptr()), dtype, mo_a,
-                             _stream_ptr(stream), ctypes.byref(out))
+    on = _stream_int(stream)
+    st = lib.const_csf_build(order, dims_a, nnz, cptr, vals.data_ptr(), dtype, mo_a, on, ctypes.byref(out))
     _check(st, "const_csf_build")
-    return CsfHandle(out.value, order, dtype)
+    return CsfHandle(out.value, order, dtype, on)
 
 
 def const_csf_from_dense(dense, mode_order: Sequence[int], stream=None) -> CsfHandle:
@@ -179,9 +196,9 @@ def const_csf_from_dense(dense, mode_order: Sequence[int], stream=None) -> CsfHa
     dims_a = (ctypes.c_int64 * order)(*[int(d) for d in dense.shape])
     mo_a = (ctypes.c_int * order)(*[int(m) for m in mode_order])
     out = ctypes.c_void_p()
-    _check(lib.const_csf_from_dense(order, dims_a, ctypes.c_void_p(dense.data_ptr()), dtype, mo_a, _stream_ptr(stream),
-                                    ctypes.byref(out)), "const_csf_from_dense")
-    return CsfHandle(out.value, order, dtype)
+    on = _stream_int(stream)
+    _check(lib.const_csf_from_dense(order, dims_a, dense.data_ptr(), dtype, mo_a, on, ctypes.byref(out)), "const_csf_from_dense")
+    return CsfHandle(out.value, order, dtype, on)
 
 
 def const_csf_build_noalloc(coords, vals, dims: Sequence[int], mode_order: Sequence[int], pos_out, crd_out,
@@ -217,15 +234,29 @@ def const_csf_build_noalloc(coords, vals, dims: Sequence[int], mode_order: Seque
     return list(sizes)
 
 
-def _dev_to_torch(ptr: Optional[int], n: int, dtype):
-    """Copy n elements from a borrowed device pointer into a fresh torch CUDA tensor."""
+_cudart = None
+
+
+def _dev_to_torch(ptr: Optional[int], n: int, dtype, csf: CsfHandle):
+    """Copy n elements of one of the handle's arrays into a fresh torch CUDA tensor.
+
+    On the stream the handle was built on the copy is ordered behind the build and in front of its release by the stream
+    itself; from any other stream everything queued on the device is waited for first.
+    """
+    global _cudart
     import torch
     out = torch.empty(n, dtype=dtype, device="cuda")
     if n:
-        cudart = ctypes.CDLL("libcudart.so.12")
-        cudart.cudaMemcpy.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_size_t, ctypes.c_int]
-        torch.cuda.synchronize()
-        rc = cudart.cudaMemcpy(out.data_ptr(), ptr, n * out.element_size(), 3)   # cudaMemcpyDeviceToDevice
+        if _cudart is None:
+            _cudart = ctypes.CDLL("libcudart.so.12")
+            _cudart.cudaMemcpy.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_size_t, ctypes.c_int]
+            _cudart.cudaMemcpyAsync.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_size_t, ctypes.c_int, ctypes.c_void_p]
+        current = _stream_int(None)
+        if current == csf.stream:                                      # 3: cudaMemcpyDeviceToDevice
+            rc = _cudart.cudaMemcpyAsync(out.data_ptr(), ptr, n * out.element_size(), 3, current)
+        else:
+            torch.cuda.synchronize()
+            rc = _cudart.cudaMemcpy(out.data_ptr(), ptr, n * out.element_size(), 3)
         if rc != 0:
             raise RuntimeError(f"cudaMemcpy failed with {rc}")
     return out
@@ -244,7 +275,7 @@ def const_csf_level(csf: CsfHandle, level: int):
         prev = ctypes.c_int64()
         _check(lib.const_csf_level(csf.ptr, level - 1, None, None, ctypes.byref(prev)), "const_csf_level")
         n_pos = prev.value + 1
-    return _dev_to_torch(pos.value, n_pos, torch.int32), _dev_to_torch(crd.value, n.value, torch.int32)
+    return _dev_to_torch(pos.value, n_pos, torch.int32, csf), _dev_to_torch(crd.value, n.value, torch.int32, csf)
 
 
 def const_csf_values(csf: CsfHandle):
@@ -252,7 +283,7 @@ def const_csf_values(csf: CsfHandle):
     lib = load_library()
     vals, nnz = ctypes.c_void_p(), ctypes.c_int64()
     _check(lib.const_csf_values(csf.ptr, ctypes.byref(vals), ctypes.byref(nnz)), "const_csf_values")
-    return _dev_to_torch(vals.value, nnz.value, torch.float32 if csf.dtype == F32 else torch.float64)
+    return _dev_to_torch(vals.value, nnz.value, torch.float32 if csf.dtype == F32 else torch.float64, csf)
 
 
 def const_csf_set_bins(csf: CsfHandle, light_max_nnz: int = 0, heavy_max_nnz: int = 0, chunk_nnz: int = 0,
@@ -277,9 +308,9 @@ def const_csf_work_lists(csf: CsfHandle):
     _check(lib.const_csf_work_lists(csf.ptr, ctypes.byref(sp), ctypes.byref(ll), ctypes.byref(n_light), ctypes.byref(it),
                                     ctypes.byref(n_items)), "const_csf_work_lists")
     _check(lib.const_csf_level(csf.ptr, 0, None, None, ctypes.byref(n0)), "const_csf_level")
-    return (_dev_to_torch(sp.value, n0.value + 1 if n0.value else 0, torch.int32),
-            _dev_to_torch(ll.value, n_light.value, torch.int32),
-            _dev_to_torch(it.value, 4 * n_items.value, torch.int32).reshape(-1, 4))
+    return (_dev_to_torch(sp.value, n0.value + 1 if n0.value else 0, torch.int32, csf),
+            _dev_to_torch(ll.value, n_light.value, torch.int32, csf),
+            _dev_to_torch(it.value, 4 * n_items.value, torch.int32, csf).reshape(-1, 4))
 
 
 BENCH_FP32_FMA, BENCH_FP64_FMA, BENCH_TF32_MMA, BENCH_ROW_GATHER, BENCH_FP64_MMA = 0, 1, 2, 3, 4
@@ -362,23 +393,19 @@ def const_plan_family(plan: PlanHandle) -> str:
 
 def const_execute(plan: PlanHandle, operands: Dict[str, Union[CsfHandle, "object"]], out, stream=None) -> None:
     """operands: name -> CsfHandle or dense torch CUDA tensor (row-major).  `out` is overwritten."""
-    lib = load_library()
-    ops = (_Operand * len(operands))()
-    keep = []
-    for slot, (name, val) in zip(ops, operands.items()):
-        b = name.encode()
-        keep.append(b)
-        slot.name = b
+    lib = _lib or load_library()
+    ops = []
+    for name, val in operands.items():
         if isinstance(val, CsfHandle):
-            slot.csf, slot.dense_dev = val.ptr, None
+            ops.append(_Operand(name.encode(), val.ptr, None))
         else:
             if not val.is_cuda or not val.is_contiguous():
                 raise ValueError(f"dense operand {name} must be a contiguous CUDA tensor")
-            slot.csf, slot.dense_dev = None, val.data_ptr()
+            ops.append(_Operand(name.encode(), None, val.data_ptr()))
     if not out.is_cuda or not out.is_contiguous():
         raise ValueError("output must be a contiguous CUDA tensor")
-    _check(lib.const_execute(plan.ptr, ops, len(operands), ctypes.c_void_p(out.data_ptr()), _stream_ptr(stream)),
-           "const_execute")
+    n = len(ops)
+    _check(lib.const_execute(plan.ptr, _operand_array(n)(*ops), n, out.data_ptr(), _stream_int(stream)), "const_execute")
 
 
 def const_plan_set_tensor_stage(plan: PlanHandle, enable: bool) -> None:
