@@ -20,7 +20,10 @@
 // sparse sum would never touch: t_kernel checks that every T it computed is finite and otherwise sets the mode word, too;
 // the gather kernel, launched last, then clears Z and does the work.
 //
-// Measured (1024 x 1024 x 128, band 32, a quarter full): see run_network.
+// Measured, 1024 x 1024 x 128, band 32, a quarter full: 4771 us in the gather form; here t_kernel 660 us (dense work at the
+// fp64 peak of 37 TFLOP/s: 480) and z_kernel 890 us (540), 1573 us together with the shape kernels.  z_kernel is held by
+// writing its slices out between the products: walking the fibres for it 1196 us, from places computed once 979, with the
+// next slice's entries on their way meanwhile 889.  331 x 331 x 61, band 17: 165 -> 136 us; 700, 100, band 21: 1198 -> 568.
 #include <algorithm>
 
 #include "common.cuh"
@@ -29,7 +32,8 @@ namespace cb {
 namespace {
 
 constexpr int kThreads = 256, kWarps = kThreads / 32;
-constexpr int kRange = 96;            // most j of a slice of U, most m of a group of slices of W
+constexpr int kRangeJ = 96;           // most j of a slice of U: two blocks of t_kernel share the memory of an SM
+constexpr int kRangeM = 80;           // most m of a group of slices of W: so do two blocks of z_kernel with the staged entries
 constexpr int kTileK = 128;           // k per tile
 constexpr int kNodes = 4;             // slices of W per z_kernel block
 constexpr int kRows = 8 * kWarps;     // slices of U per z_kernel block
@@ -92,7 +96,7 @@ __global__ void __launch_bounds__(kThreads) shape_kernel(const __grid_constant__
         a.mlen[unit - a.u.n0] = len;
         work = (unsigned long long)round_up(len, 8) * a.tk * kNodes * a.u.n0;
     }
-    if (len > kRange) a.mode[0] = 1;
+    if (len > (unit < a.u.n0 ? kRangeJ : kRangeM)) a.mode[0] = 1;
     atomicAdd(reinterpret_cast<unsigned long long *>(a.mode + 2), work);
 }
 
@@ -218,8 +222,35 @@ __global__ void __launch_bounds__(kThreads, 2) t_kernel(const __grid_constant__ 
     if (!finite) atomicExch(a.mode, 1);
 }
 
+constexpr int kStaged = 2048;         // entries of a slice of W that wait in shared memory
+
+// Entries of the next slice on their way into shared memory while the matrix tiles of this one run.
+struct Staged {
+    double v[kStaged];
+    uint32_t place[kStaged];
+    __device__ __forceinline__ void request(const uint32_t *places, const double *vals, int32_t first, int32_t last) {
+        const int n = min(last - first, kStaged);
+        for (int i = threadIdx.x; i < n; i += kThreads) {
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" :: "r"((uint32_t)__cvta_generic_to_shared(place + i)), "l"(places + first + i) : "memory");
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" :: "r"((uint32_t)__cvta_generic_to_shared(v + i)), "l"(vals + first + i) : "memory");
+        }
+    }
+    // the caller has waited (own copies) and synchronised (the other threads')
+    template <class Put>
+    __device__ __forceinline__ void write(const uint32_t *places, const double *vals, int32_t first, int32_t last, int k0, int kt, Put put) const {
+        for (int32_t p = first + threadIdx.x; p < last; p += kThreads) {
+            const int i = p - first;
+            const uint32_t pl = i < kStaged ? place[i] : __ldg(places + p);
+            const int k = (int)(pl & 4095u) - k0;
+            if ((unsigned)k < (unsigned)kt) put((int)(pl >> 12), k, i < kStaged ? v[i] : __ldg(vals + p));
+        }
+    }
+};
+
 __global__ void __launch_bounds__(kThreads, 2) z_kernel(const __grid_constant__ Net a) {
-    extern __shared__ __align__(16) double w_dense[];                     // [tile of k][range of m + 4]
+    extern __shared__ __align__(16) double z_smem[];
+    Staged &staged = *reinterpret_cast<Staged *>(z_smem);
+    double *w_dense = z_smem + sizeof(Staged) / sizeof(double);           // [tile of k][range of m + 4]
     __shared__ int skip;
     if (threadIdx.x == 0) skip = *a.mode;
     __syncthreads();
@@ -229,30 +260,29 @@ __global__ void __launch_bounds__(kThreads, 2) z_kernel(const __grid_constant__ 
     const int tiles = round_up(len, 8) / 8, ld = tiles * 8 + 4;
     const int s = a.s0 + blockIdx.y * kRows + warp * 8 + r;              // this lane's slice of U
     const bool have = s < a.s1;
-    double acc[kRange / 8][2];
+    double acc[kRangeM / 8][2];
 #pragma unroll
-    for (int t = 0; t < kRange / 8; ++t) acc[t][0] = acc[t][1] = 0.0;
+    for (int t = 0; t < kRangeM / 8; ++t) acc[t][0] = acc[t][1] = 0.0;
     const int n0 = group * kNodes, n1 = min(n0 + kNodes, a.w.n0);
-    int32_t leaf = __ldg(a.w.pos2 + __ldg(a.w.pos1 + n0));
+    int32_t leaf = __ldg(a.w.pos2 + __ldg(a.w.pos1 + n0)), leaf1 = __ldg(a.w.pos2 + __ldg(a.w.pos1 + n0 + 1));
+    staged.request(a.w_place, a.w.vals, leaf, leaf1);
     for (int node = n0; node < n1; ++node) {
         const int l = __ldg(a.w.crd0 + node);
-        const int32_t leaf1 = __ldg(a.w.pos2 + __ldg(a.w.pos1 + node + 1));
+        const int32_t leaf2 = node + 1 < n1 ? __ldg(a.w.pos2 + __ldg(a.w.pos1 + node + 2)) : leaf1;
         const double *t_row = a.T + ((size_t)(have ? s - a.s0 : 0) * a.n_l + l) * a.tk + c;
         for (int k0 = 0; k0 < a.tk; k0 += kTileK) {
             const int kt = min(kTileK, a.tk - k0), steps = kt / 4;       // steps is even
             auto t_at = [&](int st) { return have && st < steps ? __ldg(t_row + k0 + st * 4) : 0.0; };
             double x[4];
-            {
-                Entries e;
-                e.request(a.w_place, a.w.vals, leaf, leaf1);
 #pragma unroll
-                for (int z = 0; z < 4; ++z) x[z] = t_at(z);
-                __syncthreads();                                          // the tile before is used up
-                clear_shared(w_dense, kt * ld);
-                __syncthreads();
-                e.write(a.w_place, a.w.vals, k0, kt, [&](int m, int k, double v) { w_dense[k * ld + m] = v; });
-                __syncthreads();
-            }
+            for (int z = 0; z < 4; ++z) x[z] = t_at(z);
+            if (k0 == 0) asm volatile("cp.async.wait_all;" ::: "memory");
+            __syncthreads();                                              // the tile before is used up, the entries are here
+            clear_shared(w_dense, kt * ld);
+            __syncthreads();
+            staged.write(a.w_place, a.w.vals, leaf, leaf1, k0, kt, [&](int m, int k, double v) { w_dense[k * ld + m] = v; });
+            __syncthreads();
+            if (k0 + kTileK >= a.tk && node + 1 < n1) staged.request(a.w_place, a.w.vals, leaf1, leaf2);
             for (int st = 0; st < steps; st += 4) {
                 double next[4];
 #pragma unroll
@@ -262,7 +292,7 @@ __global__ void __launch_bounds__(kThreads, 2) z_kernel(const __grid_constant__ 
                     if (st + z >= steps) break;                           // uniform
                     const double *row = w_dense + ((st + z) * 4 + c) * ld + r;
 #pragma unroll
-                    for (int t = 0; t < kRange / 8; ++t)
+                    for (int t = 0; t < kRangeM / 8; ++t)
                         if (t < tiles) mma884(acc[t][0], acc[t][1], x[z], row[t * 8]);
                 }
 #pragma unroll
@@ -270,11 +300,12 @@ __global__ void __launch_bounds__(kThreads, 2) z_kernel(const __grid_constant__ 
             }
         }
         leaf = leaf1;
+        leaf1 = leaf2;
     }
     if (!have) return;
     double *z = a.Z + (size_t)__ldg(a.u.crd0 + s) * a.n_m + m0 + 2 * c;
 #pragma unroll
-    for (int t = 0; t < kRange / 8; ++t)
+    for (int t = 0; t < kRangeM / 8; ++t)
         if (t < tiles) {
             if (t * 8 + 2 * c < len) atomicAdd(z + t * 8, acc[t][0]);
             if (t * 8 + 2 * c + 1 < len) atomicAdd(z + t * 8 + 1, acc[t][1]);
@@ -301,8 +332,8 @@ const_status_t run_network_dense(const const_csf *U, const double *V, const cons
     const double sparse = (double)U->nnz * n_l + (double)W->nnz * U->n[0];
     const int64_t row_bytes = n_l * tk * 8;
     const int64_t n0 = U->n[0], groups = (W->n[0] + kNodes - 1) / kNodes;
-    // Small networks stay with the gather kernel (one launch instead of six); so does one whose T would leave fewer than
-    // 64 slices to a chunk.  What is sparser than one in kMaxDilution over all indices within kRange cannot qualify.
+    // Small networks stay with the gather kernel (one launch instead of seven, about 45 us); so does one whose T would
+    // leave fewer than 64 slices to a chunk.
     if (sparse < 2e7 || n_k > 4096 || kScratchBytes / row_bytes < std::min<int64_t>(n0, 64)) return CONST_OK;
     if (n_l > (1 << 24) || n_m > (1 << 24) || groups > 65535 * 8ll) return CONST_OK;
     int64_t chunk = std::min<int64_t>(n0, kScratchBytes / row_bytes);
@@ -346,10 +377,10 @@ const_status_t run_network_dense(const const_csf *U, const double *V, const cons
         CB_LAUNCH("network_shape", stream, decide_kernel<<<1, 1, 0, stream>>>(a.mode, (unsigned long long)sparse));
         CB_LAUNCH("network_shape", stream, place_kernel<<<(unsigned)(n0 + W->n[0]), kThreads, 0, stream>>>(a));
         const int kt = (int)std::min<int64_t>(kTileK, tk);
-        const size_t t_smem = sizeof(double) * kRange * (kt + 4), z_smem = sizeof(double) * kt * (kRange + 4);
+        const size_t t_smem = sizeof(double) * kRangeJ * (kt + 4), z_smem = sizeof(Staged) + sizeof(double) * kt * (kRangeM + 4);
         static PerDeviceOnce once;
         CB_CUDA(once_per_device(once, [] {
-            const int most = (int)sizeof(double) * std::max(kRange * (kTileK + 4), kTileK * (kRange + 4));
+            const int most = (int)(sizeof(Staged) + sizeof(double) * std::max(kRangeJ * (kTileK + 4), kTileK * (kRangeM + 4)));
             cudaError_t e = cudaFuncSetAttribute(t_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
             return e == cudaSuccess ? cudaFuncSetAttribute(z_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most) : e;
         }));

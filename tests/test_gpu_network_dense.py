@@ -24,8 +24,8 @@ def kernels_of(w):
     (331, 61, 17, 0.25),      # nothing a multiple of a tile
     (300, 128, 12, 0.3),      # a full tile of k
     (260, 150, 12, 0.3),      # two tiles of k, the second of 22
-    (200, 7, 46, 0.6),        # the widest range that qualifies with four slices together (94 of 96)
-    (200, 9, 48, 0.6),        # one that does not (98)
+    (200, 7, 39, 0.6),        # the widest range of m that qualifies with four slices together (80)
+    (200, 9, 40, 0.6),        # one that does not (82)
     (403, 33, 3, 1.0),        # narrow and full
 ])
 def test_banded(n, n_k, band, keep):
