@@ -49,7 +49,7 @@ struct Net {
     Csf3d u, w;                       // levels (i, k, j) and (l, m, k)
     const double *V;
     double *Z, *T;
-    int32_t *mode;                    // [0] nonzero: the gather kernel does the work; [2..3] dense multiply-adds (64 bits)
+    int32_t *mode;                    // [0] nonzero: the gather kernel does the work (2: from the start, 1: T was not finite); [2..3] dense multiply-adds (64 bits); [4] blocks done
     int32_t *jmin, *jlen;             // per slice of U: first j, length of the range of j
     int32_t *mmin, *mlen;             // per group of slices of W: the same of m
     uint32_t *u_place, *w_place;      // per entry (place_kernel)
@@ -64,19 +64,21 @@ __device__ __forceinline__ void mma884(double &c0, double &c1, double a, double 
 __device__ __forceinline__ int round_up(int x, int to) { return (x + to - 1) / to * to; }
 
 // One warp per slice of U and per group of slices of W: the ranges, the dense work, and whether they fit.
-__global__ void __launch_bounds__(kThreads) shape_kernel(const __grid_constant__ Net a) {
+__global__ void __launch_bounds__(kThreads) shape_kernel(const __grid_constant__ Net a, unsigned long long sparse) {
     const int lane = threadIdx.x & 31;
     const int unit = blockIdx.x * kWarps + (threadIdx.x >> 5), groups = (a.w.n0 + kNodes - 1) / kNodes;
-    if (unit >= a.u.n0 + groups) return;
+    __shared__ unsigned long long sum;
+    if (threadIdx.x == 0) sum = 0;
+    __syncthreads();
     int lo = 0x7fffffff, hi = -1;
-    unsigned long long work;
-    if (unit < a.u.n0) {
+    const bool have = unit < a.u.n0 + groups;
+    if (have && unit < a.u.n0) {
         const int f1 = __ldg(a.u.pos1 + unit + 1);
         for (int f = __ldg(a.u.pos1 + unit) + lane; f < f1; f += 32) {
             lo = min(lo, __ldg(a.u.crd2 + __ldg(a.u.pos2 + f)));
             hi = max(hi, __ldg(a.u.crd2 + __ldg(a.u.pos2 + f + 1) - 1));
         }
-    } else {
+    } else if (have) {
         const int node = (unit - a.u.n0) * kNodes + lane;
         if (lane < kNodes && node < a.w.n0) {
             lo = __ldg(a.w.crd1 + __ldg(a.w.pos1 + node));
@@ -86,23 +88,28 @@ __global__ void __launch_bounds__(kThreads) shape_kernel(const __grid_constant__
     lo = __reduce_min_sync(0xffffffffu, lo);
     hi = __reduce_max_sync(0xffffffffu, hi);
     const int len = hi - lo + 1;
-    if (lane != 0) return;
-    if (unit < a.u.n0) {
-        a.jmin[unit] = lo;
-        a.jlen[unit] = len;
-        work = (unsigned long long)round_up(len, 4) * a.tk * a.n_l;
-    } else {
-        a.mmin[unit - a.u.n0] = lo;
-        a.mlen[unit - a.u.n0] = len;
-        work = (unsigned long long)round_up(len, 8) * a.tk * kNodes * a.u.n0;
+    if (lane == 0 && have) {
+        unsigned long long work;
+        if (unit < a.u.n0) {
+            a.jmin[unit] = lo;
+            a.jlen[unit] = len;
+            work = (unsigned long long)round_up(len, 4) * a.tk * a.n_l;
+        } else {
+            a.mmin[unit - a.u.n0] = lo;
+            a.mlen[unit - a.u.n0] = len;
+            work = (unsigned long long)round_up(len, 8) * a.tk * kNodes * a.u.n0;
+        }
+        if (len > (unit < a.u.n0 ? kRangeJ : kRangeM)) a.mode[0] = 2;
+        atomicAdd(&sum, work);
     }
-    if (len > (unit < a.u.n0 ? kRangeJ : kRangeM)) a.mode[0] = 1;
-    atomicAdd(reinterpret_cast<unsigned long long *>(a.mode + 2), work);
-}
-
-// The dense form has to be worth it: sparse = multiply-adds of the gather form.
-__global__ void decide_kernel(int32_t *mode, unsigned long long sparse) {
-    if (*reinterpret_cast<unsigned long long *>(mode + 2) > kMaxDilution * sparse) mode[0] = 1;
+    // the last block to finish compares the dense work with that of the gather form: it has to be worth it
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    unsigned long long *total = reinterpret_cast<unsigned long long *>(a.mode + 2);
+    atomicAdd(total, sum);
+    __threadfence();
+    const bool last = atomicAdd(a.mode + 4, 1) == (int)gridDim.x - 1;
+    if (last && atomicAdd(total, 0ull) > kMaxDilution * sparse) a.mode[0] = 2;
 }
 
 // Where every entry goes when its slice is written out: (place in the range) << 12 | k.  One block per slice, eight lanes per
@@ -312,9 +319,9 @@ __global__ void __launch_bounds__(kThreads, 2) z_kernel(const __grid_constant__ 
         }
 }
 
-// Z back to zero where the gather kernel takes over
+// Z back to zero where the gather kernel takes over after products have been added to it
 __global__ void __launch_bounds__(256) reclear_kernel(const int32_t *mode, double *Z, int64_t n) {
-    if (!*mode) return;
+    if (*mode != 1) return;
     for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) Z[i] = 0.0;
 }
 
@@ -332,9 +339,10 @@ const_status_t run_network_dense(const const_csf *U, const double *V, const cons
     const double sparse = (double)U->nnz * n_l + (double)W->nnz * U->n[0];
     const int64_t row_bytes = n_l * tk * 8;
     const int64_t n0 = U->n[0], groups = (W->n[0] + kNodes - 1) / kNodes;
-    // Small networks stay with the gather kernel (one launch instead of seven, about 45 us); so does one whose T would
-    // leave fewer than 64 slices to a chunk.
-    if (sparse < 2e7 || n_k > 4096 || kScratchBytes / row_bytes < std::min<int64_t>(n0, 64)) return CONST_OK;
+    // Small networks stay with the gather kernel; so does one whose T would leave fewer than 64 slices to a chunk.  Where the
+    // line lies (multiply-adds of the gather form): at 1.1e8 the band at 331 takes 165 us in the gather form and 133 here,
+    // below 6e7 the six extra launches (about 25 us, also paid by operands that then do not qualify) eat the gain.
+    if (sparse < 6e7 || n_k > 4096 || kScratchBytes / row_bytes < std::min<int64_t>(n0, 64)) return CONST_OK;
     if (n_l > (1 << 24) || n_m > (1 << 24) || groups > 65535 * 8ll) return CONST_OK;
     int64_t chunk = std::min<int64_t>(n0, kScratchBytes / row_bytes);
     const int64_t chunks = (n0 + chunk - 1) / chunk;
@@ -373,8 +381,7 @@ const_status_t run_network_dense(const const_csf *U, const double *V, const cons
         a.tk = (int32_t)tk;
         a.s0 = a.s1 = 0;
         const int64_t units = n0 + groups;
-        CB_LAUNCH("network_shape", stream, shape_kernel<<<(unsigned)((units + kWarps - 1) / kWarps), kThreads, 0, stream>>>(a));
-        CB_LAUNCH("network_shape", stream, decide_kernel<<<1, 1, 0, stream>>>(a.mode, (unsigned long long)sparse));
+        CB_LAUNCH("network_shape", stream, shape_kernel<<<(unsigned)((units + kWarps - 1) / kWarps), kThreads, 0, stream>>>(a, (unsigned long long)sparse));
         CB_LAUNCH("network_shape", stream, place_kernel<<<(unsigned)(n0 + W->n[0]), kThreads, 0, stream>>>(a));
         const int kt = (int)std::min<int64_t>(kTileK, tk);
         const size_t t_smem = sizeof(double) * kRangeJ * (kt + 4), z_smem = sizeof(Staged) + sizeof(double) * kt * (kRangeM + 4);

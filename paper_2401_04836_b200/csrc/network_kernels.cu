@@ -22,6 +22,8 @@
 // 128-bit shared-memory load) and its own LT/GL entries of the V row (producer, contiguous
 // in global memory) or of the T row (consumer, contiguous in shared memory).  The partial sums of
 // the (l, m) fibres are combined with fp64 atomic adds on Z.
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace cb {
@@ -111,7 +113,7 @@ __device__ __forceinline__ void sweep(const Csf3d &x, int32_t fA, int32_t fB, co
 template <int IS, int LT, int GL>
 __global__ void __launch_bounds__(kThreads)
 network_kernel(Csf3d u, const double *__restrict__ V, Csf3d w, double *__restrict__ Z, int n_k, int n_l, int n_m,
-               int v_vec_ok, const int32_t *__restrict__ mode) {
+               int v_vec_ok, int strips, int tiles, const int32_t *__restrict__ mode) {
     constexpr int VPT_P = LT / GL;                 // entries of a V row per lane (producer)
     constexpr int VPT_C = IS / GL;                 // entries of a T row per lane (consumer)
     static_assert(LT % GL == 0 && IS % GL == 0 && LT <= kMaxLT && (VPT_P == 1 || VPT_P % 2 == 0) &&
@@ -131,10 +133,13 @@ network_kernel(Csf3d u, const double *__restrict__ V, Csf3d w, double *__restric
     __shared__ int32_t s_first;
     st.first = &s_first;
 
-    const int strip = blockIdx.x, l0 = blockIdx.y * LT;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int q = threadIdx.x % GL;                // position inside the lane group
 
+    // one tile per block, or several where a short grid is launched in case it is needed (launch_network)
+    for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    const int strip = tile % strips, l0 = tile / strips * LT;
+    __syncthreads();                               // the tile before is done with the shared tables
     for (int e = threadIdx.x; e < LT * TL; e += kThreads) T[e] = 0.0;              // "T[*,*] = 0" per fused iteration
     if (threadIdx.x <= IS) {
         const int s = strip * IS + threadIdx.x;
@@ -154,7 +159,7 @@ network_kernel(Csf3d u, const double *__restrict__ V, Csf3d w, double *__restric
     }
     __syncthreads();
     const int nodes = w_nodes;
-    if (nodes == 0) return;                        // no W nonzero has its l in this tile: nothing reaches Z
+    if (nodes == 0) continue;                      // no W nonzero has its l in this tile: nothing reaches Z
 
     // ---- producer: T[l][k][ii] = sum_j U[i,k,j] * V[j, l0 + l]
     {
@@ -241,6 +246,7 @@ network_kernel(Csf3d u, const double *__restrict__ V, Csf3d w, double *__restric
                 if (rows[c] >= 0) atomicAdd(Z + (size_t)rows[c] * n_m + m, a[c] + b[c]);
         });
     }
+    }
 }
 
 }  // namespace
@@ -260,9 +266,13 @@ const_status_t launch_network(const const_csf *U, const double *V, const const_c
     Csf3d u{U->crd[0], U->pos[1], U->crd[1], U->pos[2], U->crd[2], static_cast<const double *>(U->vals), (int32_t)U->n[0]};
     Csf3d w{W->crd[0], W->pos[1], W->crd[1], W->pos[2], W->crd[2], static_cast<const double *>(W->vals), (int32_t)W->n[0]};
     const int v_vec_ok = (n_l % 2 == 0) && (reinterpret_cast<uintptr_t>(V) % 16 == 0);
-    dim3 grid((unsigned)((U->n[0] + IS - 1) / IS), (unsigned)((n_l + LT - 1) / LT));
+    const int64_t strips = (U->n[0] + IS - 1) / IS, tiles = strips * ((n_l + LT - 1) / LT);
+    if (tiles > 0x7fffffff) return CONST_ERR_WORKSPACE;
+    // Launched behind network_dense.cu it usually has nothing to do: sixteen blocks a slot find that out in a few us, one per
+    // tile took 19 us at 16 384 tiles (four a slot are slower where there is work: their tiles cost unequal time).
+    const unsigned grid = (unsigned)(mode ? std::min<int64_t>(tiles, 148 * 2 * 16) : tiles);
     CB_LAUNCH("network_kernel", stream,
-              kernel<<<grid, kThreads, smem, stream>>>(u, V, w, Z, (int)n_k, (int)n_l, (int)n_m, v_vec_ok, mode));
+              kernel<<<grid, kThreads, smem, stream>>>(u, V, w, Z, (int)n_k, (int)n_l, (int)n_m, v_vec_ok, (int)strips, (int)tiles, mode));
     CB_CUDA(cudaGetLastError());
     return CONST_OK;
 }

@@ -24,9 +24,9 @@ def kernels_of(w):
     (331, 61, 17, 0.25),      # nothing a multiple of a tile
     (300, 128, 12, 0.3),      # a full tile of k
     (260, 150, 12, 0.3),      # two tiles of k, the second of 22
-    (200, 7, 39, 0.6),        # the widest range of m that qualifies with four slices together (80)
-    (200, 9, 40, 0.6),        # one that does not (82)
-    (403, 33, 3, 1.0),        # narrow and full
+    (400, 7, 39, 0.6),        # the widest range of m that qualifies with four slices together (80)
+    (400, 9, 40, 0.6),        # one that does not (82)
+    (603, 33, 3, 1.0),        # narrow and full
 ])
 def test_banded(n, n_k, band, keep):
     w = network_workload(n, n_k, band, keep, config_id=61)
@@ -45,18 +45,19 @@ def scattered(n, n_k, nnz, seed):
 
 
 def test_operands_without_locality():
-    w = scattered(250, 20, 60_000, 1)
-    out, _ = kernels_of(w)
+    w = scattered(400, 20, 150_000, 1)
+    out, prof = kernels_of(w)
+    assert "network_t" in prof                                 # (asked for, and handed on by the device)
     S, A = oracle(w)
     assert_close(out, S, A, np.float64)
 
 
 def test_rows_and_slices_missing():
     """Slices of U and W without nonzeros, ranges at both ends of the extents."""
-    w = network_workload(300, 40, 10, 0.5, config_id=63)
+    w = network_workload(400, 40, 10, 0.5, config_id=63)
     for name, m in (("U", 0), ("W", 1)):
         op = w.sparse[name]
-        keep = (op.coords[m] % 5 != 2) & (op.coords[m] < 290)
+        keep = (op.coords[m] % 5 != 2) & (op.coords[m] < 390)
         w.sparse[name] = gen.SparseOperand([np.ascontiguousarray(c[keep]) for c in op.coords], np.ascontiguousarray(op.vals[keep]), op.dims)
     out, _ = kernels_of(w)
     S, A = oracle(w)
@@ -66,11 +67,12 @@ def test_rows_and_slices_missing():
 @pytest.mark.parametrize("value", [np.inf, np.nan])
 def test_values_no_nonzero_reads(value):
     """A row of V that no nonzero of U reads may hold anything, though it lies inside the ranges that are written out."""
-    w = network_workload(300, 40, 10, 0.5, config_id=64)
+    w = network_workload(400, 40, 10, 0.5, config_id=64)
     U = w.sparse["U"]
     keep = U.coords[1] != 150
     w.sparse["U"] = gen.SparseOperand([np.ascontiguousarray(c[keep]) for c in U.coords], np.ascontiguousarray(U.vals[keep]), U.dims)
     S, A = oracle(w)
     w.dense["V"][150] = value
-    out, _ = kernels_of(w)
+    out, prof = kernels_of(w)
+    assert "network_t" in prof
     assert_close(out, S, A, np.float64)
