@@ -65,8 +65,9 @@ typedef struct { const char *name; const const_csf_t *csf; const void *dense_dev
  *   vals[n]    value of leaf n (bit pattern untouched; explicit zeros are kept).
  * The coordinate tuple is packed into one 64-bit key (sum of ceil(log2 extent) over modes must be
  * <= 64), radix-sorted with its value, then each level is compressed with a flag/scan/scatter pass.
- * Per-slice nonzero counts and the light / heavy / giant work lists used by const_execute are built
- * here as well (on the device; the host does not wait for them).
+ * The leaf offset of every slice is written here as well; the light / heavy / giant work lists are
+ * built on the device when something first needs them (the tensor-core stage, const_csf_bin_counts,
+ * const_csf_work_lists).
  *
  * Errors: CONST_ERR_COORD_RANGE, CONST_ERR_DUPLICATE_COORD (both detected on the device; the call
  * waits for the stream once, after the sort, to read the level sizes and the status),
@@ -135,7 +136,8 @@ const_status_t const_csf_level(const const_csf_t *csf, int level, const int32_t 
 const_status_t const_csf_values(const const_csf_t *csf, const void **vals, int64_t *nnz);
 
 /*
- * Load balancing over slices of the root level (work lists consumed by const_execute).
+ * Load balancing over slices of the root level (work lists of the kernels with the tensor-core stage; the other
+ * kernels deal out equal runs of leaves and need no lists).
  * A slice with at most light_max_nnz nonzeros is processed by one warp; up to heavy_max_nnz by one
  * thread block; a larger ("giant") slice is split into blocks of about chunk_nnz nonzeros whose
  * partial results are added atomically.  const_csf_build applies defaults; this call replaces them
@@ -273,6 +275,8 @@ const_status_t const_schedule_cin(const char *expression, const char *const *tre
  * per-term relative error below 2^-19, so the fp32 tolerance holds); enable == 0: on the fp32 FMA pipes.
  * Plans that have the stage: order-4 TTMc at rank 8 and order-3 TTMc at rank 16 x 16.  Off unless asked for: the
  * fp32 path is the faster one on both (order 4, 50 M nonzeros: 2.3 against 3.1 ms) and the more accurate one.
+ * The stage works from the tensor's work lists, which are built at its first use: inside a stream capture that first use
+ * returns CONST_ERR_UNSUPPORTED (execute once, or call const_csf_bin_counts, before capturing).
  * CONST_ERR_UNSUPPORTED for enable != 0 on any other plan.  Host-only call; takes effect at the next
  * const_execute.  A device-side wait that runs out is reported through const_last_device_status.
  */

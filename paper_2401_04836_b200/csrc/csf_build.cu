@@ -1,5 +1,5 @@
 // GPU CSF builder (Sec. 2.1, CSF representation): pack -> LSD radix sort -> per-level compression,
-// followed by the per-slice load-balancing lists used by the fused contraction kernels.
+// and, on demand, the per-slice load-balancing lists used by the kernels with the tensor-core stage.
 //
 // Layout decisions
 //   * The permuted coordinate tuple is packed into one 64-bit key, root level in the top bits, so a
@@ -10,7 +10,7 @@
 //     tiles are ranked in shared memory, the tile's digit counts are chained to earlier tiles with a
 //     decoupled look-back (every spin is bounded and reports CONST_ERR_TIMEOUT), and keys are
 //     reordered in shared memory so that global stores run over consecutive addresses.
-//   * Compression is flag / scan / scatter: element e opens a node at level l when its length-(l+1)
+//   * Compression is flag / scan / scatter, two neighbouring keys per lane in 16-byte loads: element e opens a node at level l when its length-(l+1)
 //     prefix differs from that of e-1.
 #include <algorithm>
 #include <cstring>
@@ -1075,6 +1075,10 @@ int64_t item_capacity(const const_csf *csf) {
 // the device, for the stream that built them.
 const_status_t csf_ensure_bins(const_csf *csf, cudaStream_t stream) {
     std::lock_guard<std::mutex> lock(csf->bins_mu);
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    CB_CUDA(cudaStreamIsCapturing(stream, &capture));
+    if (capture != cudaStreamCaptureStatusNone)           // lists that outlive a graph cannot be allocated inside one
+        return csf->bins_valid ? CONST_OK : CONST_ERR_UNSUPPORTED;
     if (!csf->bins_valid) return csf_rebin_locked(csf, stream);
     if (csf->bins_ready && stream != csf->bin_stream) CB_CUDA(cudaStreamWaitEvent(stream, csf->bins_ready, 0));
     return CONST_OK;
