@@ -139,7 +139,7 @@ network_kernel(Csf3d u, const double *__restrict__ V, Csf3d w, double *__restric
     // one tile per block, or several where a short grid is launched in case it is needed (launch_network)
     for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
     const int strip = tile % strips, l0 = tile / strips * LT;
-    __syncthreads();                               // the tile before is done with the shared tables
+    if (tile != (int)blockIdx.x) __syncthreads();  // the tile before is done with the shared tables
     for (int e = threadIdx.x; e < LT * TL; e += kThreads) T[e] = 0.0;              // "T[*,*] = 0" per fused iteration
     if (threadIdx.x <= IS) {
         const int s = strip * IS + threadIdx.x;

@@ -65,9 +65,10 @@ struct Stmt {
     int32_t sA[3], sB[3];          // out, lhs, rhs
     int8_t pA[3], pB[3];
     // The result is private to the group, the two loops dealt as one both index it, and the loop Q around them locates
-    // nothing: then Q and the loops outside it run in step in all threads, the fused pair is dealt to the whole group, and
-    // no two threads touch one element between two barriers, so results are updated without atomics (shared memory has
-    // none in fp64: an atomic addition there is a compare-and-swap loop).  References are affine in Q, too (sQ, pQ).
+    // nothing: then Q can run in step in all threads, the fused pair is dealt to the whole group, and
+    // no two threads touch one element between two barriers, so results are updated without atomics.  References are
+    // affine in Q, too (sQ, pQ).  In fp64 only, where an atomic addition to shared memory costs several times one in fp32
+    // (running example: 64 in fp64 1570 -> 705 us; in fp32 the barriers cost more than they save: 52, 181 -> 210).
     int8_t exclusive;
     int8_t pQ[3];
     int32_t sQ[3];

@@ -308,7 +308,7 @@ struct Compiler {
                 }
             }
         }
-        if (s.fast && s.fuse_tail && s.n_priv >= 3 && s.out.kind == kRefPrivate) {
+        if (d.dtype == CONST_F64 && s.fast && s.fuse_tail && s.n_priv == 3 && s.out.kind == kRefPrivate) {
             const Loop &LB = e.p.loops[s.priv[s.n_priv - 1]], &LA = e.p.loops[s.priv[s.n_priv - 2]], &LQ = e.p.loops[s.priv[s.n_priv - 3]];
             bool has_a = false, has_b = false;
             for (int x = 0; x < s.out.n; ++x) {
