@@ -111,7 +111,8 @@ struct Group {
 // One assignment with its private loops: loop 0 over the warps of the group (over all its threads when it is
 // the only one), loop 1 over the lanes, deeper loops in sequence.  A dense innermost loop is first merged
 // with the loop around it (Stmt::fuse_tail), so that short sparse ranges still fill the lanes.
-template <typename T, bool WARP>
+// STEP: the kernel knows exclusive statements (Stmt::exclusive); without it they are dealt out like any other.
+template <typename T, bool WARP, bool STEP>
 __device__ void run_statement(const Stmt &s, const Program &p, const Bindings &b, State &st, T *scratch) {
     using G = Group<WARP>;
     for (int k = 0; k < s.n_sparse; ++k)
@@ -129,7 +130,7 @@ __device__ void run_statement(const Stmt &s, const Program &p, const Bindings &b
     int32_t cur[kMaxPriv], end[kMaxPriv];
     // In step only where an iteration of Q has enough updates for the group (running example in fp64, updates per iteration
     // and 256 threads: 320 at extent 64 and 20 000 nonzeros, 1570 -> 705 us; 75 at 40 and 3 000, 89 -> 100; dealt out instead).
-    bool exclusive = sizeof(T) == 8 && s.exclusive != 0;            // (a constant in fp32)
+    bool exclusive = STEP && s.exclusive != 0;
     if (exclusive) {
         const Loop &LQ = p.loops[s.priv[n - 3]], &LA = p.loops[s.priv[n - 2]];
         int32_t q0, q1, lo, hi;
@@ -306,7 +307,7 @@ __device__ void run_statement(const Stmt &s, const Program &p, const Bindings &b
 }
 
 // The instructions of one iteration of the loops spread over the grid.
-template <typename T, bool WARP>
+template <typename T, bool WARP, bool STEP>
 __device__ void run_body(const Program &p, const Bindings &b, State &st, T *scratch) {
     using G = Group<WARP>;
     int32_t cur[kMaxLoops], end[kMaxLoops];
@@ -319,7 +320,7 @@ __device__ void run_body(const Program &p, const Bindings &b, State &st, T *scra
             G::sync();
             ++pc;
         } else if (in.op == kOpStmt) {
-            run_statement<T, WARP>(p.stmts[in.arg], p, b, st, scratch);
+            run_statement<T, WARP, STEP>(p.stmts[in.arg], p, b, st, scratch);
             G::sync();
             ++pc;
         } else if (in.op == kOpLoopBegin) {
@@ -343,8 +344,10 @@ __device__ void run_body(const Program &p, const Bindings &b, State &st, T *scra
 // loops are spread together).  Groups take runs of `chunk` consecutive iterations, so that the level-0 node
 // above a level-1 node is searched for once per run and followed from there.
 // local_scratch: the private workspaces of a group live in shared memory (b.scratch is then unused).
-template <typename T, bool WARP>
-__global__ void __launch_bounds__(kThreads) tree_kernel(const __grid_constant__ Program p, const __grid_constant__ Bindings b,
+// (48 registers, five blocks per SM; with exclusive statements 71: only for workspaces that leave no room for more than
+// four blocks anyway.  Spilling them to 48: 1106 instead of 703 us on the running example at 64.)
+template <typename T, bool WARP, bool STEP>
+__global__ void __launch_bounds__(kThreads, STEP ? 3 : 5) tree_kernel(const __grid_constant__ Program p, const __grid_constant__ Bindings b,
                                                         int64_t root_count, int32_t chunk, int32_t local_scratch) {
     extern __shared__ __align__(16) unsigned char dyn_smem[];
     State st;
@@ -380,7 +383,7 @@ __global__ void __launch_bounds__(kThreads) tree_kernel(const __grid_constant__ 
             } else if (p.root_loop >= 0) {
                 bind(p.loops[p.root_loop], b, st, (int32_t)it);
             }
-            run_body<T, WARP>(p, b, st, scratch);
+            run_body<T, WARP, STEP>(p, b, st, scratch);
         }
     }
 }
@@ -416,8 +419,9 @@ const_status_t run_tree(const tree::Compiled &cp, const_dtype_t dtype, const con
     // per program: who runs an iteration (block or warp), where its workspaces live, how the iterations are dealt out
     constexpr int64_t kWarpScratchBytes = 4096;                       // up to here an iteration goes to one warp
     constexpr int64_t kLocalScratchBytes = 96 * 1024;                 // up to here the workspaces live in shared memory
+    constexpr int64_t kStepBytes = 44 * 1024;                         // workspaces from which at most four blocks fit an SM
     constexpr int kWarpsPerBlock = kThreads / 32;
-    struct Launch { int64_t grid, count; int chunk; bool warp, local; size_t smem; };
+    struct Launch { int64_t grid, count; int chunk; bool warp, local, step; size_t smem; };
     std::vector<Launch> launches;
     int64_t private_bytes = 0;
     for (size_t r = 0; r < cp.programs.size(); ++r) {
@@ -431,6 +435,10 @@ const_status_t run_tree(const tree::Compiled &cp, const_dtype_t dtype, const con
         const int64_t per_group = p.block_scratch * (int64_t)esize;
         if (per_group > kScratchBudget) return CONST_ERR_WORKSPACE;
         L.warp = p.root_loop >= 0 && p.n_instr > 1 && per_group <= kWarpScratchBytes;
+        L.step = false;                                               // kept exclusive statements: see tree_kernel
+        if (dtype == CONST_F64 && !L.warp && per_group >= kStepBytes)
+            for (int i = 0; i < p.n_instr; ++i)
+                L.step = L.step || (p.instr[i].op == kOpStmt && p.stmts[p.instr[i].arg].exclusive);
         const int groups_per_block = L.warp ? kWarpsPerBlock : 1;
         L.local = per_group * groups_per_block <= kLocalScratchBytes;
         L.smem = L.local ? (size_t)(per_group * groups_per_block) : 0;
@@ -446,10 +454,11 @@ const_status_t run_tree(const tree::Compiled &cp, const_dtype_t dtype, const con
     }
     static PerDeviceOnce smem_once;
     CB_CUDA(once_per_device(smem_once, [] {
-        cudaError_t e = cudaFuncSetAttribute(tree_kernel<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLocalScratchBytes);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(tree_kernel<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLocalScratchBytes);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(tree_kernel<double, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLocalScratchBytes);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(tree_kernel<double, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLocalScratchBytes);
+        cudaError_t e = cudaFuncSetAttribute(tree_kernel<float, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLocalScratchBytes);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(tree_kernel<float, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLocalScratchBytes);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(tree_kernel<double, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLocalScratchBytes);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(tree_kernel<double, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLocalScratchBytes);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(tree_kernel<double, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLocalScratchBytes);
         return e;
     }));
     const int64_t total_bytes = shared_elems * (int64_t)esize + private_bytes + 256;
@@ -477,13 +486,15 @@ const_status_t run_tree(const tree::Compiled &cp, const_dtype_t dtype, const con
         const int32_t local = L.local ? 1 : 0;
         CB_LAUNCH("tree_kernel", stream, {
             if (dtype == CONST_F32 && L.warp)
-                tree_kernel<float, true><<<grid, kThreads, L.smem, stream>>>(cp.programs[r], b, L.count, L.chunk, local);
+                tree_kernel<float, true, false><<<grid, kThreads, L.smem, stream>>>(cp.programs[r], b, L.count, L.chunk, local);
             else if (dtype == CONST_F32)
-                tree_kernel<float, false><<<grid, kThreads, L.smem, stream>>>(cp.programs[r], b, L.count, L.chunk, local);
+                tree_kernel<float, false, false><<<grid, kThreads, L.smem, stream>>>(cp.programs[r], b, L.count, L.chunk, local);
+            else if (L.step)
+                tree_kernel<double, false, true><<<grid, kThreads, L.smem, stream>>>(cp.programs[r], b, L.count, L.chunk, local);
             else if (L.warp)
-                tree_kernel<double, true><<<grid, kThreads, L.smem, stream>>>(cp.programs[r], b, L.count, L.chunk, local);
+                tree_kernel<double, true, false><<<grid, kThreads, L.smem, stream>>>(cp.programs[r], b, L.count, L.chunk, local);
             else
-                tree_kernel<double, false><<<grid, kThreads, L.smem, stream>>>(cp.programs[r], b, L.count, L.chunk, local);
+                tree_kernel<double, false, false><<<grid, kThreads, L.smem, stream>>>(cp.programs[r], b, L.count, L.chunk, local);
         });
         e = cudaGetLastError();
     }
