@@ -344,11 +344,8 @@ __device__ void run_body(const Program &p, const Bindings &b, State &st, T *scra
 // loops are spread together).  Groups take runs of `chunk` consecutive iterations, so that the level-0 node
 // above a level-1 node is searched for once per run and followed from there.
 // local_scratch: the private workspaces of a group live in shared memory (b.scratch is then unused).
-// (48 registers, five blocks per SM; with exclusive statements 71: only for workspaces that leave no room for more than
-// four blocks anyway.  Spilling them to 48: 1106 instead of 703 us on the running example at 64.)
 template <typename T, bool WARP, bool STEP>
-__global__ void __launch_bounds__(kThreads, STEP ? 3 : 5) tree_kernel(const __grid_constant__ Program p, const __grid_constant__ Bindings b,
-                                                        int64_t root_count, int32_t chunk, int32_t local_scratch) {
+__device__ __forceinline__ void tree_body(const Program &p, const Bindings &b, int64_t root_count, int32_t chunk, int32_t local_scratch) {
     extern __shared__ __align__(16) unsigned char dyn_smem[];
     State st;
     for (int k = 0; k < kMaxSparse; ++k) st.absent[k] = kAbsentNone;
@@ -386,6 +383,19 @@ __global__ void __launch_bounds__(kThreads, STEP ? 3 : 5) tree_kernel(const __gr
             run_body<T, WARP, STEP>(p, b, st, scratch);
         }
     }
+}
+
+template <typename T, bool WARP>
+__global__ void __launch_bounds__(kThreads) tree_kernel(const __grid_constant__ Program p, const __grid_constant__ Bindings b,
+                                                        int64_t root_count, int32_t chunk, int32_t local_scratch) {
+    tree_body<T, WARP, false>(p, b, root_count, chunk, local_scratch);
+}
+
+// With the in-step form of exclusive statements: 71 registers, so only for workspaces that leave no room for more than four
+// blocks anyway (in one kernel it costs smaller schedules their occupancy, extent 40: 89 -> 108 us, or spills, 64: 703 -> 1106).
+__global__ void __launch_bounds__(kThreads, 3) tree_step_kernel(const __grid_constant__ Program p, const __grid_constant__ Bindings b,
+                                                                int64_t root_count, int32_t chunk, int32_t local_scratch) {
+    tree_body<double, false, true>(p, b, root_count, chunk, local_scratch);
 }
 
 }  // namespace
@@ -435,7 +445,7 @@ const_status_t run_tree(const tree::Compiled &cp, const_dtype_t dtype, const con
         const int64_t per_group = p.block_scratch * (int64_t)esize;
         if (per_group > kScratchBudget) return CONST_ERR_WORKSPACE;
         L.warp = p.root_loop >= 0 && p.n_instr > 1 && per_group <= kWarpScratchBytes;
-        L.step = false;                                               // kept exclusive statements: see tree_kernel
+        L.step = false;                                               // kept exclusive statements: see tree_step_kernel
         if (dtype == CONST_F64 && !L.warp && per_group >= kStepBytes)
             for (int i = 0; i < p.n_instr; ++i)
                 L.step = L.step || (p.instr[i].op == kOpStmt && p.stmts[p.instr[i].arg].exclusive);
@@ -454,11 +464,11 @@ const_status_t run_tree(const tree::Compiled &cp, const_dtype_t dtype, const con
     }
     static PerDeviceOnce smem_once;
     CB_CUDA(once_per_device(smem_once, [] {
-        cudaError_t e = cudaFuncSetAttribute(tree_kernel<float, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLocalScratchBytes);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(tree_kernel<float, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLocalScratchBytes);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(tree_kernel<double, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLocalScratchBytes);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(tree_kernel<double, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLocalScratchBytes);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(tree_kernel<double, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLocalScratchBytes);
+        cudaError_t e = cudaFuncSetAttribute(tree_kernel<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLocalScratchBytes);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(tree_kernel<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLocalScratchBytes);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(tree_kernel<double, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLocalScratchBytes);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(tree_step_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLocalScratchBytes);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(tree_kernel<double, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLocalScratchBytes);
         return e;
     }));
     const int64_t total_bytes = shared_elems * (int64_t)esize + private_bytes + 256;
@@ -486,15 +496,15 @@ const_status_t run_tree(const tree::Compiled &cp, const_dtype_t dtype, const con
         const int32_t local = L.local ? 1 : 0;
         CB_LAUNCH("tree_kernel", stream, {
             if (dtype == CONST_F32 && L.warp)
-                tree_kernel<float, true, false><<<grid, kThreads, L.smem, stream>>>(cp.programs[r], b, L.count, L.chunk, local);
+                tree_kernel<float, true><<<grid, kThreads, L.smem, stream>>>(cp.programs[r], b, L.count, L.chunk, local);
             else if (dtype == CONST_F32)
-                tree_kernel<float, false, false><<<grid, kThreads, L.smem, stream>>>(cp.programs[r], b, L.count, L.chunk, local);
+                tree_kernel<float, false><<<grid, kThreads, L.smem, stream>>>(cp.programs[r], b, L.count, L.chunk, local);
             else if (L.step)
-                tree_kernel<double, false, true><<<grid, kThreads, L.smem, stream>>>(cp.programs[r], b, L.count, L.chunk, local);
+                tree_step_kernel<<<grid, kThreads, L.smem, stream>>>(cp.programs[r], b, L.count, L.chunk, local);
             else if (L.warp)
-                tree_kernel<double, true, false><<<grid, kThreads, L.smem, stream>>>(cp.programs[r], b, L.count, L.chunk, local);
+                tree_kernel<double, true><<<grid, kThreads, L.smem, stream>>>(cp.programs[r], b, L.count, L.chunk, local);
             else
-                tree_kernel<double, false, false><<<grid, kThreads, L.smem, stream>>>(cp.programs[r], b, L.count, L.chunk, local);
+                tree_kernel<double, false><<<grid, kThreads, L.smem, stream>>>(cp.programs[r], b, L.count, L.chunk, local);
         });
         e = cudaGetLastError();
     }
