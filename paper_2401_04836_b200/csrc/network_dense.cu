@@ -343,8 +343,8 @@ const_status_t run_network_dense(const const_csf *U, const double *V, const cons
     // line lies (multiply-adds of the gather form): at 1.1e8 the band at 331 takes 165 us in the gather form and 133 here,
     // below 6e7 the six extra launches (about 25 us, also paid by operands that then do not qualify) eat the gain.
     if (sparse < 6e7 || n_k > 4096 || kScratchBytes / row_bytes < std::min<int64_t>(n0, 64)) return CONST_OK;
-    if (n_l > (1 << 24) || n_m > (1 << 24) || groups > 65535 * 8ll) return CONST_OK;
-    int64_t chunk = std::min<int64_t>(n0, kScratchBytes / row_bytes);
+    if (n_l > (1 << 24) || n_m > (1 << 24) || groups > 65535 * 8ll || n0 + W->n[0] > 0x7fffffffll) return CONST_OK;
+    int64_t chunk = std::min<int64_t>({n0, kScratchBytes / row_bytes, 65535ll * kRows});       // what T may take, and the rows of a grid
     const int64_t chunks = (n0 + chunk - 1) / chunk;
     chunk = ((n0 + chunks - 1) / chunks + kRows - 1) / kRows * kRows;     // even chunks of whole blocks, never more than fit
     if (chunk * row_bytes > kScratchBytes) chunk = kScratchBytes / row_bytes;

@@ -2,11 +2,12 @@
 written out densely: against the oracle, element by element."""
 import numpy as np
 import pytest
+import torch
 
 import paper_2401_04836_b200 as cb
 from workloads import generators as gen
 from workloads import network_workload
-from tests.gpu_util import assert_close, oracle, run_workload
+from tests.gpu_util import assert_close, oracle, run_workload, to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -76,3 +77,22 @@ def test_values_no_nonzero_reads(value):
     out, prof = kernels_of(w)
     assert "network_t" in prof
     assert_close(out, S, A, np.float64)
+
+
+def test_more_rows_than_a_grid_has():
+    """One l and eight k: a chunk of the intermediate holds 4 194 304 slices of U, 65 536 rows of blocks."""
+    n = 4_194_300
+    rng = np.random.default_rng(66)
+    i = np.arange(n, dtype=np.int32)
+    u = [i, i % 90, i % 8]
+    k, m = (x.ravel().astype(np.int32) for x in np.mgrid[0:8, 0:8])
+    uv, wv, V = rng.standard_normal(n), rng.standard_normal(64), rng.standard_normal((90, 1))
+    plan = cb.const_plan_create("Z[i,m] = U[i,j,k] * V[j,l] * W[k,l,m]", ["T[i,k,l] = U[i,j,k] * V[j,l]", "Z[i,m] = T[i,k,l] * W[k,l,m]"],
+                                {"U": (0, 2, 1), "W": (1, 2, 0)}, ["ikjl", "ilmk"], {"i": n, "j": 90, "k": 8, "l": 1, "m": 8}, cb.F64)
+    U = cb.const_csf_build([to_dev(c) for c in u], to_dev(uv), (n, 90, 8), (0, 2, 1))
+    W = cb.const_csf_build([to_dev(k), to_dev(0 * k), to_dev(m)], to_dev(wv), (8, 1, 8), (1, 2, 0))
+    out = torch.full((n, 8), float("nan"), dtype=torch.float64, device="cuda")
+    cb.const_execute(plan, {"U": U, "V": to_dev(V), "W": W}, out)
+    assert cb.const_last_device_status(plan) == 0
+    S = (uv * V[u[1], 0])[:, None] * wv.reshape(8, 8)[u[2]]
+    assert np.all(np.abs(out.cpu().numpy() - S) <= 1e-12 * np.abs(S))
