@@ -585,13 +585,20 @@ const_status_t run_any(const const_csf *X, bool mttkrp, const void *const *facto
     pad.first[3] = total;
     T *scratch = nullptr;
     if (padded) {
-        if (scratch_alloc((void **)&scratch, sizeof(T) * total, stream) != cudaSuccess) return CONST_ERR_UNSUPPORTED;
+        if (scratch_alloc((void **)&scratch, sizeof(T) * total, stream) != cudaSuccess) {
+            (void)cudaGetLastError();                   // the caller goes on without: the next launch must not find this error
+            return CONST_ERR_UNSUPPORTED;
+        }
         for (int f = 0; f < 3; ++f) {
             pad.dst[f] = scratch + pad.first[f];
             if (pad.src[f]) F[f] = pad.dst[f];
         }
         const int blocks = (int)std::min<int64_t>((total + 255) / 256, 148 * 8);
         CB_LAUNCH("pad_factors", stream, pad_factors<T><<<blocks, 256, 0, stream>>>(pad));
+        if (cudaGetLastError() != cudaSuccess) {
+            cudaFreeAsync(scratch, stream);
+            return CONST_ERR_CUDA;
+        }
     }
     const_status_t rc;
     const int rp = width[0] > 32 ? 32 : width[0];

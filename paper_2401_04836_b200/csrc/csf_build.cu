@@ -1020,6 +1020,7 @@ cudaError_t scratch_alloc(void **p, size_t bytes, cudaStream_t stream) {
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     const cudaError_t e = cudaStreamIsCapturing(stream, &capture);
     if (e != cudaSuccess) return e;
+    if (debug_knobs().no_scratch) bytes = (size_t)1 << 60;                 // more than any device has: the allocator's own error
     return capture == cudaStreamCaptureStatusNone ? pool_alloc(p, bytes, stream) : cudaMallocAsync(p, bytes, stream);
 }
 

@@ -120,3 +120,17 @@ def test_short_fibres_of_a_tensor_above_a_million(rank):
     rows = np.arange(0, 60, 7)
     S, A = oracle(w, rows)
     assert_close(out, S, A, np.float32, rows)
+
+
+@pytest.mark.parametrize("family,dims,ranks,dtype", [("ttmc", (25, 20, 30), (6, 10), cb.F32), ("mttkrp", (20, 9, 8, 7), (5, 5, 5), cb.F64)])
+def test_without_memory_for_padded_factors(family, dims, ranks, dtype):
+    """The generic executor needs none: the call succeeds there, and nothing of the failed request stays behind."""
+    X, fac = inputs(family, dims, ranks, 1500, dtype, 3)
+    cb.const_debug_set(3, 1)
+    try:
+        out, S, A = run_chain(family, dims, ranks, X, fac, dtype)
+    finally:
+        cb.const_debug_set(3, 0)
+    assert_close(out, S, A, X.vals.dtype)
+    out, S, A = run_chain(family, dims, ranks, X, fac, dtype)
+    assert_close(out, S, A, X.vals.dtype)

@@ -96,3 +96,16 @@ def test_more_rows_than_a_grid_has():
     assert cb.const_last_device_status(plan) == 0
     S = (uv * V[u[1], 0])[:, None] * wv.reshape(8, 8)[u[2]]
     assert np.all(np.abs(out.cpu().numpy() - S) <= 1e-12 * np.abs(S))
+
+
+def test_without_memory_for_the_intermediate():
+    """The gather form needs none."""
+    w = network_workload(331, 61, 17, 0.25, config_id=61)
+    cb.const_debug_set(3, 1)
+    try:
+        out, prof = kernels_of(w)
+    finally:
+        cb.const_debug_set(3, 0)
+    assert "network_t" not in prof
+    S, A = oracle(w)
+    assert_close(out, S, A, np.float64)
