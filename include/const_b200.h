@@ -284,9 +284,10 @@ const_status_t const_plan_set_tensor_stage(const_plan_t *plan, int enable);
 
 /*
  * enable != 0: const_execute runs this plan on the generic executor (family "tree" of const_plan_create)
- * although a hand-written family matches it; enable == 0: back to the family.  CONST_ERR_UNSUPPORTED when
- * the schedule exceeds the generic executor's capacities (enable != 0) or when the plan has no other
- * kernel (enable == 0).  Host-only call.
+ * although hand-written kernels take it (those of its family, or the chain kernels for a chain at other ranks or in
+ * fp64); enable == 0: back to them.  CONST_ERR_UNSUPPORTED when the schedule exceeds the generic executor's capacities
+ * (enable != 0), and for enable == 0 on a plan of family "tree" that an earlier call has not moved away from the chain
+ * kernels.  Host-only call.
  */
 const_status_t const_plan_set_generic_executor(const_plan_t *plan, int enable);
 

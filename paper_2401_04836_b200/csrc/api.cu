@@ -39,6 +39,12 @@ bool csf_matches(const const_csf *c, const PlanDesc &d, const std::string &name,
     return true;
 }
 
+// whether the leaf-balanced chain kernels can take a plan of family "tree"
+bool fused_chain(const PlanDesc &d) {
+    return d.family == Family::Tree && d.chain != PlanDesc::Chain::None &&
+           chain_covers((int)d.ranks.size() + 1, d.chain == PlanDesc::Chain::Mttkrp, d.ranks.data());
+}
+
 bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 std::atomic<int> g_spin_limit{0}, g_withhold{0}, g_variant{0}, g_no_scratch{0};
@@ -286,8 +292,7 @@ const_status_t const_execute(const_plan_t *h, const const_operand_t *operands, i
         }
     }
     // a fully fused chain at a rank or in a type without a family of its own: the leaf-balanced kernels take it
-    if (d.family == Family::Tree && !p->use_tree && d.chain != PlanDesc::Chain::None &&
-        chain_covers((int)d.ranks.size() + 1, d.chain == PlanDesc::Chain::Mttkrp, d.ranks.data())) {
+    if (!p->use_tree && fused_chain(d)) {
         const const_operand_t *x = find_operand(operands, n_operands, d.sparse_name);
         if (!x || !x->csf || x->dense_dev) return CONST_ERR_INVALID_ARG;
         const const_csf *X = as_csf(x->csf);
@@ -396,7 +401,8 @@ const_status_t const_plan_set_generic_executor(const_plan_t *h, int enable) {
     const_plan *p = const_cast<const_plan *>(as_plan(h));
     if (!p) return CONST_ERR_INVALID_ARG;
     if (enable && !p->tree_ok) return CONST_ERR_UNSUPPORTED;
-    if (!enable && p->desc.family == Family::Tree) return CONST_ERR_UNSUPPORTED;   // nothing else can run this plan
+    // family "tree": there is a way back only for a chain that was moved here from the chain kernels
+    if (!enable && p->desc.family == Family::Tree && !(p->use_tree && fused_chain(p->desc))) return CONST_ERR_UNSUPPORTED;
     p->use_tree = enable ? 1 : 0;
     return CONST_OK;
 }

@@ -78,6 +78,26 @@ def test_agrees_with_the_generic_executor(family, dims, ranks):
     assert_close(b, S, A, np.float64)
 
 
+def test_generic_executor_on_off_and_on_again():
+    """One plan of family "tree" that the chain kernels take: which kernels run is seen in the profile."""
+    w = ttmc3_workload((25, 20, 30), 1500, (6, 10), value="pm1", config_id=31)
+    S, A = oracle(w)
+    plan = cb.const_plan_create(w.expression, w.tree, w.mode_orders, w.loop_orders, w.extents, cb.F32)
+    assert cb.const_plan_family(plan) == "tree"
+    ops = {"X": build_csf(w.sparse["X"], w.mode_orders["X"])}
+    ops.update({n: to_dev(a) for n, a in w.dense.items()})
+    for generic in (None, True, False, True, True, False):
+        if generic is not None:
+            cb.const_plan_set_generic_executor(plan, generic)
+        out = torch.full(w.out_shape, float("nan"), device="cuda")
+        cb.const_profile_enable(True)
+        cb.const_execute(plan, ops, out)
+        prof = cb.const_profile_read()
+        cb.const_profile_enable(False)
+        assert ("tree_kernel" in prof) == bool(generic) and ("chain3_kernel" in prof) == (not generic), (generic, prof)
+        assert_close(out.cpu().numpy(), S, A, np.float32)
+
+
 @pytest.mark.parametrize("family,ranks", [("ttmc", (7, 10)), ("mttkrp", (6, 6))])
 def test_rows_a_tensor_does_not_name_stay_out(family, ranks):
     """A factor row that no nonzero reads may hold anything: neither padding nor unused records may touch it."""
