@@ -306,7 +306,7 @@ const_status_t launch_chain3(const Args &a, int64_t n_rows, cudaStream_t stream)
 // Same contraction as the leaf-balanced walk of chain_kernels.cu.
 const_status_t run_ttmc3_fibres(const const_csf *X, const float *U, const float *V, int R2, int R3, float *Y, int64_t n_rows,
                                 cudaStream_t s) {
-    const Args a{walk::chain_of<float, 3>(X), U, V, Y, walk::chunk_leaves(X->nnz, 16, 1536)};
+    const Args a{walk::chain_of<float, 3>(X), U, V, Y, walk::chunk_leaves(X->nnz, X->n[0], 16, 1536, 16)};
     switch (R2 * 100 + R3) {
         case 808: return launch_chain3<8, 8>(a, n_rows, s);
         case 816: return launch_chain3<8, 16>(a, n_rows, s);

@@ -41,6 +41,11 @@ using namespace walk;
 constexpr int kWarps = 4;                             // warps per block; they share nothing
 constexpr int kUnroll = 4;                            // row gathers in flight per lane
 
+// blocks an SM holds: what the registers are cut for, or the shared memory (warp_bytes per warp) allows
+constexpr int blocks_that_fit(int by_registers, size_t warp_bytes) {
+    return std::min(by_registers, (int)(227 * 1024 / (warp_bytes * kWarps + 1024)));
+}
+
 template <typename T>
 __device__ __forceinline__ void put_entry(T *dst, T v, bool whole) {
     if (whole) *dst = v;
@@ -88,9 +93,11 @@ __device__ __forceinline__ void reduce_pair(Pair<T> &p, int from) {
 template <typename T, int ORDER, int RP>
 struct MttkrpShape {
     static constexpr int N = Vec<T>::N;
-        static constexpr int LPR = RP / N;                // lanes per factor row
+    static constexpr int LPR = RP / N;                // lanes per factor row
     static constexpr int G = 32 / LPR;                // lane groups per warp
     static constexpr int W = 128;                     // leaves per window
+    static constexpr int BLOCKS = sizeof(T) == 4 ? (ORDER == 3 ? 8 : 6) : 4;          // resident blocks the registers are cut for
+    static constexpr int FIT = (sizeof(T) == 8 && ORDER == 3 ? 6 : BLOCKS) * kWarps;  // warps an SM holds (fp64, order 3: 80 registers)
     static_assert(LPR >= 1 && LPR <= 32, "rank tile");
 };
 
@@ -100,12 +107,13 @@ struct MttkrpArgs {
     Chain<T, ORDER> x;
     const T *F[ORDER - 1];
     T *out;
-    int32_t stride, R, chunk;
     size_t out_bytes;
+    int32_t stride, R;
+    int32_t chunk;                                    // leaves per warp (set by the launch)
 };
 
 template <typename T, int ORDER, int RP>
-__global__ void __launch_bounds__(kWarps * 32, sizeof(T) == 4 ? (ORDER == 3 ? 8 : 6) : 4) mttkrp_kernel(const __grid_constant__ MttkrpArgs<T, ORDER> a) {
+__global__ void __launch_bounds__(kWarps * 32, MttkrpShape<T, ORDER, RP>::BLOCKS) mttkrp_kernel(const __grid_constant__ MttkrpArgs<T, ORDER> a) {
     using S = MttkrpShape<T, ORDER, RP>;
     constexpr int N = S::N;
     __shared__ Stage<T, ORDER, S::W> stages[kWarps];
@@ -184,6 +192,7 @@ struct Ttmc3Shape {
         T t[W * R3];                                  // parked t, one row per piece
         T u[W * R2];                                  // the factor row that goes with it
     };
+    static constexpr int FIT = blocks_that_fit(BLOCKS, sizeof(Smem)) * kWarps;       // warps an SM holds
 };
 
 template <typename T>
@@ -191,8 +200,9 @@ struct Ttmc3Args {
     Chain<T, 3> x;
     const T *U, *V;                                   // rows of R2 and R3 (padded) entries
     T *out;
-    int32_t R2, R3, chunk;                            // real ranks
     size_t out_bytes;
+    int32_t R2, R3;                                   // real ranks
+    int32_t chunk;                                    // leaves per warp (set by the launch)
 };
 
 template <typename T, int R2, int R3>
@@ -297,6 +307,7 @@ struct Ttmc4Shape {
     static constexpr int N = Vec<T>::N;
     static constexpr int R = 8, SL = 4, G = 32 / SL;  // lanes per producer group, groups per warp
     static constexpr int W = 64, P = 40;              // leaves per window, parked Q (a window that would need more is halved)
+    static constexpr int BLOCKS = sizeof(T) == 4 ? 3 : 1;              // resident blocks the registers are cut for
     static constexpr int QROW = R * R + 16;           // 16 spare entries: neighbouring pieces start in other banks
     // A lane of a producer group holds 2 R entries of Q as chunks of 16 bytes; chunk c of lane h is parked at
     // (c * SL + h) * 16 bytes, so that the lanes of a group write neighbouring chunks.
@@ -305,6 +316,7 @@ struct Ttmc4Shape {
         T q[P * QROW];                                // parked Q
         T u[P * R];                                   // the factor row that goes with it
     };
+    static constexpr int FIT = blocks_that_fit(BLOCKS, sizeof(Smem)) * kWarps;
 };
 
 template <typename T>
@@ -312,12 +324,13 @@ struct Ttmc4Args {
     Chain<T, 4> x;
     const T *U, *V, *W;                               // rows of 8 entries
     T *out;
-    int32_t R2, R3, R4, chunk;                        // real ranks
     size_t out_bytes;
+    int32_t R2, R3, R4;                               // real ranks
+    int32_t chunk;                                    // leaves per warp (set by the launch)
 };
 
 template <typename T>
-__global__ void __launch_bounds__(kWarps * 32, sizeof(T) == 4 ? 3 : 1) ttmc4_kernel(const __grid_constant__ Ttmc4Args<T> a) {
+__global__ void __launch_bounds__(kWarps * 32, Ttmc4Shape<T>::BLOCKS) ttmc4_kernel(const __grid_constant__ Ttmc4Args<T> a) {
     using S = Ttmc4Shape<T>;
     constexpr int N = S::N, R = S::R, NV = R / N;
     extern __shared__ __align__(16) unsigned char smem[];
@@ -483,13 +496,15 @@ unsigned chunk_blocks(int64_t nnz, int32_t chunk) {
 }
 
 template <typename T, int ORDER, int RP>
-const_status_t launch_mttkrp(MttkrpArgs<T, ORDER> a, int tiles, cudaStream_t stream) {
+const_status_t launch_mttkrp(MttkrpArgs<T, ORDER> a, int resident, int tiles, cudaStream_t stream) {
+    a.chunk = chunk_leaves(a.x.n[ORDER - 1], a.x.n[0], resident, 4096, MttkrpShape<T, ORDER, RP>::FIT);
     const dim3 grid(chunk_blocks(a.x.n[ORDER - 1], a.chunk), (unsigned)tiles);
     return launch_on_cleared("chain3_kernel", mttkrp_kernel<T, ORDER, RP>, a, grid, kWarps * 32, 0, a.out, a.out_bytes, stream);
 }
 
 template <typename T, int R2, int R3>
-const_status_t launch_ttmc3(const Ttmc3Args<T> &a, cudaStream_t stream) {
+const_status_t launch_ttmc3(Ttmc3Args<T> a, cudaStream_t stream) {
+    a.chunk = chunk_leaves(a.x.n[2], a.x.n[0], 20, 3072, Ttmc3Shape<T, R2, R3>::FIT);
     constexpr size_t dyn = sizeof(typename Ttmc3Shape<T, R2, R3>::Smem) * kWarps;
     static PerDeviceOnce attr_once;                     // per template instance
     CB_CUDA(once_per_device(attr_once, [&] { return cudaFuncSetAttribute(ttmc3_kernel<T, R2, R3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn); }));
@@ -515,18 +530,19 @@ const_status_t dispatch_ttmc3(const Ttmc3Args<T> &a, int r2, int r3, cudaStream_
 }
 
 template <typename T, int ORDER>
-const_status_t dispatch_mttkrp(const MttkrpArgs<T, ORDER> &a, int rp, int tiles, cudaStream_t s) {
+const_status_t dispatch_mttkrp(const MttkrpArgs<T, ORDER> &a, int resident, int rp, int tiles, cudaStream_t s) {
     switch (rp) {
-        case 4: return launch_mttkrp<T, ORDER, 4>(a, tiles, s);
-        case 8: return launch_mttkrp<T, ORDER, 8>(a, tiles, s);
-        case 16: return launch_mttkrp<T, ORDER, 16>(a, tiles, s);
-        case 32: return launch_mttkrp<T, ORDER, 32>(a, tiles, s);
+        case 4: return launch_mttkrp<T, ORDER, 4>(a, resident, tiles, s);
+        case 8: return launch_mttkrp<T, ORDER, 8>(a, resident, tiles, s);
+        case 16: return launch_mttkrp<T, ORDER, 16>(a, resident, tiles, s);
+        case 32: return launch_mttkrp<T, ORDER, 32>(a, resident, tiles, s);
     }
     return CONST_ERR_UNSUPPORTED;
 }
 
 template <typename T>
-const_status_t launch_ttmc4(const Ttmc4Args<T> &a, cudaStream_t stream) {
+const_status_t launch_ttmc4(Ttmc4Args<T> a, cudaStream_t stream) {
+    a.chunk = chunk_leaves(a.x.n[3], a.x.n[0], 12, 4096, Ttmc4Shape<T>::FIT);
     constexpr size_t dyn = sizeof(typename Ttmc4Shape<T>::Smem) * kWarps;
     static PerDeviceOnce attr_once;                     // per template instance
     CB_CUDA(once_per_device(attr_once, [&] { return cudaFuncSetAttribute(ttmc4_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn); }));
@@ -603,16 +619,13 @@ const_status_t run_any(const const_csf *X, bool mttkrp, const void *const *facto
     const_status_t rc;
     const int rp = width[0] > 32 ? 32 : width[0];
     if (mttkrp && X->order == 3)
-        rc = dispatch_mttkrp<T, 3>({chain_of<T, 3>(X), {F[0], F[1]}, out, width[0], ranks[0], chunk_leaves(X->nnz, 24, 4096), bytes}, rp,
-                                   width[0] / rp, stream);
+        rc = dispatch_mttkrp<T, 3>({chain_of<T, 3>(X), {F[0], F[1]}, out, bytes, width[0], ranks[0]}, 24, rp, width[0] / rp, stream);
     else if (mttkrp)
-        rc = dispatch_mttkrp<T, 4>({chain_of<T, 4>(X), {F[0], F[1], F[2]}, out, width[0], ranks[0], chunk_leaves(X->nnz, 24, 4096), bytes}, rp,
-                                   width[0] / rp, stream);
+        rc = dispatch_mttkrp<T, 4>({chain_of<T, 4>(X), {F[0], F[1], F[2]}, out, bytes, width[0], ranks[0]}, 24, rp, width[0] / rp, stream);
     else if (X->order == 3)
-        rc = dispatch_ttmc3<T>({chain_of<T, 3>(X), F[0], F[1], out, ranks[0], ranks[1], chunk_leaves(X->nnz, 20, 3072), bytes}, width[0], width[1],
-                               stream);
+        rc = dispatch_ttmc3<T>({chain_of<T, 3>(X), F[0], F[1], out, bytes, ranks[0], ranks[1]}, width[0], width[1], stream);
     else
-        rc = launch_ttmc4<T>({chain_of<T, 4>(X), F[0], F[1], F[2], out, ranks[0], ranks[1], ranks[2], chunk_leaves(X->nnz, 12, 4096), bytes}, stream);
+        rc = launch_ttmc4<T>({chain_of<T, 4>(X), F[0], F[1], F[2], out, bytes, ranks[0], ranks[1], ranks[2]}, stream);
     if (scratch) cudaFreeAsync(scratch, stream);
     return rc;
 }
@@ -658,17 +671,20 @@ const_status_t run_ttmc3(const const_csf *X, const float *U, const float *V, int
     // Short fibres go to the record walk, whose cost is per leaf; chain3_kernel pays per fibre, but less per leaf of a long
     // one and less to start.  Measured, walk against chain3_kernel (us): 20 M leaves in fibres of one, 16 x 16: 607 / 886;
     // of two: 405 / 470; of four: 362 / 354; 32 x 32 in fibres of two: 939 / 880; 1 M leaves in fibres of one: 68 / 79, of
-    // two: 46 / 43.
-    const double per_fibre = (double)X->nnz / (double)X->n[1];
-    if (X->nnz < 1000000 || per_fibre > (R2 * R3 < 1024 ? 2.5 : 1.8)) return run_ttmc3_fibres(X, U, V, R2, R3, Y, n_rows, stream);
-    return dispatch_ttmc3<float>({chain_of<float, 3>(X), U, V, Y, R2, R3, chunk_leaves(X->nnz, 20, 3072), bytes}, R2, R3, stream);
+    // two: 46 / 43.  Below a million leaves only where the slices fill a few windows, and not at 32 x 32: 100 000 leaves in
+    // fibres of one, 16 x 16, slices of 1 / 4 / 16 / 64: 106 / 95, 51 / 51, 23 / 27, 17.4 / 18.3; 300 000: 351 / 264,
+    // 143 / 128, 47 / 54, 27 / 30; 32 x 32, 300 000: 612 / 407, 238 / 168, 83 / 69, 49 / 42.
+    const double per_fibre = (double)X->nnz / (double)X->n[1], per_slice = (double)X->nnz / (double)X->n[0];
+    const bool wide = R2 * R3 >= 1024, many = X->nnz >= 1000000 || (X->nnz >= 100000 && per_slice >= 16 && !wide);
+    if (!many || per_fibre > (wide ? 1.8 : 2.5)) return run_ttmc3_fibres(X, U, V, R2, R3, Y, n_rows, stream);
+    return dispatch_ttmc3<float>({chain_of<float, 3>(X), U, V, Y, bytes, R2, R3}, R2, R3, stream);
 }
 
 const_status_t run_mttkrp3(const const_csf *X, const float *B, const float *C, int R, float *A, int64_t n_rows,
                            int32_t *, cudaStream_t stream) {
     const size_t bytes = sizeof(float) * R * n_rows;
     if (X->nnz == 0) return clear_result(A, bytes, stream) == cudaSuccess ? CONST_OK : CONST_ERR_CUDA;
-    return dispatch_mttkrp<float, 3>({chain_of<float, 3>(X), {B, C}, A, R, R, chunk_leaves(X->nnz, 32, 4096), bytes}, R, 1, stream);
+    return dispatch_mttkrp<float, 3>({chain_of<float, 3>(X), {B, C}, A, bytes, R, R}, 32, R, 1, stream);
 }
 
 const_status_t run_ttmc4(const const_csf *X, const float *U, const float *V, const float *W, int rank, float *Y,
@@ -676,7 +692,7 @@ const_status_t run_ttmc4(const const_csf *X, const float *U, const float *V, con
     if (rank != 8) return CONST_ERR_UNSUPPORTED;
     const size_t bytes = sizeof(float) * 512 * n_rows;
     if (X->nnz == 0) return clear_result(Y, bytes, stream) == cudaSuccess ? CONST_OK : CONST_ERR_CUDA;
-    return launch_ttmc4<float>({chain_of<float, 4>(X), U, V, W, Y, rank, rank, rank, chunk_leaves(X->nnz, 12, 4096), bytes}, stream);
+    return launch_ttmc4<float>({chain_of<float, 4>(X), U, V, W, Y, bytes, rank, rank, rank}, stream);
 }
 
 }  // namespace cb

@@ -154,3 +154,29 @@ def test_without_memory_for_padded_factors(family, dims, ranks, dtype):
     assert_close(out, S, A, X.vals.dtype)
     out, S, A = run_chain(family, dims, ranks, X, fac, dtype)
     assert_close(out, S, A, X.vals.dtype)
+
+
+@pytest.mark.parametrize("dtype", [cb.F32, cb.F64])
+@pytest.mark.parametrize("family,ranks,dims", [("ttmc", (8, 8), (2000, 50, 60)), ("ttmc", (16, 8), (2000, 50, 60)), ("mttkrp", (8, 8), (2000, 50, 60)),
+                                               ("ttmc", (8, 8, 8), (150, 12, 10, 9)), ("mttkrp", (5, 5, 5), (400, 12, 10, 9))])
+@pytest.mark.parametrize("nnz", [592, 593, 2369, 9473])
+def test_short_slices_dealt_out_in_small_chunks(family, ranks, dims, dtype, nnz):
+    """Chunks of one leaf, of a few, and of up to 64: around the numbers of warps that are resident at once (148 SMs times
+    4 to 32), with slices of one leaf and of several chunks."""
+    X, fac = inputs(family, dims, ranks, nnz, dtype, nnz + len(dims))
+    hot = X.coords[0] % 7 == 0                                 # a seventh of the nonzeros into three slices
+    X = gen.SparseOperand([np.where(hot, X.coords[0] % 3, X.coords[0]).astype(np.int32)] + list(X.coords[1:]), X.vals, X.dims)
+    key = np.sort(np.unique(np.ravel_multi_index([c.astype(np.int64) for c in X.coords], dims), return_index=True)[1])
+    X = gen.SparseOperand([np.ascontiguousarray(c[key]) for c in X.coords], np.ascontiguousarray(X.vals[key]), X.dims)
+    out, S, A = run_chain(family, dims, ranks, X, fac, dtype)
+    assert_close(out, S, A, X.vals.dtype)
+
+
+def test_ttmc3_below_a_million_in_slices_of_several_windows():
+    """The size and slice length from which order-3 TTMc takes the record walk below a million nonzeros, and just below."""
+    for dims, nnz, rank in (((5000, 400, 700), 100_100, (8, 8)), ((5000, 400, 700), 99_000, (8, 8)), ((7000, 400, 700), 110_000, (16, 16)),
+                            ((7500, 400, 700), 110_000, (16, 16)), ((5000, 400, 700), 110_000, (32, 32))):
+        w = ttmc3_workload(dims, nnz, rank, slice_s=0.3, inner_s=None, value="pm1", config_id=25)
+        out, _ = run_workload(w)
+        S, A = oracle(w)
+        assert_close(out, S, A, np.float32)
