@@ -199,7 +199,9 @@ const_status_t const_csf_work_lists(const const_csf_t *csf, const int32_t **slic
  *           contractions then gather along a fibre; fused over i only (T reduced to order 2).  CONST_F64.
  *           A chain at other ranks or in fp64 (order-3 TTMc up to rank 32, order-4 TTMc up to rank 8, MTTKRP of
  *           order 3 and 4 up to rank 1024) belongs to family "tree" but runs on the fused kernels of this family,
- *           unless const_plan_set_generic_executor asks for the generic executor.
+ *           unless const_plan_set_generic_executor asks for the generic executor.  Ranks between their widths are copied
+ *           into padded factors at every execute (scratch of their size); with more than 256 padded entries per nonzero,
+ *           or without memory for them, the generic executor does the work instead.
  *   tree    the generic executor (Sec. 4.2: it walks the loop tree that Algorithm 1 prints as forall / where
  *           constructs).  Any checked schedule, any number of CSF operands, fp32 or fp64: e.g. the running
  *           example R_ijk = A_ipq B_jpr C_kqr D_jkr with X and Y as 2-D workspaces inside the fused r, j

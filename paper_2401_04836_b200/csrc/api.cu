@@ -307,7 +307,7 @@ const_status_t const_execute(const_plan_t *h, const const_operand_t *operands, i
         for (char c : d.result.idx) elems *= d.extents.at(c);
         const const_status_t rc = run_chain_any(X, d.chain == PlanDesc::Chain::Mttkrp, factors, d.ranks.data(), d.dtype, out_dev,
                                                 elems, stream);
-        if (rc != CONST_ERR_UNSUPPORTED) return rc;      // no memory for padded factors: the generic executor needs none
+        if (rc != CONST_ERR_UNSUPPORTED) return rc;      // the generic executor needs no padded factors
     }
     if (d.family == Family::Tree || p->use_tree) {
         const tree::Compiled &cp = p->tree;

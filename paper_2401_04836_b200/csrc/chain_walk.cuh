@@ -420,14 +420,14 @@ inline int32_t chunk_leaves(int64_t nnz, int64_t slices, int resident, int64_t m
     return (int32_t)((c + 63) / 64 * 64);
 }
 
-// Clears `out` ("R[*] = 0" precedes the nest) and launches the kernel so that it starts while the clearing still runs: it
+// Clears `out` ("R[*] = 0" precedes the nest; bytes = 0: the launch before has done that) and launches the kernel so that it starts while the clearing still runs: it
 // looks its place in the tensor up meanwhile and waits (after_clear) before it writes.  Clearing by a kernel of the
 // library instead of a memset is what allows that (20 000 nonzeros at rank 8, device time bound by the two launches:
 // 14.2 -> 13.9 us a call).
 template <class Args>
 inline const_status_t launch_on_cleared(const char *name, void (*kernel)(Args), const Args &args, dim3 grid, int threads, size_t smem,
                                         void *out, size_t bytes, cudaStream_t stream) {
-    CB_CUDA(clear_result(out, bytes, stream));
+    if (bytes) CB_CUDA(clear_result(out, bytes, stream));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3(threads);

@@ -161,8 +161,8 @@ const_status_t csf_build_noalloc_impl(int order, const int64_t *dims, int64_t nn
 const_status_t run_ttmc3(const const_csf *X, const float *U, const float *V, int R2, int R3, float *Y,
                          int64_t n_rows, int32_t *status, cudaStream_t stream);
 // Whether the leaf-balanced kernels take a chain of these ranks, and the chain itself at any of them, fp32 or fp64
-// (factors in level order; CONST_ERR_UNSUPPORTED when there is no memory for padded factors: nothing but the cleared
-// result has been written then).
+// (factors in level order; CONST_ERR_UNSUPPORTED when padded factors would cost more than the contraction, or there is no
+// memory for them: nothing has been written then).
 bool chain_covers(int order, bool mttkrp, const int *ranks);
 const_status_t run_chain_any(const const_csf *X, bool mttkrp, const void *const *factors, const int *ranks, const_dtype_t dtype,
                              void *out, int64_t out_elems, cudaStream_t stream);

@@ -180,3 +180,18 @@ def test_ttmc3_below_a_million_in_slices_of_several_windows():
         out, _ = run_workload(w)
         S, A = oracle(w)
         assert_close(out, S, A, np.float32)
+
+
+@pytest.mark.parametrize("extent,fused", [(40_000, True), (41_000, False)])
+def test_factors_that_dwarf_the_nonzeros(extent, fused):
+    """Copying a factor whole costs more than a few nonzeros are worth: from 256 padded entries per nonzero on the generic
+    executor, which reads only the rows that occur, does the work."""
+    w = ttmc3_workload((30, extent, extent), 5_001, (10, 12), value="pm1", config_id=33)
+    assert (2 * extent * 16 <= 256 * 5_001) == fused
+    cb.const_profile_enable(True)
+    out, _ = run_workload(w)
+    prof = cb.const_profile_read()
+    cb.const_profile_enable(False)
+    assert ("pad_factors" in prof) == fused and ("tree_kernel" in prof) == (not fused), prof
+    S, A = oracle(w)
+    assert_close(out, S, A, np.float32)
