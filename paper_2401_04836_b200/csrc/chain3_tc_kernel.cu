@@ -298,14 +298,16 @@ const_status_t run_ttmc3_tensor(const const_csf *X, const float *U, const float 
     if (R2 != R || R3 != R) return CONST_ERR_UNSUPPORTED;
     CB_CUDA(cudaMemsetAsync(Y, 0, sizeof(float) * TILE * n_rows, stream));
     if (X->nnz == 0) return CONST_OK;
-    const const_status_t bins = csf_ensure_bins(const_cast<const_csf *>(X), stream);
-    if (bins != CONST_OK) return bins;
+    BinLists bins;
+    const const_status_t rc = csf_bins(const_cast<const_csf *>(X), stream, &bins);
+    if (rc != CONST_OK) return rc;
     Csf3 x{X->crd[0], X->pos[1], X->crd[1], X->pos[2], X->crd[2], static_cast<const float *>(X->vals)};
     constexpr size_t dyn = kWarpBytes * kWarps;
     const DebugKnobs knobs = debug_knobs();
     CB_LAUNCH("chain3_tc_kernel", stream,
-              chain3_tc_kernel<<<(unsigned)X->item_cap, kWarps * 32, dyn, stream>>>(X->items, X->bin_totals, X->light_list, x, U, V, Y, status,
+              chain3_tc_kernel<<<(unsigned)bins.cap, kWarps * 32, dyn, stream>>>(bins.items, bins.totals, bins.light_list, x, U, V, Y, status,
                                                                                  knobs.spin_limit > 0 ? knobs.spin_limit : kMbarPolls, knobs.withhold));
+    if (bins.own) cudaFreeAsync(bins.own, stream);
     CB_CUDA(cudaGetLastError());
     return CONST_OK;
 }

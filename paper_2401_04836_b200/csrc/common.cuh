@@ -53,10 +53,10 @@ struct const_csf {
     void *vals = nullptr;
     unsigned char *arena = nullptr;    // pos, crd and slice_ptr live in this one allocation
     int32_t *slice_ptr = nullptr;      // [n0 + 1] leaf offset of every root-level slice
-    // load balancing: built on first use (csf_ensure_bins)
+    // load balancing: built on first use (csf_bins), in whatever stream that happens; nothing keeps that stream
     std::mutex bins_mu;
     bool bins_valid = false;
-    cudaEvent_t bins_ready = nullptr;  // recorded behind the binning: other streams wait for it
+    cudaEvent_t bins_ready = nullptr;  // recorded behind the binning: every later user waits for it
     int32_t *light_list = nullptr;     // [n0] slice ids handled one per warp (the first n_light entries are used)
     cb::WorkItem *items = nullptr;     // [item_cap] (the first n_items entries are used)
     int32_t *bin_scratch = nullptr;    // [2 * (n0 + 1) + 8 + 64] scan outputs, size-class bases and fill counters
@@ -67,7 +67,6 @@ struct const_csf {
     int64_t n_light = 0, n_heavy = 0, n_giant = 0, n_items = 0;
     int64_t light_max = 0, heavy_max = 0, chunk = 0;
     cudaStream_t stream = nullptr;     // stream of the build: the arrays are freed in its order
-    cudaStream_t bin_stream = nullptr; // stream of the last (re)binning
     int device = 0;
 };
 
@@ -138,6 +137,14 @@ struct DebugKnobs {
 };
 DebugKnobs debug_knobs();
 
+// The work lists as a kernel queued on a stream reads them.
+struct BinLists {
+    const WorkItem *items = nullptr;
+    const int32_t *totals = nullptr, *light_list = nullptr;
+    int64_t cap = 0;                   // upper bound of the number of items
+    void *own = nullptr;               // memory of lists made for this use alone: cudaFreeAsync behind the kernel (may be null)
+};
+
 // chain_kernels.cu: sets `bytes` (a multiple of 4) at the 16-byte aligned `out` to zero and lets the kernel launched next
 // start at once if its launch allows that
 cudaError_t clear_result(void *out, size_t bytes, cudaStream_t stream);
@@ -149,7 +156,7 @@ const_status_t csf_build_impl(int order, const int64_t *dims, int64_t nnz, const
 const_status_t csf_from_dense_impl(int order, const int64_t *dims, const void *dense, const_dtype_t dtype,
                                    const int *mode_order, cudaStream_t stream, const_csf **out);
 const_status_t csf_rebin(const_csf *csf, cudaStream_t stream);
-const_status_t csf_ensure_bins(const_csf *csf, cudaStream_t stream);
+const_status_t csf_bins(const_csf *csf, cudaStream_t stream, BinLists *out);
 const_status_t csf_bin_totals(const_csf *csf);      // fills the host copies n_light .. n_items (waits for the device once)
 void csf_free(const_csf *csf);
 const_status_t csf_build_noalloc_impl(int order, const int64_t *dims, int64_t nnz, const int32_t *const *coords_dev,

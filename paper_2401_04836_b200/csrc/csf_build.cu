@@ -1030,6 +1030,7 @@ void csf_free(const_csf *csf) {
     cudaGetDevice(&prev);
     cudaSetDevice(csf->device);
     auto drop = [&](void *p) { if (p) cudaFreeAsync(p, csf->stream); };
+    if (csf->bins_ready) cudaStreamWaitEvent(csf->stream, csf->bins_ready, 0);            // the lists may be another stream's work
     drop(csf->arena);
     drop(csf->vals);
     drop(csf->light_list);
@@ -1065,43 +1066,44 @@ cudaError_t wait_stream(cudaStream_t stream) {
 
 // Upper bound of the number of work items for the current thresholds: a light or heavy slice gives at most
 // one item, a giant slice of z nonzeros ceil(z / chunk) <= z / chunk + 1.
-static const_status_t csf_rebin_locked(const_csf *csf, cudaStream_t stream);
-
 int64_t item_capacity(const const_csf *csf) {
     return csf->n[0] + csf->nnz / std::max<int64_t>(csf->chunk, 1) + 1;
 }
 
-// The work lists are built when something asks for them (a kernel that works from them, const_csf_work_lists,
-// const_csf_bin_counts); most executes need none.  Safe from several threads; a later user on another stream waits, on
-// the device, for the stream that built them.
-const_status_t csf_ensure_bins(const_csf *csf, cudaStream_t stream) {
-    std::lock_guard<std::mutex> lock(csf->bins_mu);
-    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-    CB_CUDA(cudaStreamIsCapturing(stream, &capture));
-    if (capture != cudaStreamCaptureStatusNone)           // lists that outlive a graph cannot be allocated inside one
-        return csf->bins_valid ? CONST_OK : CONST_ERR_UNSUPPORTED;
-    if (!csf->bins_valid) return csf_rebin_locked(csf, stream);
-    if (csf->bins_ready && stream != csf->bin_stream) CB_CUDA(cudaStreamWaitEvent(stream, csf->bins_ready, 0));
-    return CONST_OK;
+namespace {
+
+size_t bin_scratch_ints(int64_t n0) { return 2 * (size_t)(n0 + 1) + 8 + 2 * kBinClasses; }
+
+// Nothing here waits for the device: the lists are sized by their upper bounds, the fill kernels read the counts the scan
+// left in `totals`, and so do the fused kernels later on.  Returns the totals.
+const int32_t *queue_bins(const const_csf *csf, WorkItem *items, int64_t cap, int32_t *light_list, int32_t *scratch, cudaStream_t stream) {
+    const int64_t n0 = csf->n[0];
+    ChainPtrs c;
+    c.order = csf->order;
+    for (int l = 0; l < kMaxOrder; ++l) c.pos[l] = csf->pos[l];
+    int32_t *item_off = scratch, *light_idx = scratch + (n0 + 1), *totals = scratch + 2 * (n0 + 1);
+    CB_LAUNCH("bin_scan", stream, bin_scan<<<1, 1024, 0, stream>>>(csf->slice_ptr, n0, csf->light_max, csf->heavy_max, csf->chunk, item_off,
+                                     light_idx, totals));
+    CB_LAUNCH("bin_fill", stream, bin_fill<<<(unsigned)((n0 + 255) / 256), 256, 0, stream>>>(c, csf->slice_ptr, n0, csf->light_max, csf->heavy_max,
+                                                              item_off, totals + 8, items, light_list));
+    CB_LAUNCH("bin_fill_chunks", stream, bin_fill_chunks<<<(unsigned)((cap + 127) / 128), 128, 0, stream>>>(
+                  c, csf->slice_ptr, n0, csf->heavy_max, csf->chunk, item_off, totals, items));
+    const int64_t max_groups = (n0 + kWarpsPerBlock - 1) / kWarpsPerBlock;
+    CB_LAUNCH("bin_light_items", stream, bin_light_items<<<(unsigned)((max_groups + 255) / 256), 256, 0, stream>>>(items, totals));
+    return totals;
 }
 
-const_status_t csf_rebin(const_csf *csf, cudaStream_t stream) {
-    std::lock_guard<std::mutex> lock(csf->bins_mu);
-    return csf_rebin_locked(csf, stream);
-}
-
-static const_status_t csf_rebin_locked(const_csf *csf, cudaStream_t stream) {
+// (bins_mu is held)
+const_status_t rebin(const_csf *csf, cudaStream_t stream) {
     const int64_t n0 = csf->n[0];
     csf->n_light = csf->n_heavy = csf->n_giant = csf->n_items = 0;
     csf->totals_on_host = n0 == 0;
-    csf->bin_stream = stream;
     csf->bins_valid = true;
     if (n0 == 0) { csf->item_cap = 0; return CONST_OK; }
     csf->bins_valid = false;                              // until everything below is queued
-    // Nothing below waits for the device: the lists are sized by their upper bounds, the fill kernels read
-    // the counts the scan left in `totals`, and so do the fused kernels later on.
     const int64_t cap = item_capacity(csf);
     if (cap > 0x7fffffffll) return CONST_ERR_UNSUPPORTED;
+    if (csf->bins_ready) CB_CUDA(cudaStreamWaitEvent(stream, csf->bins_ready, 0));        // lists made before, perhaps in another stream
     if (cap > csf->item_cap || !csf->items) {
         if (csf->items) cudaFreeAsync(csf->items, stream);
         csf->items = nullptr;
@@ -1109,37 +1111,58 @@ static const_status_t csf_rebin_locked(const_csf *csf, cudaStream_t stream) {
     }
     csf->item_cap = cap;
     if (!csf->light_list) CB_CUDA(pool_alloc((void **)&csf->light_list, sizeof(int32_t) * n0, stream));
-    if (!csf->bin_scratch) CB_CUDA(pool_alloc((void **)&csf->bin_scratch, sizeof(int32_t) * (2 * (n0 + 1) + 8 + 2 * kBinClasses), stream));
+    if (!csf->bin_scratch) CB_CUDA(pool_alloc((void **)&csf->bin_scratch, sizeof(int32_t) * bin_scratch_ints(n0), stream));
     if (!csf->bins_ready) CB_CUDA(cudaEventCreateWithFlags(&csf->bins_ready, cudaEventDisableTiming));
-    ChainPtrs c;
-    c.order = csf->order;
-    for (int l = 0; l < kMaxOrder; ++l) c.pos[l] = csf->pos[l];
-    int32_t *item_off = csf->bin_scratch, *light_idx = csf->bin_scratch + (n0 + 1), *totals = csf->bin_scratch + 2 * (n0 + 1);
-    csf->bin_totals = totals;
-    CB_LAUNCH("bin_scan", stream, bin_scan<<<1, 1024, 0, stream>>>(csf->slice_ptr, n0, csf->light_max, csf->heavy_max, csf->chunk, item_off,
-                                     light_idx, totals));
-    CB_LAUNCH("bin_fill", stream, bin_fill<<<(unsigned)((n0 + 255) / 256), 256, 0, stream>>>(c, csf->slice_ptr, n0, csf->light_max, csf->heavy_max,
-                                                              item_off, totals + 8, csf->items, csf->light_list));
-    CB_LAUNCH("bin_fill_chunks", stream, bin_fill_chunks<<<(unsigned)((cap + 127) / 128), 128, 0, stream>>>(
-                  c, csf->slice_ptr, n0, csf->heavy_max, csf->chunk, item_off, totals, csf->items));
-    const int64_t max_groups = (n0 + kWarpsPerBlock - 1) / kWarpsPerBlock;
-    CB_LAUNCH("bin_light_items", stream, bin_light_items<<<(unsigned)((max_groups + 255) / 256), 256, 0, stream>>>(csf->items, totals));
+    csf->bin_totals = queue_bins(csf, csf->items, cap, csf->light_list, csf->bin_scratch, stream);
     CB_CUDA(cudaGetLastError());
     CB_CUDA(cudaEventRecord(csf->bins_ready, stream));
     csf->bins_valid = true;
     return CONST_OK;
 }
 
-// Host copies of the bin totals, for callers that ask (const_csf_bin_counts, const_csf_work_lists).
+}  // namespace
+
+const_status_t csf_rebin(const_csf *csf, cudaStream_t stream) {
+    std::lock_guard<std::mutex> lock(csf->bins_mu);
+    return rebin(csf, stream);
+}
+
+// The work lists are built when something asks for them (a kernel that works from them, const_csf_work_lists,
+// const_csf_bin_counts); most executes need none.  Safe from several threads.  A later user waits, on the device, for the
+// event behind them, whichever stream they were built in: that stream may be gone by then, and its number in use again.
+const_status_t csf_bins(const_csf *csf, cudaStream_t stream, BinLists *out) {
+    std::lock_guard<std::mutex> lock(csf->bins_mu);
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    CB_CUDA(cudaStreamIsCapturing(stream, &capture));
+    if (capture != cudaStreamCaptureStatusNone) {         // lists that outlive a graph cannot be allocated inside one
+        if (!csf->bins_valid) return CONST_ERR_UNSUPPORTED;
+        *out = BinLists{csf->items, csf->bin_totals, csf->light_list, csf->item_cap, nullptr};
+        return CONST_OK;
+    }
+    if (!csf->bins_valid) {
+        const const_status_t rc = rebin(csf, stream);
+        if (rc != CONST_OK) return rc;
+    } else if (csf->bins_ready) {
+        CB_CUDA(cudaStreamWaitEvent(stream, csf->bins_ready, 0));
+    }
+    *out = BinLists{csf->items, csf->bin_totals, csf->light_list, csf->item_cap, nullptr};
+    return CONST_OK;
+}
+
+// Host copies of the bin totals, for callers that ask (const_csf_bin_counts, const_csf_work_lists): waits for the stream
+// of the build, behind the lists.
 const_status_t csf_bin_totals(const_csf *csf) {
+    std::lock_guard<std::mutex> lock(csf->bins_mu);
+    if (csf->bins_valid && csf->totals_on_host) return CONST_OK;
     int32_t h[4] = {0, 0, 0, 0};
     int prev = 0;
     CB_CUDA(cudaGetDevice(&prev));
     CB_CUDA(cudaSetDevice(csf->device));
-    const const_status_t rc = csf_ensure_bins(csf, csf->bin_stream);
+    const const_status_t rc = csf->bins_valid ? CONST_OK : rebin(csf, csf->stream);
     if (rc != CONST_OK || csf->totals_on_host) { cudaSetDevice(prev); return rc; }
-    cudaError_t e = cudaMemcpyAsync(h, csf->bin_totals, sizeof(h), cudaMemcpyDeviceToHost, csf->bin_stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(csf->bin_stream);
+    cudaError_t e = cudaStreamWaitEvent(csf->stream, csf->bins_ready, 0);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(h, csf->bin_totals, sizeof(h), cudaMemcpyDeviceToHost, csf->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(csf->stream);
     cudaSetDevice(prev);
     if (e != cudaSuccess) return CONST_ERR_CUDA;
     csf->n_light = h[1];
@@ -1248,7 +1271,6 @@ const_status_t csf_build_impl(int order, const int64_t *dims, int64_t nnz, const
                 CB_CUDA(cudaMemsetAsync(csf->slice_ptr, 0, sizeof(int32_t), stream));
             }
             CB_CUDA(cudaGetLastError());
-            csf->bin_stream = stream;
             return CONST_OK;
         };
         rc = body();

@@ -391,18 +391,20 @@ const_status_t run_ttmc4_tensor(const const_csf *X, const float *U, const float 
     if (rank != R) return CONST_ERR_UNSUPPORTED;
     CB_CUDA(cudaMemsetAsync(Y, 0, sizeof(float) * TILE * n_rows, stream));
     if (X->nnz == 0) return CONST_OK;
-    const const_status_t bins = csf_ensure_bins(const_cast<const_csf *>(X), stream);
-    if (bins != CONST_OK) return bins;
+    BinLists bins;
+    const const_status_t rc = csf_bins(const_cast<const_csf *>(X), stream, &bins);
+    if (rc != CONST_OK) return rc;
     Csf4 x{X->crd[0], X->pos[1], X->crd[1], X->pos[2], X->crd[2], X->pos[3], X->crd[3],
            static_cast<const float *>(X->vals)};
     constexpr size_t dyn = kWarpBytes * kWarps;
     static PerDeviceOnce attr_once;                     // per template instance
     CB_CUDA(once_per_device(attr_once, [&] { return cudaFuncSetAttribute(ttmc4_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn); }));
-    const unsigned grid = (unsigned)X->item_cap;
+    const unsigned grid = (unsigned)bins.cap;
     const DebugKnobs knobs = debug_knobs();
     CB_LAUNCH("ttmc4_tc_kernel", stream,
-              ttmc4_tc_kernel<<<grid, kWarps * 32, dyn, stream>>>(X->items, X->bin_totals, X->light_list, x, U, V, W, Y, status,
+              ttmc4_tc_kernel<<<grid, kWarps * 32, dyn, stream>>>(bins.items, bins.totals, bins.light_list, x, U, V, W, Y, status,
                                                                knobs.spin_limit > 0 ? knobs.spin_limit : kMbarPolls, knobs.withhold));
+    if (bins.own) cudaFreeAsync(bins.own, stream);
     CB_CUDA(cudaGetLastError());
     return CONST_OK;
 }
