@@ -277,8 +277,9 @@ const_status_t const_schedule_cin(const char *expression, const char *const *tre
  * per-term relative error below 2^-19, so the fp32 tolerance holds); enable == 0: on the fp32 FMA pipes.
  * Plans that have the stage: order-4 TTMc at rank 8 and order-3 TTMc at rank 16 x 16.  Off unless asked for: the
  * fp32 path is the faster one on both (order 4, 50 M nonzeros: 2.3 against 3.1 ms) and the more accurate one.
- * The stage works from the tensor's work lists, which are built at its first use: inside a stream capture that first use
- * returns CONST_ERR_UNSUPPORTED (execute once, or call const_csf_bin_counts, before capturing).
+ * The stage works from the tensor's work lists, which are built at its first use.  A stream capture that is the first use
+ * builds lists of its own inside the graph, at every replay; execute once, or call const_csf_bin_counts, before capturing
+ * to have them built once.  A graph keeps reading the lists it was captured with: const_csf_set_bins ends its use.
  * CONST_ERR_UNSUPPORTED for enable != 0 on any other plan.  Host-only call; takes effect at the next
  * const_execute.  A device-side wait that runs out is reported through const_last_device_status.
  */

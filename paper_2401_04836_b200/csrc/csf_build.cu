@@ -1130,20 +1130,33 @@ const_status_t csf_rebin(const_csf *csf, cudaStream_t stream) {
 // The work lists are built when something asks for them (a kernel that works from them, const_csf_work_lists,
 // const_csf_bin_counts); most executes need none.  Safe from several threads.  A later user waits, on the device, for the
 // event behind them, whichever stream they were built in: that stream may be gone by then, and its number in use again.
+// Under stream capture the wait becomes a node of the graph; lists that do not exist yet are built inside the graph, in
+// memory of its own, at every replay (lists that outlive the graph cannot be allocated in it).
 const_status_t csf_bins(const_csf *csf, cudaStream_t stream, BinLists *out) {
     std::lock_guard<std::mutex> lock(csf->bins_mu);
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     CB_CUDA(cudaStreamIsCapturing(stream, &capture));
-    if (capture != cudaStreamCaptureStatusNone) {         // lists that outlive a graph cannot be allocated inside one
-        if (!csf->bins_valid) return CONST_ERR_UNSUPPORTED;
-        *out = BinLists{csf->items, csf->bin_totals, csf->light_list, csf->item_cap, nullptr};
+    const bool capturing = capture != cudaStreamCaptureStatusNone;
+    if (capturing && !csf->bins_valid && csf->n[0] > 0) {
+        const int64_t n0 = csf->n[0];
+        out->cap = item_capacity(csf);
+        const size_t items_bytes = sizeof(WorkItem) * (size_t)out->cap;
+        unsigned char *own = nullptr;
+        CB_CUDA(scratch_alloc((void **)&own, items_bytes + sizeof(int32_t) * ((size_t)n0 + bin_scratch_ints(n0)), stream));
+        WorkItem *items = reinterpret_cast<WorkItem *>(own);
+        int32_t *light = reinterpret_cast<int32_t *>(own + items_bytes);
+        out->totals = queue_bins(csf, items, out->cap, light, light + n0, stream);
+        out->items = items;
+        out->light_list = light;
+        out->own = own;
+        CB_CUDA(cudaGetLastError());
         return CONST_OK;
     }
     if (!csf->bins_valid) {
         const const_status_t rc = rebin(csf, stream);
         if (rc != CONST_OK) return rc;
     } else if (csf->bins_ready) {
-        CB_CUDA(cudaStreamWaitEvent(stream, csf->bins_ready, 0));
+        CB_CUDA(cudaStreamWaitEvent(stream, csf->bins_ready, capturing ? cudaEventWaitExternal : cudaEventWaitDefault));
     }
     *out = BinLists{csf->items, csf->bin_totals, csf->light_list, csf->item_cap, nullptr};
     return CONST_OK;

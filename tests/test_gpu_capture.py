@@ -81,6 +81,44 @@ def tensor_workload(order):
     return ttmc3_workload((500, 300, 700), 120_000, 16, slice_s=1.1, inner_s=0.9, value="unit", config_id=2)
 
 
+@pytest.mark.parametrize("order", [3, 4])
+def test_first_use_of_the_tensor_stage_inside_a_capture(order):
+    s = Setup(tensor_workload(order), tensor_stage=True)
+    other = Setup(tensor_workload(order), tensor_stage=True)
+    other.plan = s.plan                                          # the plan has been used, the tensor has not
+    stream = torch.cuda.Stream()
+    first_execute(other, stream)
+    graph = capture(s, stream)
+    replay_twice(s, graph)
+    assert cb.const_csf_bin_counts(s.handles["X"]) == cb.const_csf_bin_counts(other.handles["X"])
+    s.execute()                                                  # and with lists of the handle's own now
+    torch.cuda.synchronize()
+    s.check()
+
+
+def test_capture_behind_lists_that_another_stream_is_still_building():
+    """The first use on one stream is not waited for: the graph has to."""
+    s = Setup(tensor_workload(4), tensor_stage=True)
+    warm = Setup(tensor_workload(4), tensor_stage=True)
+    warm.plan = s.plan
+    stream = torch.cuda.Stream()
+    first_execute(warm, stream)
+    side, scrap, graph = torch.cuda.Stream(), torch.empty_like(s.out), torch.cuda.CUDAGraph()
+    s.out.fill_(float("nan"))
+    torch.cuda.synchronize()
+    with torch.cuda.stream(side):
+        torch.cuda._sleep(400_000_000)                           # about 0.2 s in front of the lists
+        s.execute(out=scrap)
+    with torch.cuda.stream(stream):                              # (torch.cuda.graph would wait for the device first)
+        graph.capture_begin()
+        s.execute()
+        graph.capture_end()
+        graph.replay()
+    assert not side.query()                                      # the lists are still to come
+    torch.cuda.synchronize()
+    s.check()
+
+
 def test_lists_outlive_the_stream_they_were_built_in():
     """A stream of the caller's own is where the lists are first needed; it is gone when they are asked for, used on another
     stream, and released."""
