@@ -414,12 +414,13 @@ __global__ void __launch_bounds__(kWarps * 32, Ttmc4Shape<T>::BLOCKS) ttmc4_kern
                     }
 #pragma unroll
                     for (int z = 0; z < kUnroll; ++z) {
-                        if constexpr (FLAT) {         // Q[b, :] += (V[k, b] X) W[l, :]
-                            const T s0 = v0[z] * r[z].val, s1 = v1[z] * r[z].val;
+                        if constexpr (FLAT) {         // Q[b, :] += V[k, b] (X W[l, :]), multiplied in the schedule's order
 #pragma unroll
                             for (int c = 0; c < NV; ++c) {
-                                axpy(q0[c], make_pair(s0, s0), w[z][c]);
-                                axpy(q1[c], make_pair(s1, s1), w[z][c]);
+                                Vec<T> x = zero_vec<T>();
+                                axpy(x, make_pair(r[z].val, r[z].val), w[z][c]);
+                                axpy(q0[c], make_pair(v0[z], v0[z]), x);
+                                axpy(q1[c], make_pair(v1[z], v1[z]), x);
                             }
                         } else {                      // P[:] += X W[l, :];  Q[b, :] += V[k, b] P[:]
 #pragma unroll

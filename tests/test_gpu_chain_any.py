@@ -195,3 +195,22 @@ def test_factors_that_dwarf_the_nonzeros(extent, fused):
     assert ("pad_factors" in prof) == fused and ("tree_kernel" in prof) == (not fused), prof
     S, A = oracle(w)
     assert_close(out, S, A, np.float32)
+
+
+@pytest.mark.parametrize("family,ranks", [("ttmc", (8, 8)), ("ttmc", (7, 9)), ("mttkrp", (16, 16)), ("ttmc", (8, 8, 8)), ("ttmc", (5, 6, 7)), ("mttkrp", (8, 8, 8))])
+@pytest.mark.parametrize("long_fibres", [False, True])
+def test_products_are_formed_in_the_order_of_the_schedule(family, ranks, long_fibres):
+    """Leaf value times leaf factor first, then level by level upwards: large values and leaf factors small enough to bring
+    them back leave no intermediate beyond fp32, though the value times any other factor would be."""
+    dims = (12, 10, 9, 11)[: len(ranks) + 1]
+    X, fac = inputs(family, dims, ranks, 900, cb.F32, 51)
+    if not long_fibres:                                        # one leaf to a node: the leaf coordinate from the others
+        at = np.unique(np.ravel_multi_index([c.astype(np.int64) for c in X.coords[:-1]], dims[:-1]), return_index=True)[1]
+        X = gen.SparseOperand([np.ascontiguousarray(c[at]) for c in X.coords], np.ascontiguousarray(X.vals[at]), X.dims)
+    X = gen.SparseOperand(X.coords, X.vals * np.float32(2.0 ** 90), X.dims)
+    names = NAMES[family][: len(ranks)]
+    for n in names[:-1]:
+        fac[n] = fac[n] * np.float32(2.0 ** 45)
+    fac[names[-1]] = fac[names[-1]] * np.float32(2.0 ** -100)
+    out, S, A = run_chain(family, dims, ranks, X, fac, cb.F32)
+    assert_close(out, S, A, np.float32)
