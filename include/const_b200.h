@@ -321,7 +321,8 @@ const char *const_status_string(const_status_t status);
  * counts, the tensor-core stage issues and commits nothing -- so that every such wait runs out, the
  * kernel records CONST_ERR_TIMEOUT, skips its stores and returns normally;
  * what = 2: which of the tile shapes a launcher keeps for measurement is launched (0: the default; the
- * two-contraction network has variants 1..5, every one of them computes the same result);
+ * two-contraction network has variants 1..5, every one of them computes the same result, and 6, its matrix form alone: the
+ * result stays zero where that form hands the work on);
  * what = 3: value != 0 makes every request of const_execute for optional scratch (padded factors, the intermediate of the
  * two-contraction network's matrix form) fail for want of memory, so that the path that needs none runs.  Process-wide; not
  * for production use.  CONST_ERR_INVALID_ARG for an unknown `what` or a value outside [0, 2^31).

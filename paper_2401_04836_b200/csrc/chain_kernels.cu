@@ -566,11 +566,8 @@ struct Clear {
     }
 };
 
-// Lets the kernel launched next start at once, up to its own wait for this one (after_clear).
-__device__ __forceinline__ void start_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
 __global__ void __launch_bounds__(256) clear_kernel(const __grid_constant__ Clear c) {
-    start_next();
+    start_next_kernel();
     c.run();
 }
 
@@ -586,7 +583,7 @@ struct PadArgs {
 
 template <typename T>
 __global__ void __launch_bounds__(256) pad_factors(const __grid_constant__ PadArgs<T> a, const __grid_constant__ Clear result) {
-    start_next();
+    start_next_kernel();
     result.run();
     for (int64_t e = (int64_t)blockIdx.x * 256 + threadIdx.x; e < a.first[3]; e += (int64_t)gridDim.x * 256) {
 #pragma unroll

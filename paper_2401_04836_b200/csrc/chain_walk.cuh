@@ -335,9 +335,6 @@ __device__ __forceinline__ int stage_window(const Ahead<T, ORDER, W> &a, Place<O
     return pieces;
 }
 
-// Waits until the kernel launched before this one (clear_result) has finished and its stores are visible.
-__device__ __forceinline__ void after_clear() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
 // The leaves of one warp, and the end of those of its block.
 struct Share {
     int32_t e0, e1, block_end;
@@ -369,7 +366,7 @@ __device__ __forceinline__ int32_t walk_chunk(const Chain<T, ORDER> &x, const Sh
         from_start = __ldg(x.slice_ptr + place.node[0]) == e;
         end = __ldg(x.slice_ptr + place.node[0] + 1);
     }
-    after_clear();                                       // everything up to here only read
+    after_last_kernel();                                 // the result is cleared; everything up to here only read the tensor
     if (threadIdx.x == 0) first_slice = place.node[0];   // (the first warp of a block always has leaves)
     const bool joint = __syncthreads_or(threadIdx.x < 32 && end >= own.block_end) != 0;
     while (e < own.e1) {
@@ -421,25 +418,15 @@ inline int32_t chunk_leaves(int64_t nnz, int64_t slices, int resident, int64_t m
 }
 
 // Clears `out` ("R[*] = 0" precedes the nest; bytes = 0: the launch before has done that) and launches the kernel so that it starts while the clearing still runs: it
-// looks its place in the tensor up meanwhile and waits (after_clear) before it writes.  Clearing by a kernel of the
+// looks its place in the tensor up meanwhile and waits (after_last_kernel) before it writes.  Clearing by a kernel of the
 // library instead of a memset is what allows that (20 000 nonzeros at rank 8, device time bound by the two launches:
 // 14.2 -> 13.9 us a call).
 template <class Args>
 inline const_status_t launch_on_cleared(const char *name, void (*kernel)(Args), const Args &args, dim3 grid, int threads, size_t smem,
                                         void *out, size_t bytes, cudaStream_t stream) {
     if (bytes) CB_CUDA(clear_result(out, bytes, stream));
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = stream;
-    cudaLaunchAttribute early;
-    early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    early.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &early;
-    cfg.numAttrs = 1;
     cudaError_t e = cudaSuccess;
-    CB_LAUNCH(name, stream, e = cudaLaunchKernelEx(&cfg, kernel, args));
+    CB_LAUNCH(name, stream, e = launch_early(kernel, grid, threads, smem, stream, args));
     return e == cudaSuccess ? CONST_OK : CONST_ERR_CUDA;
 }
 

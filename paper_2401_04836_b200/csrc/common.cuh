@@ -127,6 +127,28 @@ private:
         __VA_ARGS__;                             \
     } while (0)
 
+// Launches a kernel so that it may start before the kernel launched last has finished: every thread of it has to wait
+// (after_last_kernel) before it touches what that kernel, or one before it, writes or reads.
+template <class... Params, class... Args>
+inline cudaError_t launch_early(void (*kernel)(Params...), dim3 grid, int threads, size_t smem, cudaStream_t stream, const Args &...args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute early;
+    early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    early.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &early;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+#ifdef __CUDACC__
+__device__ __forceinline__ void after_last_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// lets a kernel launched that way start once every block of this one has come here
+__device__ __forceinline__ void start_next_kernel() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+#endif
+
 // Test hooks (const_debug_set): limits of the bounded device-side waits and a switch that withholds the
 // signal those waits are waiting for, so that a test can see a wait run out.  0 = library defaults.
 struct DebugKnobs {

@@ -21,9 +21,13 @@
 // the gather kernel, launched last, then clears Z and does the work.
 //
 // Measured, 1024 x 1024 x 128, band 32, a quarter full: 4771 us in the gather form; here t_kernel 660 us (dense work at the
-// fp64 peak of 37 TFLOP/s: 480) and z_kernel 890 us (540), 1573 us together with the shape kernels.  z_kernel is held by
+// fp64 peak of 37 TFLOP/s: 480) and z_kernel 890 us (540), 1552 us together with clearing and shape.  z_kernel is held by
 // writing its slices out between the products: walking the fibres for it 1196 us, from places computed once 979, with the
-// next slice's entries on their way meanwhile 889.  331 x 331 x 61, band 17: 165 -> 136 us; 700, 100, band 21: 1198 -> 568.
+// next slice's entries on their way meanwhile 889.  331 x 331 x 61, band 17: 164 -> 115 us; 700, 100, band 21: 1187 -> 542.
+//
+// The launches are short ones at the small end, so they are few and start early (launch_early): clearing Z and the mode word,
+// ranges and places in one kernel, t and z once per chunk, the gather kernel.  Ranges and places in two kernels, the mode word
+// cleared apart and ordinary launches: 128 us at 331, 1566 at 1024; and 25 us instead of 8 for operands that do not qualify.
 #include <algorithm>
 
 #include "common.cuh"
@@ -38,6 +42,7 @@ constexpr int kTileK = 128;           // k per tile
 constexpr int kNodes = 4;             // slices of W per z_kernel block
 constexpr int kRows = 8 * kWarps;     // slices of U per z_kernel block
 constexpr int kMaxDilution = 8;       // dense multiply-adds per sparse one up to which the dense form is taken
+constexpr int kModeWords = 16;        // words of Net::mode
 
 struct Csf3d {
     const int32_t *crd0, *pos1, *crd1, *pos2, *crd2;
@@ -52,7 +57,7 @@ struct Net {
     int32_t *mode;                    // [0] nonzero: the gather kernel does the work (2: from the start, 1: T was not finite); [2..3] dense multiply-adds (64 bits); [4] blocks done
     int32_t *jmin, *jlen;             // per slice of U: first j, length of the range of j
     int32_t *mmin, *mlen;             // per group of slices of W: the same of m
-    uint32_t *u_place, *w_place;      // per entry (place_kernel)
+    uint32_t *u_place, *w_place;      // per entry (shape_kernel)
     int32_t n_k, n_l, n_j, n_m, tk;   // tk: n_k rounded up to 8
     int32_t s0, s1;                   // chunk of slices of U
 };
@@ -63,75 +68,79 @@ __device__ __forceinline__ void mma884(double &c0, double &c1, double a, double 
 
 __device__ __forceinline__ int round_up(int x, int to) { return (x + to - 1) / to * to; }
 
-// One warp per slice of U and per group of slices of W: the ranges, the dense work, and whether they fit.
-__global__ void __launch_bounds__(kThreads) shape_kernel(const __grid_constant__ Net a, unsigned long long sparse) {
-    const int lane = threadIdx.x & 31;
-    const int unit = blockIdx.x * kWarps + (threadIdx.x >> 5), groups = (a.w.n0 + kNodes - 1) / kNodes;
-    __shared__ unsigned long long sum;
-    if (threadIdx.x == 0) sum = 0;
-    __syncthreads();
-    int lo = 0x7fffffff, hi = -1;
-    const bool have = unit < a.u.n0 + groups;
-    if (have && unit < a.u.n0) {
-        const int f1 = __ldg(a.u.pos1 + unit + 1);
-        for (int f = __ldg(a.u.pos1 + unit) + lane; f < f1; f += 32) {
-            lo = min(lo, __ldg(a.u.crd2 + __ldg(a.u.pos2 + f)));
-            hi = max(hi, __ldg(a.u.crd2 + __ldg(a.u.pos2 + f + 1) - 1));
+// Z, and the words that steer the kernels behind, set to zero
+__global__ void __launch_bounds__(256) clear_kernel(const __grid_constant__ Net a, int64_t n) {
+    start_next_kernel();
+    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) a.Z[i] = 0.0;
+    if (blockIdx.x == 0 && threadIdx.x < kModeWords) a.mode[threadIdx.x] = 0;
+}
+
+// A block goes through slices of U and groups of slices of W: their ranges, the dense work, whether they fit, and where every
+// entry goes when its slice is written out: (place in the range) << 12 | k.  The kernels below write a slice out many times
+// (once per share of l, once per 64 slices of U); with the place beside the value they do it from two coalesced streams,
+// without walking the fibres.  The first range that does not fit ends the block's work.
+__global__ void __launch_bounds__(kThreads) shape_kernel(const __grid_constant__ Net a, int32_t units, unsigned long long sparse) {
+    __shared__ int lows[2][kWarps], highs[2][kWarps];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    unsigned long long work = 0;
+    for (int32_t at = blockIdx.x, turn = 0; at < units; at += gridDim.x, turn ^= 1) {
+        const bool of_u = at < a.u.n0;
+        const int unit = of_u ? at : at - a.u.n0;
+        const Csf3d &x = of_u ? a.u : a.w;
+        const int node0 = of_u ? unit : unit * kNodes, node1 = of_u ? unit + 1 : min(node0 + kNodes, x.n0);
+        const int32_t f0 = __ldg(x.pos1 + node0), f1 = __ldg(x.pos1 + node1);
+        int lo = 0x7fffffff, hi = -1;
+        for (int32_t f = f0 + threadIdx.x; f < f1; f += kThreads) {
+            if (of_u) {
+                lo = min(lo, __ldg(x.crd2 + __ldg(x.pos2 + f)));
+                hi = max(hi, __ldg(x.crd2 + __ldg(x.pos2 + f + 1) - 1));
+            } else {
+                const int m = __ldg(x.crd1 + f);
+                lo = min(lo, m);
+                hi = max(hi, m);
+            }
         }
-    } else if (have) {
-        const int node = (unit - a.u.n0) * kNodes + lane;
-        if (lane < kNodes && node < a.w.n0) {
-            lo = __ldg(a.w.crd1 + __ldg(a.w.pos1 + node));
-            hi = __ldg(a.w.crd1 + __ldg(a.w.pos1 + node + 1) - 1);
+        lo = __reduce_min_sync(0xffffffffu, lo);
+        hi = __reduce_max_sync(0xffffffffu, hi);
+        if (lane == 0) {
+            lows[turn][warp] = lo;
+            highs[turn][warp] = hi;
+        }
+        __syncthreads();
+        if (at == (int32_t)blockIdx.x) after_last_kernel();               // nothing has been written so far
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) {
+            lo = min(lo, lows[turn][w]);
+            hi = max(hi, highs[turn][w]);
+        }
+        const int len = hi - lo + 1;
+        if (len > (of_u ? kRangeJ : kRangeM)) {
+            if (threadIdx.x == 0) a.mode[0] = 2;
+            break;
+        }
+        if (threadIdx.x == 0) {
+            (of_u ? a.jmin : a.mmin)[unit] = lo;
+            (of_u ? a.jlen : a.mlen)[unit] = len;
+        }
+        work += of_u ? (unsigned long long)round_up(len, 4) * a.tk * a.n_l : (unsigned long long)round_up(len, 8) * a.tk * kNodes * a.u.n0;
+        uint32_t *to = of_u ? a.u_place : a.w_place;
+        const int h = threadIdx.x & 7;                                    // eight lanes per fibre
+        for (int32_t f = f0 + (threadIdx.x >> 3); f < f1; f += kThreads / 8) {
+            const uint32_t y = __ldg(x.crd1 + f);                         // k of a U fibre, m of a W fibre
+            const int32_t p1 = __ldg(x.pos2 + f + 1);
+            for (int32_t p = __ldg(x.pos2 + f) + h; p < p1; p += 8) {
+                const uint32_t z = __ldg(x.crd2 + p);
+                to[p] = of_u ? (z - lo) << 12 | y : (y - lo) << 12 | z;
+            }
         }
     }
-    lo = __reduce_min_sync(0xffffffffu, lo);
-    hi = __reduce_max_sync(0xffffffffu, hi);
-    const int len = hi - lo + 1;
-    if (lane == 0 && have) {
-        unsigned long long work;
-        if (unit < a.u.n0) {
-            a.jmin[unit] = lo;
-            a.jlen[unit] = len;
-            work = (unsigned long long)round_up(len, 4) * a.tk * a.n_l;
-        } else {
-            a.mmin[unit - a.u.n0] = lo;
-            a.mlen[unit - a.u.n0] = len;
-            work = (unsigned long long)round_up(len, 8) * a.tk * kNodes * a.u.n0;
-        }
-        if (len > (unit < a.u.n0 ? kRangeJ : kRangeM)) a.mode[0] = 2;
-        atomicAdd(&sum, work);
-    }
-    // the last block to finish compares the dense work with that of the gather form: it has to be worth it
-    __syncthreads();
+    // the last block compares the dense work with that of the gather form: it has to be worth it
     if (threadIdx.x != 0) return;
     unsigned long long *total = reinterpret_cast<unsigned long long *>(a.mode + 2);
-    atomicAdd(total, sum);
+    atomicAdd(total, work);
     __threadfence();
     const bool last = atomicAdd(a.mode + 4, 1) == (int)gridDim.x - 1;
     if (last && atomicAdd(total, 0ull) > kMaxDilution * sparse) a.mode[0] = 2;
-}
-
-// Where every entry goes when its slice is written out: (place in the range) << 12 | k.  One block per slice, eight lanes per
-// fibre.  The kernels below write a slice out many times (once per share of l, once per 64 slices of U); with the place
-// beside the value they do it from two coalesced streams, without walking the fibres.
-__global__ void __launch_bounds__(kThreads) place_kernel(const __grid_constant__ Net a) {
-    if (*a.mode) return;
-    const bool of_u = (int)blockIdx.x < a.u.n0;
-    const int node = of_u ? blockIdx.x : blockIdx.x - a.u.n0;
-    const Csf3d &x = of_u ? a.u : a.w;
-    const int32_t f1 = __ldg(x.pos1 + node + 1);
-    const int first = of_u ? a.jmin[node] : a.mmin[node / kNodes];
-    uint32_t *to = of_u ? a.u_place : a.w_place;
-    const int h = threadIdx.x & 7;
-    for (int32_t f = __ldg(x.pos1 + node) + (threadIdx.x >> 3); f < f1; f += kThreads / 8) {
-        const uint32_t y = __ldg(x.crd1 + f);                             // k of a U fibre, m of a W fibre
-        const int32_t p1 = __ldg(x.pos2 + f + 1);
-        for (int32_t p = __ldg(x.pos2 + f) + h; p < p1; p += 8) {
-            const uint32_t z = __ldg(x.crd2 + p);
-            to[p] = of_u ? (z - first) << 12 | y : (y - first) << 12 | z;
-        }
-    }
 }
 
 constexpr int kAhead = 8;             // entries per thread requested ahead of their use
@@ -171,6 +180,7 @@ __device__ __forceinline__ void clear_shared(double *d, int n) {         // n ev
 __global__ void __launch_bounds__(kThreads, 2) t_kernel(const __grid_constant__ Net a, int l_tiles_per_block) {
     extern __shared__ __align__(16) double u_dense[];                     // [range of j][tile of k + 4]
     __shared__ int skip;                                                  // one reading for the block: others may set it meanwhile
+    after_last_kernel();
     if (threadIdx.x == 0) skip = *a.mode;
     __syncthreads();
     if (skip) return;
@@ -259,6 +269,7 @@ __global__ void __launch_bounds__(kThreads, 2) z_kernel(const __grid_constant__ 
     Staged &staged = *reinterpret_cast<Staged *>(z_smem);
     double *w_dense = z_smem + sizeof(Staged) / sizeof(double);           // [tile of k][range of m + 4]
     __shared__ int skip;
+    after_last_kernel();
     if (threadIdx.x == 0) skip = *a.mode;
     __syncthreads();
     if (skip) return;
@@ -321,6 +332,7 @@ __global__ void __launch_bounds__(kThreads, 2) z_kernel(const __grid_constant__ 
 
 // Z back to zero where the gather kernel takes over after products have been added to it
 __global__ void __launch_bounds__(256) reclear_kernel(const int32_t *mode, double *Z, int64_t n) {
+    after_last_kernel();
     if (*mode != 1) return;
     for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) Z[i] = 0.0;
 }
@@ -329,8 +341,9 @@ constexpr int64_t kScratchBytes = 256ll << 20;       // T of one chunk
 
 }  // namespace
 
-// Z is cleared.  On CONST_OK with *mode_out set, the work is queued and *mode_out (device) says, once the stream gets there,
-// whether the gather kernel still has to do it; *mode_out null: nothing was queued.  release(*scratch_out) afterwards.
+// On CONST_OK with *mode_out set, the work is queued, behind the clearing of Z, and *mode_out (device) says, once the stream
+// gets there, whether the gather kernel still has to do it; *mode_out null: nothing was queued.  cudaFreeAsync(*scratch_out)
+// afterwards.
 const_status_t run_network_dense(const const_csf *U, const double *V, const const_csf *W, double *Z, int64_t n_i, int64_t n_j,
                                  int64_t n_k, int64_t n_l, int64_t n_m, int32_t **mode_out, void **scratch_out, cudaStream_t stream) {
     *mode_out = nullptr;
@@ -340,8 +353,8 @@ const_status_t run_network_dense(const const_csf *U, const double *V, const cons
     const int64_t row_bytes = n_l * tk * 8;
     const int64_t n0 = U->n[0], groups = (W->n[0] + kNodes - 1) / kNodes;
     // Small networks stay with the gather kernel; so does one whose T would leave fewer than 64 slices to a chunk.  Where the
-    // line lies (multiply-adds of the gather form): at 1.1e8 the band at 331 takes 165 us in the gather form and 133 here,
-    // below 6e7 the six extra launches (about 25 us, also paid by operands that then do not qualify) eat the gain.
+    // line lies (multiply-adds of the gather form): at 1.1e8 the band at 331 takes 164 us in the gather form and 115 here,
+    // operands that then do not qualify pay about 8 us: 3 % of a call at 1.2e8, 4 % at 7e7.
     if (sparse < 6e7 || n_k > 4096 || kScratchBytes / row_bytes < std::min<int64_t>(n0, 64)) return CONST_OK;
     if (n_l > (1 << 24) || n_m > (1 << 24) || groups > 65535 * 8ll || n0 + W->n[0] > 0x7fffffffll) return CONST_OK;
     int64_t chunk = std::min<int64_t>({n0, kScratchBytes / row_bytes, 65535ll * kRows});       // what T may take, and the rows of a grid
@@ -349,7 +362,7 @@ const_status_t run_network_dense(const const_csf *U, const double *V, const cons
     chunk = ((n0 + chunks - 1) / chunks + kRows - 1) / kRows * kRows;     // even chunks of whole blocks, never more than fit
     if (chunk * row_bytes > kScratchBytes) chunk = kScratchBytes / row_bytes;
     chunk = std::min<int64_t>(chunk, n0);
-    const size_t small = 64 + sizeof(int32_t) * (2 * (size_t)(n0 + groups) + (size_t)(U->nnz + W->nnz));
+    const size_t small = kModeWords * sizeof(int32_t) + sizeof(int32_t) * (2 * (size_t)(n0 + groups) + (size_t)(U->nnz + W->nnz));
     const size_t small_pad = (small + 255) / 256 * 256;
     unsigned char *scratch = nullptr;
     if (scratch_alloc((void **)&scratch, small_pad + (size_t)(chunk * row_bytes), stream) != cudaSuccess) {
@@ -357,7 +370,6 @@ const_status_t run_network_dense(const const_csf *U, const double *V, const cons
         return CONST_OK;
     }
     auto queue = [&]() -> const_status_t {
-        CB_CUDA(cudaMemsetAsync(scratch, 0, 64, stream));
         Net a;
         auto csf = [](const const_csf *c) {
             return Csf3d{c->crd[0], c->pos[1], c->crd[1], c->pos[2], c->crd[2], static_cast<const double *>(c->vals), (int32_t)c->n[0], (int32_t)c->n[1]};
@@ -367,7 +379,7 @@ const_status_t run_network_dense(const const_csf *U, const double *V, const cons
         a.V = V;
         a.Z = Z;
         a.mode = reinterpret_cast<int32_t *>(scratch);
-        a.jmin = reinterpret_cast<int32_t *>(scratch + 64);
+        a.jmin = a.mode + kModeWords;
         a.jlen = a.jmin + n0;
         a.mmin = a.jlen + n0;
         a.mlen = a.mmin + groups;
@@ -380,9 +392,9 @@ const_status_t run_network_dense(const const_csf *U, const double *V, const cons
         a.n_m = (int32_t)n_m;
         a.tk = (int32_t)tk;
         a.s0 = a.s1 = 0;
-        const int64_t units = n0 + groups;
-        CB_LAUNCH("network_shape", stream, shape_kernel<<<(unsigned)((units + kWarps - 1) / kWarps), kThreads, 0, stream>>>(a, (unsigned long long)sparse));
-        CB_LAUNCH("network_shape", stream, place_kernel<<<(unsigned)(n0 + W->n[0]), kThreads, 0, stream>>>(a));
+        const int clear_blocks = (int)std::max<int64_t>(1, std::min<int64_t>((n_i * n_m + 1023) / 1024, 148 * 8));
+        CB_LAUNCH("clear_result", stream, clear_kernel<<<clear_blocks, 256, 0, stream>>>(a, n_i * n_m));
+        CB_LAUNCH("network_shape", stream, CB_CUDA(launch_early(shape_kernel, dim3((unsigned)std::min<int64_t>(n0 + groups, 148 * 4)), kThreads, 0, stream, a, (int32_t)(n0 + groups), (unsigned long long)sparse)));
         const int kt = (int)std::min<int64_t>(kTileK, tk);
         const size_t t_smem = sizeof(double) * kRangeJ * (kt + 4), z_smem = sizeof(Staged) + sizeof(double) * kt * (kRangeM + 4);
         static PerDeviceOnce once;
@@ -400,11 +412,12 @@ const_status_t run_network_dense(const const_csf *U, const double *V, const cons
             const int want = std::max(1, (148 * 7 + rows * k_tiles - 1) / (rows * k_tiles));
             const int per = std::max(kWarps, ((l_tiles + want - 1) / want + kWarps - 1) / kWarps * kWarps);
             const dim3 tg((unsigned)rows, (unsigned)k_tiles, (unsigned)((l_tiles + per - 1) / per));
-            CB_LAUNCH("network_t", stream, t_kernel<<<tg, kThreads, t_smem, stream>>>(a, per));
+            CB_LAUNCH("network_t", stream, CB_CUDA(launch_early(t_kernel, tg, kThreads, t_smem, stream, a, per)));
             const dim3 zg((unsigned)groups, (unsigned)((rows + kRows - 1) / kRows));
-            CB_LAUNCH("network_z", stream, z_kernel<<<zg, kThreads, z_smem, stream>>>(a));
+            CB_LAUNCH("network_z", stream, CB_CUDA(launch_early(z_kernel, zg, kThreads, z_smem, stream, a)));
         }
-        CB_LAUNCH("network_shape", stream, reclear_kernel<<<148, 256, 0, stream>>>(a.mode, Z, n_i * n_m));
+        if (chunks > 1)          // (with one chunk every T has been looked at before the first product is added)
+            CB_LAUNCH("network_shape", stream, CB_CUDA(launch_early(reclear_kernel, dim3(148), 256, 0, stream, a.mode, Z, n_i * n_m)));
         CB_CUDA(cudaGetLastError());
         return CONST_OK;
     };

@@ -244,17 +244,21 @@ __device__ __forceinline__ void network_tile(const Csf3d &u, const double *__res
     }
 }
 
-// One tile per block; SHORT: a short grid goes through them (their numbers may need 64 bits), unless *mode, where there is
-// one, says that network_dense.cu has done the work.
-template <int IS, int LT, int GL, bool SHORT>
+// One tile per block; LOOP: a short grid goes through them (their numbers may need 64 bits).  Nothing where *mode, if there
+// is one, says that network_dense.cu has done the work.
+template <int IS, int LT, int GL, bool LOOP>
 __global__ void __launch_bounds__(kThreads)
 network_kernel(Csf3d u, const double *__restrict__ V, Csf3d w, double *__restrict__ Z, int n_k, int n_l, int n_m,
                int v_vec_ok, int64_t strips, int64_t tiles, const int32_t *__restrict__ mode) {
-    if constexpr (SHORT) {
-        if (mode && *mode == 0) return;
+    if (mode) {
+        after_last_kernel();
+        if (*mode == 0) return;
+    }
+    if constexpr (LOOP) {
         for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
             if (tile != blockIdx.x) __syncthreads();   // the tile before is done with the shared tables
-            network_tile<IS, LT, GL>(u, V, w, Z, n_k, n_l, n_m, v_vec_ok, (int)(tile % strips), (int)(tile / strips) * LT);
+            const int l_tile = (int)(tile / strips);
+            network_tile<IS, LT, GL>(u, V, w, Z, n_k, n_l, n_m, v_vec_ok, (int)(tile - l_tile * strips), l_tile * LT);
         }
     } else {
         network_tile<IS, LT, GL>(u, V, w, Z, n_k, n_l, n_m, v_vec_ok, blockIdx.x, blockIdx.y * LT);
@@ -275,20 +279,23 @@ const_status_t launch_network(const const_csf *U, const double *V, const const_c
     Csf3d w{W->crd[0], W->pos[1], W->crd[1], W->pos[2], W->crd[2], static_cast<const double *>(W->vals), (int32_t)W->n[0]};
     const int v_vec_ok = (n_l % 2 == 0) && (reinterpret_cast<uintptr_t>(V) % 16 == 0);
     const int64_t strips = (U->n[0] + IS - 1) / IS, l_tiles = (n_l + LT - 1) / LT, tiles = strips * l_tiles;
-    // A short grid behind network_dense.cu, which usually leaves nothing to do: sixteen blocks a slot find that out in a few
-    // us, one per tile took 19 us at 16 384 tiles (four a slot are slower where there is work: their tiles cost unequal
-    // time).  Also where the tiles of l outnumber a grid's rows.  Else one tile per block, which is 1 to 3 % faster than the
-    // loop (1024 x 1024 x 128 with 2 M nonzeros anywhere: 7.75 ms against 7.95).
-    auto launch = [&](auto is_short, dim3 grid) -> const_status_t {
-        auto kernel = network_kernel<IS, LT, GL, decltype(is_short)::value>;
+    // One tile per block, also behind network_dense.cu, which usually leaves nothing to do: 16 384 blocks need 15 us to find
+    // that out and 8192 need 9, but a loop over tiles costs 2.5 % where there is work (1024 x 1024 x 128 with 2 M nonzeros
+    // anywhere: 7.93 ms, one tile per block 7.77).  The loop is for tiles of l that outnumber a grid's rows.
+    auto launch = [&](auto loop, dim3 grid) -> const_status_t {
+        auto kernel = network_kernel<IS, LT, GL, decltype(loop)::value>;
         // the requested size depends on n_k: raise the limit once per device to the most a block may have
         static PerDeviceOnce attr_once;
         CB_CUDA(once_per_device(attr_once, [&] { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024); }));
-        CB_LAUNCH("network_kernel", stream,
-                  kernel<<<grid, kThreads, smem, stream>>>(u, V, w, Z, (int)n_k, (int)n_l, (int)n_m, v_vec_ok, strips, tiles, mode));
+        if (mode)
+            CB_LAUNCH("network_kernel", stream, CB_CUDA(launch_early(kernel, grid, kThreads, smem, stream, u, V, w, Z, (int)n_k, (int)n_l, (int)n_m,
+                                                                     v_vec_ok, strips, tiles, mode)));
+        else
+            CB_LAUNCH("network_kernel", stream,
+                      kernel<<<grid, kThreads, smem, stream>>>(u, V, w, Z, (int)n_k, (int)n_l, (int)n_m, v_vec_ok, strips, tiles, mode));
         return CONST_OK;
     };
-    const const_status_t rc = mode || l_tiles > 65535
+    const const_status_t rc = l_tiles > 65535
                                   ? launch(std::true_type(), dim3((unsigned)std::min<int64_t>(tiles, 148 * 2 * 16)))
                                   : launch(std::false_type(), dim3((unsigned)strips, (unsigned)l_tiles));
     if (rc != CONST_OK) return rc;
@@ -299,17 +306,23 @@ const_status_t launch_network(const const_csf *U, const double *V, const const_c
 }  // namespace
 
 // Operands with locality run on the fp64 matrix pipe (network_dense.cu), decided on the device; the gather kernel is launched
-// behind it and returns at once where that was done.
+// behind it and returns at once where that was done.  Operands it does not take pay 7 to 9 us for being looked at, more where T
+// would need several chunks (band of 41 at 331 x 331 x 61, too wide by four: 328 us without, 338 with).
 const_status_t run_network(const const_csf *U, const double *V, const const_csf *W, double *Z, int64_t n_i,
                            int64_t n_j, int64_t n_k, int64_t n_l, int64_t n_m, int32_t *, cudaStream_t stream) {
-    CB_CUDA(cudaMemsetAsync(Z, 0, sizeof(double) * n_i * n_m, stream));
-    if (U->nnz == 0 || W->nnz == 0) return CONST_OK;
     const int variant = debug_knobs().variant;
+    const bool empty = U->nnz == 0 || W->nnz == 0;
     int32_t *mode = nullptr;
     void *scratch = nullptr;
-    if (variant == 0) {
+    if ((variant == 0 || variant == 6) && !empty) {
         const const_status_t rc = run_network_dense(U, V, W, Z, n_i, n_j, n_k, n_l, n_m, &mode, &scratch, stream);
         if (rc != CONST_OK) return rc;
+    }
+    if (!mode) CB_CUDA(cudaMemsetAsync(Z, 0, sizeof(double) * n_i * n_m, stream));
+    if (empty) return CONST_OK;
+    if (variant == 6) {                                // the matrix form alone: what it hands on stays zero
+        if (scratch) cudaFreeAsync(scratch, stream);
+        return CONST_OK;
     }
     // tile shape (slices per strip, l per tile, lanes per fibre); the variants are kept for measurement
     auto gather = [&]() {

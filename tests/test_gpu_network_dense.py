@@ -37,6 +37,60 @@ def test_banded(n, n_k, band, keep):
     assert_close(out, S, A, np.float64)
 
 
+def matrix_form_alone(w):
+    """The output where only the matrix form is let run: zero if the device hands the work on."""
+    cb.const_debug_set(2, 6)
+    try:
+        out, _ = run_workload(w)
+    finally:
+        cb.const_debug_set(2, 0)
+    return out
+
+
+def bands(n, n_k, band_u, band_w, keep_u, keep_w):
+    """U and W of two bands of their own."""
+    w = network_workload(n, n_k, band_u, keep_u, config_id=65)
+    w.sparse["W"] = network_workload(n, n_k, band_w, keep_w, config_id=66).sparse["W"]
+    return w
+
+
+@pytest.mark.parametrize("band_u,band_w,keep_u,keep_w,taken", [
+    (48, 10, 0.6, 0.6, True),        # 95 neighbouring j of 96
+    (49, 10, 0.6, 0.6, False),       # 97
+    (10, 39, 0.6, 0.6, True),        # four slices of W together: 80 neighbouring m of 80
+    (10, 40, 0.6, 0.6, False),       # 82
+    (16, 16, 0.17, 0.17, True),      # 6 to 7 dense multiply-adds per sparse one
+    (16, 16, 0.1, 0.1, False),       # 11
+])
+def test_which_operands_the_matrix_form_takes(band_u, band_w, keep_u, keep_w, taken):
+    w = bands(500, 24, band_u, band_w, keep_u, keep_w)
+    S, A = oracle(w)
+    out, _ = run_workload(w)
+    assert_close(out, S, A, np.float64)
+    alone = matrix_form_alone(w)
+    if taken:
+        assert_close(alone, S, A, np.float64)
+    else:
+        assert not alone.any()
+
+
+def test_an_infinity_in_a_later_chunk():
+    """Products of the first chunk of slices have been added to Z when a T of the second turns out not to be finite: Z starts
+    again in the gather form.  (T of 1024 slices takes 335 MB, a chunk at most 256.)"""
+    w = network_workload(1024, 40, 6, 0.5, config_id=67)
+    U = w.sparse["U"]
+    keep = U.coords[1] != 1000
+    w.sparse["U"] = gen.SparseOperand([np.ascontiguousarray(c[keep]) for c in U.coords], np.ascontiguousarray(U.vals[keep]), U.dims)
+    rows = np.concatenate([np.arange(0, 1024, 61), np.arange(994, 1007)])
+    S, A = oracle(w, rows)
+    assert_close(matrix_form_alone(w), S, A, np.float64, rows)
+    w.dense["V"][1000] = np.inf
+    out, prof = kernels_of(w)
+    assert prof["network_t"][0] == 2
+    assert_close(out, S, A, np.float64, rows)
+    assert not matrix_form_alone(w).any()
+
+
 def scattered(n, n_k, nnz, seed):
     w = network_workload(n, n_k, 4, 0.25, config_id=62)
     rng = np.random.default_rng(seed)
@@ -51,6 +105,7 @@ def test_operands_without_locality():
     assert "network_t" in prof                                 # (asked for, and handed on by the device)
     S, A = oracle(w)
     assert_close(out, S, A, np.float64)
+    assert not matrix_form_alone(w).any()
 
 
 def test_rows_and_slices_missing():
@@ -77,6 +132,7 @@ def test_values_no_nonzero_reads(value):
     out, prof = kernels_of(w)
     assert "network_t" in prof
     assert_close(out, S, A, np.float64)
+    assert not matrix_form_alone(w).any()
 
 
 def test_more_rows_than_a_grid_has():
