@@ -1,8 +1,8 @@
 // Fused order-3 TTMc (Sec. 5.3) for tensors of long fibres:
 //   for i, for j (fused):  t[*] = 0;  for k: t[b] += X[i,j,k] * V[k,b];  for a,b: Y[i,a,b] += U[j,a] * t[b]      (Fig. 4(b))
 //
-// Every warp owns an equal run of the tensor's leaves, whatever the slices look like, and alternates between two phases
-// over windows of a few dozen fibres, entirely on its own:
+// Every warp owns a run of the tensor's leaves, whatever the slices look like (equal runs, or runs of equal cost, see
+// run_ttmc3_fibres), and alternates between two phases over windows of a few dozen fibres, on its own:
 //   phase 1 (producer)  A factor row of R3 floats is read by R3/4 neighbouring lanes with one 128-bit load each.  The
 //     nonzeros of the window are dealt out to the lane groups as equal contiguous runs of 4-aligned blocks, independent
 //     of fibre lengths: a block's four coordinates and four values arrive with one 128-bit load each and the four row
@@ -32,6 +32,7 @@ using walk::store_vec;
 using walk::zero_vec;
 
 constexpr int kWarps = 4;             // warps per block; they share nothing
+constexpr int kRound = 128;          // leaves that a lane group adds up before it adds the sum to those before
 constexpr int kStreamAhead = 256;   // nonzeros between the L2 prefetch of a line of the leaf arrays and its use
 
 __device__ __forceinline__ void fma4(Vec<float> &t, float x, const Vec<float> &v) { axpy(t, make_pair(x, x), v); }
@@ -79,9 +80,16 @@ __device__ __forceinline__ void phase1(const Chain<float, 3> &x, const float *__
         int f = lo;
         int32_t fend = Ps[f + 1];
         bool head = Ps[f] < pa;                                   // fibre f was begun by an earlier group
-        Vec<float> t = zero_vec<float>();
-
+        // In two levels, sum the rounds before and t the present one: the runs of a large tensor are long, and the rounding
+        // errors of a sum grow with its length (77 M, 16 x 16: relative error 5.8e-7 in one level, 3.7e-7 in two).
+        Vec<float> t = zero_vec<float>(), sum = zero_vec<float>();
+        auto round_off = [&]() {
+            axpy(sum, make_pair(1.f, 1.f), t);
+            t = zero_vec<float>();
+        };
         auto park = [&]() {                                       // hand the partial t of fibre f over
+            round_off();
+            t = sum;
             if (head) {
                 store_vec(Hs + g * R3 + 4 * q, t);
                 head_fibre = f;
@@ -92,7 +100,7 @@ __device__ __forceinline__ void phase1(const Chain<float, 3> &x, const float *__
         };
         auto leave_fibre = [&]() {                                // the run leaves fibre f
             park();
-            t = zero_vec<float>();
+            t = sum = zero_vec<float>();
             ++f;
             fend = Ps[f + 1 <= cnt ? f + 1 : cnt];
         };
@@ -149,6 +157,7 @@ __device__ __forceinline__ void phase1(const Chain<float, 3> &x, const float *__
                 if (p + 3 == fend) leave_fibre();
                 fma4(t, xc.w, v3);
                 if (p + 4 == fend) leave_fibre();
+                if (((p - m0) & (kRound - 4)) == kRound - 4) round_off();
                 v0 = w0; v1 = w1; v2 = w2; v3 = w3; xc = xw;
             }
         }
@@ -201,8 +210,35 @@ struct Args {
     Chain<float, 3> x;                                               // crd[2] and vals are readable up to the next multiple of 4
     const float *F1, *F2;
     float *out;
-    int32_t chunk;
+    int32_t chunk;                                                   // leaves per warp; with a weight, leaves + weight * fibres
+    int32_t weight;
 };
+
+// The part of the tensor between two costs, a leaf costing one and a fibre `weight`: its leaves [e0, e1), and the place of the
+// first.  Root first, as walk::place_of; both ends in one search.
+__device__ __forceinline__ void deal_weighted(const Args &a, int64_t cost, int lane, Place<3> &from, int32_t &e0, int32_t &e1) {
+    const int64_t w = a.weight, total = a.x.n[2] + w * a.x.n[1];
+    const int64_t target[2] = {cost < total ? cost : total - 1, cost + a.chunk < total ? cost + a.chunk : total - 1};
+    int32_t lo[2] = {0, 0}, hi[2] = {a.x.n[0], a.x.n[0]};
+    walk::warp_find2([&](int32_t s) { return __ldg(a.x.slice_ptr + s) + w * __ldg(a.x.pos[1] + s); }, lo, hi, target, lane);
+    from.node[0] = lo[0];
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+        hi[t] = __ldg(a.x.pos[1] + lo[t] + 1);
+        lo[t] = __ldg(a.x.pos[1] + lo[t]);
+    }
+    walk::warp_find2([&](int32_t f) { return __ldg(a.x.pos[2] + f) + w * f; }, lo, hi, target, lane);
+    from.node[1] = lo[0];
+    int32_t e[2];
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {                                    // the cost of a fibre is paid before its first leaf
+        const int32_t p = __ldg(a.x.pos[2] + lo[t]);
+        const int64_t behind = target[t] - (p + w * lo[t]) - w;
+        e[t] = behind > 0 ? max(p, (p + (int32_t)behind) & ~3) : p;  // on a block of four leaves, inside a fibre
+    }
+    e0 = cost < total ? e[0] : a.x.n[2];
+    e1 = cost + a.chunk < total ? e[1] : a.x.n[2];
+}
 
 template <int R2, int R3>
 struct __align__(16) Smem {
@@ -212,12 +248,22 @@ struct __align__(16) Smem {
 };
 
 template <int R2, int R3>
-__global__ void __launch_bounds__(kWarps * 32) chain3_kernel(const __grid_constant__ Args a) {
+__global__ void __launch_bounds__(kWarps * 32, 4) chain3_kernel(const __grid_constant__ Args a) {
     using S = Shape<R2, R3>;
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31;
     Smem<R2, R3> &sm = reinterpret_cast<Smem<R2, R3> *>(smem)[threadIdx.x >> 5];
-    const walk::Share own(a.x.n[2], a.chunk, kWarps);
+    walk::Share own;
+    Place<3> from;
+    if (a.weight == 0) {
+        own = walk::Share(a.x.n[2], a.chunk, kWarps);
+    } else {
+        __shared__ int32_t block_end;
+        deal_weighted(a, ((int64_t)blockIdx.x * kWarps + (threadIdx.x >> 5)) * a.chunk, lane, from, own.e0, own.e1);
+        if (threadIdx.x == kWarps * 32 - 1) block_end = own.e1;
+        __syncthreads();
+        own.block_end = block_end;
+    }
     Pair<float> pairs[4][4];
     auto clear = [&]() {
 #pragma unroll
@@ -246,7 +292,11 @@ __global__ void __launch_bounds__(kWarps * 32) chain3_kernel(const __grid_consta
             for (int r = 0; r < 8; ++r)
                 put((8 * rg + r) * R3 + 4 * cg, walk::make_vec(make_float4(acc[4 * r], acc[4 * r + 1], acc[4 * r + 2], acc[4 * r + 3])));
     };
-    const int32_t joint = walk::walk_chunk(a.x, own, lane, [](const Place<3> &) {},
+    const int32_t joint = walk::walk_chunk(a.x, own,
+        [&](int32_t e) {
+            return a.weight == 0 ? walk::place_of(a.x, e, lane) : from;
+        },
+        [](const Place<3> &) {},
         [&](Place<3> &place, int32_t e, int32_t limit) {
             // fibres of the window: those of the next WINDOW that begin before `limit` (all in one slice)
             constexpr int NW = S::WINDOW / 32;
@@ -296,7 +346,7 @@ const_status_t launch_chain3(const Args &a, int64_t n_rows, cudaStream_t stream)
     constexpr size_t dyn = sizeof(Smem<R2, R3>) * kWarps;
     static PerDeviceOnce attr_once;                     // per template instance
     CB_CUDA(once_per_device(attr_once, [&] { return cudaFuncSetAttribute(chain3_kernel<R2, R3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn); }));
-    const int64_t warps = ((int64_t)a.x.n[2] + a.chunk - 1) / a.chunk;
+    const int64_t warps = ((int64_t)a.x.n[2] + (int64_t)a.weight * a.x.n[1] + a.chunk - 1) / a.chunk;
     return walk::launch_on_cleared("chain3_kernel", chain3_kernel<R2, R3>, a, dim3((unsigned)((warps + kWarps - 1) / kWarps)), kWarps * 32, dyn,
                                    a.out, sizeof(float) * R2 * R3 * n_rows, stream);
 }
@@ -306,7 +356,20 @@ const_status_t launch_chain3(const Args &a, int64_t n_rows, cudaStream_t stream)
 // Same contraction as the leaf-balanced walk of chain_kernels.cu.
 const_status_t run_ttmc3_fibres(const const_csf *X, const float *U, const float *V, int R2, int R3, float *Y, int64_t n_rows,
                                 cudaStream_t s) {
-    const Args a{walk::chain_of<float, 3>(X), U, V, Y, walk::chunk_leaves(X->nnz, X->n[0], 16, 1536, 16)};
+    // From three million leaves on the warps get equal costs instead of equal leaves: a leaf of a short fibre costs several
+    // times one of a long fibre, so that with Zipf-sized slices equal leaves took unequal time, and chunks small enough to
+    // even that out paid for their searches.  A fibre counts as six leaves (four and eight are worse by 3 to 10 % on most rank
+    // pairs).  Whole waves of parts of at most 8192: larger ones are up to 5 % faster, but longer sums round more (10.5 M, 32 x
+    // 32, relative error 3.5e-7 at 16 384, 2.9e-7 at 8192, 3.2e-7 before).  Leaf chunks of 1536 against this, us (work lists):
+    // 10.5 M, slices Zipf 1.1, 8 x 8: 212 / 161 (152), 16 x 16: 324 / 231 (255), 32 x 32: 537 / 398 (459); 77 M, 16 x 16:
+    // 1102 / 1059 (1140); uniform, 20 M in fibres of 33, 8 x 8: 161 / 142 (176), 32 x 32: 307 / 311 (324); but 2 M in fibres of
+    // 25: 24.4 / 25.7, 300 000: 17.8 / 19.5 (the longer search).
+    constexpr int32_t kWeight = 6, kResident = 16;
+    constexpr int64_t kMostCost = 8192, kWave = 148 * kResident;
+    const int64_t cost = X->nnz + kWeight * X->n[1], parts = (cost + kWave * kMostCost - 1) / (kWave * kMostCost) * kWave;
+    const bool weigh = X->nnz >= 3000000;
+    const Args a{walk::chain_of<float, 3>(X), U, V, Y,
+                 weigh ? (int32_t)((cost + parts - 1) / parts) : walk::chunk_leaves(X->nnz, X->n[0], kResident, 1536, kResident), weigh ? kWeight : 0};
     switch (R2 * 100 + R3) {
         case 808: return launch_chain3<8, 8>(a, n_rows, s);
         case 816: return launch_chain3<8, 16>(a, n_rows, s);

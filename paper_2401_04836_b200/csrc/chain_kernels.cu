@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(kWarps * 32, MttkrpShape<T, ORDER, RP>::BLOCKS
     const int col = blockIdx.y * RP + q * N;
     const T *leaf = a.F[ORDER - 2] + col, *mid = ORDER == 4 ? a.F[1] + col : nullptr, *top = a.F[0] + col;
     Vec<T> acc = zero_vec<T>();
-    const int32_t joint = walk_chunk(a.x, own, lane,
+    const int32_t joint = walk_chunk(a.x, own, [&](int32_t e) { return place_of(a.x, e, lane); },
         [](const Place<ORDER> &) {},
         [&](Place<ORDER> &place, int32_t e, int32_t limit) {
             const int cnt = limit - e < S::W ? limit - e : S::W;
@@ -241,7 +241,7 @@ __global__ void __launch_bounds__(kWarps * 32, Ttmc3Shape<T, R2, R3>::BLOCKS) tt
             put(rg + 2 * i + 1, hi);
         }
     };
-    const int32_t joint = walk_chunk(a.x, own, lane,
+    const int32_t joint = walk_chunk(a.x, own, [&](int32_t e) { return place_of(a.x, e, lane); },
         [](const Place<3> &) {},
         [&](Place<3> &place, int32_t e, int32_t limit) {
             const int cnt = limit - e < S::W ? limit - e : S::W;
@@ -370,7 +370,7 @@ __global__ void __launch_bounds__(kWarps * 32, Ttmc4Shape<T>::BLOCKS) ttmc4_kern
         }
     };
     Ahead<T, 4, S::W> ahead;
-    const int32_t joint = walk_chunk(a.x, own, lane,
+    const int32_t joint = walk_chunk(a.x, own, [&](int32_t e) { return place_of(a.x, e, lane); },
         [&](const Place<4> &place) {
             request<T, 4, S::W>(a.x, place, own.e0, own.e1, lane, ahead);
         },

@@ -160,6 +160,32 @@ struct Place {
     int32_t node[ORDER - 1];
 };
 
+// Largest x in [lo, hi) with key(x) <= target, by the whole warp, for two targets at once (key(lo) <= target; key does not fall).
+template <class Key>
+__device__ __forceinline__ void warp_find2(Key key, int32_t (&lo)[2], int32_t (&hi)[2], const int64_t (&target)[2], int lane) {
+    while (hi[0] - lo[0] > 1 || hi[1] - lo[1] > 1) {
+        bool below[2][4];
+        int32_t step[2];
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+            step[t] = (int32_t)(((int64_t)hi[t] - lo[t] + 127) / 128);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int64_t at = lo[t] + (int64_t)(32 * k + lane) * step[t];
+                below[t][k] = at < hi[t] && key((int32_t)at) <= target[t];
+            }
+        }
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+            int32_t c = -1;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) c += __popc(__ballot_sync(kAll, below[t][k]));
+            lo[t] += c * step[t];
+            hi[t] = hi[t] - lo[t] < step[t] ? hi[t] : lo[t] + step[t];
+        }
+    }
+}
+
 // Root first, so that every search below is over one slice only: few steps, each a dependent load.
 template <typename T, int ORDER>
 __device__ __forceinline__ Place<ORDER> place_of(const Chain<T, ORDER> &x, int32_t leaf, int lane) {
@@ -338,6 +364,7 @@ __device__ __forceinline__ int stage_window(const Ahead<T, ORDER, W> &a, Place<O
 // The leaves of one warp, and the end of those of its block.
 struct Share {
     int32_t e0, e1, block_end;
+    Share() = default;
     __device__ __forceinline__ Share(int32_t nnz, int32_t chunk, int warps) {
         const int64_t b0 = (int64_t)blockIdx.x * warps * chunk, b1 = b0 + (int64_t)warps * chunk;
         const int64_t w0 = b0 + (int64_t)(threadIdx.x >> 5) * chunk;
@@ -349,19 +376,18 @@ struct Share {
 
 // Walks the warp's leaves: window(place, e, limit) consumes some leaves of [e, limit), all in one slice, moves the place
 // and returns how many; flush(slice, whole) ends a slice or the warp's part of it (whole: the warp had all of it).
-// start(place) is called once, at the place of the first leaf.  Returns the slice that the whole block lies in, not
+// find(e) is the place of leaf e; start(place) is called once, at the place of the first leaf.  Returns the slice that the whole block lies in, not
 // flushed, or -1: the parts of such a slice are to be added up in the block first, which keeps the number of atomic
 // additions to one row of the result (and the rounding errors they add) down where a slice is shared by many warps.
 // Every warp of the block has to call this.
-template <typename T, int ORDER, class Start, class Window, class Flush>
-__device__ __forceinline__ int32_t walk_chunk(const Chain<T, ORDER> &x, const Share &own, int lane, Start start, Window window,
-                                              Flush flush) {
+template <typename T, int ORDER, class Find, class Start, class Window, class Flush>
+__device__ __forceinline__ int32_t walk_chunk(const Chain<T, ORDER> &x, const Share &own, Find find, Start start, Window window, Flush flush) {
     __shared__ int32_t first_slice;                      // where the block's first leaf lies
     Place<ORDER> place;
     int32_t e = own.e0, end = 0;
     bool from_start = false;
     if (e < own.e1) {
-        place = place_of(x, e, lane);
+        place = find(e);
         start(place);
         from_start = __ldg(x.slice_ptr + place.node[0]) == e;
         end = __ldg(x.slice_ptr + place.node[0] + 1);

@@ -214,3 +214,23 @@ def test_products_are_formed_in_the_order_of_the_schedule(family, ranks, long_fi
     fac[names[-1]] = fac[names[-1]] * np.float32(2.0 ** -100)
     out, S, A = run_chain(family, dims, ranks, X, fac, cb.F32)
     assert_close(out, S, A, np.float32)
+
+
+@pytest.mark.parametrize("dims,slice_s,inner", [
+    ((40, 3, 60_000), None, None),         # 120 fibres of 27 000 leaves, each over many warps
+    ((1, 3000, 2500), None, None),         # one slice
+    ((3000, 5000, 400), 1.1, None),        # slices of all sizes, a hot one over hundreds of warps, fibres of a few leaves
+    ((500_000, 40, 50), 0.5, None),        # more slices than a search takes in two steps, most of them of a few leaves
+])
+def test_parts_of_equal_cost(dims, slice_s, inner):
+    """From three million nonzeros on order-3 TTMc cuts the tensor by leaves and fibres together: parts begin inside fibres,
+    at fibres, and at slices."""
+    for rank in ((8, 8), (16, 16), (32, 32)) if dims[0] <= 40 else ((8, 8), (8, 16)):
+        w = ttmc3_workload(dims, 3_100_000, rank, slice_s=slice_s, inner_s=inner, value="pm1", config_id=26)
+        out, _ = run_workload(w)
+        present = np.unique(w.sparse["X"].coords[0])
+        rows = np.unique(np.concatenate([present[:: max(1, present.size // 40)], present[-1:]]))
+        S, A = oracle(w, rows)
+        assert_close(out, S, A, np.float32, rows)
+        absent = np.setdiff1d(np.arange(dims[0]), present)
+        assert not out[absent].any()
