@@ -505,6 +505,28 @@ def measure_config(cb, torch, w, config_id, args, peaks, hbm_peak, peak_kind, ra
     }
 
 
+def short_line(line):
+    """The result line: the contract's keys, five significant digits, per configuration [step ms, execute ms, GFLOP/s, e2e GFLOP/s]."""
+    def cut(x):
+        if isinstance(x, dict):
+            return {k: cut(v) for k, v in x.items()}
+        return float(f"{x:.5g}") if isinstance(x, float) else x
+    pick = lambda d, *keys: None if d is None else {k: d.get(k) for k in keys}
+    c = line["config"]
+    out = {k: line[k] for k in ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+                                "vs_baseline", "dtype", "data")}
+    out["config"] = dict(pick(c, "workload", "scale", "step", "nnz", "l2", "replicas"),
+                         per_config={k: [cut(v["ms_per_step"]), cut(v["execute_ms"]), cut(v["value_gflops"]), cut(v["e2e"]["value"])]
+                                     for k, v in c["per_config"].items()})
+    out["roofline"] = pick(line["roofline"], "kernel", "bound", "achieved", "peak", "unit", "frac", "traffic")
+    out["cpu_baseline"] = pick(line["cpu_baseline"], "value", "unit", "cores", "kind")
+    out["max_err_ratio"] = line["max_err_ratio"]
+    out["e2e"] = pick(line["e2e"], "value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step")
+    out["gpu_launches"] = line["gpu_launches"]
+    out["clocks"] = pick(line["clocks"], "sm_mhz", "sm_max_mhz", "reasons")
+    return cut(out)
+
+
 # ------------------------------------------------------------------------------------------------
 def main():
     ap = argparse.ArgumentParser()
@@ -634,7 +656,10 @@ def main():
         "per_config": {str(cid): {k: v for k, v in results[cid].items() if k not in ("kernels", "rooflines")}
                        for cid in sorted(results)},
     }
-    print(json.dumps(line))
+    # every figure goes to standard error; the line itself stays short, so that a reader who keeps only the end of the
+    # output has all of it
+    print(json.dumps(line), file=sys.stderr)
+    print(json.dumps(short_line(line)))
     if dist is not None:
         dist.destroy_process_group()
     return 0
