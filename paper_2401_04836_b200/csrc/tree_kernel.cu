@@ -494,7 +494,7 @@ const_status_t run_tree(const tree::Compiled &cp, const_dtype_t dtype, const con
         if (L.count == 0) continue;
         const unsigned grid = (unsigned)L.grid;
         const int32_t local = L.local ? 1 : 0;
-        CB_LAUNCH("tree_kernel", stream, {
+        CB_LAUNCH(L.step ? "tree_step_kernel" : "tree_kernel", stream, {
             if (dtype == CONST_F32 && L.warp)
                 tree_kernel<float, true><<<grid, kThreads, L.smem, stream>>>(cp.programs[r], b, L.count, L.chunk, local);
             else if (dtype == CONST_F32)

@@ -110,8 +110,9 @@ def test_mttkrp_each_bin(rank, bins):
     check(w, bins)
 
 
-# order-4 TTMc: the per-slice stage Y_i = U_J^T Q_J runs on the tensor cores (split tf32 operands, the
-# default at rank 8) or on the FMA pipes; both must meet the fp32 tolerance
+# order-4 TTMc: the per-slice stage Y_i = U_J^T Q_J runs on the FMA pipes or, on request, on the tensor cores (split
+# tf32 operands); both must meet the fp32 tolerance.  Only the tensor-core kernels work from the bins: the others have to
+# give the same result whatever they are
 @pytest.mark.parametrize("tensor_stage", [False, True])
 @pytest.mark.parametrize("bins", [None, ALL_LIGHT, ALL_HEAVY, ALL_GIANT, MIXED])
 def test_ttmc4_each_bin(bins, tensor_stage):

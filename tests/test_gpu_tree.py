@@ -104,11 +104,12 @@ def test_generic_executor_on_schedules_the_families_cover():
 @pytest.mark.parametrize("rank", [4, 12, 16])
 def test_ttmc4_at_ranks_without_a_hand_written_kernel(rank):
     w = ttmc4_workload((30, 12, 10, 9), 2_500, rank, slice_s=1.0, value="pm1", config_id=3)
-    out, family = run_tree(w.expression, w.tree, w.mode_orders, w.loop_orders, w.extents, cb.F32, w.sparse, w.dense,
-                           w.out_shape)
-    assert family == "tree"
     S, A = oracle(w)
-    assert_close(out, S, A, np.float32)
+    for generic in (None, True):                                 # rank 4: the chain kernels unless asked otherwise
+        out, family = run_tree(w.expression, w.tree, w.mode_orders, w.loop_orders, w.extents, cb.F32, w.sparse, w.dense,
+                               w.out_shape, generic=generic)
+        assert family == "tree"
+        assert_close(out, S, A, np.float32)
 
 
 def test_ttmc3_in_fp64_and_with_an_unfused_consumer():
@@ -118,10 +119,11 @@ def test_ttmc3_in_fp64_and_with_an_unfused_consumer():
     dense = {n: a.astype(np.float64) for n, a in w.dense.items()}
     S, A = oc.ttmc3(X.coords, X64.vals, dense["U"], dense["V"], X.dims[0])
     for loops in (w.loop_orders, ["ijkb", "iajb"]):              # t[b] per (i,j); or t[j,b] per i with a, j swapped
-        out, family = run_tree(w.expression, w.tree, w.mode_orders, loops, w.extents, cb.F64, {"X": X64}, dense,
-                               w.out_shape)
-        assert family == "tree"
-        assert_close(out, S, A, np.float64)
+        for generic in (None, True):                             # the first is a chain that the chain kernels take
+            out, family = run_tree(w.expression, w.tree, w.mode_orders, loops, w.extents, cb.F64, {"X": X64}, dense,
+                                   w.out_shape, generic=generic)
+            assert family == "tree"
+            assert_close(out, S, A, np.float64)
 
 
 def test_order4_mttkrp():
@@ -132,10 +134,12 @@ def test_order4_mttkrp():
     expr = "M[i,r] = X[i,j,k,l] * B[j,r] * C[k,r] * D[l,r]"
     tree = ["P[i,j,k,r] = X[i,j,k,l] * D[l,r]", "Q[i,j,r] = P[i,j,k,r] * C[k,r]", "M[i,r] = Q[i,j,r] * B[j,r]"]
     ext = {"i": 20, "j": 9, "k": 8, "l": 7, "r": r}
-    out, family = run_tree(expr, tree, {"X": (0, 1, 2, 3)}, ["ijklr", "ijkr", "ijr"], ext, cb.F32, {"X": X}, fac, (20, r))
-    assert family == "tree"
     S, A = oc.nary_einsum(expr, dict(fac, X=coo(X)), ext)
-    assert_close(out, S, A, np.float32)
+    for generic in (None, True):
+        out, family = run_tree(expr, tree, {"X": (0, 1, 2, 3)}, ["ijklr", "ijkr", "ijr"], ext, cb.F32, {"X": X}, fac, (20, r),
+                               generic=generic)
+        assert family == "tree"
+        assert_close(out, S, A, np.float32)
 
 
 def test_network_scatter_form_and_unfused():
@@ -275,10 +279,11 @@ def test_medium_sizes_reach_every_way_the_iterations_are_dealt_out():
     workspaces in shared memory; (c) a 122 KB workspace per outer iteration -- workspaces in global scratch."""
     w = ttmc3_workload((4000, 300, 400), 400_000, (12, 12), slice_s=1.1, value="pm1", config_id=61)
     S, A = oracle(w)
-    out, family = run_tree(w.expression, w.tree, w.mode_orders, w.loop_orders, w.extents, cb.F32, w.sparse, w.dense,
-                           w.out_shape)
-    assert family == "tree"
-    assert_close(out, S, A, np.float32)
+    for generic in (None, True):                                  # (a chain: the chain kernels unless asked otherwise)
+        out, family = run_tree(w.expression, w.tree, w.mode_orders, w.loop_orders, w.extents, cb.F32, w.sparse, w.dense,
+                               w.out_shape, generic=generic)
+        assert family == "tree"
+        assert_close(out, S, A, np.float32)
 
     w = ttmc4_workload((300, 100, 20, 20), 60_000, 24, slice_s=1.0, value="pm1", config_id=62)
     X = w.sparse["X"]

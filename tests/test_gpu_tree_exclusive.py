@@ -16,13 +16,14 @@ pytestmark = pytest.mark.gpu
 GOLDEN = os.path.join(os.path.dirname(os.path.abspath(__file__)), "golden")
 
 
-@pytest.mark.parametrize("dtype,i,nnz_c", [
-    (cb.F64, 64, 4000),        # in step: 28 x 64 updates per value of q for 256 threads
-    (cb.F64, 61, 4000),        # rows made odd already, an extent that does not divide the group
-    (cb.F64, 64, 200),         # too few: dealt out
-    (cb.F32, 128, 4000),       # fp32: always dealt out, padded rows
+@pytest.mark.parametrize("dtype,i,nnz_c,kernel", [
+    (cb.F64, 64, 4000, "tree_step_kernel"),        # in step: 28 x 64 updates per value of q for 256 threads
+    (cb.F64, 61, 4000, "tree_step_kernel"),        # rows made odd already, an extent that does not divide the group
+    (cb.F64, 64, 200, "tree_step_kernel"),         # too few: dealt out, by the same kernel
+    (cb.F64, 40, 4000, "tree_kernel"),             # workspaces that let more than four blocks run on an SM
+    (cb.F32, 128, 4000, "tree_kernel"),            # fp32: always dealt out, padded rows
 ])
-def test_running_example_with_large_workspaces(dtype, i, nnz_c):
+def test_running_example_with_large_workspaces(dtype, i, nnz_c, kernel):
     with open(os.path.join(GOLDEN, "running_example_schedule.json")) as f:
         g = json.load(f)
     rng = np.random.default_rng(i + nnz_c)
@@ -34,7 +35,11 @@ def test_running_example_with_large_workspaces(dtype, i, nnz_c):
     plan = cb.const_plan_create(g["expression"], g["tree"], g["mode_orders"], g["loop_orders"], ext, dtype)
     ops = {n: build_csf(op, g["mode_orders"][n]) for n, op in sparse.items()}
     out = torch.full((i, 4, 48), float("nan"), dtype=torch.float32 if dtype == cb.F32 else torch.float64, device="cuda")
+    cb.const_profile_enable(True)
     cb.const_execute(plan, ops, out)
+    prof = cb.const_profile_read()
+    cb.const_profile_enable(False)
+    assert [k for k in prof if k.startswith("tree")] == [kernel]
     assert cb.const_last_device_status(plan) == 0
     S, A = oc.nary_einsum(g["expression"], {t: (op.coords, op.vals) for t, op in sparse.items()}, ext)
     assert np.count_nonzero(A) > 0
