@@ -21,13 +21,14 @@
 // the gather kernel, launched last, then clears Z and does the work.
 //
 // Measured, 1024 x 1024 x 128, band 32, a quarter full: 4771 us in the gather form; here t_kernel 660 us (dense work at the
-// fp64 peak of 37 TFLOP/s: 480) and z_kernel 890 us (540), 1552 us together with clearing and shape.  z_kernel is held by
+// fp64 peak of 37 TFLOP/s: 480) and z_kernel 820 us (540), 1499 us together with clearing and shape.  z_kernel is held by
 // writing its slices out between the products: walking the fibres for it 1196 us, from places computed once 979, with the
-// next slice's entries on their way meanwhile 889.  331 x 331 x 61, band 17: 164 -> 115 us; 700, 100, band 21: 1187 -> 542.
+// next slice's entries on their way meanwhile 889, without a test per product 820.  331 x 331 x 61, band 17: 162 -> 95 us;
+// 700, 100, band 21: 1194 -> 471.
 //
 // The launches are short ones at the small end, so they are few and start early (launch_early): clearing Z and the mode word,
 // ranges and places in one kernel, t and z once per chunk, the gather kernel.  Ranges and places in two kernels, the mode word
-// cleared apart and ordinary launches: 128 us at 331, 1566 at 1024; and 25 us instead of 8 for operands that do not qualify.
+// cleared apart and ordinary launches: 15 us more at 331 and 1024; and 25 us instead of 8 for operands that do not qualify.
 #include <algorithm>
 
 #include "common.cuh"
@@ -264,23 +265,21 @@ struct Staged {
     }
 };
 
-__global__ void __launch_bounds__(kThreads, 2) z_kernel(const __grid_constant__ Net a) {
-    extern __shared__ __align__(16) double z_smem[];
-    Staged &staged = *reinterpret_cast<Staged *>(z_smem);
-    double *w_dense = z_smem + sizeof(Staged) / sizeof(double);           // [tile of k][range of m + 4]
-    __shared__ int skip;
-    after_last_kernel();
-    if (threadIdx.x == 0) skip = *a.mode;
-    __syncthreads();
-    if (skip) return;
+// Products of kRows slices of U with the kNodes slices of W of one group, whose m span N tiles of eight.  Sums run over one
+// tile of k at a time and then join those before: in one chain over all four slices the error was a quarter above the gather
+// form's (1024: 4.3e-16 against 3.35e-16 relative 2-norm; so 2.9e-16).  N is a constant because asking at each product
+// whether its tile is there costs as much as the additions gain: 1583 us an execute at 1024 and 297 a step at 331 with up to
+// ten tiles and a test each, 1499 and 279 so.
+template <int N>
+__device__ __forceinline__ void z_group(const Net &a, int group, Staged &staged, double *w_dense) {
+    constexpr int ld = N * 8 + 4;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, r = lane >> 2, c = lane & 3;
-    const int group = blockIdx.x, m0 = a.mmin[group], len = a.mlen[group];
-    const int tiles = round_up(len, 8) / 8, ld = tiles * 8 + 4;
+    const int m0 = a.mmin[group], len = a.mlen[group];
     const int s = a.s0 + blockIdx.y * kRows + warp * 8 + r;              // this lane's slice of U
     const bool have = s < a.s1;
-    double acc[kRangeM / 8][2];
+    double acc[N][2];
 #pragma unroll
-    for (int t = 0; t < kRangeM / 8; ++t) acc[t][0] = acc[t][1] = 0.0;
+    for (int t = 0; t < N; ++t) acc[t][0] = acc[t][1] = 0.0;
     const int n0 = group * kNodes, n1 = min(n0 + kNodes, a.w.n0);
     int32_t leaf = __ldg(a.w.pos2 + __ldg(a.w.pos1 + n0)), leaf1 = __ldg(a.w.pos2 + __ldg(a.w.pos1 + n0 + 1));
     staged.request(a.w_place, a.w.vals, leaf, leaf1);
@@ -291,7 +290,7 @@ __global__ void __launch_bounds__(kThreads, 2) z_kernel(const __grid_constant__ 
         for (int k0 = 0; k0 < a.tk; k0 += kTileK) {
             const int kt = min(kTileK, a.tk - k0), steps = kt / 4;       // steps is even
             auto t_at = [&](int st) { return have && st < steps ? __ldg(t_row + k0 + st * 4) : 0.0; };
-            double x[4];
+            double x[4], part[N][2];
 #pragma unroll
             for (int z = 0; z < 4; ++z) x[z] = t_at(z);
             if (k0 == 0) asm volatile("cp.async.wait_all;" ::: "memory");
@@ -301,6 +300,8 @@ __global__ void __launch_bounds__(kThreads, 2) z_kernel(const __grid_constant__ 
             staged.write(a.w_place, a.w.vals, leaf, leaf1, k0, kt, [&](int m, int k, double v) { w_dense[k * ld + m] = v; });
             __syncthreads();
             if (k0 + kTileK >= a.tk && node + 1 < n1) staged.request(a.w_place, a.w.vals, leaf1, leaf2);
+#pragma unroll
+            for (int t = 0; t < N; ++t) part[t][0] = part[t][1] = 0.0;
             for (int st = 0; st < steps; st += 4) {
                 double next[4];
 #pragma unroll
@@ -310,11 +311,15 @@ __global__ void __launch_bounds__(kThreads, 2) z_kernel(const __grid_constant__ 
                     if (st + z >= steps) break;                           // uniform
                     const double *row = w_dense + ((st + z) * 4 + c) * ld + r;
 #pragma unroll
-                    for (int t = 0; t < kRangeM / 8; ++t)
-                        if (t < tiles) mma884(acc[t][0], acc[t][1], x[z], row[t * 8]);
+                    for (int t = 0; t < N; ++t) mma884(part[t][0], part[t][1], x[z], row[t * 8]);
                 }
 #pragma unroll
                 for (int z = 0; z < 4; ++z) x[z] = next[z];
+            }
+#pragma unroll
+            for (int t = 0; t < N; ++t) {
+                acc[t][0] += part[t][0];
+                acc[t][1] += part[t][1];
             }
         }
         leaf = leaf1;
@@ -323,11 +328,36 @@ __global__ void __launch_bounds__(kThreads, 2) z_kernel(const __grid_constant__ 
     if (!have) return;
     double *z = a.Z + (size_t)__ldg(a.u.crd0 + s) * a.n_m + m0 + 2 * c;
 #pragma unroll
-    for (int t = 0; t < kRangeM / 8; ++t)
-        if (t < tiles) {
-            if (t * 8 + 2 * c < len) atomicAdd(z + t * 8, acc[t][0]);
-            if (t * 8 + 2 * c + 1 < len) atomicAdd(z + t * 8 + 1, acc[t][1]);
-        }
+    for (int t = 0; t < N; ++t) {
+        if (t * 8 + 2 * c < len) atomicAdd(z + t * 8, acc[t][0]);
+        if (t * 8 + 2 * c + 1 < len) atomicAdd(z + t * 8 + 1, acc[t][1]);
+    }
+}
+
+__global__ void __launch_bounds__(kThreads, 2) z_kernel(const __grid_constant__ Net a) {
+    extern __shared__ __align__(16) double z_smem[];
+    Staged &staged = *reinterpret_cast<Staged *>(z_smem);
+    double *w_dense = z_smem + sizeof(Staged) / sizeof(double);           // [tile of k][range of m + 4]
+    __shared__ int skip;
+    after_last_kernel();
+    if (threadIdx.x == 0) skip = *a.mode;
+    __syncthreads();
+    if (skip) return;
+    const int group = blockIdx.x;
+    static_assert(kRangeM == 80, "one case per number of tiles");
+    switch (round_up(a.mlen[group], 8) / 8) {
+        case 1: return z_group<1>(a, group, staged, w_dense);
+        case 2: return z_group<2>(a, group, staged, w_dense);
+        case 3: return z_group<3>(a, group, staged, w_dense);
+        case 4: return z_group<4>(a, group, staged, w_dense);
+        case 5: return z_group<5>(a, group, staged, w_dense);
+        case 6: return z_group<6>(a, group, staged, w_dense);
+        case 7: return z_group<7>(a, group, staged, w_dense);
+        case 8: return z_group<8>(a, group, staged, w_dense);
+        case 9: return z_group<9>(a, group, staged, w_dense);
+        case 10: return z_group<10>(a, group, staged, w_dense);
+        default: return;                                                  // no entries
+    }
 }
 
 // Z back to zero where the gather kernel takes over after products have been added to it
@@ -353,7 +383,7 @@ const_status_t run_network_dense(const const_csf *U, const double *V, const cons
     const int64_t row_bytes = n_l * tk * 8;
     const int64_t n0 = U->n[0], groups = (W->n[0] + kNodes - 1) / kNodes;
     // Small networks stay with the gather kernel; so does one whose T would leave fewer than 64 slices to a chunk.  Where the
-    // line lies (multiply-adds of the gather form): at 1.1e8 the band at 331 takes 164 us in the gather form and 115 here,
+    // line lies (multiply-adds of the gather form): at 1.1e8 the band at 331 takes 162 us in the gather form and 95 here,
     // operands that then do not qualify pay about 8 us: 3 % of a call at 1.2e8, 4 % at 7e7.
     if (sparse < 6e7 || n_k > 4096 || kScratchBytes / row_bytes < std::min<int64_t>(n0, 64)) return CONST_OK;
     if (n_l > (1 << 24) || n_m > (1 << 24) || groups > 65535 * 8ll || n0 + W->n[0] > 0x7fffffffll) return CONST_OK;
