@@ -31,8 +31,7 @@ using walk::peek_vec;
 using walk::store_vec;
 using walk::zero_vec;
 
-constexpr int kWarps = 4;             // warps per block; they share nothing
-constexpr int kRound = 128;          // leaves that a lane group adds up before it adds the sum to those before
+constexpr int kWarps = 4;             // warps per block; they meet where a slice covers the block
 constexpr int kStreamAhead = 256;   // nonzeros between the L2 prefetch of a line of the leaf arrays and its use
 
 __device__ __forceinline__ void fma4(Vec<float> &t, float x, const Vec<float> &v) { axpy(t, make_pair(x, x), v); }
@@ -56,7 +55,7 @@ struct Shape {
 // that a group finds already begun (its run starts in the middle of it) goes to a per-group "head"
 // slot and is added to the row afterwards, one group after the other, so no atomics and no clearing
 // of the rows are needed.
-template <int R2, int R3>
+template <int R2, int R3, bool ROUNDS>
 __device__ __forceinline__ void phase1(const Chain<float, 3> &x, const float *__restrict__ F2, int cnt,
                                        int lane, float *__restrict__ Ts, const int32_t *__restrict__ Ps, float *__restrict__ Hs, int32_t *__restrict__ Hf) {
     using S = Shape<R2, R3>;
@@ -80,16 +79,19 @@ __device__ __forceinline__ void phase1(const Chain<float, 3> &x, const float *__
         int f = lo;
         int32_t fend = Ps[f + 1];
         bool head = Ps[f] < pa;                                   // fibre f was begun by an earlier group
-        // In two levels, sum the rounds before and t the present one: the runs of a large tensor are long, and the rounding
-        // errors of a sum grow with its length (77 M, 16 x 16: relative error 5.8e-7 in one level, 3.7e-7 in two).
+        // ROUNDS: in two levels, sum the rounds of 32 leaves before and t the present one.  Parts of equal cost are long, and the
+        // rounding errors of a sum grow with its length (77 M, 16 x 16: relative error 3.8e-7 in one level, 2.6e-7 in two, for
+        // 1 % of the time; a test of its own in every block of four, or for sums without a round: 3 to 6 %).
         Vec<float> t = zero_vec<float>(), sum = zero_vec<float>();
         auto round_off = [&]() {
             axpy(sum, make_pair(1.f, 1.f), t);
             t = zero_vec<float>();
         };
         auto park = [&]() {                                       // hand the partial t of fibre f over
-            round_off();
-            t = sum;
+            if constexpr (ROUNDS) {
+                round_off();
+                t = sum;
+            }
             if (head) {
                 store_vec(Hs + g * R3 + 4 * q, t);
                 head_fibre = f;
@@ -100,7 +102,8 @@ __device__ __forceinline__ void phase1(const Chain<float, 3> &x, const float *__
         };
         auto leave_fibre = [&]() {                                // the run leaves fibre f
             park();
-            t = sum = zero_vec<float>();
+            t = zero_vec<float>();
+            if constexpr (ROUNDS) sum = t;
             ++f;
             fend = Ps[f + 1 <= cnt ? f + 1 : cnt];
         };
@@ -135,9 +138,12 @@ __device__ __forceinline__ void phase1(const Chain<float, 3> &x, const float *__
                 xn = __ldg(reinterpret_cast<const float4 *>(x.vals + m0 + 4));
             }
             for (int32_t p = m0; p < m1; p += 4) {
-                if (q == 0 && ((p >> 2) & 7) == 0 && p + kStreamAhead < m1) {      // once per 128-byte line of the leaf arrays
-                    asm volatile("prefetch.global.L2 [%0];" :: "l"(x.crd[2] + p + kStreamAhead));
-                    asm volatile("prefetch.global.L2 [%0];" :: "l"(x.vals + p + kStreamAhead));
+                if (((p >> 2) & 7) == 0) {                        // once per 128-byte line of the leaf arrays
+                    if (q == 0 && p + kStreamAhead < m1) {
+                        asm volatile("prefetch.global.L2 [%0];" :: "l"(x.crd[2] + p + kStreamAhead));
+                        asm volatile("prefetch.global.L2 [%0];" :: "l"(x.vals + p + kStreamAhead));
+                    }
+                    if constexpr (ROUNDS) round_off();
                 }
                 Vec<float> w0 = v0, w1 = v1, w2 = v2, w3 = v3;
                 float4 xw = xn;
@@ -157,7 +163,6 @@ __device__ __forceinline__ void phase1(const Chain<float, 3> &x, const float *__
                 if (p + 3 == fend) leave_fibre();
                 fma4(t, xc.w, v3);
                 if (p + 4 == fend) leave_fibre();
-                if (((p - m0) & (kRound - 4)) == kRound - 4) round_off();
                 v0 = w0; v1 = w1; v2 = w2; v3 = w3; xc = xw;
             }
         }
@@ -247,7 +252,7 @@ struct __align__(16) Smem {
     int32_t j[S::WINDOW], p[S::WINDOW + 1], head_fibre[S::G1];
 };
 
-template <int R2, int R3>
+template <int R2, int R3, bool WEIGHED>
 __global__ void __launch_bounds__(kWarps * 32, 4) chain3_kernel(const __grid_constant__ Args a) {
     using S = Shape<R2, R3>;
     extern __shared__ __align__(16) unsigned char smem[];
@@ -255,7 +260,7 @@ __global__ void __launch_bounds__(kWarps * 32, 4) chain3_kernel(const __grid_con
     Smem<R2, R3> &sm = reinterpret_cast<Smem<R2, R3> *>(smem)[threadIdx.x >> 5];
     walk::Share own;
     Place<3> from;
-    if (a.weight == 0) {
+    if constexpr (!WEIGHED) {
         own = walk::Share(a.x.n[2], a.chunk, kWarps);
     } else {
         __shared__ int32_t block_end;
@@ -294,7 +299,8 @@ __global__ void __launch_bounds__(kWarps * 32, 4) chain3_kernel(const __grid_con
     };
     const int32_t joint = walk::walk_chunk(a.x, own,
         [&](int32_t e) {
-            return a.weight == 0 ? walk::place_of(a.x, e, lane) : from;
+            if constexpr (WEIGHED) return from;
+            else return walk::place_of(a.x, e, lane);
         },
         [](const Place<3> &) {},
         [&](Place<3> &place, int32_t e, int32_t limit) {
@@ -319,7 +325,7 @@ __global__ void __launch_bounds__(kWarps * 32, 4) chain3_kernel(const __grid_con
             if (lane == 0) sm.p[S::WINDOW] = last < limit ? last : limit;
             __syncwarp();
             const int32_t end = sm.p[cnt];
-            phase1<R2, R3>(a.x, a.F2, cnt, lane, sm.t, sm.p, sm.heads, sm.head_fibre);
+            phase1<R2, R3, WEIGHED>(a.x, a.F2, cnt, lane, sm.t, sm.p, sm.heads, sm.head_fibre);
             phase2<R2, R3>(a.F1, cnt, lane, sm.t, sm.j, pairs);
             place.node[1] += cnt;
             return end - e;
@@ -341,14 +347,19 @@ __global__ void __launch_bounds__(kWarps * 32, 4) chain3_kernel(const __grid_con
     }
 }
 
-template <int R2, int R3>
-const_status_t launch_chain3(const Args &a, int64_t n_rows, cudaStream_t stream) {
+template <int R2, int R3, bool WEIGHED>
+const_status_t launch_form(const Args &a, int64_t n_rows, cudaStream_t stream) {
     constexpr size_t dyn = sizeof(Smem<R2, R3>) * kWarps;
     static PerDeviceOnce attr_once;                     // per template instance
-    CB_CUDA(once_per_device(attr_once, [&] { return cudaFuncSetAttribute(chain3_kernel<R2, R3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn); }));
+    CB_CUDA(once_per_device(attr_once, [&] { return cudaFuncSetAttribute(chain3_kernel<R2, R3, WEIGHED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn); }));
     const int64_t warps = ((int64_t)a.x.n[2] + (int64_t)a.weight * a.x.n[1] + a.chunk - 1) / a.chunk;
-    return walk::launch_on_cleared("chain3_kernel", chain3_kernel<R2, R3>, a, dim3((unsigned)((warps + kWarps - 1) / kWarps)), kWarps * 32, dyn,
+    return walk::launch_on_cleared("chain3_kernel", chain3_kernel<R2, R3, WEIGHED>, a, dim3((unsigned)((warps + kWarps - 1) / kWarps)), kWarps * 32, dyn,
                                    a.out, sizeof(float) * R2 * R3 * n_rows, stream);
+}
+
+template <int R2, int R3>
+const_status_t launch_chain3(const Args &a, int64_t n_rows, cudaStream_t stream) {
+    return a.weight ? launch_form<R2, R3, true>(a, n_rows, stream) : launch_form<R2, R3, false>(a, n_rows, stream);
 }
 
 }  // namespace
@@ -359,15 +370,19 @@ const_status_t run_ttmc3_fibres(const const_csf *X, const float *U, const float 
     // From three million leaves on the warps get equal costs instead of equal leaves: a leaf of a short fibre costs several
     // times one of a long fibre, so that with Zipf-sized slices equal leaves took unequal time, and chunks small enough to
     // even that out paid for their searches.  A fibre counts as six leaves (four and eight are worse by 3 to 10 % on most rank
-    // pairs).  Whole waves of parts of at most 8192: larger ones are up to 5 % faster, but longer sums round more (10.5 M, 32 x
-    // 32, relative error 3.5e-7 at 16 384, 2.9e-7 at 8192, 3.2e-7 before).  Leaf chunks of 1536 against this, us (work lists):
-    // 10.5 M, slices Zipf 1.1, 8 x 8: 212 / 161 (152), 16 x 16: 324 / 231 (255), 32 x 32: 537 / 398 (459); 77 M, 16 x 16:
-    // 1102 / 1059 (1140); uniform, 20 M in fibres of 33, 8 x 8: 161 / 142 (176), 32 x 32: 307 / 311 (324); but 2 M in fibres of
-    // 25: 24.4 / 25.7, 300 000: 17.8 / 19.5 (the longer search).
+    // pairs).  Whole waves of parts of at most 8192, 4096 or 2048, as 8, 2 or 1 fibres are consumed side by side: larger ones are
+    // up to 5 % faster, but longer sums round more (21 M in fibres of 3.9, 16 x 32, relative error 2.9e-7 at 8192, 2.3e-7 at
+    // 4096, 2.8e-7 in leaf chunks).  Leaf chunks of 1536 against this, us (work lists):
+    // 10.5 M, slices Zipf 1.1, 8 x 8: 212 / 161 (152), 16 x 16: 324 / 231 (255), 32 x 32: 535 / 406 (453);
+    // 77 M, 16 x 16: 1100 / 1041 (1140); uniform, 20 M in fibres of 33, 8 x 8: 161 / 142 (176), 32 x 32: 307 / 311 (324).
+    // Equal leaves where they are as good: smaller tensors (2 M in fibres of 25: 24.4 / 25.7, 300 000: 17.8 / 19.5, the longer
+    // search), fibres of less than three (6 M in fibres of 2.6, 8 x 16: 110 / 117, 16 x 16: 137 / 144), and slices of more than
+    // 1024 fibres, whose sums would get longer (19 M in fibres of 3, 8 x 16, 4260 a slice: 329 / 328 us, error 1.8e-7 / 2.1e-7).
     constexpr int32_t kWeight = 6, kResident = 16;
-    constexpr int64_t kMostCost = 8192, kWave = 148 * kResident;
-    const int64_t cost = X->nnz + kWeight * X->n[1], parts = (cost + kWave * kMostCost - 1) / (kWave * kMostCost) * kWave;
-    const bool weigh = X->nnz >= 3000000;
+    constexpr int64_t kWave = 148 * kResident;
+    const int64_t cost = X->nnz + kWeight * X->n[1], most = R2 * R3 >= 1024 ? 2048 : R2 * R3 >= 512 ? 4096 : 8192;
+    const int64_t parts = (cost + kWave * most - 1) / (kWave * most) * kWave;
+    const bool weigh = X->nnz >= 3000000 && X->nnz >= 3 * X->n[1] && X->n[1] <= 1024ll * X->n[0];
     const Args a{walk::chain_of<float, 3>(X), U, V, Y,
                  weigh ? (int32_t)((cost + parts - 1) / parts) : walk::chunk_leaves(X->nnz, X->n[0], kResident, 1536, kResident), weigh ? kWeight : 0};
     switch (R2 * 100 + R3) {

@@ -221,6 +221,9 @@ def test_products_are_formed_in_the_order_of_the_schedule(family, ranks, long_fi
     ((1, 3000, 2500), None, None),         # one slice
     ((3000, 5000, 400), 1.1, None),        # slices of all sizes, a hot one over hundreds of warps, fibres of a few leaves
     ((500_000, 40, 50), 0.5, None),        # more slices than a search takes in two steps, most of them of a few leaves
+    ((900, 1050, 3000), None, None),       # slices of 1011 fibres, 3.4 leaves each
+    ((900, 1100, 3000), None, None),       # of 1052: equal leaves again
+    ((1100, 1100, 3000), None, None),      # fibres of 2.8 leaves: equal leaves again
 ])
 def test_parts_of_equal_cost(dims, slice_s, inner):
     """From three million nonzeros on order-3 TTMc cuts the tensor by leaves and fibres together: parts begin inside fibres,
