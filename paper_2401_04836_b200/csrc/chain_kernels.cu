@@ -9,7 +9,8 @@
 // and, for order 4, with one more producer: P[c] += X[i,j,k,l] * W[l,c];  Q[b,c] += V[k,b] * P[c].
 //
 // Every warp owns an equal run of the tensor's leaves and walks it in windows that it stages as flat records
-// (chain_walk.cuh), entirely on its own: no block barrier, no work list, no slice too large or too small.
+// (chain_walk.cuh), on its own: no work list, no slice too large or too small.  The warps of a block meet only where the
+// whole block lies in one slice, to add up their results.
 //   producer   Lane groups (one 128-bit load per lane and factor row) work through equal runs of the window's
 //     records, four row gathers in flight per lane.  Where a record ends a fibre, the group has the finished t.
 //   consumer, MTTKRP   The group multiplies t with the row of B whose coordinate the record carries (requested
@@ -22,8 +23,8 @@
 //
 // What bounds them, and what they measured on a B200 (before: one block or warp per slice from the work lists): the
 // gathers are served by L2 (hit rate 80-90 %, DRAM below 10 %), and the kernels are held by L2 latency and by the
-// instructions per leaf (9-12; order 4: 29), not by a bandwidth.  MTTKRP, 100 M leaves, rank 32: 1.79 -> 1.26 ms (gather
-// ceiling 1.0 ms; 64 registers for 32 warps per SM matter: 72 registers 1.42 ms); TTMc 8 x 32, 8 M leaves in fibres of
+// instructions per leaf (9-12; order 4: 29), not by a bandwidth.  MTTKRP, 100 M leaves, rank 32: 1.79 -> 1.34 ms (gather
+// ceiling 1.0 ms; 64 registers for 32 warps per SM matter: 72 registers cost 13 % more); TTMc 8 x 32, 8 M leaves in fibres of
 // 1.6: 499 -> 284 us; order-4 TTMc, 50 M leaves: 4.57 ms on these pipes, 3.11 ms with the last contraction on the tensor
 // cores -> 2.28 ms here (the factor rows of the consumer copied to shared memory behind the producer -0.4 ms, parked Q
 // laid out free of bank conflicts -0.3 ms, leaf arrays requested one window ahead -0.1 ms; the latter costs more
@@ -38,7 +39,7 @@ namespace {
 
 using namespace walk;
 
-constexpr int kWarps = 4;                             // warps per block; they share nothing
+constexpr int kWarps = 4;                             // warps per block; they meet where a slice covers the block
 constexpr int kUnroll = 4;                            // row gathers in flight per lane
 
 // blocks an SM holds: what the registers are cut for, or the shared memory (warp_bytes per warp) allows
@@ -691,12 +692,13 @@ const_status_t run_ttmc3(const const_csf *X, const float *U, const float *V, int
     // Short fibres go to the record walk, whose cost is per leaf; chain3_kernel pays per fibre, but less per leaf of a long
     // one and less to start.  Measured, walk against chain3_kernel (us): 20 M leaves in fibres of one, 16 x 16: 607 / 886;
     // of two: 405 / 470; of four: 362 / 354; 32 x 32 in fibres of two: 939 / 880; 1 M leaves in fibres of one: 68 / 79, of
-    // two: 46 / 43.  Below a million leaves only where the slices fill a few windows, and not at 32 x 32: 100 000 leaves in
-    // fibres of one, 16 x 16, slices of 1 / 4 / 16 / 64: 106 / 95, 51 / 51, 23 / 27, 17.4 / 18.3; 300 000: 351 / 264,
-    // 143 / 128, 47 / 54, 27 / 30; 32 x 32, 300 000: 612 / 407, 238 / 168, 83 / 69, 49 / 42.
+    // two: 46 / 43.  Below a million leaves only where the slices fill a few windows, with fibres of little more than one and not
+    // at R2 = 32: 100 000 leaves in fibres of one, 16 x 16, slices of 1 / 4 / 16 / 64: 106 / 95, 51 / 51, 23 / 27, 17.4 / 18.3;
+    // 300 000: 351 / 264, 143 / 128, 47 / 54, 27 / 30; 32 x 32, 300 000: 612 / 407, 238 / 168, 83 / 69, 49 / 42; 493 000 in
+    // fibres of 2.3 and slices of 425: 8 x 8 18.6 / 17.3, 8 x 32 29.3 / 25.3, 32 x 16 31.8 / 26.3.
     const double per_fibre = (double)X->nnz / (double)X->n[1], per_slice = (double)X->nnz / (double)X->n[0];
-    const bool wide = R2 * R3 >= 1024, many = X->nnz >= 1000000 || (X->nnz >= 100000 && per_slice >= 16 && !wide);
-    if (!many || per_fibre > (wide ? 1.8 : 2.5)) return run_ttmc3_fibres(X, U, V, R2, R3, Y, n_rows, stream);
+    const bool large = X->nnz >= 1000000, middle = X->nnz >= 100000 && per_slice >= 16 && R2 < 32;
+    if (per_fibre > (large ? R2 * R3 >= 1024 ? 1.8 : 2.5 : middle ? 1.5 : 0.0)) return run_ttmc3_fibres(X, U, V, R2, R3, Y, n_rows, stream);
     return dispatch_ttmc3<float>({chain_of<float, 3>(X), U, V, Y, bytes, R2, R3}, R2, R3, stream);
 }
 
