@@ -14,6 +14,11 @@
  *   - `stream` is a cudaStream_t passed as void* (NULL = the legacy default stream).
  *   - The caller owns COO inputs, dense factors and outputs.  The library owns CSF arrays, work lists
  *     and scratch (stream-ordered allocations on the given stream) until const_destroy.
+ *   - const_execute asks for optional scratch where a faster path can use it: factors padded to the kernels' widths, and
+ *     for the two-contraction network at most 256 MB for T plus 4 bytes per nonzero of U and W.  It comes from a pool of
+ *     the library's own (one per device; from the stream's capture while one is open), is returned to the pool in stream
+ *     order when the call's work is done, and the pool keeps it for later calls.  Without it the call runs on a path that
+ *     needs none.
  *   - Dense operands and outputs are row-major in the index order written in the expression, and their
  *     base addresses are 16-byte aligned (rows are read and written with 128-bit accesses).
  *   - Every function returns a const_status_t; on error no output handle is produced.
@@ -295,7 +300,8 @@ const_status_t const_plan_set_tensor_stage(const_plan_t *plan, int enable);
 const_status_t const_plan_set_generic_executor(const_plan_t *plan, int enable);
 
 /*
- * What the generic executor will do for this plan (Sec. 4.2 loop structure, as compiled): one line per loop and
+ * What the generic executor does for this plan (Sec. 4.2 loop structure, as compiled), whether or not it is the path
+ * const_execute takes (a chain that the fused kernels take has a program all the same): one line per loop and
  * per assignment -- which loop is spread over thread blocks, which CSF operand a loop walks ("walks B level 1"),
  * which operands it looks up ("locates D level 1") or that it runs over a dense range, where a workspace is
  * cleared and how many elements it has, and the private loops of every assignment.  Text protocol as for
