@@ -455,7 +455,9 @@ def measure_config(cb, torch, w, config_id, args, peaks, hbm_peak, peak_kind, ra
             return dict(common, bound="tensor", achieved=ach, peak=peaks["tf32_mma_tflops"], unit="TFLOP/s",
                         peak_source="tcgen05 tf32 microbenchmark of this run")
         per_elem = {"rs_onesweep": 2 * (8 + vbytes), "pack_hist": 4 * len(next(iter(w.sparse.values())).dims) + 8,
-                    "csf_count": 8, "csf_scatter": 8 + 4, "csf_compress": 8 + 4}.get(name)
+                    "csf_count": 8, "csf_scatter": 8 + 4, "csf_compress": 8 + 4,
+                    "split_buckets": 4 * len(next(iter(w.sparse.values())).dims) + 8 + 2 * vbytes,
+                    "split_parts": 2 * (8 + vbytes), "part_sort": 8 + 2 * vbytes + 4}.get(name)
         if per_elem is None:
             return None
         # launches alternate over the sparse operands; bytes per launch use the mean nonzero count

@@ -321,16 +321,18 @@ void const_destroy(void *handle);
 const char *const_status_string(const_status_t status);
 
 /*
- * Test hook for the bounded device-side waits (the look-back of the radix sort, the mbarrier wait of the
- * tensor-core stage).  what = 0: number of polls after which a wait gives up (0 restores the defaults);
+ * Test hook for the bounded device-side waits (the look-back of the radix sort, the chunk wait of the splitter sort, the mbarrier
+ * wait of the tensor-core stage).  what = 0: number of polls after which a wait gives up (0 restores the defaults);
  * what = 1: value != 0 withholds the signal those waits wait for -- sort tiles do not publish their
- * counts, the tensor-core stage issues and commits nothing -- so that every such wait runs out, the
+ * counts or chunks, the tensor-core stage issues and commits nothing -- so that every such wait runs out, the
  * kernel records CONST_ERR_TIMEOUT, skips its stores and returns normally;
  * what = 2: which of the tile shapes a launcher keeps for measurement is launched (0: the default; the
  * two-contraction network has variants 1..5, every one of them computes the same result, and 6, its matrix form alone: the
  * result stays zero where that form hands the work on);
  * what = 3: value != 0 makes every request of const_execute for optional scratch (padded factors, the intermediate of the
- * two-contraction network's matrix form) fail for want of memory, so that the path that needs none runs.  Process-wide; not
+ * two-contraction network's matrix form), and of const_csf_build for the splitter sort's, fail for want of memory, so that the
+ * path that needs none (less) runs;
+ * what = 4: how const_csf_build sorts, whatever the size (0: chosen by size; 1: radix passes; 2: splitters).  Process-wide; not
  * for production use.  CONST_ERR_INVALID_ARG for an unknown `what` or a value outside [0, 2^31).
  */
 const_status_t const_debug_set(int what, int64_t value);

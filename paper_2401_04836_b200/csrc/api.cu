@@ -47,12 +47,12 @@ bool fused_chain(const PlanDesc &d) {
 
 bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
-std::atomic<int> g_spin_limit{0}, g_withhold{0}, g_variant{0}, g_no_scratch{0};
+std::atomic<int> g_spin_limit{0}, g_withhold{0}, g_variant{0}, g_no_scratch{0}, g_build_path{0};
 
 }  // namespace
 
 namespace cb {
-DebugKnobs debug_knobs() { return DebugKnobs{g_spin_limit.load(), g_withhold.load(), g_variant.load(), g_no_scratch.load()}; }
+DebugKnobs debug_knobs() { return DebugKnobs{g_spin_limit.load(), g_withhold.load(), g_variant.load(), g_no_scratch.load(), g_build_path.load()}; }
 }  // namespace cb
 
 extern "C" {
@@ -445,6 +445,7 @@ const_status_t const_debug_set(int what, int64_t value) {
         case 1: g_withhold.store(value != 0); return CONST_OK;
         case 2: g_variant.store((int)value); return CONST_OK;
         case 3: g_no_scratch.store(value != 0); return CONST_OK;
+        case 4: g_build_path.store((int)value); return CONST_OK;
     }
     return CONST_ERR_INVALID_ARG;
 }

@@ -1,5 +1,5 @@
-// GPU CSF builder (Sec. 2.1, CSF representation): pack -> LSD radix sort -> per-level compression,
-// and, on demand, the per-slice load-balancing lists used by the kernels with the tensor-core stage.
+// GPU CSF builder (Sec. 2.1, CSF representation): pack -> LSD radix sort -> per-level compression (large tensors: the splitter
+// sort of csf_split.cu), and, on demand, the per-slice load-balancing lists used by the kernels with the tensor-core stage.
 //
 // Layout decisions
 //   * The permuted coordinate tuple is packed into one 64-bit key, root level in the top bits, so a
@@ -16,68 +16,10 @@
 #include <cstring>
 #include <new>
 
-#include "common.cuh"
+#include "csf_build.cuh"
 
 namespace cb {
 namespace {
-
-// ------------------------------------------------------------------------------------------------
-// pack
-// ------------------------------------------------------------------------------------------------
-struct PackArgs {
-    const int32_t *c[kMaxOrder];   // coordinates of the mode stored at level l
-    int64_t dim[kMaxOrder];
-    int shift[kMaxOrder];
-    int order;
-};
-
-enum DevErr : int32_t { kErrNone = 0 };
-
-__device__ __forceinline__ void report(int32_t *status, int32_t code) { atomicCAS(status, 0, code); }
-
-constexpr int kRsMaxBits = 9;                     // widest digit of a radix pass
-constexpr int kRsMaxBins = 1 << kRsMaxBits;
-constexpr int kMaxPasses = 8;
-
-// Digits of the radix passes.  A pass sorts on `bits[p]` key bits starting at `shift[p]`; the widths
-// are 8 or 9 bits (the width the pass kernel is instantiated for), chosen so that the key is covered
-// in as few passes as possible.
-struct DigitPlan { int shift[kMaxPasses]; int bits[kMaxPasses]; int passes; };
-
-// True in the block that is the last of its grid to arrive (`arrived` starts at zero); what the other blocks wrote before
-// is visible to it.
-__device__ __forceinline__ bool last_block(uint32_t *arrived) {
-    __shared__ bool last;
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) last = atomicAdd(arrived, 1u) == gridDim.x - 1;
-    __syncthreads();
-    if (last) __threadfence();
-    return last;
-}
-
-// Exclusive scan of one number per thread over a block of 256; the block's total in `total`.
-__device__ __forceinline__ uint32_t block_scan(uint32_t v, uint32_t &total) {
-    __shared__ uint32_t sums[8];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint32_t inc = v;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-        const uint32_t t = __shfl_up_sync(0xffffffffu, inc, off);
-        if (lane >= off) inc += t;
-    }
-    __syncthreads();                                  // the sums of a scan before are used up
-    if (lane == 31) sums[warp] = inc;
-    __syncthreads();
-    uint32_t before = 0;
-    total = 0;
-#pragma unroll
-    for (int w = 0; w < 8; ++w) {
-        if (w < warp) before += sums[w];
-        total += sums[w];
-    }
-    return before + inc - v;
-}
 
 // Pack the permuted coordinates of every nonzero into its 64-bit sort key (range-checked) and, in the
 // same read, count the digits of every radix pass.  Per-block counts live in shared memory and are
@@ -409,7 +351,6 @@ __device__ __forceinline__ void prefetch_tile_ahead(const uint64_t *__restrict__
         asm volatile("prefetch.global.L2 [%0];" :: "l"(reinterpret_cast<const char *>(keys + first) + threadIdx.x * 128));
 }
 
-struct LevelShifts { int shift[kMaxOrder]; int order; };
 
 // The 256 consecutive keys of a warp, two neighbours per lane and step (16-byte loads, all requested before the first is
 // used), and the key in front of them.
@@ -574,11 +515,6 @@ inline void launch_csf_scan(uint32_t *block_counts, int64_t nblocks, uint32_t *t
 // numbers to allocate behind the per-block counts for the chunk sums of the scan
 inline int64_t scan_partials_room(int64_t nblocks) { return kCpLevels * ((nblocks + kScanChunk - 1) / kScanChunk + 1); }
 
-struct CsfArrays {
-    int32_t *pos[kMaxOrder];
-    int32_t *crd[kMaxOrder];
-    int bits[kMaxOrder];
-};
 
 // ORDER is a template parameter so that the per-level arrays are indexed by constants and stay in registers.  The thread
 // that holds the last element closes the pos arrays; slice_ptr (may be null) receives the first leaf of every slice.
@@ -878,8 +814,8 @@ struct Scratch {            // stream-ordered temporaries of one build
         if (e == cudaSuccess) ptrs[n++] = *p;
         return e;
     }
-    void forget(void *p) {
-        for (int i = 0; i < n; ++i) if (ptrs[i] == p) ptrs[i] = nullptr;
+    void release(void *p) {                          // before the others, in the order of the stream
+        for (int i = 0; i < n; ++i) if (ptrs[i] == p) { ptrs[i] = nullptr; cudaFreeAsync(p, stream); }
     }
     ~Scratch() {
         for (int i = 0; i < n; ++i) if (ptrs[i]) cudaFreeAsync(ptrs[i], stream);
@@ -966,7 +902,6 @@ const_status_t sort_and_count(uint64_t *&keys, uint64_t *&keys_alt, const void *
     return CONST_OK;
 }
 
-struct KeyLayout { int bits[kMaxOrder]; int shift[kMaxOrder]; int total_bits; DigitPlan digits; };
 
 // Fewest passes with 8- or 9-bit digits: every pass is 8 bits wide unless 9-bit passes are needed to
 // cover the key in that number of passes (43 bits -> 9 9 9 8 8).  A digit may reach past the top of
@@ -1208,17 +1143,65 @@ const_status_t csf_build_impl(int order, const int64_t *dims, int64_t nnz, const
     const_status_t rc = CONST_OK;
     {
         Scratch tmp(stream);
-        uint64_t *keys = nullptr, *keys_alt = nullptr;
-        void *vals_sorted = nullptr;
-        uint32_t *block_counts = nullptr;
-        SortBufs sb{nullptr, nullptr, nullptr, nullptr};
         const int64_t cp_blocks = (nnz + kCpTile - 1) / kCpTile;
         const int64_t ntiles = (nnz + kRsTile - 1) / kRsTile;
         constexpr size_t kHistBytes = sizeof(uint32_t) * kMaxPasses * kRsMaxBins;
         constexpr size_t kSmallBytes = kHistBytes + 256;
-        auto body = [&]() -> const_status_t {
+        auto room = [](size_t bytes) { return (bytes + 255) / 256 * 256; };
+        const PackArgs pa = pack_args(order, dims, mode_order, coords_dev, kl);
+        int32_t *leaf_crd = nullptr;
+
+        // pos and crd of every level above the leaves, pos of the leaves and slice_ptr, behind one another in one allocation,
+        // once the level sizes are known
+        CsfArrays arr;
+        auto size_arrays = [&](const uint32_t *totals) -> const_status_t {
+            for (int l = 0; l < order - 1; ++l) csf->n[l] = totals[l];
+            csf->n[order - 1] = nnz;
+            if (item_capacity(csf) > 0x7fffffffll) return CONST_ERR_UNSUPPORTED;      // more work items than the lists can number
+            for (int l = 0; l < kMaxOrder; ++l) { arr.pos[l] = arr.crd[l] = nullptr; arr.bits[l] = kl.bits[l]; }
+            size_t at[2 * kMaxOrder + 1] = {}, bytes = 0;
+            auto put = [&](int64_t n) { const size_t o = bytes; bytes += room(sizeof(int32_t) * (size_t)n); return o; };
+            for (int l = 0; l < order; ++l) {
+                at[2 * l] = put((l == 0 ? 1 : csf->n[l - 1]) + 1);
+                if (l + 1 < order) at[2 * l + 1] = put(csf->n[l] + 4);
+            }
+            at[2 * order] = put(csf->n[0] + 1);
+            CB_CUDA(pool_alloc((void **)&csf->arena, bytes, stream));
+            for (int l = 0; l < order; ++l) {
+                arr.pos[l] = csf->pos[l] = reinterpret_cast<int32_t *>(csf->arena + at[2 * l]);
+                arr.crd[l] = csf->crd[l] = l + 1 < order ? reinterpret_cast<int32_t *>(csf->arena + at[2 * l + 1]) : leaf_crd;
+            }
+            csf->slice_ptr = reinterpret_cast<int32_t *>(csf->arena + at[2 * order]);
+            return CONST_OK;
+        };
+
+        // large tensors: splitters; `done` stays false where that sort gave up or found no memory
+        bool done = false;
+        auto by_splitters = [&]() -> const_status_t {
+            unsigned char *arena = nullptr;
+            if (debug_knobs().no_scratch || tmp.alloc((void **)&arena, split_bytes(nnz, dtype)) != cudaSuccess) {
+                cudaGetLastError();
+                return CONST_OK;
+            }
+            SplitSort sort;
+            const_status_t s = split_sort(pa, kl, nnz, vals_dev, dtype, csf->vals, leaf_crd, arena, stream, &sort);
+            if (s != CONST_OK) return s;
+            uint32_t h_small[18] = {0};          // totals at [0..3), parts at [3], status at [16], gave up at [17]
+            CB_CUDA(cudaMemcpyAsync(h_small, sort.result, sizeof(h_small), cudaMemcpyDeviceToHost, stream));
+            CB_CUDA(wait_stream(stream));
+            if (h_small[16] != 0) return (const_status_t)h_small[16];
+            if (h_small[17] != 0) {
+                tmp.release(arena);
+                return CONST_OK;
+            }
+            s = size_arrays(h_small);
+            if (s != CONST_OK) return s;
+            done = true;
+            return split_scatter(sort, arr, csf->slice_ptr, h_small[3], stream);
+        };
+
+        auto by_radix = [&]() -> const_status_t {
             // One allocation for the temporaries: small | tile states (cleared together) | block counts | keys | keys | payload
-            auto room = [](size_t bytes) { return (bytes + 255) / 256 * 256; };
             const size_t tiles_bytes = room(sizeof(unsigned long long) * std::max<int64_t>(ntiles, 1) * kRsMaxBins);
             const size_t counts_bytes = room(sizeof(uint32_t) * (kCpLevels * std::max<int64_t>(cp_blocks, 1) + scan_partials_room(cp_blocks)));
             const size_t keys_bytes = room(sizeof(uint64_t) * nnz);
@@ -1226,14 +1209,15 @@ const_status_t csf_build_impl(int order, const int64_t *dims, int64_t nnz, const
             const size_t vals_bytes = passes > 1 ? room(vsize * (nnz + 4)) : 0;
             unsigned char *arena = nullptr;
             CB_CUDA(tmp.alloc((void **)&arena, room(kSmallBytes) + tiles_bytes + counts_bytes + 2 * keys_bytes + vals_bytes));
-            CB_CUDA(pool_alloc(&csf->vals, vsize * (nnz + 4), stream));         // where the last pass leaves the payload
             unsigned char *small = arena;                                       // hist | counters | totals | status
+            SortBufs sb{nullptr, nullptr, nullptr, nullptr};
             sb.tile_status = reinterpret_cast<unsigned long long *>(arena + room(kSmallBytes));
-            block_counts = reinterpret_cast<uint32_t *>(arena + room(kSmallBytes) + tiles_bytes);
-            keys = reinterpret_cast<uint64_t *>(arena + room(kSmallBytes) + tiles_bytes + counts_bytes);
-            keys_alt = reinterpret_cast<uint64_t *>(arena + room(kSmallBytes) + tiles_bytes + counts_bytes + keys_bytes);
+            uint32_t *block_counts = reinterpret_cast<uint32_t *>(arena + room(kSmallBytes) + tiles_bytes);
+            uint64_t *keys = reinterpret_cast<uint64_t *>(arena + room(kSmallBytes) + tiles_bytes + counts_bytes);
+            uint64_t *keys_alt = reinterpret_cast<uint64_t *>(arena + room(kSmallBytes) + tiles_bytes + counts_bytes + keys_bytes);
             void *spare = passes > 1 ? (void *)(arena + room(kSmallBytes) + tiles_bytes + counts_bytes + 2 * keys_bytes) : csf->vals;
             void *vals = passes % 2 == 1 || passes == 0 ? csf->vals : spare, *vals_alt = passes % 2 == 1 || passes == 0 ? spare : csf->vals;
+            void *vals_sorted = nullptr;                                        // csf->vals: where the last pass leaves the payload
             CB_CUDA(cudaMemsetAsync(small, 0, room(kSmallBytes) + tiles_bytes, stream));
             sb.hist = reinterpret_cast<uint32_t *>(small);
             sb.counters = reinterpret_cast<uint32_t *>(small + kHistBytes);
@@ -1244,7 +1228,6 @@ const_status_t csf_build_impl(int order, const int64_t *dims, int64_t nnz, const
             ls.order = order;
             for (int l = 0; l < kMaxOrder; ++l) ls.shift[l] = kl.shift[l];
             if (nnz > 0) {
-                PackArgs pa = pack_args(order, dims, mode_order, coords_dev, kl);
                 CB_LAUNCH("pack_hist", stream, launch_pack_hist(pa, nnz, kl.digits, keys, sb.hist, status, sb.arrived, stream));
                 const_status_t s = sort_and_count(keys, keys_alt, vals_dev, vals, vals_alt, vals_sorted, nnz, kl.digits,
                                                   dtype, sb, ls, block_counts, totals, status, stream);
@@ -1254,26 +1237,8 @@ const_status_t csf_build_impl(int order, const int64_t *dims, int64_t nnz, const
             CB_CUDA(cudaMemcpyAsync(h_small, totals, sizeof(uint32_t) * 17, cudaMemcpyDeviceToHost, stream));
             CB_CUDA(wait_stream(stream));
             if (h_small[16] != 0) return (const_status_t)h_small[16];
-            for (int l = 0; l < order - 1; ++l) csf->n[l] = h_small[l];
-            csf->n[order - 1] = nnz;
-            if (item_capacity(csf) > 0x7fffffffll) return CONST_ERR_UNSUPPORTED;      // more work items than the lists can number
-
-            CsfArrays arr;
-            for (int l = 0; l < kMaxOrder; ++l) { arr.pos[l] = arr.crd[l] = nullptr; arr.bits[l] = kl.bits[l]; }
-            // pos and crd of every level and slice_ptr behind one another in one allocation
-            size_t at[2 * kMaxOrder + 1], bytes = 0;
-            auto put = [&](int64_t n) { const size_t o = bytes; bytes += (sizeof(int32_t) * (size_t)n + 255) / 256 * 256; return o; };
-            for (int l = 0; l < order; ++l) {
-                at[2 * l] = put((l == 0 ? 1 : csf->n[l - 1]) + 1);
-                at[2 * l + 1] = put(csf->n[l] + 4);
-            }
-            at[2 * order] = put(csf->n[0] + 1);
-            CB_CUDA(pool_alloc((void **)&csf->arena, bytes, stream));
-            for (int l = 0; l < order; ++l) {
-                arr.pos[l] = csf->pos[l] = reinterpret_cast<int32_t *>(csf->arena + at[2 * l]);
-                arr.crd[l] = csf->crd[l] = reinterpret_cast<int32_t *>(csf->arena + at[2 * l + 1]);
-            }
-            csf->slice_ptr = reinterpret_cast<int32_t *>(csf->arena + at[2 * order]);
+            const const_status_t s = size_arrays(h_small);
+            if (s != CONST_OK) return s;
             if (nnz > 0) {
                 CB_LAUNCH("csf_scatter", stream, launch_csf_scatter(order, cp_blocks, keys, nnz, ls, block_counts, arr, csf->slice_ptr, stream));
             } else {
@@ -1285,6 +1250,18 @@ const_status_t csf_build_impl(int order, const int64_t *dims, int64_t nnz, const
             }
             CB_CUDA(cudaGetLastError());
             return CONST_OK;
+        };
+
+        auto body = [&]() -> const_status_t {
+            // values and leaf coordinates, whose number is known, in one allocation
+            const size_t vals_room = room(vsize * (nnz + 4));
+            CB_CUDA(pool_alloc(&csf->vals, vals_room + room(sizeof(int32_t) * (nnz + 4)), stream));
+            leaf_crd = reinterpret_cast<int32_t *>(static_cast<unsigned char *>(csf->vals) + vals_room);
+            if (split_covers(nnz, kl)) {
+                const const_status_t s = by_splitters();
+                if (s != CONST_OK || done) return s;
+            }
+            return by_radix();
         };
         rc = body();
     }

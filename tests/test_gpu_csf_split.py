@@ -1,0 +1,144 @@
+"""The CSF builder's splitter sort against the CSF oracle and against its radix sort, array for array."""
+import itertools
+
+import numpy as np
+import pytest
+import torch
+
+import paper_2401_04836_b200 as cb
+from workloads import generators as gen
+from tests.gpu_util import assert_csf_equal, build_csf, csf_to_host, to_dev
+
+pytestmark = pytest.mark.gpu
+
+RADIX, SPLIT = 1, 2
+
+
+@pytest.fixture(autouse=True)
+def default_path():
+    yield
+    for what in range(5):
+        cb.const_debug_set(what, 0)
+
+
+def built(op, order, path):
+    cb.const_debug_set(4, path)
+    h = build_csf(op, order)
+    return (*csf_to_host(h), cb.const_csf_work_lists(h)[0].cpu().numpy())
+
+
+def assert_same(op, order):
+    a, b = built(op, order, RADIX), built(op, order, SPLIT)
+    for x, y in zip(a[0] + a[1] + [a[3]], b[0] + b[1] + [b[3]]):
+        np.testing.assert_array_equal(x, y)
+    assert a[2].tobytes() == b[2].tobytes()
+
+
+def operand(key, dims, dtype=np.float32, shuffle=True):
+    rng = np.random.default_rng(key.size)
+    key = rng.permutation(key) if shuffle else key
+    coords = []
+    for d in reversed(dims):
+        coords.append((key % d).astype(np.int32))
+        key = key // d
+    return gen.SparseOperand(coords[::-1], rng.standard_normal(coords[0].size).astype(dtype), dims)
+
+
+# one part, the edges of a tile (2048) and of a chunk (4096), several parts and buckets; every order, key widths up to 64 bits
+@pytest.mark.parametrize("nnz", [1, 2, 1365, 1366, 2048, 2049, 4095, 4097, 30_011, 200_003])
+def test_against_the_oracle(nnz):
+    rng = np.random.default_rng(nnz)
+    for dims, dtype in (((1700, 900), np.float32), ((90, 80, 170), np.float64), ((65536, 65536, 65536, 65536), np.float32)):
+        op = gen._uniform_tensor(dims, nnz, rng, "pm1", dtype)
+        for order in (tuple(range(len(dims))), tuple(reversed(range(len(dims))))):
+            cb.const_debug_set(4, SPLIT)
+            assert_csf_equal(build_csf(op, order), op, order)
+
+
+@pytest.mark.parametrize("dims,nnz", [((1, 1, 900_000), 400_000), ((900_000, 1, 1), 400_000), ((3, 700, 701), 1_300_000),
+                                      ((5003, 3001, 4001), 1_300_001), ((2003, 1501, 701, 301), 500_003)])
+def test_every_mode_order_against_the_radix_sort(dims, nnz):
+    rng = np.random.default_rng(nnz)
+    cells = int(np.prod(dims, dtype=np.int64))
+    key = rng.permutation(cells)[:nnz] if cells < 4 * nnz else np.unique(rng.integers(0, cells, nnz))
+    op = operand(key, dims, np.float64 if len(dims) == 4 else np.float32)
+    for order in itertools.islice(itertools.permutations(range(len(dims))), 0, None, 5 if len(dims) == 4 else 2):
+        assert_same(op, order)
+
+
+@pytest.mark.parametrize("what", ["sorted", "reversed", "banded", "clusters", "one slice"])
+def test_distributions(what):
+    """Sorted input (all lanes one way), keys crowded into a part of their range (bins of bins, then the network), a giant slice."""
+    rng = np.random.default_rng(7)
+    dims = (65536, 65536, 65536)
+    if what in ("sorted", "reversed"):
+        key = np.sort(np.unique(rng.integers(0, 2 ** 48, 600_000)))[:: 1 if what == "sorted" else -1]
+    elif what == "banded":
+        i = np.repeat(np.arange(20_000, dtype=np.int64), 30)
+        j = i + np.tile(np.arange(30), 20_000)
+        key = np.unique((i * 65536 + j) * 65536 + (7 * i + j) % 65536)
+    elif what == "clusters":
+        key = np.unique(np.exp2(rng.random(700_000) * 47.9).astype(np.int64))
+    else:
+        key = (41 << 32) + rng.permutation(2 ** 24)[:600_000].astype(np.int64)
+    op = operand(key, dims, shuffle=what not in ("sorted", "reversed"))
+    assert_same(op, (0, 1, 2))
+    assert_same(op, (2, 0, 1))
+
+
+def test_errors_and_the_way_back_to_the_radix_sort():
+    rng = np.random.default_rng(3)
+    op = gen._uniform_tensor((300, 1000, 777), 500_003, rng, "pm1", np.float32)
+    cb.const_debug_set(4, SPLIT)
+
+    def status(coords):
+        with pytest.raises(cb.ConstError) as e:
+            cb.const_csf_build([to_dev(c) for c in coords], to_dev(op.vals), op.dims, (0, 1, 2))
+        return e.value.status
+
+    twice = [c.copy() for c in op.coords]
+    for c in twice:
+        c[400_000] = c[5]
+    assert status(twice) == 4
+    assert status([np.zeros_like(c) for c in op.coords]) == 4        # one part outgrows its room: sorted again by digits
+    for bad in (-1, 1000, 2 ** 31 - 1):
+        far = [c.copy() for c in op.coords]
+        far[1][123_456] = bad
+        assert status(far) == 5
+    cb.const_debug_set(3, 1)                                         # no memory for it
+    cb.const_profile_enable(True)
+    h = build_csf(op, (0, 1, 2))
+    names = cb.const_profile_read()
+    cb.const_profile_enable(False)
+    assert "rs_onesweep" in names and "part_sort" not in names
+    assert_csf_equal(h, op, (0, 1, 2))
+
+
+def test_chunk_wait_times_out_and_recovers():
+    rng = np.random.default_rng(4)
+    op = gen._uniform_tensor((300, 1000, 777), 300_007, rng, "pm1", np.float32)
+    cb.const_debug_set(4, SPLIT)
+    cb.const_debug_set(0, 200)
+    cb.const_debug_set(1, 1)
+    with pytest.raises(cb.ConstError) as e:
+        build_csf(op, (0, 1, 2))
+    assert e.value.status == 8
+    cb.const_debug_set(1, 0)
+    cb.const_debug_set(0, 0)
+    assert_csf_equal(build_csf(op, (0, 1, 2)), op, (0, 1, 2))
+
+
+def test_which_sort_runs():
+    """The line: 400 000 nonzeros, and 1.2 M nonzeros times radix passes beyond two."""
+    for dims, nnz, split in (((2000, 3000, 4000), 590_000, False), ((2000, 3000, 4000), 610_000, True), ((512, 512, 512), 1_190_000, False),
+                             ((512, 512, 512), 1_210_000, True), ((20000, 20000, 20000, 20000), 390_000, False),
+                             ((20000, 20000, 20000, 20000), 410_000, True)):
+        coords = [torch.randint(0, d, (nnz,), device="cuda", dtype=torch.int32) for d in dims]
+        cb.const_profile_enable(True)
+        try:
+            cb.const_csf_build(coords, torch.ones(nnz, device="cuda"), dims, tuple(range(len(dims))))
+        except cb.ConstError as e:                                   # drawn with repetition: some occur twice
+            assert e.status == 4
+        names = cb.const_profile_read()
+        cb.const_profile_enable(False)
+        assert ("part_sort" in names) == split and ("rs_onesweep" in names) != split
