@@ -384,7 +384,7 @@ const_status_t run_ttmc3_fibres(const const_csf *X, const float *U, const float 
     const int64_t parts = (cost + kWave * most - 1) / (kWave * most) * kWave;
     const bool weigh = X->nnz >= 3000000 && X->nnz >= 3 * X->n[1] && X->n[1] <= 1024ll * X->n[0];
     const Args a{walk::chain_of<float, 3>(X), U, V, Y,
-                 weigh ? (int32_t)((cost + parts - 1) / parts) : walk::chunk_leaves(X->nnz, X->n[0], kResident, 1536, kResident), weigh ? kWeight : 0};
+                 weigh ? (int32_t)((cost + parts - 1) / parts) : walk::chunk_leaves(X->nnz, X->n[0], 1536, kResident), weigh ? kWeight : 0};
     switch (R2 * 100 + R3) {
         case 808: return launch_chain3<8, 8>(a, n_rows, s);
         case 816: return launch_chain3<8, 16>(a, n_rows, s);

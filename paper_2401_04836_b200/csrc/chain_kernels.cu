@@ -498,15 +498,16 @@ unsigned chunk_blocks(int64_t nnz, int32_t chunk) {
 }
 
 template <typename T, int ORDER, int RP>
-const_status_t launch_mttkrp(MttkrpArgs<T, ORDER> a, int resident, int tiles, cudaStream_t stream) {
-    a.chunk = chunk_leaves(a.x.n[ORDER - 1], a.x.n[0], resident, 4096, MttkrpShape<T, ORDER, RP>::FIT);
+const_status_t launch_mttkrp(MttkrpArgs<T, ORDER> a, int tiles, cudaStream_t stream) {
+    a.chunk = chunk_leaves(a.x.n[ORDER - 1], a.x.n[0], 4096, MttkrpShape<T, ORDER, RP>::FIT);
     const dim3 grid(chunk_blocks(a.x.n[ORDER - 1], a.chunk), (unsigned)tiles);
     return launch_on_cleared("chain3_kernel", mttkrp_kernel<T, ORDER, RP>, a, grid, kWarps * 32, 0, a.out, a.out_bytes, stream);
 }
 
 template <typename T, int R2, int R3>
 const_status_t launch_ttmc3(Ttmc3Args<T> a, cudaStream_t stream) {
-    a.chunk = chunk_leaves(a.x.n[2], a.x.n[0], 20, 3072, Ttmc3Shape<T, R2, R3>::FIT);
+    constexpr int fit = Ttmc3Shape<T, R2, R3>::FIT;
+    a.chunk = chunk_leaves(a.x.n[2], a.x.n[0], 3072, fit, (20 + fit - 1) / fit);
     constexpr size_t dyn = sizeof(typename Ttmc3Shape<T, R2, R3>::Smem) * kWarps;
     static PerDeviceOnce attr_once;                     // per template instance
     CB_CUDA(once_per_device(attr_once, [&] { return cudaFuncSetAttribute(ttmc3_kernel<T, R2, R3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn); }));
@@ -532,19 +533,19 @@ const_status_t dispatch_ttmc3(const Ttmc3Args<T> &a, int r2, int r3, cudaStream_
 }
 
 template <typename T, int ORDER>
-const_status_t dispatch_mttkrp(const MttkrpArgs<T, ORDER> &a, int resident, int rp, int tiles, cudaStream_t s) {
+const_status_t dispatch_mttkrp(const MttkrpArgs<T, ORDER> &a, int rp, int tiles, cudaStream_t s) {
     switch (rp) {
-        case 4: return launch_mttkrp<T, ORDER, 4>(a, resident, tiles, s);
-        case 8: return launch_mttkrp<T, ORDER, 8>(a, resident, tiles, s);
-        case 16: return launch_mttkrp<T, ORDER, 16>(a, resident, tiles, s);
-        case 32: return launch_mttkrp<T, ORDER, 32>(a, resident, tiles, s);
+        case 4: return launch_mttkrp<T, ORDER, 4>(a, tiles, s);
+        case 8: return launch_mttkrp<T, ORDER, 8>(a, tiles, s);
+        case 16: return launch_mttkrp<T, ORDER, 16>(a, tiles, s);
+        case 32: return launch_mttkrp<T, ORDER, 32>(a, tiles, s);
     }
     return CONST_ERR_UNSUPPORTED;
 }
 
 template <typename T>
 const_status_t launch_ttmc4(Ttmc4Args<T> a, cudaStream_t stream) {
-    a.chunk = chunk_leaves(a.x.n[3], a.x.n[0], 12, 4096, Ttmc4Shape<T>::FIT);
+    a.chunk = chunk_leaves(a.x.n[3], a.x.n[0], 4096, Ttmc4Shape<T>::FIT);
     constexpr size_t dyn = sizeof(typename Ttmc4Shape<T>::Smem) * kWarps;
     static PerDeviceOnce attr_once;                     // per template instance
     CB_CUDA(once_per_device(attr_once, [&] { return cudaFuncSetAttribute(ttmc4_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn); }));
@@ -651,9 +652,9 @@ const_status_t run_any(const const_csf *X, bool mttkrp, const void *const *facto
     const_status_t rc;
     const int rp = width[0] > 32 ? 32 : width[0];
     if (mttkrp && X->order == 3)
-        rc = dispatch_mttkrp<T, 3>({chain_of<T, 3>(X), {F[0], F[1]}, out, bytes, width[0], ranks[0]}, 24, rp, width[0] / rp, stream);
+        rc = dispatch_mttkrp<T, 3>({chain_of<T, 3>(X), {F[0], F[1]}, out, bytes, width[0], ranks[0]}, rp, width[0] / rp, stream);
     else if (mttkrp)
-        rc = dispatch_mttkrp<T, 4>({chain_of<T, 4>(X), {F[0], F[1], F[2]}, out, bytes, width[0], ranks[0]}, 24, rp, width[0] / rp, stream);
+        rc = dispatch_mttkrp<T, 4>({chain_of<T, 4>(X), {F[0], F[1], F[2]}, out, bytes, width[0], ranks[0]}, rp, width[0] / rp, stream);
     else if (X->order == 3)
         rc = dispatch_ttmc3<T>({chain_of<T, 3>(X), F[0], F[1], out, bytes, ranks[0], ranks[1]}, width[0], width[1], stream);
     else
@@ -706,7 +707,7 @@ const_status_t run_mttkrp3(const const_csf *X, const float *B, const float *C, i
                            int32_t *, cudaStream_t stream) {
     const size_t bytes = sizeof(float) * R * n_rows;
     if (X->nnz == 0) return clear_result(A, bytes, stream) == cudaSuccess ? CONST_OK : CONST_ERR_CUDA;
-    return dispatch_mttkrp<float, 3>({chain_of<float, 3>(X), {B, C}, A, bytes, R, R}, 32, R, 1, stream);
+    return dispatch_mttkrp<float, 3>({chain_of<float, 3>(X), {B, C}, A, bytes, R, R}, R, 1, stream);
 }
 
 const_status_t run_ttmc4(const const_csf *X, const float *U, const float *V, const float *W, int rank, float *Y,

@@ -428,16 +428,16 @@ inline Chain<T, ORDER> chain_of(const const_csf *X) {
     return x;
 }
 
-// Leaves per warp: as many whole waves of `resident` warps per SM as keep a chunk below `most` leaves (finding a place
+// Leaves per warp: as many whole waves of the `fit` warps that an SM holds as keep a chunk below `most` leaves (finding a place
 // and handing over a slice part are paid once per chunk, a wave that is not full leaves SMs idle), in multiples of 64.
-// A tensor that gives no warp 64 leaves is dealt out to the `fit` warps that an SM holds: windows end with their slice, so
+// A tensor that gives no warp 64 leaves is dealt out to one wave as it is: windows end with their slice, so
 // a warp with many short slices goes through as many windows one after the other (TTMc 8 x 8, 3000 leaves in slices of
 // one: 103 us at 64 leaves a warp, 14.5 here; 30 000 in slices of four: 62 and 25), and more warps than fit start late
 // (the latter with twice as many: 29).  But in chunks of half a slice on average where slices are longer than that: more
 // parts of a slice mean more atomic additions and more rounding, and gain nothing (30 000 in slices of 64: 15.0 us, in
 // chunks of 13 leaves 15.9, of 64 18.4; 20 000 in slices of 100: relative error 7.5e-8, in chunks of 9 leaves 8.3e-8).
-inline int32_t chunk_leaves(int64_t nnz, int64_t slices, int resident, int64_t most, int fit) {
-    const int64_t wave = 148 * (int64_t)resident, waves = (nnz + wave * most - 1) / (wave * most);
+inline int32_t chunk_leaves(int64_t nnz, int64_t slices, int64_t most, int fit, int64_t least_waves = 1) {
+    const int64_t wave = 148 * (int64_t)fit, waves = std::max(least_waves, (nnz + wave * most - 1) / (wave * most));
     const int64_t c = (nnz + wave * waves - 1) / (wave * waves);
     if (c < 64) return (int32_t)std::min<int64_t>(std::max((nnz + 148 * fit - 1) / (148 * fit), nnz / (2 * slices)), 64);
     return (int32_t)((c + 63) / 64 * 64);
