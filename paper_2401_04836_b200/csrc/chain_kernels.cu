@@ -110,7 +110,7 @@ struct MttkrpArgs {
     T *out;
     size_t out_bytes;
     int32_t stride, R;
-    int32_t chunk;                                    // leaves per warp (set by the launch)
+    int32_t chunk, weight;                            // cost per warp, and of a slice beyond its leaves (set by the launch)
 };
 
 template <typename T, int ORDER, int RP>
@@ -118,13 +118,13 @@ __global__ void __launch_bounds__(kWarps * 32, MttkrpShape<T, ORDER, RP>::BLOCKS
     using S = MttkrpShape<T, ORDER, RP>;
     constexpr int N = S::N;
     __shared__ Stage<T, ORDER, S::W> stages[kWarps];
-    const Share own(a.x.n[ORDER - 1], a.chunk, kWarps);
     const int lane = threadIdx.x & 31, g = lane / S::LPR, q = lane % S::LPR;
+    const Share own(a.x, a.chunk, a.weight, kWarps, lane);
     Stage<T, ORDER, S::W> &st = stages[threadIdx.x >> 5];
     const int col = blockIdx.y * RP + q * N;
     const T *leaf = a.F[ORDER - 2] + col, *mid = ORDER == 4 ? a.F[1] + col : nullptr, *top = a.F[0] + col;
     Vec<T> acc = zero_vec<T>();
-    const int32_t joint = walk_chunk(a.x, own, [&](int32_t e) { return place_of(a.x, e, lane); },
+    const int32_t joint = walk_chunk(a.x, own, [&](int32_t e) { return place_of(a.x, e, lane, own.slice); },
         [](const Place<ORDER> &) {},
         [&](Place<ORDER> &place, int32_t e, int32_t limit) {
             const int cnt = limit - e < S::W ? limit - e : S::W;
@@ -203,7 +203,7 @@ struct Ttmc3Args {
     T *out;
     size_t out_bytes;
     int32_t R2, R3;                                   // real ranks
-    int32_t chunk;                                    // leaves per warp (set by the launch)
+    int32_t chunk, weight;                            // cost per warp, and of a slice beyond its leaves (set by the launch)
 };
 
 template <typename T, int R2, int R3>
@@ -211,8 +211,8 @@ __global__ void __launch_bounds__(kWarps * 32, Ttmc3Shape<T, R2, R3>::BLOCKS) tt
     using S = Ttmc3Shape<T, R2, R3>;
     constexpr int N = S::N;
     extern __shared__ __align__(16) unsigned char smem[];
-    const Share own(a.x.n[2], a.chunk, kWarps);
     const int lane = threadIdx.x & 31, g = lane / S::LPR, q = lane % S::LPR;
+    const Share own(a.x, a.chunk, a.weight, kWarps, lane);
     typename S::Smem &sm = reinterpret_cast<typename S::Smem *>(smem)[threadIdx.x >> 5];
     const T *V = a.V + q * N;
     // consumer: the lane owns rows rg .. rg + RW - 1 and columns cg .. cg + N - 1 of the slice result; acc[i][c]: rows
@@ -242,7 +242,7 @@ __global__ void __launch_bounds__(kWarps * 32, Ttmc3Shape<T, R2, R3>::BLOCKS) tt
             put(rg + 2 * i + 1, hi);
         }
     };
-    const int32_t joint = walk_chunk(a.x, own, [&](int32_t e) { return place_of(a.x, e, lane); },
+    const int32_t joint = walk_chunk(a.x, own, [&](int32_t e) { return place_of(a.x, e, lane, own.slice); },
         [](const Place<3> &) {},
         [&](Place<3> &place, int32_t e, int32_t limit) {
             const int cnt = limit - e < S::W ? limit - e : S::W;
@@ -327,7 +327,7 @@ struct Ttmc4Args {
     T *out;
     size_t out_bytes;
     int32_t R2, R3, R4;                               // real ranks
-    int32_t chunk;                                    // leaves per warp (set by the launch)
+    int32_t chunk, weight;                            // cost per warp, and of a slice beyond its leaves (set by the launch)
 };
 
 template <typename T>
@@ -335,8 +335,8 @@ __global__ void __launch_bounds__(kWarps * 32, Ttmc4Shape<T>::BLOCKS) ttmc4_kern
     using S = Ttmc4Shape<T>;
     constexpr int N = S::N, R = S::R, NV = R / N;
     extern __shared__ __align__(16) unsigned char smem[];
-    const Share own(a.x.n[3], a.chunk, kWarps);
     const int lane = threadIdx.x & 31, g = lane / S::SL, h = lane % S::SL;
+    const Share own(a.x, a.chunk, a.weight, kWarps, lane);
     typename S::Smem &sm = reinterpret_cast<typename S::Smem *>(smem)[threadIdx.x >> 5];
     const T *V = a.V + 2 * h;
     // consumer: 16 lanes cover the 8 x 8 x 8 result; the lane owns every a for one b and four c; acc[i][c]: a = 2 i, 2 i + 1
@@ -371,7 +371,7 @@ __global__ void __launch_bounds__(kWarps * 32, Ttmc4Shape<T>::BLOCKS) ttmc4_kern
         }
     };
     Ahead<T, 4, S::W> ahead;
-    const int32_t joint = walk_chunk(a.x, own, [&](int32_t e) { return place_of(a.x, e, lane); },
+    const int32_t joint = walk_chunk(a.x, own, [&](int32_t e) { return place_of(a.x, e, lane, own.slice); },
         [&](const Place<4> &place) {
             request<T, 4, S::W>(a.x, place, own.e0, own.e1, lane, ahead);
         },
@@ -492,26 +492,28 @@ __global__ void __launch_bounds__(kWarps * 32, Ttmc4Shape<T>::BLOCKS) ttmc4_kern
 }
 
 // ---------------------------------------------------------------------------------------------- host side
-unsigned chunk_blocks(int64_t nnz, int32_t chunk) {
-    const int64_t warps = (nnz + chunk - 1) / chunk;
+template <class Args, typename T, int ORDER>
+unsigned cut_blocks(Args &a, const Chain<T, ORDER> &x, const Cut &cut) {
+    a.chunk = cut.chunk;
+    a.weight = cut.weight;
+    const int64_t warps = (x.n[ORDER - 1] + (int64_t)cut.weight * x.n[0] + cut.chunk - 1) / cut.chunk;
     return (unsigned)((warps + kWarps - 1) / kWarps);
 }
 
 template <typename T, int ORDER, int RP>
 const_status_t launch_mttkrp(MttkrpArgs<T, ORDER> a, int tiles, cudaStream_t stream) {
-    a.chunk = chunk_leaves(a.x.n[ORDER - 1], a.x.n[0], 4096, MttkrpShape<T, ORDER, RP>::FIT);
-    const dim3 grid(chunk_blocks(a.x.n[ORDER - 1], a.chunk), (unsigned)tiles);
+    const dim3 grid(cut_blocks(a, a.x, cut_leaves(a.x.n[ORDER - 1], a.x.n[0], 4096, MttkrpShape<T, ORDER, RP>::FIT, RP <= 8 ? 64 : 48)), (unsigned)tiles);
     return launch_on_cleared("chain3_kernel", mttkrp_kernel<T, ORDER, RP>, a, grid, kWarps * 32, 0, a.out, a.out_bytes, stream);
 }
 
 template <typename T, int R2, int R3>
 const_status_t launch_ttmc3(Ttmc3Args<T> a, cudaStream_t stream) {
     constexpr int fit = Ttmc3Shape<T, R2, R3>::FIT;
-    a.chunk = chunk_leaves(a.x.n[2], a.x.n[0], 3072, fit, (20 + fit - 1) / fit);
+    const dim3 grid(cut_blocks(a, a.x, cut_leaves(a.x.n[2], a.x.n[0], 3072, fit, R3 >= 32 || R2 * R3 >= 512 ? 64 : 96, (20 + fit - 1) / fit)));
     constexpr size_t dyn = sizeof(typename Ttmc3Shape<T, R2, R3>::Smem) * kWarps;
     static PerDeviceOnce attr_once;                     // per template instance
     CB_CUDA(once_per_device(attr_once, [&] { return cudaFuncSetAttribute(ttmc3_kernel<T, R2, R3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn); }));
-    return launch_on_cleared("chain3_kernel", ttmc3_kernel<T, R2, R3>, a, dim3(chunk_blocks(a.x.n[2], a.chunk)), kWarps * 32, dyn, a.out,
+    return launch_on_cleared("chain3_kernel", ttmc3_kernel<T, R2, R3>, a, grid, kWarps * 32, dyn, a.out,
                              a.out_bytes, stream);
 }
 
@@ -545,11 +547,11 @@ const_status_t dispatch_mttkrp(const MttkrpArgs<T, ORDER> &a, int rp, int tiles,
 
 template <typename T>
 const_status_t launch_ttmc4(Ttmc4Args<T> a, cudaStream_t stream) {
-    a.chunk = chunk_leaves(a.x.n[3], a.x.n[0], 4096, Ttmc4Shape<T>::FIT);
+    const dim3 grid(cut_blocks(a, a.x, cut_leaves(a.x.n[3], a.x.n[0], 4096, Ttmc4Shape<T>::FIT, 64)));
     constexpr size_t dyn = sizeof(typename Ttmc4Shape<T>::Smem) * kWarps;
     static PerDeviceOnce attr_once;                     // per template instance
     CB_CUDA(once_per_device(attr_once, [&] { return cudaFuncSetAttribute(ttmc4_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn); }));
-    return launch_on_cleared("ttmc4_kernel", ttmc4_kernel<T>, a, dim3(chunk_blocks(a.x.n[3], a.chunk)), kWarps * 32, dyn, a.out,
+    return launch_on_cleared("ttmc4_kernel", ttmc4_kernel<T>, a, grid, kWarps * 32, dyn, a.out,
                              a.out_bytes, stream);
 }
 

@@ -186,11 +186,12 @@ __device__ __forceinline__ void warp_find2(Key key, int32_t (&lo)[2], int32_t (&
     }
 }
 
-// Root first, so that every search below is over one slice only: few steps, each a dependent load.
+// Root first (slice: the leaf's, where it is known, or -1), so that every search below is over one slice only: few steps, each a
+// dependent load.
 template <typename T, int ORDER>
-__device__ __forceinline__ Place<ORDER> place_of(const Chain<T, ORDER> &x, int32_t leaf, int lane) {
+__device__ __forceinline__ Place<ORDER> place_of(const Chain<T, ORDER> &x, int32_t leaf, int lane, int32_t slice = -1) {
     Place<ORDER> p;
-    p.node[0] = warp_find(x.slice_ptr, 0, x.n[0], leaf, lane);
+    p.node[0] = slice >= 0 ? slice : warp_find(x.slice_ptr, 0, x.n[0], leaf, lane);
     const int32_t f0 = __ldg(x.pos[1] + p.node[0]), f1 = __ldg(x.pos[1] + p.node[0] + 1);
     if constexpr (ORDER == 3) {
         p.node[1] = warp_find(x.pos[2], f0, f1, leaf, lane);
@@ -364,6 +365,7 @@ __device__ __forceinline__ int stage_window(const Ahead<T, ORDER, W> &a, Place<O
 // The leaves of one warp, and the end of those of its block.
 struct Share {
     int32_t e0, e1, block_end;
+    int32_t slice = -1, begin, end;                      // slice of leaf e0 and its leaves, where the search has met them
     Share() = default;
     __device__ __forceinline__ Share(int32_t nnz, int32_t chunk, int warps) {
         const int64_t b0 = (int64_t)blockIdx.x * warps * chunk, b1 = b0 + (int64_t)warps * chunk;
@@ -371,6 +373,35 @@ struct Share {
         block_end = b1 < nnz ? (int32_t)b1 : nnz;
         e0 = w0 < nnz ? (int32_t)w0 : nnz;
         e1 = nnz - e0 < chunk ? nnz : e0 + chunk;
+    }
+    // Equal costs instead: a slice counts as `weight` leaves more than it has (weight = 0: equal leaves, no search).  Every warp of
+    // the block has to call this.
+    template <typename T, int ORDER>
+    __device__ __forceinline__ Share(const Chain<T, ORDER> &x, int32_t chunk, int32_t weight, int warps, int lane) : Share(x.n[ORDER - 1], chunk, warps) {
+        if (!weight) return;
+        const int64_t c0 = ((int64_t)blockIdx.x * warps + (threadIdx.x >> 5)) * chunk, target[2] = {c0, c0 + chunk};
+        int32_t lo[2] = {0, 0}, hi[2] = {x.n[0], x.n[0]};
+        warp_find2([&](int32_t s) { return (int64_t)__ldg(x.slice_ptr + s) + (int64_t)weight * s; }, lo, hi, target, lane);
+        int32_t at[2][3], e[2];
+#pragma unroll
+        for (int t = 0; t < 2; ++t)
+#pragma unroll
+            for (int k = 0; k < 3; ++k) at[t][k] = __ldg(x.slice_ptr + (lo[t] + k < x.n[0] ? lo[t] + k : x.n[0]));
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+            const int64_t in = target[t] - at[t][0] - (int64_t)weight * lo[t];
+            e[t] = in < at[t][1] - at[t][0] ? at[t][0] + (int32_t)in : at[t][1];
+        }
+        e0 = e[0];
+        e1 = e[1];
+        const bool next = e0 == at[0][1];                // behind the slice's leaves: the next one's first
+        slice = lo[0] + next;
+        begin = next ? at[0][1] : at[0][0];
+        end = next ? at[0][2] : at[0][1];
+        __shared__ int32_t s_end;
+        if (threadIdx.x == 32 * (warps - 1)) s_end = e1;
+        __syncthreads();
+        block_end = s_end;
     }
 };
 
@@ -384,16 +415,17 @@ template <typename T, int ORDER, class Find, class Start, class Window, class Fl
 __device__ __forceinline__ int32_t walk_chunk(const Chain<T, ORDER> &x, const Share &own, Find find, Start start, Window window, Flush flush) {
     __shared__ int32_t first_slice;                      // where the block's first leaf lies
     Place<ORDER> place;
+    place.node[0] = 0;
     int32_t e = own.e0, end = 0;
     bool from_start = false;
     if (e < own.e1) {
         place = find(e);
         start(place);
-        from_start = __ldg(x.slice_ptr + place.node[0]) == e;
-        end = __ldg(x.slice_ptr + place.node[0] + 1);
+        from_start = (own.slice >= 0 ? own.begin : __ldg(x.slice_ptr + place.node[0])) == e;
+        end = own.slice >= 0 ? own.end : __ldg(x.slice_ptr + place.node[0] + 1);
     }
     after_last_kernel();                                 // the result is cleared; everything up to here only read the tensor
-    if (threadIdx.x == 0) first_slice = place.node[0];   // (the first warp of a block always has leaves)
+    if (threadIdx.x == 0) first_slice = place.node[0];
     const bool joint = __syncthreads_or(threadIdx.x < 32 && end >= own.block_end) != 0;
     while (e < own.e1) {
         const int32_t limit = end < own.e1 ? end : own.e1;
@@ -441,6 +473,20 @@ inline int32_t chunk_leaves(int64_t nnz, int64_t slices, int64_t most, int fit, 
     const int64_t c = (nnz + wave * waves - 1) / (wave * waves);
     if (c < 64) return (int32_t)std::min<int64_t>(std::max((nnz + 148 * fit - 1) / (148 * fit), nnz / (2 * slices)), 64);
     return (int32_t)((c + 63) / 64 * 64);
+}
+
+// How the leaves are cut: cost per warp, and what a slice costs beyond its leaves (Share).  A slice's last window is not full and its
+// result is handed over: with Zipf-sized slices the warps that got the many short ones took several times as long as the
+// others.  Equal leaves against this, us: slices Zipf 1.1, TTMc 8 x 8, 1.5 M leaves in slices of 40: 219 / 77, 6 M of 400: 162 /
+// 106, 20 M of 333: 453 / 334; 32 x 32: 256 / 149, 406 / 353, 1124 / 954; order 4: 387 / 129, 407 / 301, 1080 / 853; MTTKRP rank 32: 119 / 56,
+// 122 / 103, 382 / 288; slices of equal size: within 1 % from 6 M on.  Not where slices are long anyway (from 4000 leaves on it gained
+// 1 to 3 % under Zipf 1.1 and lost 1 to 2 % on equal ones), nor where a chunk would be a few slices.
+struct Cut { int32_t chunk, weight; };
+inline Cut cut_leaves(int64_t nnz, int64_t slices, int64_t most, int fit, int32_t weight, int64_t least_waves = 1) {
+    const int64_t wave = 148 * (int64_t)fit, cost = nnz + weight * slices;
+    const int64_t waves = std::max(least_waves, (cost + wave * most - 1) / (wave * most)), c = (cost + wave * waves - 1) / (wave * waves);
+    if (c >= 4 * weight && nnz < 3000 * slices) return Cut{(int32_t)((c + 7) / 8 * 8), weight};
+    return Cut{chunk_leaves(nnz, slices, most, fit, least_waves), 0};
 }
 
 // Clears `out` ("R[*] = 0" precedes the nest; bytes = 0: the launch before has done that) and launches the kernel so that it starts while the clearing still runs: it
