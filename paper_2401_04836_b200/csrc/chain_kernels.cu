@@ -502,14 +502,14 @@ unsigned cut_blocks(Args &a, const Chain<T, ORDER> &x, const Cut &cut) {
 
 template <typename T, int ORDER, int RP>
 const_status_t launch_mttkrp(MttkrpArgs<T, ORDER> a, int tiles, cudaStream_t stream) {
-    const dim3 grid(cut_blocks(a, a.x, cut_leaves(a.x.n[ORDER - 1], a.x.n[0], 4096, MttkrpShape<T, ORDER, RP>::FIT, RP <= 8 ? 64 : 48)), (unsigned)tiles);
+    const dim3 grid(cut_blocks(a, a.x, cut_leaves(a.x.n[ORDER - 1], a.x.n[0], 4096, MttkrpShape<T, ORDER, RP>::FIT, RP <= 8 ? 64 : 48, 4)), (unsigned)tiles);
     return launch_on_cleared("chain3_kernel", mttkrp_kernel<T, ORDER, RP>, a, grid, kWarps * 32, 0, a.out, a.out_bytes, stream);
 }
 
 template <typename T, int R2, int R3>
 const_status_t launch_ttmc3(Ttmc3Args<T> a, cudaStream_t stream) {
     constexpr int fit = Ttmc3Shape<T, R2, R3>::FIT;
-    const dim3 grid(cut_blocks(a, a.x, cut_leaves(a.x.n[2], a.x.n[0], 3072, fit, R3 >= 32 || R2 * R3 >= 512 ? 64 : 96, (20 + fit - 1) / fit)));
+    const dim3 grid(cut_blocks(a, a.x, cut_leaves(a.x.n[2], a.x.n[0], 3072, fit, R3 >= 32 || R2 * R3 >= 512 ? 64 : 96, 2)));
     constexpr size_t dyn = sizeof(typename Ttmc3Shape<T, R2, R3>::Smem) * kWarps;
     static PerDeviceOnce attr_once;                     // per template instance
     CB_CUDA(once_per_device(attr_once, [&] { return cudaFuncSetAttribute(ttmc3_kernel<T, R2, R3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn); }));
@@ -547,7 +547,7 @@ const_status_t dispatch_mttkrp(const MttkrpArgs<T, ORDER> &a, int rp, int tiles,
 
 template <typename T>
 const_status_t launch_ttmc4(Ttmc4Args<T> a, cudaStream_t stream) {
-    const dim3 grid(cut_blocks(a, a.x, cut_leaves(a.x.n[3], a.x.n[0], 4096, Ttmc4Shape<T>::FIT, 64)));
+    const dim3 grid(cut_blocks(a, a.x, cut_leaves(a.x.n[3], a.x.n[0], 4096, Ttmc4Shape<T>::FIT, 64, 4)));
     constexpr size_t dyn = sizeof(typename Ttmc4Shape<T>::Smem) * kWarps;
     static PerDeviceOnce attr_once;                     // per template instance
     CB_CUDA(once_per_device(attr_once, [&] { return cudaFuncSetAttribute(ttmc4_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn); }));
