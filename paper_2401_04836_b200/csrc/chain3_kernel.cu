@@ -215,31 +215,38 @@ struct Args {
     Chain<float, 3> x;                                               // crd[2] and vals are readable up to the next multiple of 4
     const float *F1, *F2;
     float *out;
-    int32_t chunk;                                                   // leaves per warp; with a weight, leaves + weight * fibres
-    int32_t weight;
+    int32_t chunk;                                                   // cost per warp: a leaf costs one,
+    int32_t weight, slice_weight;                                    // a fibre so much, a slice so much, beyond what is in it
 };
 
-// The part of the tensor between two costs, a leaf costing one and a fibre `weight`: its leaves [e0, e1), and the place of the
-// first.  Root first, as walk::place_of; both ends in one search.
+// The part of the tensor between two costs: its leaves [e0, e1), and the place of the first.  Root first, as walk::place_of; both
+// ends in one search.
 __device__ __forceinline__ void deal_weighted(const Args &a, int64_t cost, int lane, Place<3> &from, int32_t &e0, int32_t &e1) {
-    const int64_t w = a.weight, total = a.x.n[2] + w * a.x.n[1];
-    const int64_t target[2] = {cost < total ? cost : total - 1, cost + a.chunk < total ? cost + a.chunk : total - 1};
-    int32_t lo[2] = {0, 0}, hi[2] = {a.x.n[0], a.x.n[0]};
-    walk::warp_find2([&](int32_t s) { return __ldg(a.x.slice_ptr + s) + w * __ldg(a.x.pos[1] + s); }, lo, hi, target, lane);
+    const int64_t w = a.weight, v = a.slice_weight, total = a.x.n[2] + w * a.x.n[1] + v * a.x.n[0];
+    int64_t target[2] = {cost < total ? cost : total - 1, cost + a.chunk < total ? cost + a.chunk : total - 1};
+    int32_t lo[2] = {0, 0}, hi[2] = {a.x.n[0], a.x.n[0]}, slice_end[2];
+    walk::warp_find2([&](int32_t s) { return __ldg(a.x.slice_ptr + s) + w * __ldg(a.x.pos[1] + s) + v * s; }, lo, hi, target, lane);
     from.node[0] = lo[0];
 #pragma unroll
     for (int t = 0; t < 2; ++t) {
+        target[t] -= v * lo[t];
+        slice_end[t] = __ldg(a.x.slice_ptr + lo[t] + 1);
         hi[t] = __ldg(a.x.pos[1] + lo[t] + 1);
         lo[t] = __ldg(a.x.pos[1] + lo[t]);
     }
+    const int32_t next_fibre = hi[0];
     walk::warp_find2([&](int32_t f) { return __ldg(a.x.pos[2] + f) + w * f; }, lo, hi, target, lane);
     from.node[1] = lo[0];
     int32_t e[2];
 #pragma unroll
-    for (int t = 0; t < 2; ++t) {                                    // the cost of a fibre is paid before its first leaf
+    for (int t = 0; t < 2; ++t) {                                    // the cost of a fibre is paid before its first leaf, of a slice behind its last
         const int32_t p = __ldg(a.x.pos[2] + lo[t]);
         const int64_t behind = target[t] - (p + w * lo[t]) - w;
-        e[t] = behind > 0 ? max(p, (p + (int32_t)behind) & ~3) : p;  // on a block of four leaves, inside a fibre
+        e[t] = behind >= slice_end[t] - p ? slice_end[t] : behind > 0 ? max(p, (p + (int32_t)behind) & ~3) : p;   // on a block of four leaves, inside a fibre
+    }
+    if (e[0] == slice_end[0]) {
+        ++from.node[0];
+        from.node[1] = next_fibre;
     }
     e0 = cost < total ? e[0] : a.x.n[2];
     e1 = cost + a.chunk < total ? e[1] : a.x.n[2];
@@ -261,7 +268,7 @@ __global__ void __launch_bounds__(kWarps * 32, 4) chain3_kernel(const __grid_con
     walk::Share own;
     Place<3> from;
     if constexpr (!WEIGHED) {
-        own = walk::Share(a.x.n[2], a.chunk, kWarps);
+        own = walk::Share(a.x, a.chunk, a.slice_weight, kWarps, lane);
     } else {
         __shared__ int32_t block_end;
         deal_weighted(a, ((int64_t)blockIdx.x * kWarps + (threadIdx.x >> 5)) * a.chunk, lane, from, own.e0, own.e1);
@@ -300,7 +307,7 @@ __global__ void __launch_bounds__(kWarps * 32, 4) chain3_kernel(const __grid_con
     const int32_t joint = walk::walk_chunk(a.x, own,
         [&](int32_t e) {
             if constexpr (WEIGHED) return from;
-            else return walk::place_of(a.x, e, lane);
+            else return walk::place_of(a.x, e, lane, own.slice);
         },
         [](const Place<3> &) {},
         [&](Place<3> &place, int32_t e, int32_t limit) {
@@ -352,7 +359,7 @@ const_status_t launch_form(const Args &a, int64_t n_rows, cudaStream_t stream) {
     constexpr size_t dyn = sizeof(Smem<R2, R3>) * kWarps;
     static PerDeviceOnce attr_once;                     // per template instance
     CB_CUDA(once_per_device(attr_once, [&] { return cudaFuncSetAttribute(chain3_kernel<R2, R3, WEIGHED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn); }));
-    const int64_t warps = ((int64_t)a.x.n[2] + (int64_t)a.weight * a.x.n[1] + a.chunk - 1) / a.chunk;
+    const int64_t cost = (int64_t)a.x.n[2] + (int64_t)a.weight * a.x.n[1] + (int64_t)a.slice_weight * a.x.n[0], warps = (cost + a.chunk - 1) / a.chunk;
     return walk::launch_on_cleared("chain3_kernel", chain3_kernel<R2, R3, WEIGHED>, a, dim3((unsigned)((warps + kWarps - 1) / kWarps)), kWarps * 32, dyn,
                                    a.out, sizeof(float) * R2 * R3 * n_rows, stream);
 }
@@ -378,13 +385,19 @@ const_status_t run_ttmc3_fibres(const const_csf *X, const float *U, const float 
     // Equal leaves where they are as good: smaller tensors (2 M in fibres of 25: 24.4 / 25.7, 300 000: 17.8 / 19.5, the longer
     // search), fibres of less than three (6 M in fibres of 2.6, 8 x 16: 110 / 117, 16 x 16: 137 / 144), and slices of more than
     // 1024 fibres, whose sums would get longer (19 M in fibres of 3, 8 x 16, 4260 a slice: 329 / 328 us, error 1.8e-7 / 2.1e-7).
-    constexpr int32_t kWeight = 6, kResident = 16;
+    constexpr int32_t kWeight = 6, kSliceWeight = 64, kResident = 16;
     constexpr int64_t kWave = 148 * kResident;
-    const int64_t cost = X->nnz + kWeight * X->n[1], most = R2 * R3 >= 1024 ? 2048 : R2 * R3 >= 512 ? 4096 : 8192;
+    // A slice counts as 64 leaves in either form (its result is handed over, its last window is not full): slices Zipf 1.1, 16 x 16, 281 000
+    // leaves in slices of 38: 67 / 26, 3 M of 49: 383 / 153, 12 M of 195: 320 / 283; slices of equal size within 1 %.
+    const int64_t cost = X->nnz + kWeight * X->n[1] + kSliceWeight * X->n[0], most = R2 * R3 >= 1024 ? 2048 : R2 * R3 >= 512 ? 4096 : 8192;
     const int64_t parts = (cost + kWave * most - 1) / (kWave * most) * kWave;
-    const bool weigh = X->nnz >= 3000000 && X->nnz >= 3 * X->n[1] && X->n[1] <= 1024ll * X->n[0];
-    const Args a{walk::chain_of<float, 3>(X), U, V, Y,
-                 weigh ? (int32_t)((cost + parts - 1) / parts) : walk::chunk_leaves(X->nnz, X->n[0], 1536, kResident), weigh ? kWeight : 0};
+    Args a{walk::chain_of<float, 3>(X), U, V, Y, (int32_t)((cost + parts - 1) / parts), kWeight, kSliceWeight};
+    if (X->nnz < 3000000 || X->nnz < 3 * X->n[1] || X->n[1] > 1024ll * X->n[0]) {
+        const walk::Cut cut = walk::cut_leaves(X->nnz, X->n[0], 1536, kResident, kSliceWeight, 3 * kSliceWeight);
+        a.chunk = cut.chunk;
+        a.weight = 0;
+        a.slice_weight = cut.weight;
+    }
     switch (R2 * 100 + R3) {
         case 808: return launch_chain3<8, 8>(a, n_rows, s);
         case 816: return launch_chain3<8, 16>(a, n_rows, s);

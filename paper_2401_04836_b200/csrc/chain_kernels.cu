@@ -502,14 +502,20 @@ unsigned cut_blocks(Args &a, const Chain<T, ORDER> &x, const Cut &cut) {
 
 template <typename T, int ORDER, int RP>
 const_status_t launch_mttkrp(MttkrpArgs<T, ORDER> a, int tiles, cudaStream_t stream) {
-    const dim3 grid(cut_blocks(a, a.x, cut_leaves(a.x.n[ORDER - 1], a.x.n[0], 4096, MttkrpShape<T, ORDER, RP>::FIT, RP <= 8 ? 64 : 48, 4)), (unsigned)tiles);
+    using S = MttkrpShape<T, ORDER, RP>;
+    const int64_t nnz = a.x.n[ORDER - 1], slices = a.x.n[0];
+    const int32_t weight = RP <= 8 ? 64 : 48, least = ORDER == 4 || nnz < 200 * slices ? 4 * weight : 5 * S::W;
+    const dim3 grid(cut_blocks(a, a.x, cut_leaves(nnz, slices, 4096, S::FIT, weight, least)), (unsigned)tiles);
     return launch_on_cleared("chain3_kernel", mttkrp_kernel<T, ORDER, RP>, a, grid, kWarps * 32, 0, a.out, a.out_bytes, stream);
 }
 
 template <typename T, int R2, int R3>
 const_status_t launch_ttmc3(Ttmc3Args<T> a, cudaStream_t stream) {
     constexpr int fit = Ttmc3Shape<T, R2, R3>::FIT;
-    const dim3 grid(cut_blocks(a, a.x, cut_leaves(a.x.n[2], a.x.n[0], 3072, fit, R3 >= 32 || R2 * R3 >= 512 ? 64 : 96, 2)));
+    // where only four warps fit (fp64, 32 x 32) a wave is few chunks: shorter ones even out slices of different density
+    const int64_t most = fit <= 4 ? 448 : 3072;
+    constexpr int32_t weight = R3 >= 32 || R2 * R3 >= 512 ? 64 : 96;
+    const dim3 grid(cut_blocks(a, a.x, cut_leaves(a.x.n[2], a.x.n[0], most, fit, weight, 3 * weight, true)));
     constexpr size_t dyn = sizeof(typename Ttmc3Shape<T, R2, R3>::Smem) * kWarps;
     static PerDeviceOnce attr_once;                     // per template instance
     CB_CUDA(once_per_device(attr_once, [&] { return cudaFuncSetAttribute(ttmc3_kernel<T, R2, R3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn); }));
@@ -547,7 +553,7 @@ const_status_t dispatch_mttkrp(const MttkrpArgs<T, ORDER> &a, int rp, int tiles,
 
 template <typename T>
 const_status_t launch_ttmc4(Ttmc4Args<T> a, cudaStream_t stream) {
-    const dim3 grid(cut_blocks(a, a.x, cut_leaves(a.x.n[3], a.x.n[0], 4096, Ttmc4Shape<T>::FIT, 64, 4)));
+    const dim3 grid(cut_blocks(a, a.x, cut_leaves(a.x.n[3], a.x.n[0], 4096, Ttmc4Shape<T>::FIT, 64, 256)));
     constexpr size_t dyn = sizeof(typename Ttmc4Shape<T>::Smem) * kWarps;
     static PerDeviceOnce attr_once;                     // per template instance
     CB_CUDA(once_per_device(attr_once, [&] { return cudaFuncSetAttribute(ttmc4_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn); }));
@@ -699,9 +705,20 @@ const_status_t run_ttmc3(const const_csf *X, const float *U, const float *V, int
     // at R2 = 32: 100 000 leaves in fibres of one, 16 x 16, slices of 1 / 4 / 16 / 64: 106 / 95, 51 / 51, 23 / 27, 17.4 / 18.3;
     // 300 000: 351 / 264, 143 / 128, 47 / 54, 27 / 30; 32 x 32, 300 000: 612 / 407, 238 / 168, 83 / 69, 49 / 42; 493 000 in
     // fibres of 2.3 and slices of 425: 8 x 8 18.6 / 17.3, 8 x 32 29.3 / 25.3, 32 x 16 31.8 / 26.3.
+    // With slices counted at their cost on both sides: slices of less than a hundred leaves, 16 x 16, walk / chain3_kernel, 1 M in
+    // fibres of 3.3: 54 / 67, of 20: 50 / 46; 4 M of 10.7: 135 / 157; long slices, 16 M in fibres of 3.2: 8 x 8 262 / 240, 16 x 16 333 / 354, 8 x 32
+    // 418 / 483, 32 x 8 379 / 307; of 4.1: 258 / 205, 313 / 305, 393 / 410, 365 / 265.
     const double per_fibre = (double)X->nnz / (double)X->n[1], per_slice = (double)X->nnz / (double)X->n[0];
-    const bool large = X->nnz >= 1000000, middle = X->nnz >= 100000 && per_slice >= 16 && R2 < 32;
-    if (per_fibre > (large ? R2 * R3 >= 1024 ? 1.8 : 2.5 : middle ? 1.5 : 0.0)) return run_ttmc3_fibres(X, U, V, R2, R3, Y, n_rows, stream);
+    const bool middle = X->nnz >= 100000 && per_slice >= 16 && R2 < 32;
+    double line = middle ? 1.5 : 0.0;
+    if (X->nnz >= 1000000) {
+        line = 2.5;
+        if (R2 * R3 >= 1024) line = 1.8;
+        else if (R2 == 32 && R3 == 8) line = 1.9;
+        else if (R2 < 32 && R3 < 32 && per_slice < 100) line = 8.0;
+        else if (R2 < 32 && X->nnz >= 3000000) line = R3 == 32 || R2 * R3 == 256 ? 3.5 : 2.5;
+    }
+    if (per_fibre > line) return run_ttmc3_fibres(X, U, V, R2, R3, Y, n_rows, stream);
     return dispatch_ttmc3<float>({chain_of<float, 3>(X), U, V, Y, bytes, R2, R3}, R2, R3, stream);
 }
 

@@ -467,12 +467,14 @@ inline Chain<T, ORDER> chain_of(const const_csf *X) {
 // one: 103 us at 64 leaves a warp, 14.5 here; 30 000 in slices of four: 62 and 25), and more warps than fit start late
 // (the latter with twice as many: 29).  But in chunks of half a slice on average where slices are longer than that: more
 // parts of a slice mean more atomic additions and more rounding, and gain nothing (30 000 in slices of 64: 15.0 us, in
-// chunks of 13 leaves 15.9, of 64 18.4; 20 000 in slices of 100: relative error 7.5e-8, in chunks of 9 leaves 8.3e-8).
-inline int32_t chunk_leaves(int64_t nnz, int64_t slices, int64_t most, int fit) {
+// chunks of 13 leaves 15.9, of 64 18.4; 20 000 in slices of 100: relative error 7.5e-8, in chunks of 9 leaves 8.3e-8).  Little more than
+// a window of 64 a warp would be two (one_window): rather one, and a few warps that start late (TTMc 23 x 32 in fp64, 40 000 leaves:
+// 27.7, in chunks of 128 34.6).
+inline int32_t chunk_leaves(int64_t nnz, int64_t slices, int64_t most, int fit, bool one_window = false) {
     const int64_t wave = 148 * (int64_t)fit, waves = (nnz + wave * most - 1) / (wave * most);
     const int64_t c = (nnz + wave * waves - 1) / (wave * waves);
     if (c < 64) return (int32_t)std::min<int64_t>(std::max((nnz + 148 * fit - 1) / (148 * fit), nnz / (2 * slices)), 64);
-    return (int32_t)((c + 63) / 64 * 64);
+    return one_window && c < 96 ? 64 : (int32_t)((c + 63) / 64 * 64);
 }
 
 // How the leaves are cut: cost per warp, and what a slice costs beyond its leaves (Share).  A slice's last window is not full and its
@@ -480,14 +482,15 @@ inline int32_t chunk_leaves(int64_t nnz, int64_t slices, int64_t most, int fit) 
 // others.  Equal leaves against this, us: slices Zipf 1.1, TTMc 8 x 8, 1.5 M leaves in slices of 40: 219 / 77, 6 M of 400: 162 /
 // 106, 20 M of 333: 453 / 334; 32 x 32: 256 / 149, 406 / 353, 1124 / 954; order 4: 387 / 129, 407 / 301, 1080 / 853; MTTKRP rank 32: 119 / 56,
 // 122 / 103, 382 / 288; slices of equal size: within 1 % from 6 M on.  Not where slices are long anyway (from 4000 leaves on it gained
-// 1 to 3 % under Zipf 1.1 and lost 1 to 2 % on equal ones), nor where a chunk would cost less than `least` slices and the longer search would
-// show (fp64 MTTKRP of order 4, 300 000 leaves in chunks of three: 24.1 / 26.0; TTMc 27 x 20 in fp64 gains down to two).
+// 1 to 3 % under Zipf 1.1 and lost 1 to 2 % on equal ones), nor where a chunk would cost less than `least`: the longer search shows, and
+// chunks are no whole windows any more (fp64 MTTKRP of order 4, 300 000 leaves in chunks of 154: 24.1 / 26.0; of order 3, 1.2 M equal
+// slices in chunks of two windows: 30.3 / 32.4; TTMc 32 x 16, 300 000 equal slices in chunks of 163: 27.9 / 32.0).
 struct Cut { int32_t chunk, weight; };
-inline Cut cut_leaves(int64_t nnz, int64_t slices, int64_t most, int fit, int32_t weight, int least) {
+inline Cut cut_leaves(int64_t nnz, int64_t slices, int64_t most, int fit, int32_t weight, int least, bool one_window = false) {
     const int64_t wave = 148 * (int64_t)fit, cost = nnz + weight * slices;
     const int64_t waves = (cost + wave * most - 1) / (wave * most), c = (cost + wave * waves - 1) / (wave * waves);
-    if (c >= least * weight && nnz < 3000 * slices) return Cut{(int32_t)((c + 7) / 8 * 8), weight};
-    return Cut{chunk_leaves(nnz, slices, most, fit), 0};
+    if (c >= least && nnz < 3000 * slices) return Cut{(int32_t)((c + 7) / 8 * 8), weight};
+    return Cut{chunk_leaves(nnz, slices, most, fit, one_window), 0};
 }
 
 // Clears `out` ("R[*] = 0" precedes the nest; bytes = 0: the launch before has done that) and launches the kernel so that it starts while the clearing still runs: it
