@@ -29,6 +29,7 @@ template <int ORDER>
 __global__ void __launch_bounds__(256) pack_hist(PackArgs a, int64_t nnz, DigitPlan dp, uint64_t *__restrict__ keys,
                                                  uint32_t *hist, int32_t *status, uint32_t *arrived) {
     extern __shared__ uint32_t sh[];                 // [passes][kRsMaxBins]
+    start_next_kernel();
     for (int x = threadIdx.x; x < dp.passes * kRsMaxBins; x += blockDim.x) sh[x] = 0;
     __syncthreads();
     bool bad = false;
@@ -79,7 +80,7 @@ inline void launch_pack_hist(const PackArgs &pa, int64_t nnz, const DigitPlan &d
 // ------------------------------------------------------------------------------------------------
 constexpr int kRsThreads = 256;
 constexpr int kRsItems = 16;
-constexpr int kRsTile = kRsThreads * kRsItems;     // 4096 keys per tile
+constexpr int kRsTile = kRsThreads * kRsItems;     // 4096 keys per tile; at least 1024, see tile_items
 constexpr int kRsWarps = kRsThreads / 32;
 constexpr int kSpinLimit = 1 << 21;
 // Distance, in tiles, of the pass kernel's L2 prefetch: half a wave of its resident blocks (148 SMs x 3).  Measured on
@@ -95,19 +96,21 @@ __device__ __forceinline__ unsigned long long status_word(unsigned epoch, unsign
     return ((unsigned long long)((epoch << 2) | flag) << 32) | count;
 }
 
-// One radix pass over BITS key bits.  Thread t owns digits t, t + 256, ... (DPT of them).
-template <typename V, int BITS>
-__global__ void __launch_bounds__(kRsThreads, 3) rs_onesweep(const uint64_t *__restrict__ kin, uint64_t *__restrict__ kout,
-                                                            const V *__restrict__ vin, V *__restrict__ vout, int64_t n,
-                                                            int shift, const uint32_t *__restrict__ digit_base,
+// One radix pass over BITS key bits in tiles of ITEMS keys per thread.  Thread t owns digits t, t + 256, ... (DPT of them).
+// (Kernels that start early have no __restrict__ on what the kernel before writes: the compiler would take its loads for ones of
+// constant data and may move them in front of the wait.)
+template <typename V, int BITS, int ITEMS>
+__global__ void __launch_bounds__(kRsThreads, 3) rs_onesweep(const uint64_t *kin, uint64_t *kout,
+                                                            const V *vin, V *vout, int64_t n,
+                                                            int shift, const uint32_t *digit_base,
                                                             unsigned long long *status, uint32_t *counter,
                                                             int32_t *err, unsigned epoch, int spin_limit, int withhold, int ahead_tiles) {
-    constexpr int kBins = 1 << BITS;
+    constexpr int kBins = 1 << BITS, kTile = kRsThreads * ITEMS;
     constexpr unsigned kDigitMask = kBins - 1;
     constexpr int DPT = kBins / kRsThreads;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     uint64_t *keybuf = reinterpret_cast<uint64_t *>(smem_raw);
-    V *valbuf = reinterpret_cast<V *>(smem_raw + kRsTile * sizeof(uint64_t));
+    V *valbuf = reinterpret_cast<V *>(smem_raw + kTile * sizeof(uint64_t));
     __shared__ uint32_t warp_hist[kRsWarps][kBins];
     __shared__ uint32_t digit_excl[kBins];
     __shared__ uint32_t s_gbase[kBins];
@@ -116,34 +119,36 @@ __global__ void __launch_bounds__(kRsThreads, 3) rs_onesweep(const uint64_t *__r
     __shared__ int s_abort;
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (threadIdx.x == 0) { s_tile = atomicAdd(counter, 1u); s_abort = 0; }
     for (int x = threadIdx.x; x < kRsWarps * kBins; x += kRsThreads) (&warp_hist[0][0])[x] = 0;
+    after_last_kernel();
+    start_next_kernel();
+    if (threadIdx.x == 0) { s_tile = atomicAdd(counter, 1u); s_abort = 0; }
     __syncthreads();
     const uint32_t tile = s_tile;
-    const int64_t tile_base = (int64_t)tile * kRsTile;
+    const int64_t tile_base = (int64_t)tile * kTile;
     if (tile_base >= n) return;                       // never happens: the grid has exactly ceil(n / tile) blocks
     const int64_t left = n - tile_base;
-    const int nvalid = left < kRsTile ? (int)left : kRsTile;
+    const int nvalid = left < kTile ? (int)left : kTile;
 
     // A tile that will be taken soon (half a wave of resident blocks ahead) is requested into L2 now, so that the
     // loads of the block that takes it find it there instead of in DRAM.
     {
-        const int64_t ahead = tile_base + (int64_t)ahead_tiles * kRsTile;
+        const int64_t ahead = tile_base + (int64_t)ahead_tiles * kTile;
         const int64_t kb = ahead * (int64_t)sizeof(uint64_t) + (int64_t)threadIdx.x * 128;       // keys: 32 KB = 256 lines
-        if (ahead + kRsTile <= n) {
+        if (ahead + kTile <= n) {
             asm volatile("prefetch.global.L2 [%0];" :: "l"(reinterpret_cast<const char *>(kin) + kb));
             const int64_t vb = ahead * (int64_t)sizeof(V) + (int64_t)threadIdx.x * 128;
-            if ((int64_t)threadIdx.x * 128 < (int64_t)kRsTile * (int64_t)sizeof(V))
+            if ((int64_t)threadIdx.x * 128 < (int64_t)kTile * (int64_t)sizeof(V))
                 asm volatile("prefetch.global.L2 [%0];" :: "l"(reinterpret_cast<const char *>(vin) + vb));
         }
     }
 
     // this thread's slots of the tile: local indices mine + 32 i
-    const int mine = warp * (32 * kRsItems) + lane;
+    const int mine = warp * (32 * ITEMS) + lane;
     const uint64_t *ktile = kin + tile_base + mine;
-    uint64_t key[kRsItems];
+    uint64_t key[ITEMS];
 #pragma unroll
-    for (int i = 0; i < kRsItems; ++i)
+    for (int i = 0; i < ITEMS; ++i)
         key[i] = mine + i * 32 < nvalid ? ktile[i * 32] : ~0ull;   // padding sorts after every real key of the tile
 
     // Digit counts of the tile first, so that later tiles can see them as early as possible:
@@ -157,10 +162,10 @@ __global__ void __launch_bounds__(kRsThreads, 3) rs_onesweep(const uint64_t *__r
     // In pairs: the ballots of both, then both counter additions, then the ranks, so that the additions' round trips overlap
     // (77 M keys: 569 -> 559 us a pass; four at a time 566, eight 568: registers.  Lane words built with atomicOr instead of
     // ballots: 647).
-    int rank[kRsItems];
+    int rank[ITEMS];
     constexpr int kBatch = 2;
 #pragma unroll
-    for (int i0 = 0; i0 < kRsItems; i0 += kBatch) {
+    for (int i0 = 0; i0 < ITEMS; i0 += kBatch) {
         unsigned peers[kBatch];
         uint32_t old[kBatch];
 #pragma unroll
@@ -237,7 +242,7 @@ __global__ void __launch_bounds__(kRsThreads, 3) rs_onesweep(const uint64_t *__r
     {
         const V *vtile = vin + tile_base + mine;
 #pragma unroll
-        for (int i = 0; i < kRsItems; ++i) {
+        for (int i = 0; i < ITEMS; ++i) {
             const V val = mine + i * 32 < nvalid ? vtile[i * 32] : V(0);
             const unsigned dg = (unsigned)(key[i] >> shift) & kDigitMask;
             const int p = (int)digit_excl[dg] + (int)warp_hist[warp][dg] + rank[i];
@@ -322,7 +327,7 @@ __global__ void __launch_bounds__(kRsThreads, 3) rs_onesweep(const uint64_t *__r
 
     // store runs of consecutive addresses
 #pragma unroll
-    for (int m = 0; m < kRsItems; ++m) {
+    for (int m = 0; m < ITEMS; ++m) {
         const int p = threadIdx.x + m * kRsThreads;
         if (p < nvalid) {
             const uint64_t k = keybuf[p];
@@ -345,7 +350,7 @@ constexpr int kCpLevels = kMaxOrder - 1;                      // levels that nee
 constexpr int kCpAheadTiles = 592;                            // L2 prefetch distance of the one-shot tile kernels (half a wave)
 
 // Requests the keys of the tile `kCpAheadTiles` after this block's into L2 (threads 0..127 take one line each).
-__device__ __forceinline__ void prefetch_tile_ahead(const uint64_t *__restrict__ keys, int64_t n) {
+__device__ __forceinline__ void prefetch_tile_ahead(const uint64_t *keys, int64_t n) {
     const int64_t first = ((int64_t)blockIdx.x + kCpAheadTiles) * kCpTile;
     if (threadIdx.x < kCpTile * (int)sizeof(uint64_t) / 128 && first + kCpTile <= n)
         asm volatile("prefetch.global.L2 [%0];" :: "l"(reinterpret_cast<const char *>(keys + first) + threadIdx.x * 128));
@@ -358,15 +363,15 @@ struct WarpKeys {
     ulonglong2 k[kCpSteps];
     uint64_t carry;
     int64_t base;
-    __device__ __forceinline__ void load(const uint64_t *__restrict__ keys, int64_t n, int64_t warp_base, int lane) {
+    __device__ __forceinline__ void load(const uint64_t *keys, int64_t n, int64_t warp_base, int lane) {
         base = warp_base;
-        carry = warp_base > 0 && warp_base <= n ? __ldg(keys + warp_base - 1) : 0ull;
+        carry = warp_base > 0 && warp_base <= n ? keys[warp_base - 1] : 0ull;
 #pragma unroll
         for (int it = 0; it < kCpSteps; ++it) {
             const int64_t e = warp_base + it * 64 + 2 * lane;
             k[it] = make_ulonglong2(0ull, 0ull);
-            if (e + 1 < n) k[it] = __ldg(reinterpret_cast<const ulonglong2 *>(keys + e));
-            else if (e < n) k[it].x = __ldg(keys + e);
+            if (e + 1 < n) k[it] = *reinterpret_cast<const ulonglong2 *>(keys + e);
+            else if (e < n) k[it].x = keys[e];
         }
     }
     // the key in front of this lane's first key of step `it`
@@ -379,10 +384,11 @@ struct WarpKeys {
 
 // Per-block node counts of every level; with few blocks the last one to finish also scans them (launch_csf_count).
 template <int ORDER>
-__global__ void __launch_bounds__(kCpThreads) csf_count(const uint64_t *__restrict__ keys, int64_t n, LevelShifts ls,
+__global__ void __launch_bounds__(kCpThreads) csf_count(const uint64_t *keys, int64_t n, LevelShifts ls,
                                                        uint32_t *block_counts, int32_t *status, uint32_t *totals, uint32_t *arrived) {
     __shared__ uint32_t sh[kCpLevels];
     if (threadIdx.x < kCpLevels) sh[threadIdx.x] = 0;
+    after_last_kernel();
     prefetch_tile_ahead(keys, n);
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -613,10 +619,11 @@ inline void launch_csf_count(int order, int64_t blocks, const uint64_t *keys, in
     const bool alone = blocks <= kCpScanBlocks;
     uint32_t *t = alone ? totals : nullptr;
     CB_LAUNCH("csf_count", stream, {
+        const dim3 grid((unsigned)blocks);
         switch (order) {
-            case 2: csf_count<2><<<(unsigned)blocks, kCpThreads, 0, stream>>>(keys, n, ls, block_counts, status, t, arrived); break;
-            case 3: csf_count<3><<<(unsigned)blocks, kCpThreads, 0, stream>>>(keys, n, ls, block_counts, status, t, arrived); break;
-            default: csf_count<4><<<(unsigned)blocks, kCpThreads, 0, stream>>>(keys, n, ls, block_counts, status, t, arrived); break;
+            case 2: launch_early(csf_count<2>, grid, kCpThreads, 0, stream, keys, n, ls, block_counts, status, t, arrived); break;
+            case 3: launch_early(csf_count<3>, grid, kCpThreads, 0, stream, keys, n, ls, block_counts, status, t, arrived); break;
+            default: launch_early(csf_count<4>, grid, kCpThreads, 0, stream, keys, n, ls, block_counts, status, t, arrived); break;
         }
     });
     if (!alone) launch_csf_scan(block_counts, blocks, totals, stream);
@@ -829,23 +836,41 @@ struct SortBufs {
     uint32_t *counters;                // [kMaxPasses] tile tickets
     unsigned long long *tile_status;   // [ntiles][kRsMaxBins], cleared by the caller
     uint32_t *arrived;                 // [2] blocks that have finished the pack and the count kernel, zero at first
+    int items;                         // keys per thread and tile of a pass
 };
+
+// Keys per thread of a pass: small tensors in small tiles, which are more tiles, each done sooner.  Build of an order-3 tensor at
+// 4 / 8 / 16, us: 20 000 nonzeros 62 / 70 / 70, 150 000 83 / 85 / 98, 300 000 98 / 97 / 100, 700 000 122 / 111 / 122, 1 M
+// 145 / 135 / 135, 2 M (three passes) 158 / 135 / 121.
+int tile_items(int64_t n) { return n <= 200000 ? 4 : n <= 900000 ? 8 : kRsItems; }
+
+
+template <typename V, int BITS, int ITEMS>
+const_status_t launch_tiles(const uint64_t *kin, uint64_t *kout, const V *vin, V *vout, int64_t n, int shift,
+                            const uint32_t *digit_base, const SortBufs &b, uint32_t *counter, int32_t *status,
+                            unsigned epoch, cudaStream_t stream) {
+    const int64_t ntiles = (n + kRsThreads * ITEMS - 1) / (kRsThreads * ITEMS);
+    const size_t dyn = kRsThreads * ITEMS * (sizeof(uint64_t) + sizeof(V));
+    static PerDeviceOnce attr_once;                     // per template instance
+    CB_CUDA(once_per_device(attr_once, [&] { return cudaFuncSetAttribute(rs_onesweep<V, BITS, ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn); }));
+    const DebugKnobs knobs = debug_knobs();
+    cudaError_t e = cudaSuccess;
+    CB_LAUNCH("rs_onesweep", stream,
+              e = launch_early(rs_onesweep<V, BITS, ITEMS>, dim3((unsigned)ntiles), kRsThreads, dyn, stream, kin, kout, vin, vout, n, shift,
+                               digit_base, b.tile_status, counter, status, epoch,
+                               (int)(knobs.spin_limit > 0 ? knobs.spin_limit : kSpinLimit), (int)knobs.withhold, (int)kRsAheadTiles));
+    return e == cudaSuccess ? CONST_OK : CONST_ERR_CUDA;
+}
 
 template <typename V, int BITS>
 const_status_t launch_onesweep(const uint64_t *kin, uint64_t *kout, const V *vin, V *vout, int64_t n, int shift,
                                const uint32_t *digit_base, const SortBufs &b, uint32_t *counter, int32_t *status,
                                unsigned epoch, cudaStream_t stream) {
-    const int64_t ntiles = (n + kRsTile - 1) / kRsTile;
-    const size_t dyn = kRsTile * (sizeof(uint64_t) + sizeof(V));
-    static PerDeviceOnce attr_once;                     // per template instance
-    CB_CUDA(once_per_device(attr_once, [&] { return cudaFuncSetAttribute(rs_onesweep<V, BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn); }));
-    const DebugKnobs knobs = debug_knobs();
-    CB_LAUNCH("rs_onesweep", stream,
-              rs_onesweep<V, BITS><<<(unsigned)ntiles, kRsThreads, dyn, stream>>>(
-                  kin, kout, vin, vout, n, shift, digit_base, b.tile_status, counter, status, epoch,
-                  knobs.spin_limit > 0 ? knobs.spin_limit : kSpinLimit, knobs.withhold,
-                  kRsAheadTiles));
-    return CONST_OK;
+    switch (b.items) {
+        case 4: return launch_tiles<V, BITS, 4>(kin, kout, vin, vout, n, shift, digit_base, b, counter, status, epoch, stream);
+        case 8: return launch_tiles<V, BITS, 8>(kin, kout, vin, vout, n, shift, digit_base, b, counter, status, epoch, stream);
+        default: return launch_tiles<V, BITS, kRsItems>(kin, kout, vin, vout, n, shift, digit_base, b, counter, status, epoch, stream);
+    }
 }
 
 // Sorts (keys, payload) by key.  The first pass reads the payload from `vals_src` (the caller's
@@ -1144,7 +1169,8 @@ const_status_t csf_build_impl(int order, const int64_t *dims, int64_t nnz, const
     {
         Scratch tmp(stream);
         const int64_t cp_blocks = (nnz + kCpTile - 1) / kCpTile;
-        const int64_t ntiles = (nnz + kRsTile - 1) / kRsTile;
+        const int items = tile_items(nnz);
+        const int64_t ntiles = (nnz + kRsThreads * items - 1) / (kRsThreads * items);
         constexpr size_t kHistBytes = sizeof(uint32_t) * kMaxPasses * kRsMaxBins;
         constexpr size_t kSmallBytes = kHistBytes + 256;
         auto room = [](size_t bytes) { return (bytes + 255) / 256 * 256; };
@@ -1210,7 +1236,7 @@ const_status_t csf_build_impl(int order, const int64_t *dims, int64_t nnz, const
             unsigned char *arena = nullptr;
             CB_CUDA(tmp.alloc((void **)&arena, room(kSmallBytes) + tiles_bytes + counts_bytes + 2 * keys_bytes + vals_bytes));
             unsigned char *small = arena;                                       // hist | counters | totals | status
-            SortBufs sb{nullptr, nullptr, nullptr, nullptr};
+            SortBufs sb{nullptr, nullptr, nullptr, nullptr, items};
             sb.tile_status = reinterpret_cast<unsigned long long *>(arena + room(kSmallBytes));
             uint32_t *block_counts = reinterpret_cast<uint32_t *>(arena + room(kSmallBytes) + tiles_bytes);
             uint64_t *keys = reinterpret_cast<uint64_t *>(arena + room(kSmallBytes) + tiles_bytes + counts_bytes);
@@ -1335,7 +1361,7 @@ const_status_t csf_build_noalloc_impl(int order, const int64_t *dims, int64_t nn
     uint32_t *block_counts = reinterpret_cast<uint32_t *>(base + kNaOffBlockCounts);
     SortBufs sb{reinterpret_cast<uint32_t *>(base + kNaOffHist), reinterpret_cast<uint32_t *>(base + kNaOffSmall),
                 reinterpret_cast<unsigned long long *>(base + kNaOffTileStatus),
-                reinterpret_cast<uint32_t *>(base + kNaOffSmall + 192)};
+                reinterpret_cast<uint32_t *>(base + kNaOffSmall + 192), kRsItems};
     uint32_t *totals = reinterpret_cast<uint32_t *>(base + kNaOffSmall + 64);
     int32_t *status = reinterpret_cast<int32_t *>(base + kNaOffSmall + 128);
     // everything that must start at zero: digit histograms, pass counters, level totals, status word

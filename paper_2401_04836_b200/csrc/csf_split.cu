@@ -100,6 +100,7 @@ template <int ORDER>
 __global__ void __launch_bounds__(kThreads) split_sample(PackArgs a, Tables t, uint32_t samples) {
     const uint32_t x = blockIdx.x * kThreads + threadIdx.x;
     bool bad = false;
+    start_next_kernel();
     if (x >= samples) return;
     const int64_t e = sample_at(x, samples, t.n);
     uint32_t c[ORDER];
@@ -158,6 +159,8 @@ __device__ __forceinline__ void fill_cells(uint32_t *cells, const uint64_t *spli
 __global__ void __launch_bounds__(kThreads) split_rank(Tables t, uint32_t samples) {
     extern __shared__ __align__(16) unsigned char smem[];
     uint64_t *all = reinterpret_cast<uint64_t *>(smem);
+    after_last_kernel();
+    start_next_kernel();
     for (uint32_t x = threadIdx.x; x < samples; x += kThreads) all[x] = t.samples[x];
     __syncthreads();
     const uint32_t me = blockIdx.x * (kThreads / 8) + threadIdx.x / 8, sub = threadIdx.x % 8;
@@ -198,8 +201,8 @@ __device__ __forceinline__ uint32_t take_chunk(const Tables &t, uint32_t b, uint
 // the phases of a tile, too few loads under way.  77 M: 822 us and 680 us for the two levels, 2.6 and 2.7 TB/s; a radix pass over the same
 // data takes 560.
 template <typename V, int ORDER>
-__global__ void __launch_bounds__(kThreads, tile_blocks(ORDER > 0)) split_tile(PackArgs a, Tables t, const uint64_t *__restrict__ kin,
-                                                                 const V *__restrict__ vin, uint64_t *__restrict__ kout, V *__restrict__ vout,
+__global__ void __launch_bounds__(kThreads, tile_blocks(ORDER > 0)) split_tile(PackArgs a, Tables t, const uint64_t *kin,
+                                                                 const V *vin, uint64_t *kout, V *vout,
                                                                  int spin_limit, int withhold) {
     constexpr bool kFirst = ORDER > 0;
     constexpr int kWays = kFirst ? kMaxBuckets : kMaxParts, kPer = kWays / kThreads;
@@ -219,6 +222,8 @@ __global__ void __launch_bounds__(kThreads, tile_blocks(ORDER > 0)) split_tile(P
     int shift = t.bucket_shift;
     int64_t base = (int64_t)blockIdx.x * kTile, end = t.n, stride = (int64_t)gridDim.x * kTile;
     if (!kFirst) {
+        after_last_kernel();
+        start_next_kernel();
         if (tid == 0) s_bad = *reinterpret_cast<volatile uint32_t *>(t.gave_up()) != 0;
         __syncthreads();
         if (s_bad || blockIdx.x >= *t.next_chunk) return;
@@ -257,7 +262,11 @@ __global__ void __launch_bounds__(kThreads, tile_blocks(ORDER > 0)) split_tile(P
         else at([&](int i) { return min(i * kThreads + tid, last); });
     };
     if (base >= end) return;
-    load(base);
+    load(base);                                                         // (first level: the caller's arrays, no earlier kernel's)
+    if (kFirst) {
+        after_last_kernel();
+        start_next_kernel();
+    }
     const int splits = kFirst ? t.buckets - 1 : (int)t.bucket_parts[b] - 1;
     const uint64_t *from_split = kFirst ? t.bucket_split : t.part_split + (size_t)b * kMaxParts;
     const uint32_t *from_cells = kFirst ? t.bucket_cells : t.part_cells + (size_t)b * kCells;
@@ -593,11 +602,13 @@ __device__ __forceinline__ void sort_block(K *buf, uint16_t *order, uint32_t *bi
 __device__ __forceinline__ uint32_t parts_of(uint32_t size) { return min((size + kPartMean - 1) / kPartMean, (uint32_t)kMaxParts); }
 
 // One block per bucket: where it starts, how many parts it gets, and their splitters from a sorted sample of it.
-__global__ void __launch_bounds__(kSampleThreads, 1) split_parts(Tables t, const uint64_t *__restrict__ keys) {
+__global__ void __launch_bounds__(kSampleThreads, 1) split_parts(Tables t, const uint64_t *keys) {
     extern __shared__ __align__(16) unsigned char smem[];
     uint64_t *keybuf = reinterpret_cast<uint64_t *>(smem);
     uint32_t *bins = reinterpret_cast<uint32_t *>(smem + (kSampleThreads * kItems + kPad) * sizeof(uint64_t));
     __shared__ uint64_t split[kMaxParts];
+    after_last_kernel();
+    start_next_kernel();
     if (*t.gave_up()) return;
     const int tid = threadIdx.x, b = blockIdx.x;
     uint32_t parts_before = 0, first_part;
@@ -638,6 +649,8 @@ __global__ void __launch_bounds__(kSampleThreads, 1) split_parts(Tables t, const
 
 // Where every part begins and what its keys lie between: one block per bucket, one thread per part.
 __global__ void __launch_bounds__(kWide) part_jobs(Tables t) {
+    after_last_kernel();
+    start_next_kernel();
     if (*t.gave_up()) return;
     const int tid = threadIdx.x, b = blockIdx.x;
     uint32_t before = 0, start, total;
@@ -659,8 +672,8 @@ __global__ void __launch_bounds__(kWide) part_jobs(Tables t) {
 // have beyond `base`, the root coordinate of the part's lowest key: 32 bits wherever those suffice.
 template <typename K, int NT, typename V, int ORDER>
 __device__ __forceinline__ void sort_part(unsigned char *smem, const Tables &t, const LevelShifts &ls, uint32_t leaf_mask, uint32_t g, const PartJob &job,
-                                          uint64_t base, const uint64_t (&key)[kItems], const V (&val)[kItems], V *__restrict__ vals_out,
-                                          int32_t *__restrict__ leaf_crd, uint64_t *__restrict__ list_keys, uint32_t *__restrict__ list_pos) {
+                                          uint64_t base, const uint64_t (&key)[kItems], const V (&val)[kItems], V *vals_out,
+                                          int32_t *leaf_crd, uint64_t *list_keys, uint32_t *list_pos) {
     constexpr int D = ORDER - 2;                                        // the level above the leaves
     constexpr int kRoom = kItems * NT, kWarps = NT / 32;
     __shared__ uint32_t opened[kWarps][D + 1];
@@ -746,12 +759,13 @@ __device__ __forceinline__ void sort_part(unsigned char *smem, const Tables &t, 
 // launch comes first and lets the other one start beside it.  What bounds it: instruction issue (230 thread instructions per nonzero, a
 // third of them in the search through the bins) at 30 warps per SM.  77 M: 914 us; 5 M uniform: 62 us.
 template <typename V, int ORDER, int NT>
-__global__ void __launch_bounds__(NT, 1024 / NT) part_sort(Tables t, LevelShifts ls, int leaf_bits, const uint64_t *__restrict__ keys,
-                                                          const V *__restrict__ vals, V *__restrict__ vals_out, int32_t *__restrict__ leaf_crd,
-                                                          uint64_t *__restrict__ list_keys, uint32_t *__restrict__ list_pos) {
+__global__ void __launch_bounds__(NT, 1024 / NT) part_sort(Tables t, LevelShifts ls, int leaf_bits, const uint64_t *keys,
+                                                          const V *vals, V *vals_out, int32_t *leaf_crd,
+                                                          uint64_t *list_keys, uint32_t *list_pos) {
     extern __shared__ __align__(16) unsigned char smem[];
     constexpr bool kLarge = NT == kWide;
-    if (kLarge) start_next_kernel();
+    if (kLarge) after_last_kernel();
+    start_next_kernel();
     if (!kLarge && blockIdx.x == gridDim.x - 1) after_last_kernel();     // this launch ends after the one beside it
     if (*t.gave_up()) return;
     const uint32_t leaf_mask = (uint32_t)((1ull << leaf_bits) - 1ull);
@@ -784,6 +798,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) part_sort(Tables t, LevelShifts
 template <int ORDER>
 __global__ void __launch_bounds__(kWide) part_scan(Tables t, LevelShifts ls) {
     constexpr int L = ORDER - 1;
+    after_last_kernel();
     if (*t.gave_up()) return;
     const int tid = threadIdx.x, b = blockIdx.x;
     const uint32_t parts = t.bucket_parts[b], g = t.part_base[b] + tid;
@@ -903,12 +918,12 @@ __global__ void __launch_bounds__(kNodeThreads) part_nodes(const PartInfo *__res
 // ------------------------------------------------------------------------------------------------
 // host
 // ------------------------------------------------------------------------------------------------
-// The splitter sort has eleven launches and two samplings where the radix sort has three and one per pass: it takes tensors of
-// at least 400 000 nonzeros whose count, times the passes beyond two, is 1.2 M or more.  Both sides around the line (build, us,
-// radix / splitters): 400 K nonzeros and five passes 133 / 117, four passes 103 / 110 (skewed) and 108 / 104; 740 K and three
-// passes 117 / 118; 800 K and four passes 128 / 116; 1.6 M and three passes 159 / 152; at 30 M between 0.64 and 0.78 of the time.
-// Above 110 M a bucket would need more parts than there are ways.
-constexpr int64_t kSplitMin = 400000, kSplitWork = 1200000, kSplitMax = 110000000;
+// The splitter sort has nine launches and two samplings where the radix sort has two and one per pass: it takes tensors of
+// at least 200 000 nonzeros whose count, times the passes beyond two, is 700 000 or more.  Both sides around the line (build, us,
+// radix / splitters, uniform; Zipf-sized slices cost the splitters some 10 us more): 200 K nonzeros and five passes 97 / 88, four 84 / 89;
+// 300 K and four 96 / 92, three 93 / 91; 500 K and three 99 / 93; 700 K and three 105 / 101; 2.5 M and five 221 / 153; at 30 M, with
+// both as they were before they started early, between 0.64 and 0.78 of the time.  Above 110 M a bucket would need more parts than there are ways.
+constexpr int64_t kSplitMin = 200000, kSplitWork = 700000, kSplitMax = 110000000;
 
 int bucket_count(int64_t nnz) {
     int k = 16;
@@ -967,9 +982,14 @@ const_status_t queue_tile(const char *name, unsigned blocks, const PackArgs &pa,
     static PerDeviceOnce once;                                           // per template instance
     CB_CUDA(allow_smem(split_tile<V, ORDER>, smem, once));
     const DebugKnobs knobs = debug_knobs();
-    CB_LAUNCH(name, stream, split_tile<V, ORDER><<<blocks, kThreads, smem, stream>>>(
-                                pa, t, kin, vin, kout, vout, knobs.spin_limit > 0 ? knobs.spin_limit : kSpinLimit, knobs.withhold));
-    return CONST_OK;
+    const int spins = knobs.spin_limit > 0 ? knobs.spin_limit : kSpinLimit, withhold = knobs.withhold;
+    // Blocks that stay for several tiles wait for an empty machine: started early they lie unevenly on the SMs, for good (build of
+    // 77 M: 2735 us against 2509; of 5 M: 224 against 226).
+    const bool stays = ORDER > 0 && (int64_t)blocks * kTile < t.n;
+    cudaError_t e = cudaSuccess;
+    CB_LAUNCH(name, stream, if (stays) split_tile<V, ORDER><<<blocks, kThreads, smem, stream>>>(pa, t, kin, vin, kout, vout, spins, withhold);
+                            else e = launch_early(split_tile<V, ORDER>, dim3(blocks), kThreads, smem, stream, pa, t, kin, vin, kout, vout, spins, withhold));
+    return e == cudaSuccess ? CONST_OK : CONST_ERR_CUDA;
 }
 
 template <typename V, int ORDER>
@@ -982,7 +1002,7 @@ const_status_t queue_sort(const PackArgs &pa, const KeyLayout &k, const LevelShi
     static PerDeviceOnce once_rank, once_parts, once_sort, once_large;
     CB_CUDA(allow_smem(split_rank, sizeof(uint64_t) * kMaxBuckets * kOverBuckets, once_rank));
     CB_LAUNCH("split_rank", stream,
-              split_rank<<<samples / (kThreads / 8), kThreads, sizeof(uint64_t) * samples, stream>>>(t, samples));
+              CB_CUDA(launch_early(split_rank, dim3(samples / (kThreads / 8)), kThreads, sizeof(uint64_t) * samples, stream, t, samples)));
     const_status_t s = queue_tile<V, ORDER>("split_buckets", (unsigned)std::min<int64_t>((t.n + kTile - 1) / kTile, 148 * tile_blocks(true)), pa, t, nullptr, vals, keys1, vals1, stream);
     if (s != CONST_OK) return s;
     // keys' pad, bins and their starts (see sort_block)
@@ -990,7 +1010,7 @@ const_status_t queue_sort(const PackArgs &pa, const KeyLayout &k, const LevelShi
     constexpr size_t smem_sample = with_bins(kSampleThreads * kItems * sizeof(uint64_t), kBins<kSampleThreads>);
     CB_CUDA(allow_smem(split_parts, smem_sample, once_parts));
     CB_LAUNCH("split_sample2", stream,
-              split_parts<<<(unsigned)at.buckets, kSampleThreads, smem_sample, stream>>>(t, keys1));
+              CB_CUDA(launch_early(split_parts, dim3((unsigned)at.buckets), kSampleThreads, smem_sample, stream, t, (const uint64_t *)keys1)));
     s = queue_tile<V, 0>("split_parts", at.max_chunks, pa, t, keys1, vals1, keys2, vals2, stream);
     if (s != CONST_OK) return s;
     constexpr size_t smem = with_bins(kTile * (sizeof(uint64_t) + sizeof(V)), kBins<kThreads>);
@@ -998,13 +1018,14 @@ const_status_t queue_sort(const PackArgs &pa, const KeyLayout &k, const LevelShi
     CB_CUDA(allow_smem(part_sort<V, ORDER, kThreads>, smem, once_sort));
     CB_CUDA(allow_smem(part_sort<V, ORDER, kWide>, smem_large, once_large));
     uint32_t *pos1 = reinterpret_cast<uint32_t *>(vals1);
-    CB_LAUNCH("part_jobs", stream, part_jobs<<<(unsigned)at.buckets, kWide, 0, stream>>>(t));
-    CB_LAUNCH("part_sort_large", stream, part_sort<V, ORDER, kWide><<<148, kWide, smem_large, stream>>>(
-                                             t, ls, k.bits[ORDER - 1], keys2, vals2, vals_out, leaf_crd, keys1, pos1));
+    CB_LAUNCH("part_jobs", stream, CB_CUDA(launch_early(part_jobs, dim3((unsigned)at.buckets), kWide, 0, stream, t)));
+    CB_LAUNCH("part_sort_large", stream,
+              CB_CUDA(launch_early(part_sort<V, ORDER, kWide>, dim3(148), kWide, smem_large, stream, t, ls, (int)k.bits[ORDER - 1],
+                                   (const uint64_t *)keys2, (const V *)vals2, vals_out, leaf_crd, keys1, pos1)));
     CB_LAUNCH("part_sort", stream,
               CB_CUDA(launch_early(part_sort<V, ORDER, kThreads>, dim3(at.max_parts), kThreads, smem, stream, t, ls, (int)k.bits[ORDER - 1],
                                    (const uint64_t *)keys2, (const V *)vals2, vals_out, leaf_crd, keys1, pos1)));
-    CB_LAUNCH("part_scan", stream, part_scan<ORDER><<<(unsigned)at.buckets, kWide, 0, stream>>>(t, ls));
+    CB_LAUNCH("part_scan", stream, CB_CUDA(launch_early(part_scan<ORDER>, dim3((unsigned)at.buckets), kWide, 0, stream, t, ls)));
     CB_CUDA(cudaGetLastError());
     return CONST_OK;
 }

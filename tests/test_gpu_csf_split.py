@@ -129,10 +129,10 @@ def test_chunk_wait_times_out_and_recovers():
 
 
 def test_which_sort_runs():
-    """The line: 400 000 nonzeros, and 1.2 M nonzeros times radix passes beyond two."""
-    for dims, nnz, split in (((2000, 3000, 4000), 590_000, False), ((2000, 3000, 4000), 610_000, True), ((512, 512, 512), 1_190_000, False),
-                             ((512, 512, 512), 1_210_000, True), ((20000, 20000, 20000, 20000), 390_000, False),
-                             ((20000, 20000, 20000, 20000), 410_000, True)):
+    """The line: 200 000 nonzeros, and 700 000 nonzeros times radix passes beyond two."""
+    for dims, nnz, split in (((2000, 3000, 4000), 340_000, False), ((2000, 3000, 4000), 360_000, True), ((512, 512, 512), 690_000, False),
+                             ((512, 512, 512), 710_000, True), ((20000, 20000, 20000, 20000), 190_000, False),
+                             ((20000, 20000, 20000, 20000), 210_000, True)):
         coords = [torch.randint(0, d, (nnz,), device="cuda", dtype=torch.int32) for d in dims]
         cb.const_profile_enable(True)
         try:
@@ -142,3 +142,16 @@ def test_which_sort_runs():
         names = cb.const_profile_read()
         cb.const_profile_enable(False)
         assert ("part_sort" in names) == split and ("rs_onesweep" in names) != split
+
+
+@pytest.mark.parametrize("nnz", [1023, 1025, 50_000, 199_999, 200_001, 410_001, 900_001])
+def test_tile_sizes_of_the_radix_sort(nnz):
+    """Tiles of 1024, 2048 and 4096 keys, whose passes start before the one before has ended."""
+    rng = np.random.default_rng(nnz)
+    for dims, dtype in (((331, 331, 64), np.float64), ((1201, 993, 1503), np.float32)):
+        op = gen._uniform_tensor(dims, nnz, rng, "pm1", dtype)
+        for order in ((0, 1, 2), (2, 0, 1)):
+            cb.const_debug_set(4, RADIX)
+            for _ in range(3):
+                h = build_csf(op, order)
+            assert_csf_equal(h, op, order)
