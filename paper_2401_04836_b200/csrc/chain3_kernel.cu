@@ -393,7 +393,7 @@ const_status_t run_ttmc3_fibres(const const_csf *X, const float *U, const float 
     const int64_t parts = (cost + kWave * most - 1) / (kWave * most) * kWave;
     Args a{walk::chain_of<float, 3>(X), U, V, Y, (int32_t)((cost + parts - 1) / parts), kWeight, kSliceWeight};
     if (X->nnz < 3000000 || X->nnz < 3 * X->n[1] || X->n[1] > 1024ll * X->n[0]) {
-        const walk::Cut cut = walk::cut_leaves(X->nnz, X->n[0], 1536, kResident, kSliceWeight, 3 * kSliceWeight);
+        const walk::Cut cut = walk::cut_leaves(X->nnz, X->n[0], 1536, kResident, kSliceWeight, 96);
         a.chunk = cut.chunk;
         a.weight = 0;
         a.slice_weight = cut.weight;

@@ -504,7 +504,9 @@ template <typename T, int ORDER, int RP>
 const_status_t launch_mttkrp(MttkrpArgs<T, ORDER> a, int tiles, cudaStream_t stream) {
     using S = MttkrpShape<T, ORDER, RP>;
     const int64_t nnz = a.x.n[ORDER - 1], slices = a.x.n[0];
-    const int32_t weight = RP <= 8 ? 64 : 48, least = ORDER == 4 || nnz < 200 * slices ? 4 * weight : 5 * S::W;
+    // (fp64, rank 32, order 4, slices Zipf 1.1 of 25 leaves, 800 000 of them, weights 32 / 48 / 64, us: 77 / 92 / 108; fp32, rank 8: 61 / 55 / 53)
+    constexpr int32_t weight = RP >= 32 && (ORDER == 4 || sizeof(T) == 8) ? 32 : RP >= 16 || sizeof(T) == 8 ? 48 : 64;
+    const int32_t least = ORDER == 4 ? 96 : nnz < 200 * slices ? 4 * weight : 5 * S::W;
     const dim3 grid(cut_blocks(a, a.x, cut_leaves(nnz, slices, 4096, S::FIT, weight, least)), (unsigned)tiles);
     return launch_on_cleared("chain3_kernel", mttkrp_kernel<T, ORDER, RP>, a, grid, kWarps * 32, 0, a.out, a.out_bytes, stream);
 }
@@ -514,8 +516,12 @@ const_status_t launch_ttmc3(Ttmc3Args<T> a, cudaStream_t stream) {
     constexpr int fit = Ttmc3Shape<T, R2, R3>::FIT;
     // where only four warps fit (fp64, 32 x 32) a wave is few chunks: shorter ones even out slices of different density
     const int64_t most = fit <= 4 ? 448 : 3072;
-    constexpr int32_t weight = R3 >= 32 || R2 * R3 >= 512 ? 64 : 96;
-    const dim3 grid(cut_blocks(a, a.x, cut_leaves(a.x.n[2], a.x.n[0], most, fit, weight, 3 * weight, true)));
+    // The more a leaf costs, the less a slice counts.  Slices Zipf 1.1, fp64, weights 32 / 64 / 96, us: 20 x 27, 400 000 leaves in slices of 100
+    // 106 / 118 / 127; 8 x 32, in slices of 25 61 / 76 / 93, but 4 M in slices of 400 and fibres of several leaves 225 / 212 / -; fp32, 16 x 8,
+    // 800 000 in slices of 25 73 / 64 / 61.
+    constexpr bool wide = R3 >= 32 || R2 * R3 >= 512;
+    constexpr int32_t weight = sizeof(T) == 8 && R2 * R3 > 64 ? (wide ? 48 : 80) : wide ? 64 : 96;
+    const dim3 grid(cut_blocks(a, a.x, cut_leaves(a.x.n[2], a.x.n[0], most, fit, weight, 96, true)));
     constexpr size_t dyn = sizeof(typename Ttmc3Shape<T, R2, R3>::Smem) * kWarps;
     static PerDeviceOnce attr_once;                     // per template instance
     CB_CUDA(once_per_device(attr_once, [&] { return cudaFuncSetAttribute(ttmc3_kernel<T, R2, R3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn); }));
@@ -553,7 +559,7 @@ const_status_t dispatch_mttkrp(const MttkrpArgs<T, ORDER> &a, int rp, int tiles,
 
 template <typename T>
 const_status_t launch_ttmc4(Ttmc4Args<T> a, cudaStream_t stream) {
-    const dim3 grid(cut_blocks(a, a.x, cut_leaves(a.x.n[3], a.x.n[0], 4096, Ttmc4Shape<T>::FIT, 64, 256)));
+    const dim3 grid(cut_blocks(a, a.x, cut_leaves(a.x.n[3], a.x.n[0], 4096, Ttmc4Shape<T>::FIT, 64, 64)));
     constexpr size_t dyn = sizeof(typename Ttmc4Shape<T>::Smem) * kWarps;
     static PerDeviceOnce attr_once;                     // per template instance
     CB_CUDA(once_per_device(attr_once, [&] { return cudaFuncSetAttribute(ttmc4_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn); }));

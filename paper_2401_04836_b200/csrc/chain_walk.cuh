@@ -482,9 +482,11 @@ inline int32_t chunk_leaves(int64_t nnz, int64_t slices, int64_t most, int fit, 
 // others.  Equal leaves against this, us: slices Zipf 1.1, TTMc 8 x 8, 1.5 M leaves in slices of 40: 219 / 77, 6 M of 400: 162 /
 // 106, 20 M of 333: 453 / 334; 32 x 32: 256 / 149, 406 / 353, 1124 / 954; order 4: 387 / 129, 407 / 301, 1080 / 853; MTTKRP rank 32: 119 / 56,
 // 122 / 103, 382 / 288; slices of equal size: within 1 % from 6 M on.  Not where slices are long anyway (from 4000 leaves on it gained
-// 1 to 3 % under Zipf 1.1 and lost 1 to 2 % on equal ones), nor where a chunk would cost less than `least`: the longer search shows, and
-// chunks are no whole windows any more (fp64 MTTKRP of order 4, 300 000 leaves in chunks of 154: 24.1 / 26.0; of order 3, 1.2 M equal
-// slices in chunks of two windows: 30.3 / 32.4; TTMc 32 x 16, 300 000 equal slices in chunks of 163: 27.9 / 32.0).
+// 1 to 3 % under Zipf 1.1 and lost 1 to 2 % on equal ones), nor where a chunk would cost less than `least`, which is no less than
+// `weight` (a warp may end up without leaves, a block may not).  Short chunks, equal leaves against this, us: 10 x 12, 200 000 leaves in
+// slices of 143, equal / Zipf 1.1: 25.9 / 28.6 against 21.3 / 19.8; fp64 18 x 23, 40 000 of 133: 35.2 / 33.9 against 24.9 / 23.6; order 4, TTMc,
+// 150 000: 0.93 of the time on average.  MTTKRP of order 3 keeps a longer `least` where slices are long: 400 000 equal ones of 100 in
+// chunks of 138 17.6 / 19.8.
 struct Cut { int32_t chunk, weight; };
 inline Cut cut_leaves(int64_t nnz, int64_t slices, int64_t most, int fit, int32_t weight, int least, bool one_window = false) {
     const int64_t wave = 148 * (int64_t)fit, cost = nnz + weight * slices;

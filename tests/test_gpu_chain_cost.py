@@ -31,11 +31,14 @@ def sizes_of(what, rng):
         return np.ones(60_000, np.int64)
     if what == "giant in front":                           # one slice over hundreds of warps, then a tail of short ones
         return np.concatenate([[180_000], rng.integers(1, 9, 20_000)])
+    if what.startswith("short chunks"):                    # of little more than a slice's own cost: some warps get no leaf
+        n, k = (110_000, 1800) if what == "short chunks" else (240_000, 4000)
+        return (n / 6 * np.arange(1, k + 1) ** -1.1).astype(np.int64) + rng.integers(1, 40, k)
     z = (180_000 * np.arange(1, 24_001) ** -1.1).astype(np.int64) + 1
     return np.concatenate([z[:1], rng.permutation(z[1:])])
 
 
-@pytest.mark.parametrize("what", ["ones", "giant in front", "zipf"])
+@pytest.mark.parametrize("what", ["ones", "giant in front", "zipf", "short chunks", "short chunks, more of them"])
 @pytest.mark.parametrize("family,order,ranks,dtype", [
     ("ttmc", 3, (8, 8), cb.F32), ("ttmc", 3, (16, 32), cb.F32), ("ttmc", 3, (20, 27), cb.F64), ("mttkrp", 3, (8,), cb.F32),
     ("mttkrp", 3, (32,), cb.F32), ("mttkrp", 4, (12,), cb.F64), ("ttmc", 4, (8, 8, 8), cb.F32), ("long fibres", 3, (16, 16), cb.F32)])
