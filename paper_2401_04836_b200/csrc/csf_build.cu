@@ -6,7 +6,8 @@
 //     single key sort orders the nonzeros lexicographically by the chosen mode order.
 //   * The value travels with its key as the sort payload, so no gather pass is needed afterwards and
 //     the sorted payload buffer *is* the leaf value array.
-//   * The sort is a least-significant-digit radix sort with 8-bit digits.  Each pass is one kernel:
+//   * The sort is a least-significant-digit radix sort with 8- or 9-bit digits.  Each pass is one kernel, which may start before
+//     the one before it has ended (its loads of what that one wrote are plain ones: cached read-only loads could move above the wait):
 //     tiles are ranked in shared memory, the tile's digit counts are chained to earlier tiles with a
 //     decoupled look-back (every spin is bounded and reports CONST_ERR_TIMEOUT), and keys are
 //     reordered in shared memory so that global stores run over consecutive addresses.
