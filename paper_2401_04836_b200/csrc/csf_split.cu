@@ -461,6 +461,11 @@ __device__ __forceinline__ uint32_t scan_bins(uint32_t *counts, uint16_t *start,
     return s_squares;
 }
 
+// Whether `other` comes in front of `x`, `earlier` settling it between equal ones.  32-bit numbers stay below 2^32 - 1 (part_sort), 64-bit
+// ones may be any.
+__device__ __forceinline__ bool in_front(uint32_t other, uint32_t x, bool earlier) { return other < x + earlier; }
+__device__ __forceinline__ bool in_front(uint64_t other, uint64_t x, bool earlier) { return earlier ? other <= x : other < x; }
+
 // Sorts m <= kItems x NT numbers of type K: thread x holds dist[i] for element i * NT + x.
 // They are dealt to bins of equal ranges -- where that leaves many in few bins, to new ones whose borders follow the counts of
 // the old -- and every one then finds its place among those of its bin (a warp works on neighbouring places, so its lanes meet
@@ -537,14 +542,14 @@ __device__ __forceinline__ void sort_block(K *buf, uint16_t *order, uint32_t *bi
 #pragma unroll
                 for (int z = 0; z < kTogether; ++z) {
                     const uint32_t q = from[z] + x;
-                    rank[i0 + z] += (q < to[z]) & (other[z] < dist[i0 + z] + (q < (uint32_t)((i0 + z) * NT + tid)));
+                    rank[i0 + z] += (q < to[z]) & in_front(other[z], dist[i0 + z], q < (uint32_t)((i0 + z) * NT + tid));
                 }
             }
 #pragma unroll
             for (int z = 0; z < kTogether; ++z) {
                 const uint32_t p = (i0 + z) * NT + tid;
                 if (p >= (uint32_t)m) continue;
-                for (uint32_t q = from[z] + kSlack; q < to[z]; ++q) rank[i0 + z] += buf[q] < dist[i0 + z] + (q < p);
+                for (uint32_t q = from[z] + kSlack; q < to[z]; ++q) rank[i0 + z] += in_front(buf[q], dist[i0 + z], q < p);
                 put(rank[i0 + z], dist[i0 + z], p);
             }
         }

@@ -86,6 +86,25 @@ def test_distributions(what):
     assert_same(op, (2, 0, 1))
 
 
+@pytest.mark.parametrize("tail", [3, 200, 500, 1300])
+@pytest.mark.parametrize("dims", [(2, 1 << 21, 1 << 21, 1 << 21), (4, 1 << 21, 1 << 21, 1 << 20), (1 << 16,) * 4])
+def test_largest_key_of_64_bits(dims, tail):
+    """The last corner of extents that fill 64 bits, in a part that begins in the first slice: its number is the largest there is."""
+    rng = np.random.default_rng(tail)
+    nnz = 300_000
+    for shrink in (0, 4, 8) * 2:                           # the tail, in the last slice, is spread over it or lies close to the corner
+        coords = [rng.integers(0, d, nnz).astype(np.int32) for d in dims]
+        coords[0][:] = 0
+        near = [d >> shrink for d in dims[2:]]
+        inside = rng.permutation(np.unique(rng.integers(0, near[0] * near[1], 2 * tail)))[:tail]
+        inside[0] = 0
+        for c, d, back in zip(coords, dims, (0, 0, inside // near[1], inside % near[1])):
+            c[:tail] = d - 1 - back
+        perm = rng.permutation(nnz)
+        op = gen.SparseOperand([c[perm] for c in coords], rng.standard_normal(nnz).astype(np.float32), dims)
+        assert_same(op, (0, 1, 2, 3))
+
+
 def test_errors_and_the_way_back_to_the_radix_sort():
     rng = np.random.default_rng(3)
     op = gen._uniform_tensor((300, 1000, 777), 500_003, rng, "pm1", np.float32)
