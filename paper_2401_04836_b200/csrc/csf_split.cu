@@ -637,8 +637,9 @@ __global__ void __launch_bounds__(kSampleThreads, 1) split_parts(Tables t, const
             dist[i] = lo;
             if (x < m) {
                 const uint32_t v = (uint32_t)sample_at(x, m, size);
-                const uint32_t ch = t.chunk_of[(size_t)b * t.chunk_rows + v / kChunk] - 1;
-                dist[i] = keys[(size_t)ch * kChunk + v % kChunk];
+                const uint32_t ch = t.chunk_of[(size_t)b * t.chunk_rows + v / kChunk];
+                if (ch) dist[i] = keys[(size_t)(ch - 1) * kChunk + v % kChunk];
+                else report(t.status(), CONST_ERR_TIMEOUT);             // not published (const_debug_set), and no tile had to wait for it
             }
         }
         sort_block<kSampleThreads>(keybuf, (uint16_t *)nullptr, bins, reinterpret_cast<uint16_t *>(bins + kBins<kSampleThreads> + 4), (int)m,

@@ -147,6 +147,20 @@ def test_chunk_wait_times_out_and_recovers():
     assert_csf_equal(build_csf(op, (0, 1, 2)), op, (0, 1, 2))
 
 
+@pytest.mark.parametrize("nnz", [1366, 2048, 4097])
+def test_chunks_that_nobody_waits_for(nnz):
+    """One coordinate throughout: one bucket of several parts, which up to a tile no other tile appends to.  Its chunk is not published, so
+    it cannot be sampled; published, the coordinate occurs twice."""
+    op = operand(np.full(nnz, 123_456_789), (300, 1000, 777))
+    for withhold, status in ((1, 8), (0, 4)):
+        cb.const_debug_set(4, SPLIT)
+        cb.const_debug_set(0, 200)
+        cb.const_debug_set(1, withhold)
+        with pytest.raises(cb.ConstError) as e:
+            build_csf(op, (0, 1, 2))
+        assert e.value.status == status
+
+
 def test_which_sort_runs():
     """The line: 200 000 nonzeros, and 700 000 nonzeros times radix passes beyond two."""
     for dims, nnz, split in (((2000, 3000, 4000), 340_000, False), ((2000, 3000, 4000), 360_000, True), ((512, 512, 512), 690_000, False),
