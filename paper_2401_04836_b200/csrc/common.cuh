@@ -128,7 +128,8 @@ private:
     } while (0)
 
 // Launches a kernel so that it may start before the kernel launched last has finished: every thread of it has to wait
-// (after_last_kernel) before it touches what that kernel, or one before it, writes or reads.
+// (after_last_kernel) before it touches what that kernel, or one before it, writes or reads.  (part_sort may acquire a word instead
+// that a kernel which has waited releases.)
 template <class... Params, class... Args>
 inline cudaError_t launch_early(void (*kernel)(Params...), dim3 grid, int threads, size_t smem, cudaStream_t stream, const Args &...args) {
     cudaLaunchConfig_t cfg = {};

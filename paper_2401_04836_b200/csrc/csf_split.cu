@@ -60,7 +60,7 @@ struct PartJob {                                   // a part as part_sort takes 
 
 struct Tables {
     uint32_t *result;                              // totals [0..3), parts [3], status [16], gave up [17]
-    uint32_t *arrived, *next_chunk, *large, *cursor, *part_count, *chunk_of;     // cleared
+    uint32_t *arrived, *next_chunk, *large, *ready, *cursor, *part_count, *chunk_of;     // cleared
     uint64_t *samples, *bucket_split, *part_split;
     uint32_t *bucket_cells, *part_cells;
     uint32_t *part_base, *bucket_parts, *part_owner, *part_nodes, *bucket_nodes;
@@ -762,20 +762,36 @@ __device__ __forceinline__ void sort_part(unsigned char *smem, const Tables &t, 
 }
 
 // NT = kThreads: a block takes one part of at most kTile nonzeros.  NT = kWide: few blocks go over the list of the larger ones; that
-// launch comes first and lets the other one start beside it.  What bounds it: instruction issue (230 thread instructions per nonzero, a
+// launch comes first and lets the other one start beside it, which therefore may not wait for its end to read what part_jobs and the
+// kernels before left: the wide launch, having waited for part_jobs, releases the number of parts, and a block that acquires it sees all
+// that the releasing thread could see.  A block that does not find it waits like any other, and so does the last one, so
+// that the narrow launch ends after the wide one (builds, us, this against all blocks waiting: 77 M 2600 / 2626, 5 M 241 / 251, 1 M of Zipf
+// slices 124 / 137).  What bounds it: instruction issue (230 thread instructions per nonzero, a
 // third of them in the search through the bins) at 30 warps per SM.  77 M: 914 us; 5 M uniform: 62 us.
 template <typename V, int ORDER, int NT>
 __global__ void __launch_bounds__(NT, 1024 / NT) part_sort(Tables t, LevelShifts ls, int leaf_bits, const uint64_t *keys,
                                                           const V *vals, V *vals_out, int32_t *leaf_crd,
-                                                          uint64_t *list_keys, uint32_t *list_pos) {
+                                                          uint64_t *list_keys, uint32_t *list_pos, int withhold) {
     extern __shared__ __align__(16) unsigned char smem[];
     constexpr bool kLarge = NT == kWide;
-    if (kLarge) after_last_kernel();
-    start_next_kernel();
-    if (!kLarge && blockIdx.x == gridDim.x - 1) after_last_kernel();     // this launch ends after the one beside it
-    if (*t.gave_up()) return;
+    auto parts = [&]() { return *t.gave_up() ? 0u : t.result[3]; };
+    uint32_t todo;
+    if (kLarge) {
+        after_last_kernel();
+        todo = *t.gave_up() ? 0u : *t.large;
+        if (blockIdx.x == 0 && threadIdx.x == 0 && !withhold)
+            asm volatile("st.release.gpu.global.u32 [%0], %1;" :: "l"(t.ready), "r"(parts() + 1) : "memory");
+        start_next_kernel();
+    } else {
+        start_next_kernel();
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(todo) : "l"(t.ready) : "memory");
+        if (todo == 0 || blockIdx.x == gridDim.x - 1) {
+            after_last_kernel();
+            todo = parts() + 1;
+        }
+        --todo;
+    }
     const uint32_t leaf_mask = (uint32_t)((1ull << leaf_bits) - 1ull);
-    const uint32_t todo = kLarge ? *t.large : t.result[3];
     for (uint32_t turn = blockIdx.x; turn < todo; turn += gridDim.x) {
         const uint32_t g = kLarge ? t.large_parts[turn] : turn;
         const PartJob job = t.jobs[g];
@@ -1024,13 +1040,14 @@ const_status_t queue_sort(const PackArgs &pa, const KeyLayout &k, const LevelShi
     CB_CUDA(allow_smem(part_sort<V, ORDER, kThreads>, smem, once_sort));
     CB_CUDA(allow_smem(part_sort<V, ORDER, kWide>, smem_large, once_large));
     uint32_t *pos1 = reinterpret_cast<uint32_t *>(vals1);
+    const int withhold = debug_knobs().withhold;
     CB_LAUNCH("part_jobs", stream, CB_CUDA(launch_early(part_jobs, dim3((unsigned)at.buckets), kWide, 0, stream, t)));
     CB_LAUNCH("part_sort_large", stream,
               CB_CUDA(launch_early(part_sort<V, ORDER, kWide>, dim3(148), kWide, smem_large, stream, t, ls, (int)k.bits[ORDER - 1],
-                                   (const uint64_t *)keys2, (const V *)vals2, vals_out, leaf_crd, keys1, pos1)));
+                                   (const uint64_t *)keys2, (const V *)vals2, vals_out, leaf_crd, keys1, pos1, withhold)));
     CB_LAUNCH("part_sort", stream,
               CB_CUDA(launch_early(part_sort<V, ORDER, kThreads>, dim3(at.max_parts), kThreads, smem, stream, t, ls, (int)k.bits[ORDER - 1],
-                                   (const uint64_t *)keys2, (const V *)vals2, vals_out, leaf_crd, keys1, pos1)));
+                                   (const uint64_t *)keys2, (const V *)vals2, vals_out, leaf_crd, keys1, pos1, withhold)));
     CB_LAUNCH("part_scan", stream, CB_CUDA(launch_early(part_scan<ORDER>, dim3((unsigned)at.buckets), kWide, 0, stream, t, ls)));
     CB_CUDA(cudaGetLastError());
     return CONST_OK;
@@ -1067,6 +1084,7 @@ const_status_t split_sort(const PackArgs &pa, const KeyLayout &k, int64_t nnz, c
     t.arrived = t.result + 32;
     t.next_chunk = t.result + 48;
     t.large = t.result + 56;
+    t.ready = t.result + 60;
     t.large_parts = u32(at.large_parts);
     t.cursor = u32(at.cursor);
     t.part_count = u32(at.part_count);

@@ -161,6 +161,16 @@ def test_chunks_that_nobody_waits_for(nnz):
         assert e.value.status == status
 
 
+@pytest.mark.parametrize("nnz", [1, 500, 2048])
+def test_parts_are_sorted_without_the_early_word(nnz):
+    """Signals withheld where nothing has to wait for a chunk: the blocks that sort parts are not told that they may start, and wait."""
+    op = operand(np.arange(nnz, dtype=np.int64) * 99_991, (300, 1000, 777))
+    cb.const_debug_set(4, SPLIT)
+    cb.const_debug_set(1, 1)
+    assert_csf_equal(build_csf(op, (0, 1, 2)), op, (0, 1, 2))
+    assert_csf_equal(build_csf(op, (2, 0, 1)), op, (2, 0, 1))
+
+
 def test_which_sort_runs():
     """The line: 200 000 nonzeros, and 700 000 nonzeros times radix passes beyond two."""
     for dims, nnz, split in (((2000, 3000, 4000), 340_000, False), ((2000, 3000, 4000), 360_000, True), ((512, 512, 512), 690_000, False),
