@@ -332,8 +332,9 @@ const char *const_status_string(const_status_t status);
  * what = 3: value != 0 makes every request of const_execute for optional scratch (padded factors, the intermediate of the
  * two-contraction network's matrix form), and of const_csf_build for the splitter sort's, fail for want of memory, so that the
  * path that needs none (less) runs;
- * what = 4: how const_csf_build sorts, whatever the size (0: chosen by size; 1: radix passes; 2: splitters).  Process-wide; not
- * for production use.  CONST_ERR_INVALID_ARG for an unknown `what` or a value outside [0, 2^31).
+ * what = 4: how const_csf_build sorts, whatever the size (0: chosen by size; 1: radix passes; 2: splitters; 3 and 4: splitters, and
+ * then radix passes, as if a part had outgrown its room (3) or no memory were left for the arrays of the upper levels (4)).
+ * Process-wide; not for production use.  CONST_ERR_INVALID_ARG for an unknown `what` or a value outside [0, 2^31) (what = 4: above 4).
  */
 const_status_t const_debug_set(int what, int64_t value);
 

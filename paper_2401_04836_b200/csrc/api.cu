@@ -445,7 +445,10 @@ const_status_t const_debug_set(int what, int64_t value) {
         case 1: g_withhold.store(value != 0); return CONST_OK;
         case 2: g_variant.store((int)value); return CONST_OK;
         case 3: g_no_scratch.store(value != 0); return CONST_OK;
-        case 4: g_build_path.store((int)value); return CONST_OK;
+        case 4:
+            if (value > 4) return CONST_ERR_INVALID_ARG;
+            g_build_path.store((int)value);
+            return CONST_OK;
     }
     return CONST_ERR_INVALID_ARG;
 }

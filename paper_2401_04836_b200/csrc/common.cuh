@@ -157,7 +157,7 @@ struct DebugKnobs {
     int withhold;        // nonzero: producers do not publish / the tensor-core stage does not commit
     int variant;         // kernel variant to launch where a launcher keeps several for measurement (0: the default)
     int no_scratch;      // nonzero: scratch_alloc finds no memory
-    int build_path;      // sort of the CSF build: 0 by size, 1 radix, 2 splitters
+    int build_path;      // sort of the CSF build: 0 by size, 1 radix, 2 splitters; then, as if 3 a part had outgrown its room, 4 memory had run out
 };
 DebugKnobs debug_knobs();
 

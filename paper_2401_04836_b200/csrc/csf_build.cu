@@ -1202,11 +1202,12 @@ const_status_t csf_build_impl(int order, const int64_t *dims, int64_t nnz, const
             return CONST_OK;
         };
 
-        // large tensors: splitters; `done` stays false where that sort gave up or found no memory
+        // large tensors: splitters; `done` stays false where that sort gave up or there was no memory for it or beside it
         bool done = false;
         auto by_splitters = [&]() -> const_status_t {
             unsigned char *arena = nullptr;
-            if (debug_knobs().no_scratch || tmp.alloc((void **)&arena, split_bytes(nnz, dtype)) != cudaSuccess) {
+            const DebugKnobs knobs = debug_knobs();
+            if (knobs.no_scratch || tmp.alloc((void **)&arena, split_bytes(nnz, dtype)) != cudaSuccess) {
                 cudaGetLastError();
                 return CONST_OK;
             }
@@ -1217,11 +1218,17 @@ const_status_t csf_build_impl(int order, const int64_t *dims, int64_t nnz, const
             CB_CUDA(cudaMemcpyAsync(h_small, sort.result, sizeof(h_small), cudaMemcpyDeviceToHost, stream));
             CB_CUDA(wait_stream(stream));
             if (h_small[16] != 0) return (const_status_t)h_small[16];
-            if (h_small[17] != 0) {
+            if (h_small[17] != 0 || knobs.build_path == 3) {
                 tmp.release(arena);
                 return CONST_OK;
             }
-            s = size_arrays(h_small);
+            s = knobs.build_path == 4 ? CONST_ERR_CUDA : size_arrays(h_small);
+            if (s == CONST_ERR_CUDA) {                   // no memory for the arrays beside this arena: beside the radix sort's there may be
+                cudaGetLastError();
+                csf->arena = nullptr;
+                tmp.release(arena);
+                return CONST_OK;
+            }
             if (s != CONST_OK) return s;
             done = true;
             return split_scatter(sort, arr, csf->slice_ptr, h_small[3], stream);

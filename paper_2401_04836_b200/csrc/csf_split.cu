@@ -1070,7 +1070,7 @@ const_status_t queue_order(const PackArgs &pa, const KeyLayout &k, const LevelSh
 bool split_covers(int64_t nnz, const KeyLayout &k) {
     const int path = debug_knobs().build_path;
     if (nnz < 1 || nnz > kSplitMax || path == 1) return false;
-    return path == 2 || (nnz >= kSplitMin && nnz * (k.digits.passes - 2) >= kSplitWork);
+    return path >= 2 || (nnz >= kSplitMin && nnz * (k.digits.passes - 2) >= kSplitWork);
 }
 
 size_t split_bytes(int64_t nnz, const_dtype_t dtype) { return Layout(nnz, dtype == CONST_F32 ? 4 : 8).bytes; }

@@ -133,6 +133,24 @@ def test_errors_and_the_way_back_to_the_radix_sort():
     assert_csf_equal(h, op, (0, 1, 2))
 
 
+@pytest.mark.parametrize("path", [3, 4])
+def test_the_radix_sort_runs_behind_the_splitters(path):
+    """A valid tensor whose build gives up (3), or finds no memory for the upper levels beside its arena (4), when the values and leaf
+    coordinates have been written already."""
+    rng = np.random.default_rng(5)
+    for dims, dtype in (((300, 1000, 777), np.float32), ((70, 80, 90, 100), np.float64), ((5003, 3001), np.float32)):
+        op = gen._uniform_tensor(dims, 300_007, rng, "pm1", dtype)
+        cb.const_debug_set(4, path)
+        cb.const_profile_enable(True)
+        h = build_csf(op, tuple(range(len(dims))))
+        names = cb.const_profile_read()
+        cb.const_profile_enable(False)
+        assert "part_sort" in names and "rs_onesweep" in names and "part_nodes" not in names
+        assert_csf_equal(h, op, tuple(range(len(dims))))
+    with pytest.raises(cb.ConstError):
+        cb.const_debug_set(4, 5)
+
+
 def test_chunk_wait_times_out_and_recovers():
     rng = np.random.default_rng(4)
     op = gen._uniform_tensor((300, 1000, 777), 300_007, rng, "pm1", np.float32)
