@@ -81,11 +81,11 @@ inline void launch_pack_hist(const PackArgs &pa, int64_t nnz, const DigitPlan &d
 // ------------------------------------------------------------------------------------------------
 constexpr int kRsThreads = 256;
 constexpr int kRsItems = 16;
-constexpr int kRsTile = kRsThreads * kRsItems;     // 4096 keys per tile; at least 1024, see tile_items
+constexpr int kRsTile = kRsThreads * kRsItems;     // 4096 keys per tile; 1024 and 2048 too, see tile_items
 constexpr int kRsWarps = kRsThreads / 32;
 constexpr int kSpinLimit = 1 << 21;
 // Distance, in tiles, of the pass kernel's L2 prefetch: half a wave of its resident blocks (148 SMs x 3).  Measured on
-// 38.5 M nonzeros: none 0.326 ms per pass, 56 to 444 tiles 0.311 ms, 888 and more 0.336 ms (evicted before use).
+// 38.5 M nonzeros in tiles of 4096: none 0.326 ms per pass, 56 to 444 tiles 0.311 ms, 888 and more 0.336 ms (evicted before use).
 constexpr int kRsAheadTiles = 222;
 // A tile's state for one digit is one 64-bit word: the count in the low half; in the high half
 // (pass number << 2) | flag, flag 1 = the tile's own count, flag 2 = the count summed over this and
@@ -131,16 +131,16 @@ __global__ void __launch_bounds__(kRsThreads, 3) rs_onesweep(const uint64_t *kin
     const int64_t left = n - tile_base;
     const int nvalid = left < kTile ? (int)left : kTile;
 
-    // A tile that will be taken soon (half a wave of resident blocks ahead) is requested into L2 now, so that the
-    // loads of the block that takes it find it there instead of in DRAM.
+    // A tile that will be taken soon (kRsAheadTiles) is requested into L2 now, so that the loads of the block that takes it find it
+    // there instead of in DRAM.  (Sorts in tiles of 1024 keys are too small to have one.)
     {
         const int64_t ahead = tile_base + (int64_t)ahead_tiles * kTile;
-        const int64_t kb = ahead * (int64_t)sizeof(uint64_t) + (int64_t)threadIdx.x * 128;       // keys: 32 KB = 256 lines
-        if (ahead + kTile <= n) {
-            asm volatile("prefetch.global.L2 [%0];" :: "l"(reinterpret_cast<const char *>(kin) + kb));
-            const int64_t vb = ahead * (int64_t)sizeof(V) + (int64_t)threadIdx.x * 128;
-            if ((int64_t)threadIdx.x * 128 < (int64_t)kTile * (int64_t)sizeof(V))
-                asm volatile("prefetch.global.L2 [%0];" :: "l"(reinterpret_cast<const char *>(vin) + vb));
+        if (ahead + kTile <= n) {                     // one line of 128 bytes per thread, as far as the tile goes
+            const int line = (int)threadIdx.x * 128;
+            if (line < kTile * (int)sizeof(uint64_t))
+                asm volatile("prefetch.global.L2 [%0];" :: "l"(reinterpret_cast<const char *>(kin + ahead) + line));
+            if (line < kTile * (int)sizeof(V))
+                asm volatile("prefetch.global.L2 [%0];" :: "l"(reinterpret_cast<const char *>(vin + ahead) + line));
         }
     }
 
