@@ -8,7 +8,8 @@
 //       for a,b: Y[i,a,b] += U[j,a] * t[b]          (consumer contraction; MTTKRP: A[i,r] += B[j,r] * t[r])
 // and, for order 4, with one more producer: P[c] += X[i,j,k,l] * W[l,c];  Q[b,c] += V[k,b] * P[c].
 //
-// Every warp owns an equal run of the tensor's leaves and walks it in windows that it stages as flat records
+// Every warp owns a run of the tensor's leaves -- of equal cost, a slice counting as some leaves beyond its own, or of equal
+// leaves (cut_leaves) -- and walks it in windows that it stages as flat records
 // (chain_walk.cuh), on its own: no work list, no slice too large or too small.  The warps of a block meet only where the
 // whole block lies in one slice, to add up their results.
 //   producer   Lane groups (one 128-bit load per lane and factor row) work through equal runs of the window's

@@ -6,7 +6,7 @@
 //      counts, whatever the distribution (split_sample, split_rank);
 //   2. every tile packs its coordinates, deals them to the buckets and appends each run to its bucket, which is a list of
 //      fixed chunks that are handed out as it grows (split_tile, first level);
-//   3. per bucket a sample gives splitters for parts of about kPartMean nonzeros (split_parts), and every chunk deals its
+//   3. per bucket a sample gives splitters for parts of about kPartMean nonzeros (split_sample2), and every chunk deals its
 //      nonzeros to the parts, each of which has room for kPartRoom (split_tile, second level);
 //   4. a block sorts a part in shared memory, writes values and leaf coordinates to their final places and lists the nodes that
 //      open at the level above the leaves (part_sort); a scan numbers the nodes (part_scan), and once the host has sized the
@@ -47,7 +47,7 @@ constexpr int kPartBits = 9;                       // part_owner: bucket << kPar
 static_assert(kMaxParts <= 1 << kPartBits && kMaxParts <= kWide && kMaxBuckets <= kWide && kTile <= kChunk, "one thread per part");
 
 struct PartInfo {
-    uint64_t first, last, prev;                    // keys: the part's ends, and the last one in front of it
+    uint64_t first, last;                          // keys: the part's ends
     uint32_t count, start;                         // nonzeros, position of the first one
     uint32_t opened[kMaxOrder - 1];                // nodes that open in the part, its first element counted at every level
     uint32_t cont;                                 // bit l: at level l the first element goes on with a node of an earlier part
@@ -71,7 +71,7 @@ struct Tables {
     uint64_t key_max;
     int64_t n;
     int buckets, bucket_shift, chunk_rows;
-    uint32_t max_chunks, max_parts;
+    uint32_t max_chunks;
     __device__ __forceinline__ int32_t *status() const { return reinterpret_cast<int32_t *>(result + 16); }
     __device__ __forceinline__ uint32_t *gave_up() const { return result + 17; }
 };
@@ -607,7 +607,7 @@ __device__ __forceinline__ void sort_block(K *buf, uint16_t *order, uint32_t *bi
 __device__ __forceinline__ uint32_t parts_of(uint32_t size) { return min((size + kPartMean - 1) / kPartMean, (uint32_t)kMaxParts); }
 
 // One block per bucket: where it starts, how many parts it gets, and their splitters from a sorted sample of it.
-__global__ void __launch_bounds__(kSampleThreads, 1) split_parts(Tables t, const uint64_t *keys) {
+__global__ void __launch_bounds__(kSampleThreads, 1) split_sample2(Tables t, const uint64_t *keys) {
     extern __shared__ __align__(16) unsigned char smem[];
     uint64_t *keybuf = reinterpret_cast<uint64_t *>(smem);
     uint32_t *bins = reinterpret_cast<uint32_t *>(smem + (kSampleThreads * kItems + kPad) * sizeof(uint64_t));
@@ -837,7 +837,6 @@ __global__ void __launch_bounds__(kWide) part_scan(Tables t, LevelShifts ls) {
             cont |= (uint32_t)same << l;
             count[l] = info.opened[l] - same;
         }
-        info.prev = prev;
         info.cont = cont;
     }
 #pragma unroll
@@ -850,20 +849,10 @@ __global__ void __launch_bounds__(kWide) part_scan(Tables t, LevelShifts ls) {
     if (!last_block(t.arrived + 1)) return;
 #pragma unroll
     for (int l = 0; l < L; ++l) {
-        uint32_t c[1], sum = 0, total;
-#pragma unroll
-        for (int q = 0; q < 1; ++q) {
-            const int x = tid * (1) + q;
-            c[q] = x < t.buckets ? __ldcg(t.bucket_nodes + x * (kMaxOrder - 1) + l) : 0;
-            sum += c[q];
-        }
-        uint32_t at = block_scan<kWide>(sum, total);
-#pragma unroll
-        for (int q = 0; q < 1; ++q) {
-            const int x = tid * (1) + q;
-            if (x < t.buckets) t.bucket_nodes[x * (kMaxOrder - 1) + l] = at;
-            at += c[q];
-        }
+        uint32_t total;
+        const uint32_t in_bucket = tid < t.buckets ? __ldcg(t.bucket_nodes + tid * (kMaxOrder - 1) + l) : 0;
+        const uint32_t at = block_scan<kWide>(in_bucket, total);
+        if (tid < t.buckets) t.bucket_nodes[tid * (kMaxOrder - 1) + l] = at;
         if (tid == 0) t.result[l] = total;
     }
 }
@@ -1021,7 +1010,7 @@ const_status_t queue_sort(const PackArgs &pa, const KeyLayout &k, const LevelShi
     uint64_t *keys1 = reinterpret_cast<uint64_t *>(arena + at.keys1), *keys2 = reinterpret_cast<uint64_t *>(arena + at.keys2);
     V *vals1 = reinterpret_cast<V *>(arena + at.vals1), *vals2 = reinterpret_cast<V *>(arena + at.vals2);
     CB_LAUNCH("split_sample", stream, split_sample<ORDER><<<(samples + kThreads - 1) / kThreads, kThreads, 0, stream>>>(pa, t, samples));
-    static PerDeviceOnce once_rank, once_parts, once_sort, once_large;
+    static PerDeviceOnce once_rank, once_sample, once_sort, once_large;
     CB_CUDA(allow_smem(split_rank, sizeof(uint64_t) * kMaxBuckets * kOverBuckets, once_rank));
     CB_LAUNCH("split_rank", stream,
               CB_CUDA(launch_early(split_rank, dim3(samples / (kThreads / 8)), kThreads, sizeof(uint64_t) * samples, stream, t, samples)));
@@ -1030,9 +1019,9 @@ const_status_t queue_sort(const PackArgs &pa, const KeyLayout &k, const LevelShi
     // keys' pad, bins and their starts (see sort_block)
     constexpr auto with_bins = [](size_t bytes, int bins) { return bytes + kPad * sizeof(uint64_t) + (bins + 4) * sizeof(uint32_t) + (bins + 8) * sizeof(uint16_t); };
     constexpr size_t smem_sample = with_bins(kSampleThreads * kItems * sizeof(uint64_t), kBins<kSampleThreads>);
-    CB_CUDA(allow_smem(split_parts, smem_sample, once_parts));
+    CB_CUDA(allow_smem(split_sample2, smem_sample, once_sample));
     CB_LAUNCH("split_sample2", stream,
-              CB_CUDA(launch_early(split_parts, dim3((unsigned)at.buckets), kSampleThreads, smem_sample, stream, t, (const uint64_t *)keys1)));
+              CB_CUDA(launch_early(split_sample2, dim3((unsigned)at.buckets), kSampleThreads, smem_sample, stream, t, (const uint64_t *)keys1)));
     s = queue_tile<V, 0>("split_parts", at.max_chunks, pa, t, keys1, vals1, keys2, vals2, stream);
     if (s != CONST_OK) return s;
     constexpr size_t smem = with_bins(kTile * (sizeof(uint64_t) + sizeof(V)), kBins<kThreads>);
@@ -1109,7 +1098,6 @@ const_status_t split_sort(const PackArgs &pa, const KeyLayout &k, int64_t nnz, c
     t.bucket_shift = std::max(0, k.total_bits - 10);
     t.chunk_rows = at.chunk_rows;
     t.max_chunks = at.max_chunks;
-    t.max_parts = at.max_parts;
     LevelShifts ls;
     ls.order = pa.order;
     for (int l = 0; l < kMaxOrder; ++l) ls.shift[l] = k.shift[l];
