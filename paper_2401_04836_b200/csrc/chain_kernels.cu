@@ -515,14 +515,17 @@ const_status_t launch_mttkrp(MttkrpArgs<T, ORDER> a, int tiles, cudaStream_t str
 template <typename T, int R2, int R3>
 const_status_t launch_ttmc3(Ttmc3Args<T> a, cudaStream_t stream) {
     constexpr int fit = Ttmc3Shape<T, R2, R3>::FIT;
-    // where only four warps fit (fp64, 32 x 32) a wave is few chunks: shorter ones even out slices of different density
-    const int64_t most = fit <= 4 ? 448 : 3072;
+    // Only four warps fit (fp64, 32 x 32): six waves, nine where slices are long.  Chunks that cost 448 throughout / equal leaves in
+    // chunks of 256 to 3072 / this, us: slices of equal size, 1.5 M leaves in slices of 5 2147 / 1928 / 1941, 8 M of 100 2265 / 2079 /
+    // 2070, 8 M of 1000 1661 / 1510 / 1529; slices Zipf 1.1, 400 000 of 25 196 / 272 / 178, 8 M of 1000 1163 / 1351 / 1166 (in six
+    // waves 1232); geometric mean over 258 tensors, this to 448 0.97, to equal leaves 0.84.
+    const int even = fit > 4 ? 1 : a.x.n[2] >= 700 * (int64_t)a.x.n[0] ? 9 : 6;
     // The more a leaf costs, the less a slice counts.  Slices Zipf 1.1, fp64, weights 32 / 64 / 96, us: 20 x 27, 400 000 leaves in slices of 100
     // 106 / 118 / 127; 8 x 32, in slices of 25 61 / 76 / 93, but 4 M in slices of 400 and fibres of several leaves 225 / 212 / -; fp32, 16 x 8,
     // 800 000 in slices of 25 73 / 64 / 61.
     constexpr bool wide = R3 >= 32 || R2 * R3 >= 512;
     constexpr int32_t weight = sizeof(T) == 8 && R2 * R3 > 64 ? (wide ? 48 : 80) : wide ? 64 : 96;
-    const dim3 grid(cut_blocks(a, a.x, cut_leaves(a.x.n[2], a.x.n[0], most, fit, weight, 96, true)));
+    const dim3 grid(cut_blocks(a, a.x, cut_leaves(a.x.n[2], a.x.n[0], 3072, fit, weight, 96, true, even)));
     constexpr size_t dyn = sizeof(typename Ttmc3Shape<T, R2, R3>::Smem) * kWarps;
     static PerDeviceOnce attr_once;                     // per template instance
     CB_CUDA(once_per_device(attr_once, [&] { return cudaFuncSetAttribute(ttmc3_kernel<T, R2, R3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn); }));

@@ -487,12 +487,16 @@ inline int32_t chunk_leaves(int64_t nnz, int64_t slices, int64_t most, int fit, 
 // slices of 143, equal / Zipf 1.1: 25.9 / 28.6 against 21.3 / 19.8; fp64 18 x 23, 40 000 of 133: 35.2 / 33.9 against 24.9 / 23.6; order 4, TTMc,
 // 150 000: 0.93 of the time on average.  MTTKRP of order 3 keeps a longer `least` where slices are long: 400 000 equal ones of 100 in
 // chunks of 138 17.6 / 19.8.
+// Where a wave is few warps, one of long chunks leaves slices of different density uneven: up to `even` waves then, in chunks of no less
+// than 448 leaves each (equal leaves: in any number of waves).
 struct Cut { int32_t chunk, weight; };
-inline Cut cut_leaves(int64_t nnz, int64_t slices, int64_t most, int fit, int32_t weight, int least, bool one_window = false) {
+inline Cut cut_leaves(int64_t nnz, int64_t slices, int64_t most, int fit, int32_t weight, int least, bool one_window = false, int even = 1) {
+    constexpr int64_t kShort = 448;
     const int64_t wave = 148 * (int64_t)fit, cost = nnz + weight * slices;
-    const int64_t waves = (cost + wave * most - 1) / (wave * most), c = (cost + wave * waves - 1) / (wave * waves);
+    const int64_t waves = std::max<int64_t>((cost + wave * most - 1) / (wave * most), std::min<int64_t>(even, (nnz + wave * kShort - 1) / (wave * kShort)));
+    const int64_t c = (cost + wave * waves - 1) / (wave * waves);
     if (c >= least && nnz < 3000 * slices) return Cut{(int32_t)((c + 7) / 8 * 8), weight};
-    return Cut{chunk_leaves(nnz, slices, most, fit, one_window), 0};
+    return Cut{chunk_leaves(nnz, slices, even > 1 ? kShort : most, fit, one_window), 0};
 }
 
 // Clears `out` ("R[*] = 0" precedes the nest; bytes = 0: the launch before has done that) and launches the kernel so that it starts while the clearing still runs: it
