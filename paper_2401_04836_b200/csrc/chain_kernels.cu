@@ -715,8 +715,10 @@ const_status_t run_ttmc3(const const_csf *X, const float *U, const float *V, int
     // at R2 = 32: 100 000 leaves in fibres of one, 16 x 16, slices of 1 / 4 / 16 / 64: 106 / 95, 51 / 51, 23 / 27, 17.4 / 18.3;
     // 300 000: 351 / 264, 143 / 128, 47 / 54, 27 / 30; 32 x 32, 300 000: 612 / 407, 238 / 168, 83 / 69, 49 / 42; 493 000 in
     // fibres of 2.3 and slices of 425: 8 x 8 18.6 / 17.3, 8 x 32 29.3 / 25.3, 32 x 16 31.8 / 26.3.
-    // With slices counted at their cost on both sides: slices of less than a hundred leaves, 16 x 16, walk / chain3_kernel, 1 M in
-    // fibres of 3.3: 54 / 67, of 20: 50 / 46; 4 M of 10.7: 135 / 157; long slices, 16 M in fibres of 3.2: 8 x 8 262 / 240, 16 x 16 333 / 354, 8 x 32
+    // With slices counted at their cost on both sides: slices of less than a hundred leaves, 16 x 16, walk / chain3_kernel, slices of 40,
+    // 4 M in fibres of 11: 174 / 228 (Zipf 1.1: 171 / 185; but slices of 25, 9 M of 12, 8 x 16, Zipf 1.1: 504 / 479), 1 M of 18, Zipf 1.1: 50 / 52; slices of 85, of 11, 1 M: 37.1 / 35.9 (Zipf 1.1:
+    // 34.6 / 41.0), 4 M: 117 / 123; at 32 x 8 slices of 600, 4 M of 1.6: 102 / 101, of 2.2: 97 / 86, 1 M of 1.6: 36 / 33, of 2.2, Zipf
+    // 1.1: 33 / 34; long slices, 16 M in fibres of 3.2: 8 x 8 262 / 240, 16 x 16 333 / 354, 8 x 32
     // 418 / 483, 32 x 8 379 / 307; of 4.1: 258 / 205, 313 / 305, 393 / 410, 365 / 265.
     const double per_fibre = (double)X->nnz / (double)X->n[1], per_slice = (double)X->nnz / (double)X->n[0];
     const bool middle = X->nnz >= 100000 && per_slice >= 16 && R2 < 32;
@@ -725,7 +727,7 @@ const_status_t run_ttmc3(const const_csf *X, const float *U, const float *V, int
         line = 2.5;
         if (R2 * R3 >= 1024) line = 1.8;
         else if (R2 == 32 && R3 == 8) line = 1.9;
-        else if (R2 < 32 && R3 < 32 && per_slice < 100) line = 8.0;
+        else if (R2 < 32 && R3 < 32 && per_slice < 100) line = per_slice < 64 ? 20.0 : 8.0;
         else if (R2 < 32 && X->nnz >= 3000000) line = R3 == 32 || R2 * R3 == 256 ? 3.5 : 2.5;
     }
     if (per_fibre > line) return run_ttmc3_fibres(X, U, V, R2, R3, Y, n_rows, stream);

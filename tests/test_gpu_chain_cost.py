@@ -27,6 +27,8 @@ def coordinates(sizes, dims, rng):
 
 
 def sizes_of(what, rng):
+    if what == "forties":                                  # with long fibres: a million leaves in short slices
+        return np.full(26_000, 40)
     if what == "ones":                                     # every slice one leaf: chunks end in the cost behind a leaf
         return np.ones(60_000, np.int64)
     if what == "giant in front":                           # one slice over hundreds of warps, then a tail of short ones
@@ -36,6 +38,11 @@ def sizes_of(what, rng):
         return (n / 6 * np.arange(1, k + 1) ** -1.1).astype(np.int64) + rng.integers(1, 40, k)
     z = (180_000 * np.arange(1, 24_001) ** -1.1).astype(np.int64) + 1
     return np.concatenate([z[:1], rng.permutation(z[1:])])
+
+
+@pytest.mark.parametrize("ranks", [(8, 16), (16, 16)])
+def test_short_slices_of_long_fibres(ranks):
+    test_slices_of_all_sizes("long fibres", 3, ranks, cb.F32, "forties")
 
 
 @pytest.mark.parametrize("what", ["ones", "giant in front", "zipf", "short chunks", "short chunks, more of them"])
