@@ -69,7 +69,9 @@ typedef struct { const char *name; const const_csf_t *csf; const void *dense_dev
  *              pos[0] = {0, n_0};
  *   vals[n]    value of leaf n (bit pattern untouched; explicit zeros are kept).
  * The coordinate tuple is packed into one 64-bit key (sum of ceil(log2 extent) over modes must be
- * <= 64), radix-sorted with its value, then each level is compressed with a flag/scan/scatter pass.
+ * <= 64), sorted with its value (by radix passes, tensors from some 200 000 to 110 M nonzeros by sampled splitters), then each level
+ * is compressed.  Temporaries come from the library's pool, which keeps them for later calls: about 20 bytes per nonzero (fp64: 24) for
+ * the radix sort, 48 (64) for the splitter sort; where those cannot be had, the radix sort runs.
  * The leaf offset of every slice is written here as well; the light / heavy / giant work lists are
  * built on the device when something first needs them (the tensor-core stage, const_csf_bin_counts,
  * const_csf_work_lists).

@@ -24,13 +24,14 @@ namespace {
 // Measured on 77 M nonzeros of Zipf slices (43-bit keys, fp32) unless it says otherwise, us for the kernel named.
 // A tile of 2048 (4096: split_buckets 1573 against 1094).
 constexpr int kThreads = 256, kItems = 8, kTile = kThreads * kItems;
-// blocks of split_tile resident per SM: three of 80 registers for the first level, which keeps coordinates (four: 907 against 822), four of 64 for
-// the second (three: 733 against 680)
+// Blocks of split_tile resident per SM: three of 80 registers for the first level, which keeps coordinates (four: 907 against 822, two: 894
+// against 821; fp64 uniform, two: 814 against 757; order 4, which spills a few registers at three, 30 M, two against three: fp32 316 / 305,
+// fp64 361 / 361), four of 64 for the second (three: 733 against 680).
 constexpr int tile_blocks(bool first) { return first ? 3 : 4; }
 constexpr int kWide = 512;                         // threads of the blocks that sort up to kPartRoom numbers, kItems each
 constexpr int kChunk = 4096;                       // elements of a bucket's chunk, at least a tile: a run spans two at most
-// Parts of 1365 on average: one in a hundred is larger than the 2048 of an ordinary block, and one that outgrows its room of
-// three times the average is to be expected once in some hundred builds of 77 M with kOverParts samples a part.
+// Parts of 1365 on average: with kOverParts samples a part, one in seventy is larger than the 2048 of an ordinary block, and one in
+// 10^10 outgrows its room of three times the average.
 constexpr int kPartRoom = kWide * kItems, kPartMean = 1365;
 constexpr int kSampleThreads = 1024;               // of the block that sorts a bucket's sample
 // Two levels of ways about alike: 256 buckets of up to 512 parts (both levels together 1645; 512 of 256: 1720; 128 of 512: 1665).
@@ -197,9 +198,9 @@ __device__ __forceinline__ uint32_t take_chunk(const Tables &t, uint32_t b, uint
 // Deals tiles to their buckets (ORDER > 0: packs the coordinates first) or a chunk of a bucket to the bucket's parts (ORDER 0),
 // appending each run to its target.  A block goes over several tiles, with the tables loaded once; the loads of the next tile are
 // under way while the present one is written out.
-// What bounds it: the shared-memory pipe (some 45 wavefronts per 32 nonzeros: cells and splitters, counters, the reorder) and, between
-// the phases of a tile, too few loads under way.  77 M: 822 us and 680 us for the two levels, 2.6 and 2.7 TB/s; a radix pass over the same
-// data takes 560.
+// What bounds it: the shared-memory pipe (52 and 40 wavefronts per 32 nonzeros in the two levels: cells and splitters, counters, the
+// reorder; it is 72 and 79 % busy) and, between the phases of a tile, too few loads under way.  77 M: 821 us and 691 us for the two
+// levels, 2.6 and 2.7 TB/s (uniform: 662 and 687); a radix pass over the same data takes 560.
 template <typename V, int ORDER>
 __global__ void __launch_bounds__(kThreads, tile_blocks(ORDER > 0)) split_tile(PackArgs a, Tables t, const uint64_t *kin,
                                                                  const V *vin, uint64_t *kout, V *vout,
@@ -766,8 +767,9 @@ __device__ __forceinline__ void sort_part(unsigned char *smem, const Tables &t, 
 // kernels before left: the wide launch, having waited for part_jobs, releases the number of parts, and a block that acquires it sees all
 // that the releasing thread could see.  A block that does not find it waits like any other, and so does the last one, so
 // that the narrow launch ends after the wide one (builds, us, this against all blocks waiting: 77 M 2600 / 2626, 5 M 241 / 251, 1 M of Zipf
-// slices 124 / 137).  What bounds it: instruction issue (230 thread instructions per nonzero, a
-// third of them in the search through the bins) at 30 warps per SM.  77 M: 914 us; 5 M uniform: 62 us.
+// slices 124 / 137).  What bounds it: instruction issue (250 thread instructions per
+// nonzero), 66 % busy at 30 warps per SM.  77 M: 835 us beside 47 of the wide launch (uniform: 857);
+// 5 M uniform: 70.
 template <typename V, int ORDER, int NT>
 __global__ void __launch_bounds__(NT, 1024 / NT) part_sort(Tables t, LevelShifts ls, int leaf_bits, const uint64_t *keys,
                                                           const V *vals, V *vals_out, int32_t *leaf_crd,
@@ -931,9 +933,11 @@ __global__ void __launch_bounds__(kNodeThreads) part_nodes(const PartInfo *__res
 // ------------------------------------------------------------------------------------------------
 // The splitter sort has nine launches and two samplings where the radix sort has two and one per pass: it takes tensors of
 // at least 200 000 nonzeros whose count, times the passes beyond two, is 700 000 or more.  Both sides around the line (build, us,
-// radix / splitters, uniform; Zipf-sized slices cost the splitters some 10 us more): 200 K nonzeros and five passes 97 / 88, four 84 / 89;
-// 300 K and four 96 / 92, three 93 / 91; 500 K and three 99 / 93; 700 K and three 105 / 101; 2.5 M and five 221 / 153; at 30 M, with
-// both as they were before they started early, between 0.64 and 0.78 of the time.  Above 110 M a bucket would need more parts than there are ways.
+// radix / splitters; uniform, Zipf-sized slices): five passes, keys of 44 bits, 150 K 102 / 93, 103 / 95, 200 K 112 / 94, 114 / 96, 260 K
+// 114 / 95, 116 / 101; of 41 bits, 150 K 97 / 94, 96 / 92, 200 K 101 / 94, 101 / 93; four passes, 150 K 84 / 86, 82 / 94, 200 K 85 / 89,
+// 86 / 91, 260 K 90 / 92, 91 / 93, 300 K 98 / 90, 98 / 93, 500 K 98 / 93, 98 / 97; three, uniform, 500 K 99 / 93, 700 K 105 / 101.  The
+// line lies where no number of passes loses; five would gain up to 15 % from 150 K on.  Beyond it the splitters take 0.62 to 0.80 of
+// the time from 3 M on, in fp32 and fp64, orders 2 to 4, sorted or not.  Above 110 M a bucket would need more parts than there are ways.
 constexpr int64_t kSplitMin = 200000, kSplitWork = 700000, kSplitMax = 110000000;
 
 int bucket_count(int64_t nnz) {
