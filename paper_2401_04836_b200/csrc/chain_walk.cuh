@@ -481,7 +481,9 @@ inline int32_t chunk_leaves(int64_t nnz, int64_t slices, int64_t most, int fit, 
 // result is handed over: with Zipf-sized slices the warps that got the many short ones took several times as long as the
 // others.  Equal leaves against this, us: slices Zipf 1.1, TTMc 8 x 8, 1.5 M leaves in slices of 40: 219 / 77, 6 M of 400: 162 /
 // 106, 20 M of 333: 453 / 334; 32 x 32: 256 / 149, 406 / 353, 1124 / 954; order 4: 387 / 129, 407 / 301, 1080 / 853; MTTKRP rank 32: 119 / 56,
-// 122 / 103, 382 / 288; slices of equal size: within 1 % from 6 M on.  Not where slices are long anyway, 3000 leaves (from 4000 leaves on it gained
+// 122 / 103, 382 / 288; slices of equal size: within 1 % from 6 M on, below that 0.88 to 0.99 of the time
+// by family, but up to a tenth slower where equal leaves are just whole windows (8 x 32, 300 000 leaves in slices of 400: 17.6 / 19.3; Zipf
+// 1.1: 25.4 / 23.3) and in very short slices (order-4 MTTKRP, 50 000 in slices of five: 17.5 / 20.7; 300 000: 0.8 of the time).  Not where slices are long anyway, 3000 leaves (from 4000 leaves on it gained
 // 1 to 3 % under Zipf 1.1 and lost 1 to 2 % on equal ones), nor where a chunk would cost less than `least`, which is no less than
 // `weight` (a warp may end up without leaves, a block may not).  Short chunks, equal leaves against this, us: 10 x 12, 200 000 leaves in
 // slices of 143, equal / Zipf 1.1: 25.9 / 28.6 against 21.3 / 19.8; fp64 18 x 23, 40 000 of 133: 35.2 / 33.9 against 24.9 / 23.6; order 4, TTMc,
