@@ -66,6 +66,14 @@ def test_every_mode_order_against_the_radix_sort(dims, nnz):
         assert_same(op, order)
 
 
+def test_scan_over_many_blocks():
+    """Above 4096 blocks of the count kernel (8.4 M nonzeros) the radix path scans them with kernels of their own."""
+    dims = (3001, 2503, 4007)
+    key = np.unique(np.random.default_rng(9).integers(0, int(np.prod(dims, dtype=np.int64)), 9_000_000))
+    assert key.size > 4096 * 2048
+    assert_same(operand(key, dims), (1, 0, 2))
+
+
 @pytest.mark.parametrize("what", ["sorted", "reversed", "banded", "clusters", "one slice"])
 def test_distributions(what):
     """Sorted input (all lanes one way), keys crowded into a part of their range (bins of bins, then the network), a giant slice."""
